@@ -15,7 +15,7 @@ namespace {
 
 enum WsSlot {
     kWsNv = 0, kWsOut, kWsPcap, kWsS32, kWsS64, kWsScap, kWsPartial, kWsMisc,
-    kWsP32, kWsP64, kWsAdjPartial, kWsSamples, kWsShell, kWsFar, kWsLoops, kWsQueue, kWsConeMeta, kWsCut, kWsFlat, kWsClF, kWsAlm, kWsPF2, kWsSort, kWsMid, kWsFar64, kWsCount
+    kWsP32, kWsP64, kWsAdjPartial, kWsSamples, kWsShell, kWsFar, kWsLoops, kWsQueue, kWsConeMeta, kWsCut, kWsFlat, kWsClF, kWsAlm, kWsPF2, kWsSort, kWsMid, kWsFar64, kWsTree, kWsCount
 };
 static_assert(kWsCount <= kMaxWorkspaces, "isw_ctx holds kMaxWorkspaces workspace slots");
 
@@ -192,6 +192,60 @@ void timing_end(isw_ctx *c, int k, cudaStream_t s)
     c->n_timed = k + 1;
 }
 
+// Whether a map runs over the cluster tree (a variant or a chunk count set by the caller asks for the
+// direct kernels).
+bool use_tree(const isw_ctx *c, int64_t nside, int64_t npix, int64_t n, int prec, bool full_sky)
+{
+    return prec == ISW_F32C && full_sky && c->tile_override < 0 && c->split_override == 0 && tree_rule(nside, npix, n);
+}
+
+// isw_map over the cluster tree of a full sky
+int map_tree_impl(isw_ctx *c, int64_t nside, const double *samples, int64_t n, int64_t ld, const double xo[3], double GU,
+                  int prec, int accumulate, double *theta, cudaStream_t s)
+{
+    const TreePlan p = tree_plan(prec, nside, 12, n, c->num_sms);
+    const int64_t tot = p.ncl[0] * p.leaf * p.leaf;
+    int r;
+    if ((r = ensure_ws(c, kWsNv, (size_t)tot * 3 * sizeof(double)))) return r;
+    if ((r = ensure_ws(c, kWsOut, (size_t)tot * sizeof(int64_t)))) return r;
+    if ((r = ensure_ws(c, kWsS32, (size_t)p.n_pad * sizeof(Seg32)))) return r;
+    if ((r = ensure_ws(c, kWsS64, (size_t)p.n_pad * sizeof(Seg64)))) return r;
+    if ((r = ensure_ws(c, kWsSort, sort_scratch_bytes(n, 2)))) return r;
+    if ((r = ensure_ws(c, kWsTree, p.bytes))) return r;
+    TreeMapArgs m{};
+    m.theta_pix = std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
+    double *nv = (double *)c->ws[kWsNv];
+    int64_t *outidx = (int64_t *)c->ws[kWsOut];
+    Seg32 *s32 = (Seg32 *)c->ws[kWsS32];
+    Seg64 *s64 = (Seg64 *)c->ws[kWsS64];
+    launch_pixel_table(nside, 0, 0, 12 * nside * nside, nullptr, p.leaf, p.leaf, p.ncl[0], nv, tot, outidx,
+                       nullptr, c->d_status, s);
+    const uint32_t *perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], c->ws[kWsSort], 2, s);
+    launch_pack(samples, n, ld, xo[0], xo[1], xo[2], GU, m.theta_pix, c->near_k, p.n_pad, perm, s32, s64, nullptr, nullptr,
+                nullptr, c->d_status, s);
+    c->n_launch += spatial_order_launches() + 2;
+    m.nv = nv;
+    m.ldn = tot;
+    m.outidx = outidx;
+    m.diag = 1;
+    m.s32 = s32;
+    m.s64 = s64;
+    m.perm = perm;
+    m.n = n;
+    m.b_min = (float)c->b_min;
+    m.theta = theta;
+    m.accumulate = accumulate;
+    m.st = c->d_status;
+    m.scratch = c->ws[kWsTree];
+    const int ti = timing_begin(c, s);
+    cudaError_t e = launch_map_tree(p, m, s);
+    if (e != cudaSuccess) return cuda_err(c, e, "isw_map launch");
+    c->n_launch += tree_launches(p);
+    c->n_pair += 1;
+    timing_end(c, ti, s);
+    return check_launch(c, "isw_map launch");
+}
+
 // Shared body of isw_map: pixel table, sample records, caps, map kernel, partial reduce.
 int map_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_t *pix_list, const double *samples,
              int64_t n, int64_t ld, const double *x_obs, double GU, int prec, int accumulate, double *theta,
@@ -206,6 +260,8 @@ int map_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_
         }
         return ISW_OK;
     }
+    if (tune_waves == 0 && !patch && use_tree(c, nside, npix, n, prec, !pix_list && pix0 == 0 && npix == 12 * nside * nside))
+        return map_tree_impl(c, nside, samples, n, ld, xo, GU, prec, accumulate, theta, s);
     int vidx = 0;
     if (prec == ISW_F32C) {
         if (c->tile_override >= 0 && c->tile_override < num_f32_variants()) vidx = c->tile_override;
@@ -236,7 +292,7 @@ int map_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_
     if (prec == ISW_F64 && (r = ensure_ws(c, kWsFar64, (size_t)n_pad * sizeof(Far64)))) return r;
     if (split > 1 && (r = ensure_ws(c, kWsPartial, (size_t)split * pp.tot * sizeof(double)))) return r;
     if ((r = ensure_ws(c, kWsQueue, 2 * sizeof(unsigned long long)))) return r;
-    if (prec == ISW_F32C && (r = ensure_ws(c, kWsSort, sort_scratch_bytes(n)))) return r;
+    if (prec == ISW_F32C && (r = ensure_ws(c, kWsSort, sort_scratch_bytes(n, 1)))) return r;
 
     const double theta_pix = patch ? patch->width / (double)patch->M
                                    : std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
@@ -256,7 +312,7 @@ int map_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_
     // FP32 path: records in the spatial order of the samples (tight segment-tile caps)
     const uint32_t *perm = nullptr;
     if (prec == ISW_F32C) {
-        perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], c->ws[kWsSort], s);
+        perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], c->ws[kWsSort], 1, s);
         c->n_launch += spatial_order_launches();
     }
     launch_pack(samples, n, ld, xo[0], xo[1], xo[2], GU, theta_pix, c->near_k, n_pad, perm, s32, s64, far, mid,
@@ -1022,6 +1078,7 @@ int isw_map_batched(isw_ctx *c, int64_t nside, const double *nodes, int64_t ld, 
 
     // autotuner: time every FP32 variant on a prefix of the samples, keep the fastest
     if ((flags & ISW_AUTOTUNE) && prec == ISW_F32C && n > 0 && c->tile_override < 0 &&
+        !use_tree(c, nside, npix, n, prec, true) &&
         !(c->tuned_nside == nside && c->tuned_n == n)) {
         if (!skip_lc) {
             launch_lightcone_shells(nodes, n, ld, d_off, nshell, d_tbox, d_mode, loop_params, nloops, ldp, xo[0],

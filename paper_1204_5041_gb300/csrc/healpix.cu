@@ -203,7 +203,7 @@ void launch_pixel_table(int64_t N, int mode, int64_t pix0, int64_t npix, const i
     if (blocks > 152 * 64) blocks = 152 * 64;
     k_pixel_table<<<(unsigned)blocks, threads, 0, s>>>(N, mode, pix0, npix, pix_list, tx, ty, ntiles, nv, ldn, outidx,
                                                        st);
-    k_pixel_caps<<<(unsigned)ntiles, 256, 0, s>>>(nv, ldn, outidx, tx * ty, caps);
+    if (caps) k_pixel_caps<<<(unsigned)ntiles, 256, 0, s>>>(nv, ldn, outidx, tx * ty, caps);
 }
 
 }  // namespace isw

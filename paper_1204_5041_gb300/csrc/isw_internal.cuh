@@ -418,6 +418,8 @@ __device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b)
     return d;
 }
 
+__device__ __forceinline__ uint64_t f2_neg(uint64_t a) { return a ^ 0x8000000080000000ull; }
+
 struct __align__(16) Seg64 {
     double xh[3], xl[3], xd[3], xp[3], c, om, X, cu;   // X = |X_s - x_obs|
 };

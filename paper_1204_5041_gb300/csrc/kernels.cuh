@@ -82,10 +82,11 @@ void launch_cone_cut(const double *S, int64_t ld, int64_t n, const int64_t *off,
                      int64_t *count, cudaStream_t s);
 
 // sort.cu: spatial order of the samples (stable radix sort of the Morton code of Xhat); returns the
-// device array perm[n] (record s holds sample perm[s]), inside scratch of sort_scratch_bytes(n)
-size_t sort_scratch_bytes(int64_t n);
+// device array perm[n] (record s holds sample perm[s]), inside scratch of sort_scratch_bytes(n, orders).
+// With orders = 2 perm[n + k] is the k-th sample in the Morton order of Xdot.
+size_t sort_scratch_bytes(int64_t n, int orders);
 const uint32_t *launch_spatial_order(const double *S, int64_t n, int64_t ld, double xo0, double xo1, double xo2,
-                                     void *scratch, cudaStream_t s);
+                                     void *scratch, int orders, cudaStream_t s);
 int spatial_order_launches();
 
 // pack.cu: per-sample records of the map kernels and per-tile caps
@@ -138,6 +139,49 @@ void launch_map_f32c(int idx, const MapArgs &a, int grid, cudaStream_t s);
 void launch_map_f32c_near(int idx, const MapArgs &a, int num_sms, cudaStream_t s);
 void launch_map_f64(const MapArgs &a, int grid, cudaStream_t s);
 void launch_reduce_partials(const MapArgs &a, int tile_sz, cudaStream_t s);
+
+// tree.cu: the map over a cluster tree of the pixels
+constexpr int kTreeLevels = 20;
+constexpr int64_t kTreeMinSide = 32;
+constexpr double kTreeMinPairs = 1e8;
+// Whether a full-sky FP32 map of default settings runs over the tree: from 1e8 pairs, where its dozen
+// extra launches (0.15 ms) are made up for (N_side 64 with 10,240 samples, 5e8 pairs: 0.6 against 2.5
+// ms).  The list entries hold 30-bit record numbers.
+inline bool tree_rule(int64_t nside, int64_t npix, int64_t n)
+{
+    return nside >= kTreeMinSide && npix == 12 * nside * nside && (double)npix * (double)n >= kTreeMinPairs &&
+           n < (int64_t(1) << 30);
+}
+struct TreePlan {
+    int leaf, nn, nface, levels;          // leaf side in pixels, nodes per cluster
+    int nb[kTreeLevels];                  // clusters per face side, from the finest level
+    int64_t ncl[kTreeLevels];             // clusters of the level
+    int64_t n_pad, nst;                   // padded samples, sample tiles
+    int nslots, pslots;                   // resident CTAs of the node and pixel kernels
+    int pool, ppool;                      // chunk pool entries of a level and of the pixels
+    size_t off_queue, off_crit, off_vcrit, off_caps, off_sup, off_vidx, off_inv, off_rec, off_work, off_pool, off_partial;
+    size_t off_geo[kTreeLevels], off_F[kTreeLevels], bytes;   // scratch layout
+};
+struct TreeMapArgs {
+    const double *nv;         // pixel table: leaf x leaf slots per finest cluster, clusters in (face, y, x) order
+    int64_t ldn;
+    const int64_t *outidx;
+    int diag;                 // slots in anti-diagonal order (full sky) or row by row (patch)
+    double theta_pix;
+    const Seg32 *s32;
+    const Seg64 *s64;
+    const uint32_t *perm;     // sample of each record, and of each velocity-order entry (perm + n)
+    int64_t n;
+    float b_min;
+    double *theta;
+    int accumulate;
+    DevStatus *st;
+    void *scratch;            // TreePlan::bytes
+};
+int tree_leaf(int prec);
+TreePlan tree_plan(int prec, int64_t N, int nface, int64_t n, int num_sms);
+cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_t s);
+inline int tree_launches(const TreePlan &p) { return 2 * p.levels + 7; }
 
 // adjoint.cu
 struct AdjArgs {

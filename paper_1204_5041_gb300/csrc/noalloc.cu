@@ -12,8 +12,9 @@
 // share it and it keeps the previous call's contents: each call clears the status word and
 // overwrites every other byte it reads, and two calls that overlap on the GPU (different
 // streams, no ordering between them) race on it and give wrong maps.  The launch sequence,
-// kernel variant and segment-chunk rule are those of isw_map with default settings (the chunk
-// count is capped by the scratch left), so within that cap the map equals isw_map's bit for bit.
+// kernels and the rules that choose them are those of isw_map with default settings, so the map equals
+// isw_map's bit for bit as long as the same kernels fit: the cluster tree of larger full-sky maps
+// (tree.cu), else the direct kernels with their chunk count capped by the scratch left.
 // A caller that passes status_out gets the status the kernels recorded (skipped samples, a
 // bounded wait that ran out), read back after a stream synchronisation.
 #include <cmath>
@@ -81,6 +82,64 @@ int scratch_address(int dev, void **addr, int *sms)
     return ISW_OK;
 }
 
+// After the launches: the status that the kernels recorded in the first word of the scratch, read back
+// when the caller asked for it (waits for them; no allocation).
+int finish(void *base, int32_t *status_out, cudaStream_t s)
+{
+    if (cudaGetLastError() != cudaSuccess) return ISW_ECUDA;
+    if (status_out) {
+        DevStatus h;
+        if (cudaMemcpyAsync(&h, base, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess) {
+            cudaGetLastError();
+            return ISW_ECUDA;
+        }
+        *status_out = status_code(h);
+    }
+    return ISW_OK;
+}
+
+// A full-sky map over the cluster tree, with isw_map's launch sequence; ISW_EINVAL when it does not fit
+// the scratch (the direct kernels, which need less, are then tried).
+int map_tree_noalloc(int64_t nside, const double *samples, int64_t n, int64_t ld, const double *x_obs, double GU,
+                     double *theta, unsigned char *b, int sms, cudaStream_t s)
+{
+    const TreePlan p = tree_plan(ISW_F32C, nside, 12, n, sms);
+    const int64_t tot = p.ncl[0] * p.leaf * p.leaf;
+    size_t at = up256(sizeof(DevStatus));
+    auto take = [&](size_t bytes) {
+        const size_t o = at;
+        at += up256(bytes);
+        return o;
+    };
+    const size_t off_nv = take((size_t)tot * 3 * sizeof(double)), off_out = take((size_t)tot * sizeof(int64_t));
+    const size_t off_s32 = take((size_t)p.n_pad * sizeof(Seg32)), off_s64 = take((size_t)p.n_pad * sizeof(Seg64));
+    const size_t off_sort = take(sort_scratch_bytes(n, 2)), off_tree = take(p.bytes);
+    if (at > kStaticScratchBytes) return ISW_EINVAL;
+    DevStatus *st = (DevStatus *)b;
+    if (cudaMemsetAsync(st, 0, sizeof(DevStatus), s) != cudaSuccess) return ISW_ECUDA;
+    const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
+    TreeMapArgs m{};
+    m.theta_pix = std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
+    launch_pixel_table(nside, 0, 0, 12 * nside * nside, nullptr, p.leaf, p.leaf, p.ncl[0], (double *)(b + off_nv), tot,
+                       (int64_t *)(b + off_out), nullptr, st, s);
+    m.perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], b + off_sort, 2, s);
+    m.nv = (const double *)(b + off_nv);
+    m.ldn = tot;
+    m.outidx = (const int64_t *)(b + off_out);
+    m.diag = 1;
+    m.s32 = (const Seg32 *)(b + off_s32);
+    m.s64 = (const Seg64 *)(b + off_s64);
+    launch_pack(samples, n, ld, xo[0], xo[1], xo[2], GU, m.theta_pix, kNearK, p.n_pad, m.perm, (Seg32 *)(b + off_s32),
+                (Seg64 *)(b + off_s64), nullptr, nullptr, nullptr, st, s);
+    m.n = n;
+    m.b_min = (float)kBMin;
+    m.theta = theta;
+    m.st = st;
+    m.scratch = b + off_tree;
+    return launch_map_tree(p, m, s) == cudaSuccess ? ISW_OK : ISW_ECUDA;
+}
+
 }  // namespace
 
 extern "C" int isw_map_f32c_noalloc(int64_t nside, int64_t pix0, int64_t npix, const double *samples, int64_t n,
@@ -104,6 +163,15 @@ extern "C" int isw_map_f32c_noalloc(int64_t nside, int64_t pix0, int64_t npix, c
     if (n == 0) return cudaMemsetAsync(theta_out, 0, (size_t)npix * sizeof(double), s) == cudaSuccess ? ISW_OK
                                                                                                          : ISW_ECUDA;
 
+    void *base = nullptr;
+    int sms = 0;
+    int r = scratch_address(dev, &base, &sms);
+    if (r) return r;
+    if (pix0 == 0 && tree_rule(nside, npix, n)) {   // the cluster tree, as isw_map, when it fits
+        r = map_tree_noalloc(nside, samples, n, ld, x_obs, GU, theta_out, (unsigned char *)base, sms, s);
+        if (r != ISW_EINVAL) return r == ISW_OK ? finish(base, status_out, s) : r;
+    }
+
     // ---- scratch layout for the FP32 pair kernel's first variant (the one isw_map uses by default)
     const Variant v = f32_variant(0);
     const int S = v.seg_tile, tile = v.tx * v.ty;
@@ -124,16 +192,11 @@ extern "C" int isw_map_f32c_noalloc(int64_t nside, int64_t pix0, int64_t npix, c
     off[6] = at; at += up256((size_t)nst * sizeof(SegCap));
     const size_t off_far = at; at += up256((size_t)(n_pad / 2) * sizeof(Far2));
     const size_t off_mid = at; at += up256((size_t)n_pad * sizeof(Mid2));
-    const size_t off_sort = at; at += up256(sort_scratch_bytes(n));
+    const size_t off_sort = at; at += up256(sort_scratch_bytes(n, 1));
     off[7] = at;
     if (at > kStaticScratchBytes) return ISW_EINVAL;  // problem too large for the static scratch
     // segment-chunk partials fit for at most `room` chunks
     const int64_t room = (int64_t)((kStaticScratchBytes - at) / ((size_t)tot * sizeof(double)));
-
-    void *base = nullptr;
-    int sms = 0;
-    int r = scratch_address(dev, &base, &sms);
-    if (r) return r;
 
     // segment chunks: the rule isw_map uses, capped by the scratch left
     const int slots = map_f32c_slots(0, sms);
@@ -157,7 +220,7 @@ extern "C" int isw_map_f32c_noalloc(int64_t nside, int64_t pix0, int64_t npix, c
     const double theta_pix = std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
     launch_pixel_table(nside, full ? 0 : 1, pix0, npix, nullptr, v.tx, v.ty, ntiles, nv, tot, outidx, pcaps, st, s);
     Far2 *far = (Far2 *)(b + off_far);
-    const uint32_t *perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], b + off_sort, s);
+    const uint32_t *perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], b + off_sort, 1, s);
     Mid2 *mid = (Mid2 *)(b + off_mid);
     launch_pack(samples, n, ld, xo[0], xo[1], xo[2], GU, theta_pix, kNearK, n_pad, perm, s32, s64, far, mid, nullptr, st,
                 s);
@@ -189,16 +252,5 @@ extern "C" int isw_map_f32c_noalloc(int64_t nside, int64_t pix0, int64_t npix, c
     launch_map_f32c(0, a, (int)(items < slots ? items : slots), s);
     launch_map_f32c_near(0, a, sms, s);
     if (split > 1) launch_reduce_partials(a, tile, s);
-    if (cudaGetLastError() != cudaSuccess) return ISW_ECUDA;
-    if (status_out) {
-        // what the kernels recorded: wait for them, then read the status word (no allocation)
-        DevStatus h;
-        if (cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) {
-            cudaGetLastError();
-            return ISW_ECUDA;
-        }
-        *status_out = status_code(h);
-    }
-    return ISW_OK;
+    return finish(base, status_out, s);
 }

@@ -37,6 +37,27 @@ __device__ __forceinline__ double rcp64(double x)
     return fma(r, fma(e, e, e), r);
 }
 
+// pair64 with the third-order reciprocal in the place of the IEEE division (an ulp or two; B and Q
+// are far above the float range's lower end: Q >= 1e-30 for distinct directions, B > 1e-12)
+__device__ __forceinline__ double pair64_fast(double nx, double ny, double nz, const Seg64 &g, unsigned &zero)
+{
+    const double dx = (nx - g.xh[0]) - g.xl[0];
+    const double dy = (ny - g.xh[1]) - g.xl[1];
+    const double dz = (nz - g.xh[2]) - g.xl[2];
+    const double Q = dx * dx + dy * dy + dz * dz;
+    const double A = nx * g.xp[0] + ny * g.xp[1] + nz * g.xp[2];
+    const double B = 1.0 + (nx * g.xd[0] + ny * g.xd[1] + nz * g.xd[2]);
+    const double Pd = g.xd[0] * dx + g.xd[1] * dy + g.xd[2] * dz;
+    const double Qd = g.xp[0] * dx + g.xp[1] * dy + g.xp[2] * dz;
+    const double den = B * Q, num = g.c * (B * Pd - A * Qd);
+    if (fabs(den) > 1e-30 && fabs(den) < 1e30) return num * rcp64(den);
+    if (Q == 0.0) {
+        ++zero;
+        return 0.0;
+    }
+    return num / den;
+}
+
 __device__ __forceinline__ void fold(float &hi, float &lo, float x)
 {
     const float s = hi + x;

@@ -6,10 +6,12 @@
 // the order of a 3-D Morton code of the unit vector Xhat quantised to 8 bits per axis.  The sort
 // is a stable least-significant-digit radix sort of (key, index) in three passes of 8 bits, so
 // the order, and with it the rounding of the map's sums, is reproducible.
-//   k_sort_keys     key = Morton code of Xhat (invalid samples last), index = input position
+// The cluster-tree maps need a second order of the same samples, by the Morton code of Xdot (tree.cuh);
+// both are sorted by the same launches (blockIdx.y).
+//   k_sort_keys     keys (invalid samples last), index = input position
 //   k_sort_hist     per block of 1024 elements, the 256-bin histogram of the pass's digit
-//   k_sort_scan     exclusive scan of the histograms in (digit, block) order: each block's first
-//                   output position for each digit
+//   k_sort_scan     one block per digit: exclusive scan of the digit's counts over the blocks, and the
+//                   digit's total (one block for all digits took 42 us a pass at 2e5 samples, now 3)
 //   k_sort_scatter  the block's elements in input order, ranked within their digit by a warp
 //                   match and per-warp counts, written to their positions (stable)
 #include "isw_internal.cuh"
@@ -30,24 +32,33 @@ __device__ __forceinline__ uint32_t spread3(uint32_t x)   // bits b0..b7 -> posi
     return x;
 }
 
+__device__ __forceinline__ uint32_t morton(double x, double y, double z)   // of a point in [-1, 1]^3
+{
+    const double r[3] = {x, y, z};
+    uint32_t q[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double u = floor((r[c] + 1.0) * 128.0);
+        q[c] = (uint32_t)(u < 0.0 ? 0.0 : (u > 255.0 ? 255.0 : u));
+    }
+    return spread3(q[0]) | (spread3(q[1]) << 1) | (spread3(q[2]) << 2);
+}
+
 __global__ void k_sort_keys(const double *__restrict__ S, int64_t n, int64_t ld, double xo0, double xo1, double xo2,
                             uint32_t *__restrict__ key, uint32_t *__restrict__ idx)
 {
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
-        const double r[3] = {S[s] - xo0, S[ld + s] - xo1, S[2 * ld + s] - xo2};
-        const double nrm = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
         uint32_t k = kInvalidKey;
-        if (nrm > 0.0 && isfinite(nrm)) {
-            uint32_t q[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const double u = floor((r[c] / nrm + 1.0) * 128.0);
-                q[c] = (uint32_t)(u < 0.0 ? 0.0 : (u > 255.0 ? 255.0 : u));
-            }
-            k = spread3(q[0]) | (spread3(q[1]) << 1) | (spread3(q[2]) << 2);
+        if (blockIdx.y == 0) {
+            const double r[3] = {S[s] - xo0, S[ld + s] - xo1, S[2 * ld + s] - xo2};
+            const double nrm = sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
+            if (nrm > 0.0 && isfinite(nrm)) k = morton(r[0] / nrm, r[1] / nrm, r[2] / nrm);
+        } else {
+            const double v[3] = {S[3 * ld + s], S[4 * ld + s], S[5 * ld + s]};
+            if (isfinite(v[0] + v[1] + v[2])) k = morton(v[0], v[1], v[2]);
         }
-        key[s] = k;
-        idx[s] = (uint32_t)s;
+        key[blockIdx.y * n + s] = k;
+        idx[blockIdx.y * n + s] = (uint32_t)s;
     }
 }
 
@@ -57,6 +68,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t *__re
     __shared__ uint32_t h[kRadix];
     const int tid = threadIdx.x;
     const int64_t b = blockIdx.x;
+    key += blockIdx.y * n;
     h[tid] = 0;
     __syncthreads();
     for (int i = tid; i < kSortBlock; i += kSortThreads) {
@@ -64,46 +76,65 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t *__re
         if (e < n) atomicAdd(&h[(key[e] >> shift) & (kRadix - 1)], 1u);
     }
     __syncthreads();
-    hist[(int64_t)tid * nblocks + b] = h[tid];
+    hist[((int64_t)blockIdx.y * kRadix + tid) * nblocks + b] = h[tid];
 }
 
-// One block of 1024 threads: each thread scans a contiguous run serially, then the run totals
-// are scanned across the block.
-__global__ void __launch_bounds__(1024) k_sort_scan(uint32_t *__restrict__ hist, int64_t total)
+// Inclusive scan over the block's kSortThreads values; wtot is shared scratch of kSortWarps words.
+__device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t *wtot)
 {
-    __shared__ uint32_t part[1024];
-    const int tid = threadIdx.x;
-    const int64_t per = (total + 1023) / 1024;
-    const int64_t a = tid * per, e = a + per < total ? a + per : total;
-    uint32_t s = 0;
-    for (int64_t i = a; i < e; ++i) s += hist[i];
-    part[tid] = s;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wtot[w] = x;
     __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {   // inclusive scan of the run totals
-        const uint32_t v = tid >= o ? part[tid - o] : 0u;
+    for (int i = 0; i < w; ++i) x += wtot[i];
+    __syncthreads();
+    return x;
+}
+
+// Row blockIdx.x (one digit) of array blockIdx.y: exclusive scan in place, total to tot.
+__global__ void __launch_bounds__(kSortThreads) k_sort_scan(uint32_t *__restrict__ hist, int nblocks,
+                                                            uint32_t *__restrict__ tot)
+{
+    __shared__ uint32_t wtot[kSortWarps];
+    __shared__ uint32_t last;
+    const int tid = threadIdx.x;
+    uint32_t *row = hist + ((int64_t)blockIdx.y * kRadix + blockIdx.x) * nblocks;
+    uint32_t carry = 0;
+    for (int b0 = 0; b0 < nblocks; b0 += kSortThreads) {
+        const int b = b0 + tid;
+        const uint32_t v = b < nblocks ? row[b] : 0u;
+        const uint32_t x = block_scan(v, wtot);
+        if (b < nblocks) row[b] = carry + x - v;
+        if (tid == kSortThreads - 1) last = x;
         __syncthreads();
-        part[tid] += v;
+        carry += last;
         __syncthreads();
     }
-    uint32_t run = tid > 0 ? part[tid - 1] : 0u;
-    for (int64_t i = a; i < e; ++i) {
-        const uint32_t h = hist[i];
-        hist[i] = run;
-        run += h;
-    }
+    if (tid == 0) tot[blockIdx.y * kRadix + blockIdx.x] = carry;
 }
 
 __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const uint32_t *__restrict__ key_in,
                                                                const uint32_t *__restrict__ idx_in, int64_t n,
                                                                int shift, const uint32_t *__restrict__ offs,
-                                                               int nblocks, uint32_t *__restrict__ key_out,
+                                                               const uint32_t *__restrict__ tot, int nblocks,
+                                                               uint32_t *__restrict__ key_out,
                                                                uint32_t *__restrict__ idx_out)
 {
+    __shared__ uint32_t wtot[kSortWarps];
     __shared__ uint32_t base[kRadix];                // next output position of each digit
     __shared__ uint32_t wcnt[kSortWarps][kRadix];    // elements of each digit per warp, this round
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int64_t b = blockIdx.x;
-    base[tid] = offs[(int64_t)tid * nblocks + b];
+    key_in += blockIdx.y * n;
+    idx_in += blockIdx.y * n;
+    key_out += blockIdx.y * n;
+    idx_out += blockIdx.y * n;
+    const uint32_t all = tot[blockIdx.y * kRadix + tid];
+    base[tid] = block_scan(all, wtot) - all + offs[((int64_t)blockIdx.y * kRadix + tid) * nblocks + b];
     for (int r = 0; r < kSortBlock / kSortThreads; ++r) {
 #pragma unroll
         for (int w = 0; w < kSortWarps; ++w) wcnt[w][tid] = 0u;
@@ -132,29 +163,30 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const uint32_t *_
 }
 }  // namespace
 
-size_t sort_scratch_bytes(int64_t n)
+size_t sort_scratch_bytes(int64_t n, int orders)
 {
     const int64_t nblocks = (n + kSortBlock - 1) / kSortBlock;
-    return (size_t)4 * n * sizeof(uint32_t) + (size_t)kRadix * nblocks * sizeof(uint32_t) + 4 * 256;
+    return (size_t)orders * ((size_t)4 * n + (size_t)kRadix * (nblocks + 1)) * sizeof(uint32_t) + 4 * 256;
 }
 
 const uint32_t *launch_spatial_order(const double *S, int64_t n, int64_t ld, double xo0, double xo1, double xo2,
-                                     void *scratch, cudaStream_t s)
+                                     void *scratch, int orders, cudaStream_t s)
 {
     if (n <= 0) return nullptr;
-    const int64_t nblocks = (n + kSortBlock - 1) / kSortBlock;
+    const int64_t nblocks = (n + kSortBlock - 1) / kSortBlock, m = orders * n;
     uint32_t *p = reinterpret_cast<uint32_t *>(scratch);
-    uint32_t *key[2] = {p, p + n}, *idx[2] = {p + 2 * n, p + 3 * n};
-    uint32_t *hist = p + 4 * n;
+    uint32_t *key[2] = {p, p + m}, *idx[2] = {p + 2 * m, p + 3 * m};
+    uint32_t *hist = p + 4 * m, *tot = hist + (int64_t)orders * kRadix * nblocks;
     int64_t kb = (n + 255) / 256;
     if (kb > 152 * 32) kb = 152 * 32;
-    k_sort_keys<<<(unsigned)kb, 256, 0, s>>>(S, n, ld, xo0, xo1, xo2, key[0], idx[0]);
+    k_sort_keys<<<dim3((unsigned)kb, orders), 256, 0, s>>>(S, n, ld, xo0, xo1, xo2, key[0], idx[0]);
     int cur = 0;
+    const dim3 grid((unsigned)nblocks, orders);
     for (int shift = 0; shift < 24; shift += 8) {
-        k_sort_hist<<<(unsigned)nblocks, kSortThreads, 0, s>>>(key[cur], n, shift, hist, (int)nblocks);
-        k_sort_scan<<<1, 1024, 0, s>>>(hist, (int64_t)kRadix * nblocks);
-        k_sort_scatter<<<(unsigned)nblocks, kSortThreads, 0, s>>>(key[cur], idx[cur], n, shift, hist, (int)nblocks,
-                                                                    key[cur ^ 1], idx[cur ^ 1]);
+        k_sort_hist<<<grid, kSortThreads, 0, s>>>(key[cur], n, shift, hist, (int)nblocks);
+        k_sort_scan<<<dim3(kRadix, orders), kSortThreads, 0, s>>>(hist, (int)nblocks, tot);
+        k_sort_scatter<<<grid, kSortThreads, 0, s>>>(key[cur], idx[cur], n, shift, hist, tot, (int)nblocks, key[cur ^ 1],
+                                                     idx[cur ^ 1]);
         cur ^= 1;
     }
     return idx[cur];

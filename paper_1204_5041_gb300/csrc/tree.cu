@@ -1,0 +1,1120 @@
+// The map of Eq. (1)-(2) over a cluster tree of the pixels (tree.cuh says which pairs are summed
+// where and why the result is the all-pairs sum to the working precision).
+//
+//   k_tree_crit      per sample and per tile of 64 samples, what the near/far decision reads
+//   k_tree_leaf_geo  finest clusters (T x T pixel blocks): centre, frame, extent, near radius
+//   k_tree_up_geo    parents (2 x 2 children), level by level
+//   k_tree_nodes_*   per level from the coarsest: the level's samples summed at the p^2 nodes of every
+//                    cluster, plus the parent's interpolant at the same nodes
+//   k_tree_pixels_*  per finest cluster: the interpolant at its pixels plus the near samples pixel by
+//                    pixel
+// Sums over chunks of samples go to separate partial arrays, added in a fixed order by the reader, so
+// maps are reproducible.
+//
+// FP32 maps, 8 x 8 nodes, near radius 3.5 half-sizes, leaves of 16 x 16 pixels: N_side 512 with 2e5 samples
+// 309 -> 8.3 ms (6.3e11 pairs; 3e9 pair terms at nodes, 6e8 at pixels), N_side 64 with 10,240 samples
+// 2.5 -> 0.6 ms; error against FP64 2.6e-8 of the rms (direct kernels 6.9e-8), largest 3e-7 (9e-7).  The
+// node kernels are bound by FP32 issue (FMA pipe 40-50%), the pixel kernel by its FP64 near pairs (a
+// quarter of its time) and by the tests that find them.
+#include "tree.cuh"
+
+namespace isw {
+
+namespace {
+
+// Near radius in stereographic half-sizes: 4 gives 2.2e-8 of the rms at N_side 100 and 10.1 ms at N_side 512
+// with 2e5 samples, 3.5 2.6e-8 and 9.2 ms, 3 5.1e-8 and 8.5 ms.
+constexpr double kKappa = 3.5;
+
+__device__ __forceinline__ double near_radius(double a)
+{
+    // chord of stereographic radius kappa a
+    const double z = kKappa * a;
+    return 2.0 * z / sqrt(1.0 + z * z);
+}
+
+__device__ __forceinline__ float warp_sum(float v)
+{
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ float warp_max(float v)
+{
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+// ball around the mean of the lane's two points (w = enlargement, < 0: no point); radius < 0 when empty
+__device__ __forceinline__ TreeCap warp_ball(const float4 (&x)[2])
+{
+    float sx = 0.f, sy = 0.f, sz = 0.f, cnt = 0.f, r = -1.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (x[h].w >= 0.f) {
+            sx += x[h].x;
+            sy += x[h].y;
+            sz += x[h].z;
+            cnt += 1.f;
+        }
+    cnt = fmaxf(warp_sum(cnt), 1.f);
+    sx = warp_sum(sx) / cnt;
+    sy = warp_sum(sy) / cnt;
+    sz = warp_sum(sz) / cnt;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (x[h].w >= 0.f) {
+            const float dx = x[h].x - sx, dy = x[h].y - sy, dz = x[h].z - sz;
+            r = fmaxf(r, sqrtf(dx * dx + dy * dy + dz * dz) * 1.0001f + 1e-6f + x[h].w);
+        }
+    TreeCap c;
+    c.a = make_float4(sx, sy, sz, warp_max(r));
+    return c;
+}
+
+// One warp per tile of 64 records (position order): decision data, evaluation records, caps, and the
+// record of every input sample.
+__global__ void __launch_bounds__(256) k_tree_crit(const Seg32 *__restrict__ s32, const Seg64 *__restrict__ s64,
+                                                   const uint32_t *__restrict__ perm, int64_t n, int64_t ntile,
+                                                   TreeCrit *__restrict__ crit, TreeCap *__restrict__ caps,
+                                                   TreeRec *__restrict__ rec, uint32_t *__restrict__ inv)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (t >= ntile) return;
+    float4 x[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int64_t s = t * kTreeS + 32 * h + lane;
+        TreeCrit cr;
+        cr.a = make_float4(0.f, 0.f, 0.f, 0.f);
+        cr.b = make_float4(0.f, 0.f, 0.f, kCritSkip);
+        x[h] = make_float4(0.f, 0.f, 0.f, -1.f);
+        const Seg32 f = s32[s];
+        if (s < n) {
+            inv[perm[s]] = (uint32_t)s;
+            if (f.b.w >= 0.f) {
+                cr.a = make_float4(f.a.x, f.a.y, f.a.z, sqrtf(f.b.w) * 1.0001f);
+                cr.b = make_float4(-f.k.x, -f.k.y, -f.k.z, (float)s64[s].om);
+                x[h] = cr.a;
+            }
+        }
+        crit[s] = cr;
+        if (rec) {
+            float4 *dst = rec[s].v;
+            dst[0] = f.a;
+            dst[1] = make_float4(f.b.x, f.b.y, f.b.z, f.e.w);
+            dst[2] = make_float4(f.d.x, f.d.y, f.d.z, f.k.w);
+            dst[3] = make_float4(f.e.x, f.e.y, f.e.z, f.b.w);
+        }
+    }
+    const TreeCap c = warp_ball(x);
+    if (lane == 0) caps[t] = c;
+}
+
+// One warp per tile of 64 samples in velocity order.
+__global__ void __launch_bounds__(256) k_tree_vcrit(const TreeCrit *__restrict__ crit, const Seg32 *__restrict__ s32,
+                                                    const uint32_t *__restrict__ vperm,
+                                                    const uint32_t *__restrict__ inv, int64_t n, int64_t ntile,
+                                                    TreeCrit *__restrict__ vcrit, TreeCap *__restrict__ vcaps,
+                                                    uint32_t *__restrict__ vidx)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (t >= ntile) return;
+    float4 x[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int64_t k = t * kTreeS + 32 * h + lane;
+        TreeCrit cr;
+        cr.a = make_float4(0.f, 0.f, 0.f, 0.f);
+        cr.b = make_float4(0.f, 0.f, 0.f, kCritSkip);
+        x[h] = make_float4(0.f, 0.f, 0.f, -1.f);
+        uint32_t r = 0;
+        if (k < n) {
+            r = inv[vperm[k]];
+            cr = crit[r];
+            if (cr.b.w < kCritSkip) {
+                const float4 d = s32[r].d;
+                x[h] = make_float4(d.x, d.y, d.z, 0.f);
+            }
+        }
+        vcrit[k] = cr;
+        vidx[k] = r;
+    }
+    const TreeCap c = warp_ball(x);
+    if (lane == 0) vcaps[t] = c;
+}
+
+// Balls over kTreeSuper tiles, one warp each: around the mean of the tiles' centres.  Position order in
+// blockIdx.y = 0, velocity order in 1 (caps and sup hold both, nst and nsup apart).
+__global__ void __launch_bounds__(128) k_tree_super(const TreeCap *__restrict__ caps, int64_t nst, int64_t nsup,
+                                                    TreeCap *__restrict__ sup)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t u = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (u >= nsup) return;
+    const int64_t t = u * kTreeSuper + lane;
+    float4 a = make_float4(0.f, 0.f, 0.f, -1.f);
+    if (t < nst) a = caps[blockIdx.y * nst + t].a;
+    const float on = a.w >= 0.f ? 1.f : 0.f, cnt = fmaxf(warp_sum(on), 1.f);
+    const float sx = warp_sum(on * a.x) / cnt, sy = warp_sum(on * a.y) / cnt, sz = warp_sum(on * a.z) / cnt;
+    const float dx = a.x - sx, dy = a.y - sy, dz = a.z - sz;
+    const float r = warp_max(on > 0.f ? sqrtf(dx * dx + dy * dy + dz * dz) * 1.0001f + 1e-6f + a.w : -1.f);
+    TreeCap c;
+    c.a = make_float4(sx, sy, sz, r);
+    if (lane == 0) sup[blockIdx.y * nsup + u] = c;
+}
+
+// frame from a centre direction and a rough tangent; extents are filled in by the caller
+__device__ __forceinline__ void make_frame(double cx, double cy, double cz, double tx, double ty, double tz,
+                                           TreeGeo &g)
+{
+    const double r = 1.0 / sqrt(cx * cx + cy * cy + cz * cz);
+    g.n0[0] = cx * r;
+    g.n0[1] = cy * r;
+    g.n0[2] = cz * r;
+    double t = tx * g.n0[0] + ty * g.n0[1] + tz * g.n0[2];
+    double ux = tx - t * g.n0[0], uy = ty - t * g.n0[1], uz = tz - t * g.n0[2];
+    double u2 = ux * ux + uy * uy + uz * uz;
+    if (!(u2 > 1e-12 * (tx * tx + ty * ty + tz * tz)) || !(u2 > 0.0)) {   // no tangent: any will do
+        ux = fabs(g.n0[2]) < 0.9 ? -g.n0[1] : 0.0;
+        uy = fabs(g.n0[2]) < 0.9 ? g.n0[0] : -g.n0[2];
+        uz = fabs(g.n0[2]) < 0.9 ? 0.0 : g.n0[1];
+        u2 = ux * ux + uy * uy + uz * uz;
+    }
+    const double ru = 1.0 / sqrt(u2);
+    g.e1[0] = ux * ru;
+    g.e1[1] = uy * ru;
+    g.e1[2] = uz * ru;
+    // once more against the rounding of the first projection
+    t = g.e1[0] * g.n0[0] + g.e1[1] * g.n0[1] + g.e1[2] * g.n0[2];
+    for (int c = 0; c < 3; ++c) g.e1[c] -= t * g.n0[c];
+    const double rv = 1.0 / sqrt(g.e1[0] * g.e1[0] + g.e1[1] * g.e1[1] + g.e1[2] * g.e1[2]);
+    for (int c = 0; c < 3; ++c) g.e1[c] *= rv;
+    g.e2[0] = g.n0[1] * g.e1[2] - g.n0[2] * g.e1[1];
+    g.e2[1] = g.n0[2] * g.e1[0] - g.n0[0] * g.e1[2];
+    g.e2[2] = g.n0[0] * g.e1[1] - g.n0[1] * g.e1[0];
+}
+
+// the float copies of a finished geometry, with the near radius D
+__device__ __forceinline__ void finish_geo(TreeGeo &g, double D)
+{
+    g.pad = 0.0;
+    g.c = make_float4((float)g.n0[0], (float)g.n0[1], (float)g.n0[2], (float)D);
+    g.l = make_float4((float)(g.n0[0] - (double)g.c.x), (float)(g.n0[1] - (double)g.c.y),
+                      (float)(g.n0[2] - (double)g.c.z), 0.f);
+    g.f1 = make_float4((float)g.e1[0], (float)g.e1[1], (float)g.e1[2], (float)(1.0 / g.a1));
+    g.f2 = make_float4((float)g.e2[0], (float)g.e2[1], (float)g.e2[2], (float)(1.0 / g.a2));
+}
+
+// One CTA of T*T/4 threads per finest cluster.  Sums in float are enough: they only choose the
+// centre and frame, and the extents are measured from the pixels afterwards.
+template <int T>
+__global__ void __launch_bounds__(T *T / 4) k_tree_leaf_geo(const double *__restrict__ nv, int64_t ldn,
+                                                            const int64_t *__restrict__ outidx, int diag,
+                                                            double theta_pix, TreeGeo *__restrict__ geo)
+{
+    constexpr int NT = T * T / 4, W = NT / 32;
+    __shared__ float red[6][W];
+    __shared__ TreeGeo g;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int64_t t = blockIdx.x;
+    float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int l = tid; l < T * T; l += NT) {
+        const int64_t k = t * T * T + l;
+        if (outidx[k] < 0) continue;
+        int lx, ly;
+        if (diag) diag_slot_square(l, T, lx, ly);
+        else lx = l % T;
+        const float f = (float)lx - 0.5f * (float)(T - 1);
+        for (int c = 0; c < 3; ++c) {
+            const float v = (float)nv[c * ldn + k];
+            s[c] += v;
+            s[3 + c] += f * v;
+        }
+    }
+    for (int c = 0; c < 6; ++c) {
+        for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
+        if (lane == 0) red[c][w] = s[c];
+    }
+    __syncthreads();
+    if (tid == 0) {
+        double a[6];
+        for (int c = 0; c < 6; ++c) {
+            a[c] = 0.0;
+            for (int i = 0; i < W; ++i) a[c] += red[c][i];
+        }
+        make_frame(a[0], a[1], a[2], a[3], a[4], a[5], g);
+    }
+    __syncthreads();
+    const float e1x = (float)g.e1[0], e1y = (float)g.e1[1], e1z = (float)g.e1[2];
+    const float e2x = (float)g.e2[0], e2y = (float)g.e2[1], e2z = (float)g.e2[2];
+    float m1 = 0.f, m2 = 0.f;
+    for (int l = tid; l < T * T; l += NT) {
+        const int64_t k = t * T * T + l;
+        if (outidx[k] < 0) continue;
+        const float dx = (float)(nv[k] - g.n0[0]), dy = (float)(nv[ldn + k] - g.n0[1]),
+                    dz = (float)(nv[2 * ldn + k] - g.n0[2]);
+        const float s = 1.f / (2.f - 0.5f * (dx * dx + dy * dy + dz * dz));
+        m1 = fmaxf(m1, fabsf(dx * e1x + dy * e1y + dz * e1z) * s);
+        m2 = fmaxf(m2, fabsf(dx * e2x + dy * e2y + dz * e2z) * s);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+        m2 = fmaxf(m2, __shfl_xor_sync(0xffffffffu, m2, o));
+    }
+    __syncthreads();
+    if (lane == 0) {
+        red[0][w] = m1;
+        red[1][w] = m2;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int i = 0; i < W; ++i) {
+            m1 = fmaxf(m1, red[0][i]);
+            m2 = fmaxf(m2, red[1][i]);
+        }
+        // margin for the float arithmetic; a single pixel still gets a square of a quarter pixel
+        g.a1 = fmax((double)m1 * 1.00001, 0.125 * theta_pix);
+        g.a2 = fmax((double)m2 * 1.00001, 0.125 * theta_pix);
+        finish_geo(g, near_radius(fmax(g.a1, g.a2)) * 1.00001 + 1e-7);
+        geo[t] = g;
+    }
+}
+
+// One warp per parent cluster (nb x nb per face) of the child level (cnb x cnb per face): lane l
+// takes point l % 8 (corners and edge midpoints) of the rectangle of child l / 8.  Offsets from the
+// parent's centre are differences of FP64 centres plus a float offset, so they keep their relative
+// accuracy for small clusters.
+__global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__ child, int cnb,
+                                                     TreeGeo *__restrict__ geo, int nb, int nface)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (t >= (int64_t)nface * nb * nb) return;
+    const int64_t f = t / (nb * nb);
+    const int by = (int)(t - f * nb * nb) / nb, bx = (int)(t - f * nb * nb) % nb;
+    const int i = 2 * bx + (lane >> 3 & 1), j = 2 * by + (lane >> 4);
+    const bool has = i < cnb && j < cnb;
+    const TreeGeo k = child[has ? (f * cnb + j) * cnb + i : (f * cnb + 2 * by) * cnb + 2 * bx];
+    const float on = has && (lane & 7) == 0 ? 1.f : 0.f;
+    const float cx = warp_sum(on * k.c.x), cy = warp_sum(on * k.c.y), cz = warp_sum(on * k.c.z);
+    const float ux = warp_sum(on * k.f1.x), uy = warp_sum(on * k.f1.y), uz = warp_sum(on * k.f1.z);
+    TreeGeo g;
+    make_frame(cx, cy, cz, ux, uy, uz, g);
+    const float d0 = (float)(k.n0[0] - g.n0[0]), d1 = (float)(k.n0[1] - g.n0[1]), d2 = (float)(k.n0[2] - g.n0[2]);
+    const int q = lane & 7, pt = q < 4 ? q : q + 1;   // 3 x 3 points without the middle one
+    const float xi = (float)(pt % 3 - 1) * (float)k.a1, eta = (float)(pt / 3 - 1) * (float)k.a2;
+    const float r2 = xi * xi + eta * eta, s = 2.f / (1.f + r2);
+    const float x = d0 + s * (xi * k.f1.x + eta * k.f2.x - r2 * k.c.x);
+    const float y = d1 + s * (xi * k.f1.y + eta * k.f2.y - r2 * k.c.y);
+    const float z = d2 + s * (xi * k.f1.z + eta * k.f2.z - r2 * k.c.z);
+    const float ps = 1.f / (2.f - 0.5f * (x * x + y * y + z * z));
+    const float m1 = fabsf(x * (float)g.e1[0] + y * (float)g.e1[1] + z * (float)g.e1[2]) * ps;
+    const float m2 = fabsf(x * (float)g.e2[0] + y * (float)g.e2[1] + z * (float)g.e2[2]) * ps;
+    g.a1 = (double)warp_max(m1) * 1.002;
+    g.a2 = (double)warp_max(m2) * 1.002;
+    // near at a child implies near here
+    const float cd = (k.c.w + sqrtf(d0 * d0 + d1 * d1 + d2 * d2)) * 1.00003f + 2e-6f;
+    const double D = fmax(near_radius(fmax(g.a1, g.a2)) * 1.00001 + 1e-7, (double)warp_max(cd));
+    if (lane == 0) {
+        finish_geo(g, D);
+        geo[t] = g;
+    }
+}
+
+struct TreeNodeArgs {
+    TreeSamples S;
+    const TreeRec *rec;
+    const TreeGeo *geo, *pgeo;   // this level, the parent level (NULL at the coarsest)
+    int nb, pnb;
+    TreeWork W, Wp;              // items of this level, chunks of the parent's
+    double *F;                   // [ncl + pool][64]
+    const double *Fp;            // the parent level's
+    unsigned long long *queue;
+};
+
+constexpr int kNP = 8, kNN = kNP * kNP;   // FP32: 8 x 8 nodes
+constexpr int kLeaf = 16;                 // and 16 x 16 pixel leaves
+// Samples per chunk, at least.  Strings put up to 30 times the mean number of samples on a few clusters;
+// cut by the planned chunks N_side 100 with 3e4 samples takes 1.1 ms, with the same number of chunks for
+// every cluster (50, to spread the heavy ones) 1.9.
+constexpr int kNodeTarget = 1024, kPixTarget = 256;
+
+// Samples staged for one cluster, relative to its centre, each value twice as the (v, v) operand of a
+// packed instruction over two targets: with D = n0 - Xhat and target n = n0 + m, d = D + m and
+//   |d|^2 = K + 2 D.m + |m|^2,  Xdot.d = P + Xdot.m,  X'.d = Q + X'.m,  B = B0 + Xdot.m
+// from the per-sample K = |D|^2, P = Xdot.D, Q = X'.D and B0 = 1 + n0.Xdot (free of cancellation), so
+// a pair costs 18 FP32 operations instead of the 25 of the form that subtracts float pairs, and needs
+// neither the far-field form nor a test of B.  |m| < 0.36 |D| on a cluster whose samples are far, so
+// every sum keeps its relative accuracy.
+// Entry (9 x 16 B, an odd stride: the staging threads' stores meet no bank conflict):
+//   (2Dx, 2Dy) (2Dz, K) (Xdot x, y) (Xdot z, P) (-X' x, y) (-X' z, -Q) (B0, f) (c, -)
+constexpr int kNodeRec = 9;
+// Pixels may be close to their samples or in their beams: (c, rho^2 | 1 - |Xdot|), the low parts of D
+// (its high parts are the 2D / 2) and W = n0 + Xdot/|Xdot|, as (Dx, Dy) (Dz, Wx) (Wy, Wz).
+constexpr int kPixRec = 11;
+
+struct __align__(16) TreeSmem32 {
+    ulonglong2 rec[kTreeBatch * kPixRec];   // also the tables of the interpolation, before or after
+    TreeScanSmem scan;
+    TreeGeo geo, pgeo;
+    double coef[kNN], tmp[kNN];
+    int64_t item;
+};
+
+__device__ __forceinline__ void load_geo(TreeGeo *dst, const TreeGeo *src)
+{
+    constexpr int W = sizeof(TreeGeo) / 4;
+    static_assert(sizeof(TreeGeo) % 4 == 0 && W <= kTreeNT, "geometry copy");
+    if ((int)threadIdx.x < W) reinterpret_cast<uint32_t *>(dst)[threadIdx.x] = reinterpret_cast<const uint32_t *>(src)[threadIdx.x];
+}
+
+__device__ __forceinline__ float comp(const float4 &v, int c) { return c == 0 ? v.x : (c == 1 ? v.y : v.z); }
+
+// x = hi + lo + off as a new (hi, lo) pair
+__device__ __forceinline__ void pair_add(float h, float l, float off, float &hi, float &lo)
+{
+    const float s = h + off;
+    const float bb = s - h;
+    const float e = ((h - (s - bb)) + (off - bb)) + l;
+    hi = s + e;
+    lo = e - (hi - s);
+}
+
+// The interpolant with coefficients coef (FP64, shared) at (x, y) in [-1, 1]^2: everything but the
+// mean in FP32, the mean added in FP64.
+__device__ __forceinline__ double interp32(const double *coef, const float *cf, float x, float y)
+{
+    float tx[kNP];
+    tx[0] = 1.f;
+    tx[1] = x;
+#pragma unroll
+    for (int i = 2; i < kNP; ++i) tx[i] = fmaf(2.f * x, tx[i - 1], -tx[i - 2]);
+    float v = 0.f, t0 = 1.f, t1 = y;
+#pragma unroll
+    for (int j = 0; j < kNP; ++j) {
+        const float4 a = reinterpret_cast<const float4 *>(cf)[2 * j], b = reinterpret_cast<const float4 *>(cf)[2 * j + 1];
+        const float r = fmaf(b.w, tx[7], fmaf(b.z, tx[6], fmaf(b.y, tx[5], fmaf(b.x, tx[4],
+                        fmaf(a.w, tx[3], fmaf(a.z, tx[2], fmaf(a.y, tx[1], a.x)))))));
+        v = fmaf(r, t0, v);
+        const float t2 = fmaf(2.f * y, t1, -t0);
+        t0 = t1;
+        t1 = t2;
+    }
+    return coef[0] + (double)v;
+}
+
+// coefficients in float with the mean taken out (interp32 adds it in FP64)
+__device__ __forceinline__ void coefs_to_float(const double *coef, float *cf)
+{
+    for (int k = threadIdx.x; k < kNN; k += blockDim.x) cf[k] = k == 0 ? 0.f : (float)coef[k];
+    __syncthreads();
+}
+
+// Coordinates in [-1, 1]^2 of direction n0 + d (float offset d from the centre)
+__device__ __forceinline__ void local_xy(const TreeGeo &g, float dx, float dy, float dz, float &x, float &y)
+{
+    const float s = __fdividef(1.f, 2.f - 0.5f * fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
+    x = fmaf(dz, g.f1.z, fmaf(dy, g.f1.y, dx * g.f1.x)) * (s * g.f1.w);
+    y = fmaf(dz, g.f2.z, fmaf(dy, g.f2.y, dx * g.f2.x)) * (s * g.f2.w);
+}
+
+// chord from the centre to the farthest point of the cluster's rectangle
+__device__ __forceinline__ float target_radius(const TreeGeo &g)
+{
+    const float r2 = (float)(g.a1 * g.a1 + g.a2 * g.a2);
+    return 2.f * sqrtf(r2 / (1.f + r2)) * 1.0001f + 1e-7f;
+}
+
+__device__ __forceinline__ uint64_t dup2(float v) { return f2_pack(v, v); }
+
+// One sample relative to the centre of g, into its shared entry.
+template <int REC>
+__device__ __forceinline__ void stage_sample(const float4 (&q)[4], const TreeGeo &g, ulonglong2 *dst)
+{
+    float D[3], Dl[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {   // (n0 hi + lo) - (Xhat hi + lo) as a float pair
+        const float nh = comp(g.c, c), xh = comp(q[0], c), t = nh - xh, bb = t - nh;
+        const float e = ((nh - (t - bb)) - (xh + bb)) + (comp(g.l, c) - comp(q[1], c));
+        D[c] = t + e;
+        Dl[c] = e - (D[c] - t);
+    }
+    const float P = fmaf(q[2].z, D[2], fmaf(q[2].y, D[1], q[2].x * D[0]));
+    const float Q = fmaf(q[3].z, D[2], fmaf(q[3].y, D[1], q[3].x * D[0]));
+    const float K = fmaf(D[2], D[2], fmaf(D[1], D[1], D[0] * D[0]));
+    const float om = q[2].w, v = 1.f - om, iv = v > 0.f ? 1.f / v : 0.f;
+    const float wx = fmaf(q[2].x, iv, g.c.x), wy = fmaf(q[2].y, iv, g.c.y), wz = fmaf(q[2].z, iv, g.c.z);
+    const float B0 = fmaf(0.5f * v, fmaf(wz, wz, fmaf(wy, wy, wx * wx)), om);   // 1 - v + v |n0 + Xdot/v|^2 / 2
+    dst[0] = make_ulonglong2(dup2(2.f * D[0]), dup2(2.f * D[1]));
+    dst[1] = make_ulonglong2(dup2(2.f * D[2]), dup2(K));
+    dst[2] = make_ulonglong2(dup2(q[2].x), dup2(q[2].y));
+    dst[3] = make_ulonglong2(dup2(q[2].z), dup2(P));
+    dst[4] = make_ulonglong2(dup2(-q[3].x), dup2(-q[3].y));
+    dst[5] = make_ulonglong2(dup2(-q[3].z), dup2(-Q));
+    dst[6] = make_ulonglong2(dup2(B0), dup2(q[1].w));
+    dst[7] = make_ulonglong2(dup2(q[0].w), f2_pack(q[3].w, om));
+    if (REC > 9) {
+        dst[8] = make_ulonglong2(dup2(Dl[0]), dup2(Dl[1]));
+        dst[9] = make_ulonglong2(dup2(Dl[2]), dup2(wx));
+        dst[10] = make_ulonglong2(dup2(wy), dup2(wz));
+    }
+}
+
+// Stages count records of the scan's list in batches, one sample per thread; the next batch's records
+// are in flight while eval(entries, first list entry, batch size) runs.  Whole block.
+template <int REC, typename Eval>
+__device__ __forceinline__ void tree_batches(TreeSmem32 &sm, const TreeRec *__restrict__ recs, int count, Eval &&eval)
+{
+    const int tid = threadIdx.x;
+    float4 q[4];
+    auto fetch = [&](int b0) {
+        if (b0 + tid < count) {
+            const float4 *src = recs[sm.scan.list[b0 + tid] & kTreeIndex].v;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) q[k] = src[k];
+        }
+    };
+    fetch(0);
+#pragma unroll 1
+    for (int b0 = 0; b0 < count; b0 += kTreeBatch) {
+        if (b0 + tid < count) stage_sample<REC>(q, sm.geo, sm.rec + tid * REC);
+        fetch(b0 + kTreeBatch);
+        __syncthreads();
+        eval(sm.rec, b0, count - b0 < kTreeBatch ? count - b0 : kTreeBatch);
+        __syncthreads();
+    }
+}
+
+// offset from the centre of the node at (xi, eta)
+__device__ __forceinline__ void node_offset(const TreeGeo &g, int k, float (&m)[3])
+{
+    const float xi = (float)(g.a1 * cheb_at<kNP>(1, k % kNP)), eta = (float)(g.a2 * cheb_at<kNP>(1, k / kNP));
+    const float r2 = fmaf(xi, xi, eta * eta), s = 2.f / (1.f + r2);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) m[c] = s * fmaf(xi, comp(g.f1, c), fmaf(eta, comp(g.f2, c), -r2 * comp(g.c, c)));
+}
+
+// The samples of one level at the nodes of its clusters.  A half-warp holds the 64 nodes of the
+// cluster, four per lane as two f32x2 pairs, and takes every eighth sample of a batch (two samples per
+// warp at a time: one 16-byte shared load then feeds four nodes of two samples; with two nodes per
+// lane of one sample the loads bound the loop).  The eight half-warps are added up at the end.
+template <bool ROOT>
+__global__ void __launch_bounds__(kTreeNT, 4) k_tree_nodes_f32(TreeNodeArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TreeSmem32 &sm = *reinterpret_cast<TreeSmem32 *>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, half = lane >> 4, hl = lane & 15;
+    const int np = *a.W.npool;
+    TreeQueue queue{a.queue, 0ull};
+    for (int64_t item = queue.first(&sm.item); item < a.W.ncl + np; item = queue.next(&sm.item)) {
+        int kc, nch;
+        int64_t at;
+        const int64_t cl = tree_item(a.W, item, np, kc, nch, at);
+        if (cl < 0) continue;
+        int64_t pcl = 0;
+        if (!ROOT) {
+            const int64_t f = cl / ((int64_t)a.nb * a.nb), rem = cl - f * a.nb * a.nb;
+            pcl = (f * a.pnb + rem / a.nb / 2) * a.pnb + rem % a.nb / 2;
+            load_geo(&sm.pgeo, a.pgeo + pcl);
+        }
+        load_geo(&sm.geo, a.geo + cl);
+        __syncthreads();
+        const float4 self = sm.geo.c, parent = ROOT ? self : sm.pgeo.c;
+        uint64_t m[2][3], mm[2];   // node offsets from the centre, |m|^2
+#pragma unroll
+        for (int pp = 0; pp < 2; ++pp) {
+            float o[2][3];
+            node_offset(sm.geo, 32 * pp + hl, o[0]);
+            node_offset(sm.geo, 32 * pp + 16 + hl, o[1]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) m[pp][c] = f2_pack(o[0][c], o[1][c]);
+            mm[pp] = f2_fma(m[pp][2], m[pp][2], f2_fma(m[pp][1], m[pp][1], f2_mul(m[pp][0], m[pp][0])));
+        }
+        float ahi[4] = {0.f, 0.f, 0.f, 0.f}, alo[4] = {0.f, 0.f, 0.f, 0.f};
+        auto consume = [&](int count) {
+            tree_batches<kNodeRec>(sm, a.rec, count, [&](const ulonglong2 *mr, int b0, int cnt) {
+                uint64_t part[2] = {0ull, 0ull};
+#pragma unroll 1
+                for (int s0 = 2 * w; s0 < cnt; s0 += 2 * (kTreeNT / 32)) {
+                    const bool on = s0 + half < cnt;
+                    const ulonglong2 *r = mr + kNodeRec * (on ? s0 + half : s0);
+                    const ulonglong2 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3], r4 = r[4], r5 = r[5], r6 = r[6];
+                    const uint64_t c = on ? r[7].x : 0ull;   // no second sample: zero weight
+#pragma unroll
+                    for (int pp = 0; pp < 2; ++pp) {
+                        const uint64_t Q = f2_fma(m[pp][2], r1.x, f2_fma(m[pp][1], r0.y, f2_fma(m[pp][0], r0.x, f2_add(mm[pp], r1.y))));
+                        const uint64_t g = f2_fma(m[pp][2], r3.x, f2_fma(m[pp][1], r2.y, f2_mul(m[pp][0], r2.x)));
+                        const uint64_t Qdn = f2_fma(m[pp][2], r5.x, f2_fma(m[pp][1], r4.y, f2_fma(m[pp][0], r4.x, r5.y)));
+                        const uint64_t B = f2_add(g, r6.x), Pd = f2_add(g, r3.y), A = f2_sub(r6.y, Qdn);
+                        const uint64_t num = f2_fma(A, Qdn, f2_mul(B, Pd));
+                        float u0, u1;
+                        f2_unpack(f2_mul(B, Q), u0, u1);
+                        part[pp] = f2_fma(f2_mul(c, num), f2_pack(rcp_approx(u0), rcp_approx(u1)), part[pp]);
+                    }
+                }
+#pragma unroll
+                for (int pp = 0; pp < 2; ++pp) {
+                    float p0, p1;
+                    f2_unpack(part[pp], p0, p1);
+                    fold(ahi[2 * pp], alo[2 * pp], p0);
+                    fold(ahi[2 * pp + 1], alo[2 * pp + 1], p1);
+                }
+            });
+        };
+        tree_scan<ROOT, false>(a.S, kc, nch, self, parent, 0.f, 0.f, sm.scan, consume);
+        double (*red)[kNN] = reinterpret_cast<double (*)[kNN]>(sm.rec);   // the batches are done
+#pragma unroll
+        for (int q = 0; q < 4; ++q) red[2 * w + half][16 * q + hl] = (double)ahi[q] + (double)alo[q];
+        __syncthreads();
+        double v = 0.0;
+        if (tid < kNN) {
+#pragma unroll
+            for (int i = 0; i < kTreeNT / 16; ++i) v += red[i][tid];
+        }
+        if (!ROOT && kc == 0) {   // the parent's interpolant at this cluster's nodes
+            cheb_coefs<kNP>(a.Fp, a.Wp, pcl, sm.coef, sm.tmp);
+            float *cf = reinterpret_cast<float *>(sm.rec + kTreeNT / 16 * kNN / 2);
+            coefs_to_float(sm.coef, cf);
+            if (tid < kNN) {
+                float d[3], x, y;
+                node_offset(sm.geo, tid, d);
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    d[c] += (comp(sm.geo.c, c) - comp(sm.pgeo.c, c)) + (comp(sm.geo.l, c) - comp(sm.pgeo.l, c));
+                local_xy(sm.pgeo, d[0], d[1], d[2], x, y);
+                v += interp32(sm.coef, cf, x, y);
+            }
+        }
+        if (tid < kNN) a.F[at * kNN + tid] = v;
+        __syncthreads();
+    }
+}
+
+struct TreePixArgs {
+    TreeSamples S;
+    const TreeRec *rec;
+    const Seg64 *s64;
+    const TreeGeo *geo;          // finest clusters
+    const double *nv;            // pixel table, T * T slots per cluster
+    int64_t ldn;
+    const int64_t *outidx;
+    TreeWork W, Wf;              // items of the pixel stage, chunks of the finest level's node sums
+    const double *F;
+    double *theta;
+    double *partial;             // [pool][T * T]
+    int accumulate;
+    float b_min;
+    DevStatus *st;
+    unsigned long long *queue;
+};
+
+// FP64 pairs of one warp's 64 pixels: queued as (record, pixel) and evaluated 32 at a time, one per
+// lane.  Evaluated where they are found, a warp spent the FP64 unit's 64 cycles per instruction on
+// one or two lanes, and the tiles that hold a string took 1.5 ms at N_side 64.
+struct TreeNearQueue {
+    uint32_t src[64];
+    double val[32];
+    double acc[64];
+    uint8_t pix[64];
+};
+struct __align__(16) TreeSmemPix {
+    TreeSmem32 s;
+    TreeNearQueue q[kTreeNT / 32];
+};
+
+// Evaluate the first cnt <= 32 entries of the warp's queue and add them to the pixels' sums in queue
+// order (entries of one pixel by the lowest lane that holds it).
+__device__ __noinline__ void near_flush(TreeNearQueue &q, int cnt, const Seg64 *__restrict__ s64,
+                                        const double *__restrict__ nv, int64_t ldn, int64_t kw, unsigned &zerocnt)
+{
+    const int lane = threadIdx.x & 31;
+    const bool on = lane < cnt;
+    const int px = on ? q.pix[lane] : 64 + lane;
+    double v = 0.0;
+    if (on) {
+        const Seg64 g = s64[q.src[lane]];
+        const int64_t k = kw + px;
+        v = pair64_fast(nv[k], nv[ldn + k], nv[2 * ldn + k], g, zerocnt);
+    }
+    q.val[lane] = v;
+    __syncwarp();
+    const unsigned peers = __match_any_sync(0xffffffffu, px);
+    if (on && (peers & ((1u << lane) - 1u)) == 0u) {
+        double s = q.acc[px];
+        for (unsigned m = peers; m; m &= m - 1u) s += q.val[__ffs(m) - 1];
+        q.acc[px] = s;
+    }
+    __syncwarp();
+}
+
+// The pixels of the finest clusters: a half-warp holds 64 of them, four per lane as two f32x2 pairs, and
+// every warp takes all near samples, one per half-warp at a time.  A sample that may come within
+// max(rho, R / 2) of some pixel takes d from float pairs; pairs with |d| < rho or B < b_min / 1000 go to
+// the warp's FP64 queue.
+__global__ void __launch_bounds__(kTreeNT, 4) k_tree_pixels_f32(TreePixArgs a)
+{
+    constexpr int TILE = kLeaf * kLeaf;
+    static_assert(TILE == 2 * kTreeNT, "64 pixels per warp");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TreeSmem32 &sm = reinterpret_cast<TreeSmemPix *>(smem_raw)->s;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, half = lane >> 4, hl = lane & 15;
+    TreeNearQueue &nq = reinterpret_cast<TreeSmemPix *>(smem_raw)->q[w];
+    const uint64_t half2 = f2_pack(0.5f, 0.5f);
+    unsigned nearcnt = 0, zerocnt = 0;
+    const int np = *a.W.npool;
+    TreeQueue queue{a.queue, 0ull};
+    for (int64_t item = queue.first(&sm.item); item < a.W.ncl + np; item = queue.next(&sm.item)) {
+        int kc, nch;
+        int64_t at;
+        const int64_t cl = tree_item(a.W, item, np, kc, nch, at);
+        if (cl < 0) continue;
+        load_geo(&sm.geo, a.geo + cl);
+        nq.acc[lane] = 0.0;
+        nq.acc[32 + lane] = 0.0;
+        __syncthreads();
+        const float4 self = sm.geo.c;
+        float ahi[4] = {0.f, 0.f, 0.f, 0.f}, alo[4] = {0.f, 0.f, 0.f, 0.f};
+        unsigned valid = 0;
+        int qlen = 0;
+        uint64_t m[2][3], ml[2][3], mm[2];   // offsets from the centre as float pairs, |m|^2
+        const int64_t kw = cl * TILE + w * 64;   // pixel 16 q + hl of the warp is the lane's q-th
+#pragma unroll
+        for (int pp = 0; pp < 2; ++pp) {
+            float h[2][3], l[2][3];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int64_t k = kw + 16 * (2 * pp + u) + hl;
+                if (a.outidx[k] >= 0) valid |= 1u << (2 * pp + u);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const double v = a.nv[c * a.ldn + k] - sm.geo.n0[c];
+                    h[u][c] = __double2float_rn(v);
+                    l[u][c] = __double2float_rn(v - (double)h[u][c]);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                m[pp][c] = f2_pack(h[0][c], h[1][c]);
+                ml[pp][c] = f2_pack(l[0][c], l[1][c]);
+            }
+            mm[pp] = f2_fma(m[pp][2], m[pp][2], f2_fma(m[pp][1], m[pp][1], f2_mul(m[pp][0], m[pp][0])));
+        }
+        double far[2] = {0.0, 0.0};   // of the lane's pixels 2 half and 2 half + 1
+        if (kc == 0) {
+            cheb_coefs<kNP>(a.F, a.Wf, cl, sm.coef, sm.tmp);
+            float *cf = reinterpret_cast<float *>(sm.rec);
+            coefs_to_float(sm.coef, cf);
+            float d[2][3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) f2_unpack(half ? m[1][c] : m[0][c], d[0][c], d[1][c]);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                float x, y;
+                local_xy(sm.geo, d[u][0], d[u][1], d[u][2], x, y);
+                far[u] = interp32(sm.coef, cf, x, y);
+            }
+            __syncthreads();   // the coefficients' buffer is the first batch's
+        }
+        const float b_tiny = a.b_min * 1e-3f;
+        auto consume = [&](int count) {
+            tree_batches<kPixRec>(sm, a.rec, count, [&](const ulonglong2 *mr, int b0, int cnt) {
+                uint64_t part[2] = {0ull, 0ull};
+#pragma unroll 1
+                for (int s0 = 0; s0 < cnt; s0 += 2) {
+                    const bool on = s0 + half < cnt;
+                    const int s = on ? s0 + half : s0;
+                    const ulonglong2 *r = mr + kPixRec * s;
+                    const ulonglong2 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3], r4 = r[4], r5 = r[5], r6 = r[6], r7 = r[7];
+                    const uint64_t c = on ? r7.x : 0ull;   // no second sample: zero weight
+                    const uint32_t src = sm.scan.list[b0 + s];
+                    if (!__any_sync(0xffffffffu, (src & (kTreeBeam | kTreeClose)) != 0u)) {
+#pragma unroll
+                        for (int pp = 0; pp < 2; ++pp) {
+                            const uint64_t Q = f2_fma(m[pp][2], r1.x, f2_fma(m[pp][1], r0.y, f2_fma(m[pp][0], r0.x, f2_add(mm[pp], r1.y))));
+                            const uint64_t g = f2_fma(m[pp][2], r3.x, f2_fma(m[pp][1], r2.y, f2_mul(m[pp][0], r2.x)));
+                            const uint64_t Qdn = f2_fma(m[pp][2], r5.x, f2_fma(m[pp][1], r4.y, f2_fma(m[pp][0], r4.x, r5.y)));
+                            const uint64_t B = f2_add(g, r6.x), Pd = f2_add(g, r3.y), A = f2_sub(r6.y, Qdn);
+                            const uint64_t num = f2_fma(A, Qdn, f2_mul(B, Pd));
+                            float u0, u1;
+                            f2_unpack(f2_mul(B, Q), u0, u1);
+                            part[pp] = f2_fma(f2_mul(c, num), f2_pack(rcp_approx(u0), rcp_approx(u1)), part[pp]);
+                        }
+                        continue;
+                    }
+                    const ulonglong2 r8 = r[8], r9 = r[9], r10 = r[10];
+                    float rho2, om;
+                    f2_unpack(r7.y, rho2, om);
+                    const uint64_t om2 = dup2(om), hv2 = dup2(fmaf(-0.5f, om, 0.5f));   // 1 - v, v / 2
+                    unsigned near = 0;
+#pragma unroll
+                    for (int pp = 0; pp < 2; ++pp) {
+                        const uint64_t dx = f2_add(f2_fma(half2, r0.x, m[pp][0]), f2_add(ml[pp][0], r8.x));
+                        const uint64_t dy = f2_add(f2_fma(half2, r0.y, m[pp][1]), f2_add(ml[pp][1], r8.y));
+                        const uint64_t dz = f2_add(f2_fma(half2, r1.x, m[pp][2]), f2_add(ml[pp][2], r9.x));
+                        const uint64_t Q = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
+                        const uint64_t Pd = f2_fma(r3.x, dz, f2_fma(r2.y, dy, f2_mul(r2.x, dx)));
+                        const uint64_t Qdn = f2_fma(r5.x, dz, f2_fma(r4.y, dy, f2_mul(r4.x, dx)));
+                        const uint64_t A = f2_sub(r6.y, Qdn);
+                        const uint64_t wx = f2_add(r9.y, m[pp][0]), wy = f2_add(r10.x, m[pp][1]), wz = f2_add(r10.y, m[pp][2]);
+                        const uint64_t B = f2_fma(hv2, f2_fma(wz, wz, f2_fma(wy, wy, f2_mul(wx, wx))), om2);
+                        const uint64_t num = f2_fma(A, Qdn, f2_mul(B, Pd));
+                        float u0, u1, q0, q1, c0, c1;
+                        f2_unpack(f2_mul(B, Q), u0, u1);
+                        f2_unpack(Q, q0, q1);
+                        f2_unpack(B, c0, c1);
+                        u0 = rcp_approx(u0);
+                        u1 = rcp_approx(u1);
+                        if (q0 < rho2 || c0 < b_tiny) {
+                            near |= 1u << (2 * pp);
+                            u0 = 0.f;   // queued: zero weight here
+                        }
+                        if (q1 < rho2 || c1 < b_tiny) {
+                            near |= 2u << (2 * pp);
+                            u1 = 0.f;
+                        }
+                        part[pp] = f2_fma(f2_mul(c, num), f2_pack(u0, u1), part[pp]);
+                    }
+                    if (!__any_sync(0xffffffffu, near != 0u)) continue;
+                    near &= on ? valid : 0u;
+                    const unsigned below = (1u << lane) - 1u;
+#pragma unroll 1
+                    for (int q = 0; q < 4; ++q) {
+                        const bool hit = near >> q & 1u;
+                        const unsigned m = __ballot_sync(0xffffffffu, hit);
+                        if (!m) continue;
+                        if (hit) {
+                            const int p = qlen + __popc(m & below);
+                            nq.src[p] = src & kTreeIndex;
+                            nq.pix[p] = (uint8_t)(16 * q + hl);
+                            ++nearcnt;
+                        }
+                        qlen += __popc(m);
+                        __syncwarp();
+                        if (qlen >= 32) {
+                            near_flush(nq, 32, a.s64, a.nv, a.ldn, kw, zerocnt);
+                            const uint32_t ms = nq.src[32 + lane];
+                            const uint8_t mp = nq.pix[32 + lane];
+                            __syncwarp();
+                            nq.src[lane] = ms;
+                            nq.pix[lane] = mp;
+                            qlen -= 32;
+                            __syncwarp();
+                        }
+                    }
+                }
+#pragma unroll
+                for (int pp = 0; pp < 2; ++pp) {
+                    float p0, p1;
+                    f2_unpack(part[pp], p0, p1);
+                    fold(ahi[2 * pp], alo[2 * pp], p0);
+                    fold(ahi[2 * pp + 1], alo[2 * pp + 1], p1);
+                }
+            });
+        };
+        tree_scan<false, true>(a.S, kc, nch, self, self, target_radius(sm.geo), a.b_min, sm.scan, consume);
+        if (qlen > 0) near_flush(nq, qlen, a.s64, a.nv, a.ldn, kw, zerocnt);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {   // both half-warps' sums of a pixel; half q / 2 writes it
+            double v = (double)ahi[q] + (double)alo[q];
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            if (half != q / 2) continue;
+            v = (v + nq.acc[16 * q + hl]) + far[q & 1];
+            const int64_t k = kw + 16 * q + hl;
+            if (nch == 1) {
+                const int64_t oi = a.outidx[k];
+                if (oi >= 0) a.theta[oi] = a.accumulate ? a.theta[oi] + v : v;
+            } else {
+                a.partial[item * TILE + w * 64 + 16 * q + hl] = v;   // pool entry of the chunk
+            }
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        nearcnt += __shfl_xor_sync(0xffffffffu, nearcnt, o);
+        zerocnt += __shfl_xor_sync(0xffffffffu, zerocnt, o);
+    }
+    if (lane == 0 && (nearcnt | zerocnt)) {
+        atomicAdd(&a.st->near_pairs, (unsigned long long)nearcnt);
+        atomicAdd(&a.st->zero_pairs, (unsigned long long)zerocnt);
+    }
+}
+
+// theta of the clusters that were cut into chunks: their partial sums added in chunk order.
+__global__ void __launch_bounds__(kLeaf *kLeaf) k_tree_reduce(TreeWork W, const double *__restrict__ partial,
+                                                              const int64_t *__restrict__ outidx,
+                                                              double *__restrict__ theta, int accumulate)
+{
+    constexpr int TILE = kLeaf * kLeaf;
+    const int np = *W.npool;
+    for (int e = blockIdx.x; e < np; e += gridDim.x) {
+        const int2 it = W.pool[e];
+        if (it.y != 0) continue;
+        const int64_t oi = outidx[(int64_t)it.x * TILE + threadIdx.x];
+        const int nch = W.nch[it.x];
+        double hi = 0.0, lo = 0.0;
+        for (int c = 0; c < nch; ++c) fold64(hi, lo, partial[(int64_t)(e + c) * TILE + threadIdx.x]);
+        if (oi >= 0) theta[oi] = accumulate ? theta[oi] + (hi + lo) : hi + lo;
+    }
+}
+
+// The stages to plan: node sums of the levels, then the pixels.
+constexpr int kTargets = 8;             // chunk sizes tried: target, 2 target, ...
+// work counters, totals per chunk size and pool lengths of the stages
+constexpr size_t kTreeZero = (kTreeLevels + 1) * ((1 + kTargets) * sizeof(unsigned long long) + sizeof(int));
+struct TreeStages {
+    int n;
+    int64_t first[kTreeLevels + 2];     // prefix of the stages' cluster counts
+    const TreeGeo *geo[kTreeLevels + 1], *pgeo[kTreeLevels + 1];   // the clusters, their parents (nodes only)
+    int nb[kTreeLevels + 1], pnb[kTreeLevels + 1];
+    int pool[kTreeLevels + 1];          // pool entries
+    int target[kTreeLevels + 1];        // smallest chunk
+    int2 *entries[kTreeLevels + 1];
+};
+
+// Share of a tile's samples that lies within the near chord of a cluster, from the tile's ball (a
+// linear ramp across the ball): position tiles by distance, beam tiles by B.
+__device__ __forceinline__ float tile_share(const TreeCap &t, const float4 &c, int pass)
+{
+    if (t.a.w < 0.f) return 0.f;
+    float x;
+    if (pass) {
+        const float b = 1.f + (c.x * t.a.x + c.y * t.a.y + c.z * t.a.z);
+        x = 0.5f * c.w * c.w - b;
+    } else {
+        const float dx = c.x - t.a.x, dy = c.y - t.a.y, dz = c.z - t.a.z;
+        x = c.w - sqrtf(dx * dx + dy * dy + dz * dz);
+    }
+    return fminf(fmaxf(0.5f + 0.5f * x / (t.a.w + 1e-6f), 0.f), 1.f);
+}
+
+// Estimate of every cluster's samples from the tile balls; all of them at the root.  And, for each chunk
+// size, the pool entries that it would take.  One warp per (stage, cluster).
+__global__ void __launch_bounds__(128) k_tree_count(TreeStages g, TreeSamples S, int64_t n, int *__restrict__ est,
+                                                    unsigned long long *__restrict__ total)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (k >= g.first[g.n]) return;
+    int st = 0;
+    while (k >= g.first[st + 1]) ++st;
+    const int64_t c = k - g.first[st];
+    const bool leaf = st == g.n - 1;
+    int64_t v = n;
+    if (leaf || g.pgeo[st]) {
+        const float4 self = g.geo[st][c].c;
+        float4 outer = self;
+        if (!leaf) {
+            const int64_t nb = g.nb[st], f = c / (nb * nb), rem = c - f * nb * nb;
+            outer = g.pgeo[st][(f * g.pnb[st] + rem / nb / 2) * g.pnb[st] + rem % nb / 2].c;
+        }
+        float share = 0.f;
+        const int nsup = (int)((S.nst + kTreeSuper - 1) / kTreeSuper);
+        for (int pass = 0; pass < 2; ++pass) {
+            const TreeCap *sup = pass ? S.vsup : S.sup, *caps = pass ? S.vcaps : S.caps;
+            for (int u0 = 0; u0 < nsup; u0 += 32) {
+                bool in = false;
+                if (u0 + lane < nsup) {
+                    const TreeCap cap = sup[u0 + lane];
+                    in = pass ? tree_tile_beam(cap, outer) : tree_tile_pos(cap, outer);
+                }
+                unsigned m = __ballot_sync(0xffffffffu, in);
+                for (; m; m &= m - 1u) {
+                    const int64_t t = (int64_t)(u0 + __ffs(m) - 1) * kTreeSuper + lane;
+                    if (t < S.nst) {
+                        const TreeCap cap = caps[t];
+                        const float f = tile_share(cap, outer, pass);
+                        share += leaf || pass ? f : fmaxf(f - tile_share(cap, self, pass), 0.f);
+                    }
+                }
+            }
+        }
+        v = (int64_t)(warp_sum(share) * (float)kTreeS);
+        if (v > n) v = n;
+    }
+    if (lane == 0) est[k] = (int)v;
+    if (lane < kTargets) {
+        const int64_t T = (int64_t)g.target[st] << lane;
+        if (v >= T) atomicAdd(total + st * kTargets + lane, (unsigned long long)(1 + v / T));
+    }
+}
+
+// Chunks per cluster: with the smallest chunk size whose entries fit the pool (none: no cluster is
+// cut).  Where a cluster's entries lie in the pool depends on the order of the atomics; what they hold
+// does not.
+__global__ void __launch_bounds__(128) k_tree_plan(TreeStages g, const int *__restrict__ est,
+                                                   const unsigned long long *__restrict__ total, int *__restrict__ nch,
+                                                   int *__restrict__ pbase, int *__restrict__ npool)
+{
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= g.first[g.n]) return;
+    int st = 0;
+    while (k >= g.first[st + 1]) ++st;
+    int j = 0;
+    while (j < kTargets && total[st * kTargets + j] > (unsigned long long)g.pool[st]) ++j;
+    const int64_t T = (int64_t)g.target[st] << j;
+    const int m = j == kTargets || est[k] < T ? 1 : (int)(1 + est[k] / T);
+    int b = 0;
+    if (m > 1) {
+        b = atomicAdd(npool + st, m);
+        for (int i = 0; i < m; ++i) g.entries[st][b + i] = make_int2((int)(k - g.first[st]), i);
+    }
+    nch[k] = m;
+    pbase[k] = b;
+}
+
+size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
+
+int slots_of(const void *fn, size_t smem, int num_sms)
+{
+    int nb = 0;
+    if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kTreeNT, smem);
+    return (nb > 0 ? nb : 1) * num_sms;
+}
+
+}  // namespace
+
+int tree_leaf(int prec) { return kLeaf; }
+
+TreePlan tree_plan(int prec, int64_t N, int nface, int64_t n, int num_sms)
+{
+    TreePlan p{};
+    p.leaf = kLeaf;
+    p.nn = kNN;
+    p.nface = nface;
+    p.n_pad = (n + kTreeS - 1) / kTreeS * kTreeS;
+    p.nst = p.n_pad / kTreeS;
+    int64_t nb = (N + p.leaf - 1) / p.leaf;
+    p.nslots = slots_of((const void *)&k_tree_nodes_f32<false>, sizeof(TreeSmem32), num_sms);
+    p.pslots = slots_of((const void *)&k_tree_pixels_f32, sizeof(TreeSmemPix), num_sms);
+    int64_t all = 0;
+    for (;;) {
+        const int L = p.levels++;
+        p.nb[L] = (int)nb;
+        p.ncl[L] = nface * nb * nb;
+        all += p.ncl[L];
+        if (nb <= 2 || p.levels == kTreeLevels) break;
+        nb = (nb + 1) / 2;
+    }
+    all += p.ncl[0];
+    p.pool = 8 * p.nslots;
+    p.ppool = 8 * p.pslots;
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = at;
+        at += up256(bytes);
+        return o;
+    };
+    p.off_queue = take(kTreeZero);   // zeroed per call
+    p.off_crit = take((size_t)p.n_pad * sizeof(TreeCrit));
+    p.off_vcrit = take((size_t)p.n_pad * sizeof(TreeCrit));
+    p.off_caps = take((size_t)2 * p.nst * sizeof(TreeCap));
+    p.off_sup = take((size_t)2 * ((p.nst + kTreeSuper - 1) / kTreeSuper) * sizeof(TreeCap));
+    p.off_vidx = take((size_t)p.n_pad * sizeof(uint32_t));
+    p.off_inv = take((size_t)n * sizeof(uint32_t));
+    p.off_rec = take((size_t)p.n_pad * sizeof(TreeRec));
+    p.off_work = take((size_t)3 * all * sizeof(int));
+    p.off_pool = take(((size_t)p.levels * p.pool + p.ppool) * sizeof(int2));
+    p.off_partial = take((size_t)p.ppool * p.leaf * p.leaf * sizeof(double));
+    for (int L = 0; L < p.levels; ++L) {
+        p.off_geo[L] = take((size_t)p.ncl[L] * sizeof(TreeGeo));
+        p.off_F[L] = take((size_t)(p.ncl[L] + p.pool) * p.nn * sizeof(double));
+    }
+    p.bytes = at;
+    return p;
+}
+
+cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_t s)
+{
+    unsigned char *b = (unsigned char *)m.scratch;
+    TreeCrit *crit = (TreeCrit *)(b + p.off_crit), *vcrit = (TreeCrit *)(b + p.off_vcrit);
+    TreeCap *caps = (TreeCap *)(b + p.off_caps), *sup = (TreeCap *)(b + p.off_sup);
+    uint32_t *vidx = (uint32_t *)(b + p.off_vidx), *inv = (uint32_t *)(b + p.off_inv);
+    TreeRec *rec = (TreeRec *)(b + p.off_rec);
+    unsigned long long *queue = (unsigned long long *)(b + p.off_queue), *total = queue + kTreeLevels + 1;
+    int *npool = (int *)(total + (kTreeLevels + 1) * kTargets);
+    cudaError_t e = cudaMemsetAsync(queue, 0, kTreeZero, s);
+    if (e != cudaSuccess) return e;
+    const unsigned tb = (unsigned)((p.nst * 32 + 255) / 256);
+    k_tree_crit<<<tb, 256, 0, s>>>(m.s32, m.s64, m.perm, m.n, p.nst, crit, caps, rec, inv);
+    k_tree_vcrit<<<tb, 256, 0, s>>>(crit, m.s32, m.perm + m.n, inv, m.n, p.nst, vcrit, caps + p.nst, vidx);
+    const int64_t nsup = (p.nst + kTreeSuper - 1) / kTreeSuper;
+    k_tree_super<<<dim3((unsigned)((nsup + 3) / 4), 2), 128, 0, s>>>(caps, p.nst, nsup, sup);
+    const TreeSamples S{crit, vcrit, caps, caps + p.nst, sup, sup + nsup, vidx, p.nst};
+    k_tree_leaf_geo<kLeaf><<<(unsigned)p.ncl[0], kLeaf * kLeaf / 4, 0, s>>>(m.nv, m.ldn, m.outidx, m.diag, m.theta_pix,
+                                                                             (TreeGeo *)(b + p.off_geo[0]));
+    for (int L = 1; L < p.levels; ++L)
+        k_tree_up_geo<<<(unsigned)((p.ncl[L] + 3) / 4), 128, 0, s>>>((const TreeGeo *)(b + p.off_geo[L - 1]), p.nb[L - 1],
+                                                                     (TreeGeo *)(b + p.off_geo[L]), p.nb[L], p.nface);
+    // stages 0 .. levels - 1: node sums of the level; stage `levels`: the pixels
+    TreeStages g{};
+    g.n = p.levels + 1;
+    int2 *entries = (int2 *)(b + p.off_pool);
+    for (int st = 0; st <= p.levels; ++st) {
+        const bool pix = st == p.levels;
+        const int L = pix ? 0 : st;
+        g.first[st + 1] = g.first[st] + p.ncl[L];
+        g.geo[st] = (const TreeGeo *)(b + p.off_geo[L]);
+        g.nb[st] = p.nb[L];
+        if (st + 1 < p.levels) {
+            g.pgeo[st] = (const TreeGeo *)(b + p.off_geo[st + 1]);
+            g.pnb[st] = p.nb[st + 1];
+        }
+        g.pool[st] = pix ? p.ppool : p.pool;
+        g.target[st] = pix ? kPixTarget : kNodeTarget;
+        g.entries[st] = entries + (size_t)st * p.pool;
+    }
+    const int64_t all = g.first[g.n];
+    int *est = (int *)(b + p.off_work), *nch = est + all, *pbase = nch + all;
+    k_tree_count<<<(unsigned)((all + 3) / 4), 128, 0, s>>>(g, S, m.n, est, total);
+    k_tree_plan<<<(unsigned)((all + 127) / 128), 128, 0, s>>>(g, est, total, nch, pbase, npool);
+    auto work = [&](int st) {
+        return TreeWork{nch + g.first[st], pbase + g.first[st], g.entries[st], npool + st, g.first[st + 1] - g.first[st]};
+    };
+    for (int L = p.levels - 1; L >= 0; --L) {
+        const bool root = L == p.levels - 1;
+        TreeNodeArgs a{};
+        a.S = S;
+        a.rec = rec;
+        a.geo = (const TreeGeo *)(b + p.off_geo[L]);
+        a.nb = p.nb[L];
+        a.W = work(L);
+        a.F = (double *)(b + p.off_F[L]);
+        if (!root) {
+            a.pgeo = (const TreeGeo *)(b + p.off_geo[L + 1]);
+            a.pnb = p.nb[L + 1];
+            a.Fp = (const double *)(b + p.off_F[L + 1]);
+            a.Wp = work(L + 1);
+        }
+        a.queue = queue + L;
+        const void *fn = root ? (const void *)&k_tree_nodes_f32<true> : (const void *)&k_tree_nodes_f32<false>;
+        const int64_t items = p.ncl[L] + p.pool;
+        void *args[] = {(void *)&a};
+        cudaLaunchKernel(fn, dim3((unsigned)(items < p.nslots ? items : p.nslots)), dim3(kTreeNT), args,
+                         sizeof(TreeSmem32), s);
+    }
+    TreePixArgs a{};
+    a.S = S;
+    a.rec = rec;
+    a.s64 = m.s64;
+    a.geo = (const TreeGeo *)(b + p.off_geo[0]);
+    a.nv = m.nv;
+    a.ldn = m.ldn;
+    a.outidx = m.outidx;
+    a.W = work(p.levels);
+    a.Wf = work(0);
+    a.F = (const double *)(b + p.off_F[0]);
+    a.theta = m.theta;
+    a.partial = (double *)(b + p.off_partial);
+    a.accumulate = m.accumulate;
+    a.b_min = m.b_min;
+    a.st = m.st;
+    a.queue = queue + kTreeLevels;
+    const int64_t items = p.ncl[0] + p.ppool;
+    k_tree_pixels_f32<<<(unsigned)(items < p.pslots ? items : p.pslots), kTreeNT, sizeof(TreeSmemPix), s>>>(a);
+    k_tree_reduce<<<(unsigned)p.pslots, kLeaf * kLeaf, 0, s>>>(a.W, a.partial, m.outidx, m.theta, m.accumulate);
+    return cudaSuccess;
+}
+
+}  // namespace isw

@@ -1,0 +1,450 @@
+// Cluster tree over the pixels of a map (device side shared by tree.cu and treeadj.cu).
+//
+// The pair term of Eq. (1)-(2) is a smooth function of the direction n away from two places: n
+// near the sample (1 - n.Xhat -> 0) and n in its beam (B = 1 + n.Xdot -> 0).  In the stereographic
+// coordinates (xi, eta) about a cluster centre n0,
+//   n = (2 xi e1 + 2 eta e2 + (1 - xi^2 - eta^2) n0) / (1 + xi^2 + eta^2),
+// every factor of the pair term is a polynomial over 1 + xi^2 + eta^2, those denominators cancel,
+// and the term is a rational function whose only poles are
+//   (xi - xi_s)^2 + (eta - eta_s)^2 = 0        at distance |z_s|^2 = (1 - n0.Xhat) / (1 + n0.Xhat),
+//   (xi - xi_b)^2 + (eta - eta_b)^2 = -beta^2  with |z_b|^2 + beta^2 = (1 + n0.Xdot) / (1 - n0.Xdot).
+// So when n0.Xhat and -n0.Xdot are both below one threshold, i.e. the chord |n0 - Xhat| and the
+// "beam chord" sqrt(2 (1 + n0.Xdot)) both exceed the cluster's near radius D, the sum of such
+// samples over the cluster's square [-a, a]^2 is its polynomial interpolant in p x p Chebyshev
+// points to within ~rho^-p, rho = (kappa - 1) + sqrt((kappa - 1)^2 + 1) for D = the chord of
+// stereographic radius kappa a.  The pair terms are then evaluated at p^2 nodes instead of at every
+// pixel of the cluster.
+//
+// Every (sample, pixel) pair is accounted for exactly once: at the first level, from the coarsest
+// down, at which the sample is far from the pixel's cluster, or, if it is near at the finest level
+// too, directly at the pixel.  Near at a cluster implies near at its parent (D_parent >= D_child +
+// the distance of the two centres, both chords being 1-Lipschitz in n0), so that a level takes the
+// samples that are near at the parent and far at itself.  The decision is one function of
+// explicitly rounded operations, so every kernel takes the same one.
+#pragma once
+
+#include "isw_internal.cuh"
+#include "kernels.cuh"
+#include "pipeline.cuh"
+
+namespace isw {
+
+// Per sample: a = (Xhat, near-field radius rho), b = (-Xdot/|Xdot|, 1 - |Xdot|); a sample to be
+// skipped (zero weight or padding) has b.w = kCritSkip.
+constexpr float kCritSkip = 4.f;
+struct __align__(16) TreeCrit {
+    float4 a, b;
+};
+// Per tile of kTreeS samples, in the order that the tile is cut from: a ball (centre, radius; < 0 when
+// the tile has no sample to sum) that holds the tile's Xhat vectors, enlarged by the largest rho
+// (position order), or its Xdot vectors (velocity order).
+struct __align__(16) TreeCap {
+    float4 a;
+};
+// The samples in two orders.  Position order (Morton code of Xhat) is the order of the records; the
+// velocity order (Morton code of Xdot) finds the samples whose beam meets a cluster: -Xdot near n0 has
+// little to do with where the sample is, and in position order nearly every tile of a loop's samples
+// holds some beam (N_side 512 with 2e5 samples: the tests of samples in such tiles took 1-2 ms a level).
+struct TreeSamples {
+    const TreeCrit *crit, *vcrit;
+    const TreeCap *caps, *vcaps;
+    const TreeCap *sup, *vsup; // the same balls over kTreeSuper consecutive tiles
+    const uint32_t *vidx;      // record of a velocity-order entry
+    int64_t nst;               // tiles of either order
+};
+// FP32 evaluation record (64 B): Xhat hi (3), c | Xhat lo (3), f = X'.Xhat | Xdot (3), 1 - |Xdot| | X' (3),
+// rho^2.
+struct __align__(16) TreeRec {
+    float4 v[4];
+};
+// Cluster geometry: centre and tangent frame, half-sizes of the rectangle in stereographic
+// coordinates that holds the cluster's pixels (or its children's rectangles), and the float centre
+// with the near radius D that decides near and far.
+struct __align__(16) TreeGeo {
+    double n0[3], e1[3], e2[3], a1, a2;
+    double pad;
+    float4 c;    // n0, D
+    float4 l;    // n0 - (float)n0
+    float4 f1;   // e1, 1 / a1
+    float4 f2;   // e2, 1 / a2
+};
+
+// Work of one stage (a level's node sums, or the pixels): clusters with many samples are cut into
+// chunks, listed in the pool; the others are one item each.
+struct TreeWork {
+    const int *nch;        // chunks of a cluster
+    const int *pbase;      // first pool entry of a cluster with nch > 1
+    const int2 *pool;      // (cluster, chunk)
+    const int *npool;      // pool entries in use
+    int64_t ncl;
+};
+
+constexpr int kTreeS = 64;        // samples per tile of the scan
+constexpr int kTreeNT = 128;      // threads per CTA of the evaluation kernels
+constexpr int kTreeBatch = 128;   // samples per staged batch, one per thread
+constexpr int kTreeGroup = 32;    // candidate tiles tested sample by sample at a time
+constexpr int kTreeSuper = 32;    // tiles per super tile
+constexpr int kTreeList = kTreeGroup * kTreeS + kTreeBatch;
+
+// cos(pi m / 32): Chebyshev points x_k = cos(pi (2k + 1) / (2p)) and values T_i(x_k) for p = 8, 16
+__device__ __constant__ const double kCos32[64] = {
+    1.0, 0.99518472667219688624, 0.98078528040323044913, 0.95694033573220886494,
+    0.92387953251128675613, 0.88192126434835502971, 0.83146961230254523708, 0.77301045336273696081,
+    0.7071067811865475244, 0.63439328416364549822, 0.55557023301960222474, 0.47139673682599764856,
+    0.38268343236508977173, 0.29028467725446236764, 0.19509032201612826785, 0.098017140329560601994,
+    0.0, -0.098017140329560601994, -0.19509032201612826785, -0.29028467725446236764,
+    -0.38268343236508977173, -0.47139673682599764856, -0.55557023301960222474, -0.63439328416364549822,
+    -0.7071067811865475244, -0.77301045336273696081, -0.83146961230254523708, -0.88192126434835502971,
+    -0.92387953251128675613, -0.95694033573220886494, -0.98078528040323044913, -0.99518472667219688624,
+    -1.0, -0.99518472667219688624, -0.98078528040323044913, -0.95694033573220886494,
+    -0.92387953251128675613, -0.88192126434835502971, -0.83146961230254523708, -0.77301045336273696081,
+    -0.7071067811865475244, -0.63439328416364549822, -0.55557023301960222474, -0.47139673682599764856,
+    -0.38268343236508977173, -0.29028467725446236764, -0.19509032201612826785, -0.098017140329560601994,
+    0.0, 0.098017140329560601994, 0.19509032201612826785, 0.29028467725446236764,
+    0.38268343236508977173, 0.47139673682599764856, 0.55557023301960222474, 0.63439328416364549822,
+    0.7071067811865475244, 0.77301045336273696081, 0.83146961230254523708, 0.88192126434835502971,
+    0.92387953251128675613, 0.95694033573220886494, 0.98078528040323044913, 0.99518472667219688624};
+
+// T_i at the k-th of NP Chebyshev points (i = 1: the point itself)
+template <int NP>
+__device__ __forceinline__ double cheb_at(int i, int k)
+{
+    static_assert(32 % (2 * NP) == 0 || NP == 16, "kCos32 holds multiples of pi / 32");
+    return kCos32[(i * (2 * k + 1) * (16 / NP)) & 63];
+}
+
+// The near decision, by position and by beam: explicitly rounded operations, the same result in
+// every kernel.
+__device__ __forceinline__ bool tree_near_pos(const float4 &a, const float4 &c)
+{
+    const float dx = __fsub_rn(c.x, a.x), dy = __fsub_rn(c.y, a.y), dz = __fsub_rn(c.z, a.z);
+    const float d2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+    const float r = __fadd_rn(c.w, a.w);
+    return d2 < __fmul_rn(r, r);
+}
+// 2 B at the centre, and the decision from it
+__device__ __forceinline__ float tree_beam2(const float4 &b, const float4 &c)
+{
+    const float wx = __fsub_rn(c.x, b.x), wy = __fsub_rn(c.y, b.y), wz = __fsub_rn(c.z, b.z);
+    const float w2 = __fmaf_rn(wz, wz, __fmaf_rn(wy, wy, __fmul_rn(wx, wx)));
+    // 2 B = 2 (1 - v) + v |n0 + Xdot/v|^2 without cancellation
+    return __fmaf_rn(__fsub_rn(1.f, b.w), w2, __fmul_rn(2.f, b.w));
+}
+__device__ __forceinline__ bool tree_near_beam(const float4 &b, const float4 &c)
+{
+    return tree_beam2(b, c) < __fmul_rn(c.w, c.w);
+}
+
+// Whether a tile may hold a sample that is near, with margins.
+__device__ __forceinline__ bool tree_tile_pos(const TreeCap &t, const float4 &c)
+{
+    const float dx = c.x - t.a.x, dy = c.y - t.a.y, dz = c.z - t.a.z;
+    const float r = c.w + t.a.w + 1e-5f;
+    return t.a.w >= 0.f && dx * dx + dy * dy + dz * dz < r * r * 1.0001f;
+}
+__device__ __forceinline__ bool tree_tile_beam(const TreeCap &t, const float4 &c)
+{
+    const float b = 1.f + (c.x * t.a.x + c.y * t.a.y + c.z * t.a.z) - t.a.w;   // lower bound of B
+    return t.a.w >= 0.f && 2.f * b < c.w * c.w + 1e-5f;
+}
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+struct TreeScanSmem {
+    uint32_t list[kTreeList];
+    uint32_t cand[kTreeGroup * kTreeSuper];   // candidate tiles
+    uint32_t sup[kTreeNT];                    // candidate super tiles
+    int wcnt[kTreeNT / 32];
+    int tcnt[kTreeGroup];
+};
+
+// List entries: the record and, for LEAF, what the evaluation has to watch for at the cluster's pixels
+// (all within chord R of the centre): kTreeBeam when some B may be below b_min, kTreeClose when some
+// |d| may be below max(rho, R / 2).
+constexpr uint32_t kTreeBeam = 0x80000000u, kTreeClose = 0x40000000u, kTreeIndex = 0x3fffffffu;
+
+// Exclusive prefix of 32 counts (tcnt, in warp order) and their total, for every thread.
+__device__ __forceinline__ int tree_prefix(const int *tcnt, int &total)
+{
+    const int lane = threadIdx.x & 31;
+    const int own = tcnt[lane];
+    int incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    total = __shfl_sync(0xffffffffu, incl, 31);
+    return incl - own;
+}
+
+// Tests the samples of up to kTreeGroup tiles (tile(i), i < n) and appends those of the cluster to
+// sm.list after the `held` entries there; whole block, returns the new length.
+template <bool ROOT, bool LEAF, typename Tile>
+__device__ __forceinline__ int tree_select(const TreeSamples &S, int pass, const float4 self, const float4 outer,
+                                           float R, float beam2, int n, int held, TreeScanSmem &sm, Tile &&tile)
+{
+    constexpr int W = kTreeNT / 32, NR = kTreeGroup / W;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    const TreeCrit *crit = pass ? S.vcrit : S.crit;
+    unsigned mk[NR][2];
+    uint32_t fl = 0;   // two flag bits per tested sample
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+        const int idx = i * W + w;
+        mk[i][0] = mk[i][1] = 0u;
+        if (idx < n) {
+            const int64_t s = (int64_t)tile(idx) * kTreeS + lane;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float4 a = crit[s + 32 * h].a, b = crit[s + 32 * h].b;
+                bool sel = b.w < kCritSkip;
+                if (!ROOT) {
+                    const bool pos = tree_near_pos(a, outer);
+                    sel = sel && (pass ? !pos && tree_near_beam(b, outer) : pos);
+                }
+                if (!LEAF) {
+                    sel = sel && !tree_near_pos(a, self) && !tree_near_beam(b, self);
+                } else {
+                    if (tree_beam2(b, self) < beam2) fl |= 1u << (4 * i + 2 * h);
+                    float4 c = self;
+                    c.w = 1.5f * R + 1e-6f;   // the chord limit of tree_near_pos adds rho
+                    if (tree_near_pos(a, c)) fl |= 2u << (4 * i + 2 * h);
+                }
+                mk[i][h] = __ballot_sync(0xffffffffu, sel);
+            }
+        }
+        if (lane == 0) sm.tcnt[idx] = __popc(mk[i][0]) + __popc(mk[i][1]);
+    }
+    __syncthreads();
+    int total;
+    const int excl = tree_prefix(sm.tcnt, total);
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+        const int idx = i * W + w;
+        int pos = held + __shfl_sync(0xffffffffu, excl, idx);
+        if ((mk[i][0] | mk[i][1]) == 0u) continue;
+        const int64_t s = (int64_t)tile(idx) * kTreeS + lane;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (mk[i][h] >> lane & 1u)
+                sm.list[pos + __popc(mk[i][h] & below)] =
+                    (pass ? S.vidx[s + 32 * h] : (uint32_t)s + 32 * h) |
+                    (LEAF ? (fl >> (4 * i + 2 * h) & 1u) << 31 | (fl >> (4 * i + 2 * h + 1) & 1u) << 30 : 0u);
+            pos += __popc(mk[i][h]);
+        }
+    }
+    __syncthreads();
+    return held + total;
+}
+
+// Selects, in a fixed order, the samples of the tiles kc, kc + split, ... that belong to one cluster
+// (every split-th tile: strings are dense on a few clusters and consecutive in either order, so chunks
+// of consecutive tiles would leave all near samples of such a cluster in one chunk).  ROOT: all
+// samples far from it; LEAF: those near it; otherwise those near the parent and far from it.  The
+// position order gives all samples (ROOT) or those near by position, the velocity order those near by
+// beam only.  consume(n) is called by the whole block with n entries in sm.list: a multiple of
+// kTreeBatch, except for the last call.  Super tiles are tested first, 128 at a time, then the tiles of
+// 32 candidates, then the samples of 32 tiles; entries left over wait, so that batches stay full.
+template <bool ROOT, bool LEAF, typename Consume>
+__device__ __forceinline__ void tree_scan(const TreeSamples &S, int kc, int split, const float4 self,
+                                          const float4 parent, float R, float b_min, TreeScanSmem &sm,
+                                          Consume &&consume)
+{
+    constexpr int W = kTreeNT / 32, NR = kTreeGroup / W;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    const float4 outer = LEAF ? self : parent;
+    const float rb = sqrtf(2.f * b_min) * 1.001f + R + 1e-5f, beam2 = rb * rb;
+    int held = 0;
+    auto drain = [&]() {   // full batches
+        if (held < kTreeBatch) return;
+        const int full = held & ~(kTreeBatch - 1);
+        consume(full);
+        __syncthreads();
+        const int rem = held - full;
+        uint32_t v = 0;
+        if (tid < rem) v = sm.list[full + tid];
+        __syncthreads();
+        if (tid < rem) sm.list[tid] = v;
+        held = rem;
+        __syncthreads();
+    };
+    if (ROOT) {
+        const int64_t j1 = (S.nst - kc + split - 1) / split;   // tile j of the chunk is tile kc + j split
+#pragma unroll 1
+        for (int64_t g0 = 0; g0 < j1; g0 += kTreeGroup) {
+            const int n = (int)(j1 - g0 < kTreeGroup ? j1 - g0 : kTreeGroup);
+            held = tree_select<true, false>(S, 0, self, self, R, beam2, n, held, sm,
+                                            [&](int i) { return kc + (g0 + i) * split; });
+            drain();
+        }
+    } else {
+        const int nsup = (int)((S.nst + kTreeSuper - 1) / kTreeSuper);
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+            const TreeCap *caps = pass ? S.vcaps : S.caps, *sup = pass ? S.vsup : S.sup;
+#pragma unroll 1
+            for (int u0 = 0; u0 < nsup; u0 += kTreeNT) {
+                bool in = false;
+                if (u0 + tid < nsup) {
+                    const TreeCap cap = sup[u0 + tid];
+                    in = pass ? tree_tile_beam(cap, outer) : tree_tile_pos(cap, outer);
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, in);
+                if (lane == 0) sm.wcnt[w] = __popc(m);
+                __syncthreads();
+                int ns = 0, at = 0;
+#pragma unroll
+                for (int i = 0; i < W; ++i) {
+                    if (i == w) at = ns;
+                    ns += sm.wcnt[i];
+                }
+                if (in) sm.sup[at + __popc(m & below)] = u0 + tid;
+                __syncthreads();
+#pragma unroll 1
+                for (int v0 = 0; v0 < ns; v0 += kTreeGroup) {
+                    unsigned mk[NR];
+#pragma unroll
+                    for (int i = 0; i < NR; ++i) {
+                        const int idx = v0 + i * W + w;
+                        bool hit = false;
+                        if (idx < ns) {
+                            const uint32_t t = sm.sup[idx] * kTreeSuper + lane;
+                            if (t < (uint32_t)S.nst && (split == 1 || t % (uint32_t)split == (uint32_t)kc)) {
+                                const TreeCap cap = caps[t];
+                                hit = pass ? tree_tile_beam(cap, outer) : tree_tile_pos(cap, outer);
+                            }
+                        }
+                        mk[i] = __ballot_sync(0xffffffffu, hit);
+                        if (lane == 0) sm.tcnt[i * W + w] = __popc(mk[i]);
+                    }
+                    __syncthreads();
+                    int ncand;
+                    const int excl = tree_prefix(sm.tcnt, ncand);
+#pragma unroll
+                    for (int i = 0; i < NR; ++i) {
+                        const int pos = __shfl_sync(0xffffffffu, excl, i * W + w);
+                        if (mk[i] >> lane & 1u)
+                            sm.cand[pos + __popc(mk[i] & below)] = sm.sup[v0 + i * W + w] * kTreeSuper + lane;
+                    }
+                    __syncthreads();
+#pragma unroll 1
+                    for (int g0 = 0; g0 < ncand; g0 += kTreeGroup) {
+                        const int n = ncand - g0 < kTreeGroup ? ncand - g0 : kTreeGroup;
+                        held = tree_select<false, LEAF>(S, pass, self, outer, R, beam2, n, held, sm,
+                                                        [&](int i) { return sm.cand[g0 + i]; });
+                        drain();
+                    }
+                }
+            }
+        }
+    }
+    if (held > 0) consume(held);
+    __syncthreads();
+}
+
+// Item -> (cluster, chunk): pool entries first (the heavy clusters), then one item per cluster, -1 for
+// a cluster whose chunks are in the pool.  `at` is the slot of the item's sums.
+__device__ __forceinline__ int64_t tree_item(const TreeWork &W, int64_t item, int np, int &kc, int &nch, int64_t &at)
+{
+    if (item < np) {
+        const int2 e = W.pool[item];
+        kc = e.y;
+        nch = W.nch[e.x];
+        at = W.ncl + item;
+        return e.x;
+    }
+    const int64_t c = item - np;
+    kc = 0;
+    nch = W.nch[c];
+    at = c;
+    return nch == 1 ? c : -1;
+}
+
+// Dynamic distribution with the next item's number already on its way: the counter is read by thread 0
+// when an item starts and handed over when it ends.
+struct TreeQueue {
+    unsigned long long *counter;
+    unsigned long long nx;
+    __device__ __forceinline__ int64_t first(int64_t *slot)
+    {
+        if (threadIdx.x == 0) *slot = (int64_t)atomicAdd(counter, 1ull);
+        __syncthreads();
+        const int64_t item = *slot;
+        if (threadIdx.x == 0) nx = atomicAdd(counter, 1ull);
+        __syncthreads();
+        return item;
+    }
+    __device__ __forceinline__ int64_t next(int64_t *slot)
+    {
+        if (threadIdx.x == 0) *slot = (int64_t)nx;
+        __syncthreads();
+        const int64_t item = *slot;
+        if (threadIdx.x == 0) nx = atomicAdd(counter, 1ull);
+        __syncthreads();
+        return item;
+    }
+};
+
+// Values of cluster cl at its NP x NP nodes (the sum of its chunks) -> their Chebyshev coefficients in
+// shared memory (coef, tmp: NP * NP doubles); whole block.
+template <int NP>
+__device__ __forceinline__ void cheb_coefs(const double *__restrict__ F, const TreeWork &W, int64_t cl, double *coef,
+                                           double *tmp)
+{
+    constexpr int NN = NP * NP;
+    const int nch = W.nch[cl];
+    const int64_t at = nch == 1 ? cl : W.ncl + W.pbase[cl];
+    for (int k = threadIdx.x; k < NN; k += blockDim.x) {
+        double v = 0.0;
+        for (int c = 0; c < nch; ++c) v += F[(at + c) * NN + k];
+        coef[k] = v;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < NN; k += blockDim.x) {   // along xi: node k = j NP + i
+        const int j = k / NP, m = k % NP;
+        double v = 0.0;
+#pragma unroll
+        for (int i = 0; i < NP; ++i) v = fma(coef[j * NP + i], cheb_at<NP>(m, i), v);
+        tmp[k] = v * (m == 0 ? 1.0 / NP : 2.0 / NP);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < NN; k += blockDim.x) {
+        const int q = k / NP, m = k % NP;
+        double v = 0.0;
+#pragma unroll
+        for (int j = 0; j < NP; ++j) v = fma(tmp[j * NP + m], cheb_at<NP>(q, j), v);
+        coef[k] = v * (q == 0 ? 1.0 / NP : 2.0 / NP);
+    }
+    __syncthreads();
+}
+
+// Position (lx, ly) of slot l in a T x T block enumerated by anti-diagonals from the largest
+// lx + ly down (the slot order of the full-sky pixel tables).
+__device__ __forceinline__ void diag_slot_square(int l, int T, int &lx, int &ly)
+{
+    const int half = T * (T + 1) / 2;
+    const bool upper = l < half;
+    const int m = upper ? l : T * T - 1 - l;
+    int k = (int)((sqrtf(8.f * (float)m + 1.f) - 1.f) * 0.5f);
+    while (k * (k + 1) / 2 > m) --k;
+    while ((k + 1) * (k + 2) / 2 <= m) ++k;
+    const int o = m - k * (k + 1) / 2;
+    if (upper) {
+        lx = T - 1 - k + o;
+        ly = T - 1 - o;
+    } else {
+        lx = k - o;
+        ly = o;
+    }
+}
+
+}  // namespace isw
