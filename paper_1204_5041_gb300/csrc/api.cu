@@ -883,13 +883,13 @@ int isw_map_cl(isw_ctx *c, int64_t nside, const double *theta, int64_t lmax, dou
     int r;
     if ((r = set_device(c))) return r;
     const size_t L1 = (size_t)lmax + 1;
-    if ((r = ensure_ws(c, kWsClF, 2 * (size_t)(4 * nside - 1) * L1 * sizeof(double)))) return r;
+    if ((r = ensure_ws(c, kWsClF, cl_scratch_bytes(nside, lmax)))) return r;
     if (!alm) {
         if ((r = ensure_ws(c, kWsAlm, 2 * L1 * L1 * sizeof(double)))) return r;
         alm = (double *)c->ws[kWsAlm];
     }
-    launch_map_cl(nside, theta, lmax, (double *)c->ws[kWsClF], alm, cl, (cudaStream_t)stream);
-    c->n_launch += 3;
+    launch_map_cl(nside, theta, lmax, c->ws[kWsClF], alm, cl, (cudaStream_t)stream);
+    c->n_launch += 4;
     return check_launch(c, "isw_map_cl launch");
 }
 

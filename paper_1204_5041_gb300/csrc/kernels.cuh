@@ -47,9 +47,10 @@ void launch_map_flat(bool f64, const void *r32, const void *r64, const int64_t *
                      int split, int64_t M, double pitch, double *theta, double *partial, int accumulate,
                      DevStatus *st, unsigned long long *queue, uint32_t wait_polls, int grid, cudaStream_t s);
 
-// cl.cu: angular power spectrum (F: double[2][4N-1][lmax+1] workspace; alm: double[2][lmax+1][lmax+1])
+// cl.cu: angular power spectrum (scratch: cl_scratch_bytes; alm: double[2][lmax+1][lmax+1])
 int cl_max_nside();
-void launch_map_cl(int64_t N, const double *map, int64_t lmax, double *F, double *alm, double *cl, cudaStream_t s);
+size_t cl_scratch_bytes(int64_t N, int64_t lmax);
+void launch_map_cl(int64_t N, const double *map, int64_t lmax, void *scratch, double *alm, double *cl, cudaStream_t s);
 
 // lightcone.cu
 void launch_lightcone(int mode, const double *nodes, int64_t n, int64_t ld, const double *P, int64_t nloops,
