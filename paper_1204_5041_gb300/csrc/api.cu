@@ -194,45 +194,65 @@ void timing_end(isw_ctx *c, int k, cudaStream_t s)
 
 // Whether a map runs over the cluster tree (a variant or a chunk count set by the caller asks for the
 // direct kernels).
-bool use_tree(const isw_ctx *c, int64_t nside, int64_t npix, int64_t n, int prec, bool full_sky)
+bool use_tree(const isw_ctx *c, int64_t npix, int64_t n, int prec)
 {
-    return prec == ISW_F32C && full_sky && c->tile_override < 0 && c->split_override == 0 && tree_rule(nside, npix, n);
+    return c->split_override == 0 && (prec == ISW_F64 || c->tile_override < 0) && tree_rule(prec, npix, n) &&
+           npix < (int64_t(1) << 32);
 }
 
-// isw_map over the cluster tree of a full sky
-int map_tree_impl(isw_ctx *c, int64_t nside, const double *samples, int64_t n, int64_t ld, const double xo[3], double GU,
+// isw_map over the cluster tree: a full sky, a patch (M x M, one face), or a list or range of pixels in
+// spatial order.
+int map_tree_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_t *pix_list,
+                  const PatchSpec *patch, const double *samples, int64_t n, int64_t ld, const double xo[3], double GU,
                   int prec, int accumulate, double *theta, cudaStream_t s)
 {
-    const TreePlan p = tree_plan(prec, nside, 12, n, c->num_sms);
+    const bool full = !patch && !pix_list && pix0 == 0 && npix == 12 * nside * nside, list = !patch && !full;
+    const TreePlan p = tree_plan(prec, patch ? patch->M : nside, patch ? 1 : (full ? 12 : 0), npix, n, c->num_sms);
     const int64_t tot = p.ncl[0] * p.leaf * p.leaf;
+    const size_t sort_bytes = (sort_scratch_bytes(n, 2) + 255) / 256 * 256;
     int r;
     if ((r = ensure_ws(c, kWsNv, (size_t)tot * 3 * sizeof(double)))) return r;
     if ((r = ensure_ws(c, kWsOut, (size_t)tot * sizeof(int64_t)))) return r;
     if ((r = ensure_ws(c, kWsS32, (size_t)p.n_pad * sizeof(Seg32)))) return r;
     if ((r = ensure_ws(c, kWsS64, (size_t)p.n_pad * sizeof(Seg64)))) return r;
-    if ((r = ensure_ws(c, kWsSort, sort_scratch_bytes(n, 2)))) return r;
+    if (prec == ISW_F64 && (r = ensure_ws(c, kWsFar64, (size_t)p.n_pad * sizeof(Far64)))) return r;
+    if ((r = ensure_ws(c, kWsSort, sort_bytes + (list ? sort_scratch_bytes(npix, 1) : 0)))) return r;
     if ((r = ensure_ws(c, kWsTree, p.bytes))) return r;
     TreeMapArgs m{};
-    m.theta_pix = std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
+    m.theta_pix = patch ? patch->width / (double)patch->M : std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
     double *nv = (double *)c->ws[kWsNv];
     int64_t *outidx = (int64_t *)c->ws[kWsOut];
     Seg32 *s32 = (Seg32 *)c->ws[kWsS32];
     Seg64 *s64 = (Seg64 *)c->ws[kWsS64];
-    launch_pixel_table(nside, 0, 0, 12 * nside * nside, nullptr, p.leaf, p.leaf, p.ncl[0], nv, tot, outidx,
-                       nullptr, c->d_status, s);
-    const uint32_t *perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], c->ws[kWsSort], 2, s);
+    Far64 *far64 = prec == ISW_F64 ? (Far64 *)c->ws[kWsFar64] : nullptr;
+    unsigned char *sort = (unsigned char *)c->ws[kWsSort];
+    if (patch) {
+        launch_patch_table(*patch, p.leaf, p.leaf, p.ncl[0], nv, tot, outidx, nullptr, s);
+        m.order = kSlotsRows;
+    } else if (full) {
+        launch_pixel_table(nside, 0, 0, npix, nullptr, p.leaf, p.leaf, p.ncl[0], nv, tot, outidx, nullptr, c->d_status, s);
+        m.order = kSlotsDiag;
+    } else {
+        const uint32_t *pp = launch_pixel_order(nside, pix0, npix, pix_list, sort + sort_bytes, s);
+        launch_pixel_table(nside, pix_list ? 2 : 1, pix0, npix, pix_list, p.leaf, p.leaf, p.ncl[0], nv, tot, outidx,
+                           nullptr, c->d_status, s, pp);
+        m.order = kSlotsList;
+        c->n_launch += spatial_order_launches();
+    }
+    const uint32_t *perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], sort, 2, s);
     launch_pack(samples, n, ld, xo[0], xo[1], xo[2], GU, m.theta_pix, c->near_k, p.n_pad, perm, s32, s64, nullptr, nullptr,
-                nullptr, c->d_status, s);
+                far64, c->d_status, s);
     c->n_launch += spatial_order_launches() + 2;
     m.nv = nv;
     m.ldn = tot;
     m.outidx = outidx;
-    m.diag = 1;
     m.s32 = s32;
     m.s64 = s64;
+    m.far64 = far64;
     m.perm = perm;
     m.n = n;
     m.b_min = (float)c->b_min;
+    m.d_far = (float)c->d_far;
     m.theta = theta;
     m.accumulate = accumulate;
     m.st = c->d_status;
@@ -260,8 +280,8 @@ int map_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_
         }
         return ISW_OK;
     }
-    if (tune_waves == 0 && !patch && use_tree(c, nside, npix, n, prec, !pix_list && pix0 == 0 && npix == 12 * nside * nside))
-        return map_tree_impl(c, nside, samples, n, ld, xo, GU, prec, accumulate, theta, s);
+    if (tune_waves == 0 && use_tree(c, npix, n, prec))
+        return map_tree_impl(c, nside, pix0, npix, pix_list, patch, samples, n, ld, xo, GU, prec, accumulate, theta, s);
     int vidx = 0;
     if (prec == ISW_F32C) {
         if (c->tile_override >= 0 && c->tile_override < num_f32_variants()) vidx = c->tile_override;
@@ -1078,7 +1098,7 @@ int isw_map_batched(isw_ctx *c, int64_t nside, const double *nodes, int64_t ld, 
 
     // autotuner: time every FP32 variant on a prefix of the samples, keep the fastest
     if ((flags & ISW_AUTOTUNE) && prec == ISW_F32C && n > 0 && c->tile_override < 0 &&
-        !use_tree(c, nside, npix, n, prec, true) &&
+        !use_tree(c, npix, n, prec) &&
         !(c->tuned_nside == nside && c->tuned_n == n)) {
         if (!skip_lc) {
             launch_lightcone_shells(nodes, n, ld, d_off, nshell, d_tbox, d_mode, loop_params, nloops, ldp, xo[0],

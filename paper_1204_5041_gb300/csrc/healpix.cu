@@ -48,10 +48,10 @@ __device__ __forceinline__ void diag_slot(int l, int tx, int ty, int &lx, int &l
 // index its value is written to (RING index for full-sky maps, list position otherwise),
 // or -1 for padding.  Full-sky tiles are tx x ty blocks of face coordinates (compact
 // patches) with their slots in anti-diagonal (RING-following) order; range / list tiles are
-// consecutive chunks of tx*ty pixels.
+// consecutive chunks of tx*ty pixels, in the order perm when one is given.
 __global__ void k_pixel_table(int64_t N, int mode, int64_t pix0, int64_t npix, const int64_t *__restrict__ pix_list,
                               int tx, int ty, int64_t ntiles, double *__restrict__ nv, int64_t ldn,
-                              int64_t *__restrict__ outidx, DevStatus *st)
+                              int64_t *__restrict__ outidx, const uint32_t *__restrict__ perm, DevStatus *st)
 {
     const int tile_sz = tx * ty;
     const int64_t total = ntiles * tile_sz;
@@ -73,8 +73,9 @@ __global__ void k_pixel_table(int64_t N, int mode, int64_t pix0, int64_t npix, c
                 oi = ring;
             }
         } else if (k < npix) {
-            ring = (mode == 2) ? pix_list[k] : pix0 + k;
-            oi = k;
+            const int64_t pos = perm ? (int64_t)perm[k] : k;   // position in the list or range
+            ring = (mode == 2) ? pix_list[pos] : pix0 + pos;
+            oi = pos;
             if (ring < 0 || ring >= npix_all) {
                 atomicOr(&st->bits, kStatBadIndex);
                 ring = -1;
@@ -179,7 +180,7 @@ void launch_patch_table(const PatchSpec &p, int tx, int ty, int64_t ntiles, doub
     int64_t blocks = (total + 255) / 256;
     if (blocks > 152 * 64) blocks = 152 * 64;
     k_patch_table<<<(unsigned)blocks, 256, 0, s>>>(p, tx, ty, ntiles, nv, ldn, outidx);
-    k_pixel_caps<<<(unsigned)ntiles, 256, 0, s>>>(nv, ldn, outidx, tx * ty, caps);
+    if (caps) k_pixel_caps<<<(unsigned)ntiles, 256, 0, s>>>(nv, ldn, outidx, tx * ty, caps);
 }
 
 int launch_pix2vec(int64_t N, int64_t pix0, int64_t npix, const int64_t *pix_list, double *out, int64_t ld,
@@ -195,14 +196,14 @@ int launch_pix2vec(int64_t N, int64_t pix0, int64_t npix, const int64_t *pix_lis
 
 void launch_pixel_table(int64_t N, int mode, int64_t pix0, int64_t npix, const int64_t *pix_list, int tx, int ty,
                         int64_t ntiles, double *nv, int64_t ldn, int64_t *outidx, float4 *caps, DevStatus *st,
-                        cudaStream_t s)
+                        cudaStream_t s, const uint32_t *perm)
 {
     const int64_t total = ntiles * tx * ty;
     const int threads = 256;
     int64_t blocks = (total + threads - 1) / threads;
     if (blocks > 152 * 64) blocks = 152 * 64;
     k_pixel_table<<<(unsigned)blocks, threads, 0, s>>>(N, mode, pix0, npix, pix_list, tx, ty, ntiles, nv, ldn, outidx,
-                                                       st);
+                                                       perm, st);
     if (caps) k_pixel_caps<<<(unsigned)ntiles, 256, 0, s>>>(nv, ldn, outidx, tx * ty, caps);
 }
 

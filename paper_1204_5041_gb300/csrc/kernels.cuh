@@ -21,7 +21,7 @@ int launch_pix2vec(int64_t N, int64_t pix0, int64_t npix, const int64_t *pix_lis
                    DevStatus *st, cudaStream_t s);
 void launch_pixel_table(int64_t N, int mode, int64_t pix0, int64_t npix, const int64_t *pix_list, int tx, int ty,
                         int64_t ntiles, double *nv, int64_t ldn, int64_t *outidx, float4 *caps, DevStatus *st,
-                        cudaStream_t s);
+                        cudaStream_t s, const uint32_t *perm = nullptr);
 
 // A gnomonic patch: orthonormal frame (e1, e2, e3) with e3 the centre, M x M pixels of
 // coordinate pitch width / M; pixel (i, j) at (xi, eta) = ((i + 1/2 - M/2), (j + 1/2 - M/2)) * pitch,
@@ -89,6 +89,9 @@ size_t sort_scratch_bytes(int64_t n, int orders);
 const uint32_t *launch_spatial_order(const double *S, int64_t n, int64_t ld, double xo0, double xo1, double xo2,
                                      void *scratch, int orders, cudaStream_t s);
 int spatial_order_launches();
+// the same for the selected pixels (a range, or a list when pix_list is given): perm[npix] of positions
+const uint32_t *launch_pixel_order(int64_t N, int64_t pix0, int64_t npix, const int64_t *pix_list, void *scratch,
+                                   cudaStream_t s);
 
 // pack.cu: per-sample records of the map kernels and per-tile caps
 // perm (may be NULL): record s is built from sample perm[s] (else from sample s)
@@ -143,19 +146,22 @@ void launch_reduce_partials(const MapArgs &a, int tile_sz, cudaStream_t s);
 
 // tree.cu: the map over a cluster tree of the pixels
 constexpr int kTreeLevels = 20;
-constexpr int64_t kTreeMinSide = 32;
-constexpr double kTreeMinPairs = 1e8;
-// Whether a full-sky FP32 map of default settings runs over the tree: from 1e8 pairs, where its dozen
-// extra launches (0.15 ms) are made up for (N_side 64 with 10,240 samples, 5e8 pairs: 0.6 against 2.5
-// ms).  The list entries hold 30-bit record numbers.
-inline bool tree_rule(int64_t nside, int64_t npix, int64_t n)
+// Whether a map of default settings runs over the tree: from 1e8 pairs in FP32, where its dozen extra
+// launches (0.15 ms) are made up for (N_side 64 with 10,240 samples, 5e8 pairs: 0.6 against 2.5 ms), and
+// from 2e7 in FP64; with enough pixels for the leaves' nodes to be fewer than the pixels.  The list
+// entries hold 30-bit record numbers.
+inline bool tree_rule(int prec, int64_t npix, int64_t n)
 {
-    return nside >= kTreeMinSide && npix == 12 * nside * nside && (double)npix * (double)n >= kTreeMinPairs &&
+    const bool f64 = prec == ISW_F64;
+    return npix >= (f64 ? 48 * 1024 : 12 * 1024) && (double)npix * (double)n >= (f64 ? 2e7 : 1e8) &&
            n < (int64_t(1) << 30);
 }
+// slot order of the pixel tables: anti-diagonals (full sky), rows (patch), spatially sorted list
+enum : int { kSlotsDiag = 0, kSlotsRows = 1, kSlotsList = 2 };
 struct TreePlan {
-    int leaf, nn, nface, levels;          // leaf side in pixels, nodes per cluster
-    int nb[kTreeLevels];                  // clusters per face side, from the finest level
+    int prec;
+    int leaf, nn, levels;                 // leaf side in pixels, doubles per cluster's node sums
+    int nb[kTreeLevels];                  // clusters per face side, from the finest level (0: a list)
     int64_t ncl[kTreeLevels];             // clusters of the level
     int64_t n_pad, nst;                   // padded samples, sample tiles
     int nslots, pslots;                   // resident CTAs of the node and pixel kernels
@@ -167,20 +173,22 @@ struct TreeMapArgs {
     const double *nv;         // pixel table: leaf x leaf slots per finest cluster, clusters in (face, y, x) order
     int64_t ldn;
     const int64_t *outidx;
-    int diag;                 // slots in anti-diagonal order (full sky) or row by row (patch)
+    int order;                // slots of a cluster
     double theta_pix;
     const Seg32 *s32;
     const Seg64 *s64;
+    const Far64 *far64;       // FP64 maps
     const uint32_t *perm;     // sample of each record, and of each velocity-order entry (perm + n)
     int64_t n;
-    float b_min;
+    float b_min, d_far;
     double *theta;
     int accumulate;
     DevStatus *st;
     void *scratch;            // TreePlan::bytes
 };
 int tree_leaf(int prec);
-TreePlan tree_plan(int prec, int64_t N, int nface, int64_t n, int num_sms);
+// nface faces of N x N pixels, or (nface = 0) a list of npix
+TreePlan tree_plan(int prec, int64_t N, int nface, int64_t npix, int64_t n, int num_sms);
 cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_t s);
 inline int tree_launches(const TreePlan &p) { return 2 * p.levels + 7; }
 

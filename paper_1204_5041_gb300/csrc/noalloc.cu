@@ -99,12 +99,13 @@ int finish(void *base, int32_t *status_out, cudaStream_t s)
     return ISW_OK;
 }
 
-// A full-sky map over the cluster tree, with isw_map's launch sequence; ISW_EINVAL when it does not fit
+// A map over the cluster tree, with isw_map's launch sequence; ISW_EINVAL when it does not fit
 // the scratch (the direct kernels, which need less, are then tried).
-int map_tree_noalloc(int64_t nside, const double *samples, int64_t n, int64_t ld, const double *x_obs, double GU,
+int map_tree_noalloc(int64_t nside, int64_t pix0, int64_t npix, const double *samples, int64_t n, int64_t ld, const double *x_obs, double GU,
                      double *theta, unsigned char *b, int sms, cudaStream_t s)
 {
-    const TreePlan p = tree_plan(ISW_F32C, nside, 12, n, sms);
+    const bool full = pix0 == 0 && npix == 12 * nside * nside;
+    const TreePlan p = tree_plan(ISW_F32C, nside, full ? 12 : 0, npix, n, sms);
     const int64_t tot = p.ncl[0] * p.leaf * p.leaf;
     size_t at = up256(sizeof(DevStatus));
     auto take = [&](size_t bytes) {
@@ -115,19 +116,21 @@ int map_tree_noalloc(int64_t nside, const double *samples, int64_t n, int64_t ld
     const size_t off_nv = take((size_t)tot * 3 * sizeof(double)), off_out = take((size_t)tot * sizeof(int64_t));
     const size_t off_s32 = take((size_t)p.n_pad * sizeof(Seg32)), off_s64 = take((size_t)p.n_pad * sizeof(Seg64));
     const size_t off_sort = take(sort_scratch_bytes(n, 2)), off_tree = take(p.bytes);
+    const size_t off_psort = full ? 0 : take(sort_scratch_bytes(npix, 1));
     if (at > kStaticScratchBytes) return ISW_EINVAL;
     DevStatus *st = (DevStatus *)b;
     if (cudaMemsetAsync(st, 0, sizeof(DevStatus), s) != cudaSuccess) return ISW_ECUDA;
     const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
     TreeMapArgs m{};
     m.theta_pix = std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
-    launch_pixel_table(nside, 0, 0, 12 * nside * nside, nullptr, p.leaf, p.leaf, p.ncl[0], (double *)(b + off_nv), tot,
-                       (int64_t *)(b + off_out), nullptr, st, s);
+    const uint32_t *pp = full ? nullptr : launch_pixel_order(nside, pix0, npix, nullptr, b + off_psort, s);
+    launch_pixel_table(nside, full ? 0 : 1, pix0, npix, nullptr, p.leaf, p.leaf, p.ncl[0], (double *)(b + off_nv), tot,
+                       (int64_t *)(b + off_out), nullptr, st, s, pp);
     m.perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], b + off_sort, 2, s);
     m.nv = (const double *)(b + off_nv);
     m.ldn = tot;
     m.outidx = (const int64_t *)(b + off_out);
-    m.diag = 1;
+    m.order = full ? kSlotsDiag : kSlotsList;
     m.s32 = (const Seg32 *)(b + off_s32);
     m.s64 = (const Seg64 *)(b + off_s64);
     launch_pack(samples, n, ld, xo[0], xo[1], xo[2], GU, m.theta_pix, kNearK, p.n_pad, m.perm, (Seg32 *)(b + off_s32),
@@ -167,8 +170,8 @@ extern "C" int isw_map_f32c_noalloc(int64_t nside, int64_t pix0, int64_t npix, c
     int sms = 0;
     int r = scratch_address(dev, &base, &sms);
     if (r) return r;
-    if (pix0 == 0 && tree_rule(nside, npix, n)) {   // the cluster tree, as isw_map, when it fits
-        r = map_tree_noalloc(nside, samples, n, ld, x_obs, GU, theta_out, (unsigned char *)base, sms, s);
+    if (tree_rule(ISW_F32C, npix, n)) {   // the cluster tree, as isw_map, when it fits
+        r = map_tree_noalloc(nside, pix0, npix, samples, n, ld, x_obs, GU, theta_out, (unsigned char *)base, sms, s);
         if (r != ISW_EINVAL) return r == ISW_OK ? finish(base, status_out, s) : r;
     }
 

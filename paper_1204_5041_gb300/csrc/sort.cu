@@ -161,6 +161,63 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const uint32_t *_
         __syncthreads();
     }
 }
+// Keys of pixels: the Morton code of the centre, from float coordinates (they only order the pixels).
+__global__ void k_pixel_keys(int64_t N, int64_t pix0, int64_t npix, const int64_t *__restrict__ pix_list,
+                             uint32_t *__restrict__ key, uint32_t *__restrict__ idx)
+{
+    const int64_t all = 12 * N * N, cap = 2 * N * (N - 1);
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < npix; k += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t p = pix_list ? pix_list[k] : pix0 + k;
+        uint32_t v = kInvalidKey;
+        if (p >= 0 && p < all) {
+            float z, phi;
+            if (p >= cap && p < all - cap) {
+                const int64_t q = p - cap;
+                z = (float)((4.0 * (double)N - 2.0 * (double)(q / (4 * N) + N)) / (3.0 * (double)N));
+                phi = (float)(q % (4 * N)) / (float)(4 * N);
+            } else {
+                const int64_t q = p < cap ? p : all - 1 - p, i = (1 + isqrt64(1 + 2 * q)) / 2;
+                const float t = (float)i / (float)N;
+                z = 1.f - t * t / 3.f;
+                phi = ((float)(q - 2 * i * (i - 1)) + 0.5f) / (float)(4 * i);
+                if (p >= cap) {
+                    z = -z;
+                    phi = 1.f - phi;
+                }
+            }
+            const float st = sqrtf(fmaxf(1.f - z * z, 0.f));
+            float s, c;
+            sincospif(2.f * phi, &s, &c);
+            v = morton(st * c, st * s, z);
+        }
+        key[k] = v;
+        idx[k] = (uint32_t)k;
+    }
+}
+
+// Sorts the key arrays in the scratch (orders of n each); returns the sorted indices.
+const uint32_t *sort_passes(int64_t n, int orders, uint32_t *p, cudaStream_t s)
+{
+    const int64_t nblocks = (n + kSortBlock - 1) / kSortBlock, m = orders * n;
+    uint32_t *key[2] = {p, p + m}, *idx[2] = {p + 2 * m, p + 3 * m};
+    uint32_t *hist = p + 4 * m, *tot = hist + (int64_t)orders * kRadix * nblocks;
+    int cur = 0;
+    const dim3 grid((unsigned)nblocks, orders);
+    for (int shift = 0; shift < 24; shift += 8) {
+        k_sort_hist<<<grid, kSortThreads, 0, s>>>(key[cur], n, shift, hist, (int)nblocks);
+        k_sort_scan<<<dim3(kRadix, orders), kSortThreads, 0, s>>>(hist, (int)nblocks, tot);
+        k_sort_scatter<<<grid, kSortThreads, 0, s>>>(key[cur], idx[cur], n, shift, hist, tot, (int)nblocks, key[cur ^ 1],
+                                                     idx[cur ^ 1]);
+        cur ^= 1;
+    }
+    return idx[cur];
+}
+
+unsigned key_blocks(int64_t n)
+{
+    const int64_t b = (n + 255) / 256;
+    return (unsigned)(b < 152 * 32 ? b : 152 * 32);
+}
 }  // namespace
 
 size_t sort_scratch_bytes(int64_t n, int orders)
@@ -173,23 +230,17 @@ const uint32_t *launch_spatial_order(const double *S, int64_t n, int64_t ld, dou
                                      void *scratch, int orders, cudaStream_t s)
 {
     if (n <= 0) return nullptr;
-    const int64_t nblocks = (n + kSortBlock - 1) / kSortBlock, m = orders * n;
     uint32_t *p = reinterpret_cast<uint32_t *>(scratch);
-    uint32_t *key[2] = {p, p + m}, *idx[2] = {p + 2 * m, p + 3 * m};
-    uint32_t *hist = p + 4 * m, *tot = hist + (int64_t)orders * kRadix * nblocks;
-    int64_t kb = (n + 255) / 256;
-    if (kb > 152 * 32) kb = 152 * 32;
-    k_sort_keys<<<dim3((unsigned)kb, orders), 256, 0, s>>>(S, n, ld, xo0, xo1, xo2, key[0], idx[0]);
-    int cur = 0;
-    const dim3 grid((unsigned)nblocks, orders);
-    for (int shift = 0; shift < 24; shift += 8) {
-        k_sort_hist<<<grid, kSortThreads, 0, s>>>(key[cur], n, shift, hist, (int)nblocks);
-        k_sort_scan<<<dim3(kRadix, orders), kSortThreads, 0, s>>>(hist, (int)nblocks, tot);
-        k_sort_scatter<<<grid, kSortThreads, 0, s>>>(key[cur], idx[cur], n, shift, hist, tot, (int)nblocks, key[cur ^ 1],
-                                                     idx[cur ^ 1]);
-        cur ^= 1;
-    }
-    return idx[cur];
+    k_sort_keys<<<dim3(key_blocks(n), orders), 256, 0, s>>>(S, n, ld, xo0, xo1, xo2, p, p + 2 * orders * n);
+    return sort_passes(n, orders, p, s);
+}
+
+const uint32_t *launch_pixel_order(int64_t N, int64_t pix0, int64_t npix, const int64_t *pix_list, void *scratch,
+                                   cudaStream_t s)
+{
+    uint32_t *p = reinterpret_cast<uint32_t *>(scratch);
+    k_pixel_keys<<<key_blocks(npix), 256, 0, s>>>(N, pix0, npix, pix_list, p, p + 2 * npix);
+    return sort_passes(npix, 1, p, s);
 }
 
 int spatial_order_launches() { return 1 + 3 * 3; }

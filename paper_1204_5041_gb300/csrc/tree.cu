@@ -22,14 +22,16 @@ namespace isw {
 
 namespace {
 
-// Near radius in stereographic half-sizes: 4 gives 2.2e-8 of the rms at N_side 100 and 10.1 ms at N_side 512
+// Near radius in stereographic half-sizes.  FP32 (8 x 8 nodes): 4 gives 2.2e-8 of the rms at N_side 100 and 10.1 ms at N_side 512
 // with 2e5 samples, 3.5 2.6e-8 and 9.2 ms, 3 5.1e-8 and 8.5 ms.
-constexpr double kKappa = 3.5;
+// FP64 (16 x 16 nodes): in 80-bit arithmetic, with clusters set next to the strings, the truncation is
+// 9e-16 of the rms at 4 and 1e-17 at 5; 4.5 keeps it below the rounding of the sums.
+constexpr double kKappa32 = 3.5, kKappa64 = 4.5;
 
-__device__ __forceinline__ double near_radius(double a)
+__device__ __forceinline__ double near_radius(double kappa, double a)
 {
     // chord of stereographic radius kappa a
-    const double z = kKappa * a;
+    const double z = kappa * a;
     return 2.0 * z / sqrt(1.0 + z * z);
 }
 
@@ -211,8 +213,8 @@ __device__ __forceinline__ void finish_geo(TreeGeo &g, double D)
 // centre and frame, and the extents are measured from the pixels afterwards.
 template <int T>
 __global__ void __launch_bounds__(T *T / 4) k_tree_leaf_geo(const double *__restrict__ nv, int64_t ldn,
-                                                            const int64_t *__restrict__ outidx, int diag,
-                                                            double theta_pix, TreeGeo *__restrict__ geo)
+                                                            const int64_t *__restrict__ outidx, int order,
+                                                            double theta_pix, double kappa, TreeGeo *__restrict__ geo)
 {
     constexpr int NT = T * T / 4, W = NT / 32;
     __shared__ float red[6][W];
@@ -223,10 +225,11 @@ __global__ void __launch_bounds__(T *T / 4) k_tree_leaf_geo(const double *__rest
     for (int l = tid; l < T * T; l += NT) {
         const int64_t k = t * T * T + l;
         if (outidx[k] < 0) continue;
-        int lx, ly;
-        if (diag) diag_slot_square(l, T, lx, ly);
-        else lx = l % T;
-        const float f = (float)lx - 0.5f * (float)(T - 1);
+        int lx = T / 2, ly;
+        if (order == kSlotsDiag) diag_slot_square(l, T, lx, ly);
+        else if (order == kSlotsRows) lx = l % T;
+        // a list has no axis of its own: the frame is then any
+        const float f = order == kSlotsList ? 0.f : (float)lx - 0.5f * (float)(T - 1);
         for (int c = 0; c < 3; ++c) {
             const float v = (float)nv[c * ldn + k];
             s[c] += v;
@@ -277,26 +280,36 @@ __global__ void __launch_bounds__(T *T / 4) k_tree_leaf_geo(const double *__rest
         // margin for the float arithmetic; a single pixel still gets a square of a quarter pixel
         g.a1 = fmax((double)m1 * 1.00001, 0.125 * theta_pix);
         g.a2 = fmax((double)m2 * 1.00001, 0.125 * theta_pix);
-        finish_geo(g, near_radius(fmax(g.a1, g.a2)) * 1.00001 + 1e-7);
+        finish_geo(g, near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7);
         geo[t] = g;
     }
 }
 
-// One warp per parent cluster (nb x nb per face) of the child level (cnb x cnb per face): lane l
+// One warp per parent cluster (tree_parent of the child level): lane l
 // takes point l % 8 (corners and edge midpoints) of the rectangle of child l / 8.  Offsets from the
 // parent's centre are differences of FP64 centres plus a float offset, so they keep their relative
 // accuracy for small clusters.
-__global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__ child, int cnb,
-                                                     TreeGeo *__restrict__ geo, int nb, int nface)
+__global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__ child, int cnb, int64_t cncl,
+                                                     TreeGeo *__restrict__ geo, int nb, int64_t ncl, double kappa)
 {
     const int lane = threadIdx.x & 31;
     const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (t >= (int64_t)nface * nb * nb) return;
-    const int64_t f = t / (nb * nb);
-    const int by = (int)(t - f * nb * nb) / nb, bx = (int)(t - f * nb * nb) % nb;
-    const int i = 2 * bx + (lane >> 3 & 1), j = 2 * by + (lane >> 4);
-    const bool has = i < cnb && j < cnb;
-    const TreeGeo k = child[has ? (f * cnb + j) * cnb + i : (f * cnb + 2 * by) * cnb + 2 * bx];
+    if (t >= ncl) return;
+    int64_t kid, kid0;
+    bool has;
+    if (nb == 0) {
+        kid0 = 4 * t;
+        kid = kid0 + (lane >> 3);
+        has = kid < cncl;
+    } else {
+        const int64_t f = t / ((int64_t)nb * nb);
+        const int by = (int)(t - f * nb * nb) / nb, bx = (int)(t - f * nb * nb) % nb;
+        const int i = 2 * bx + (lane >> 3 & 1), j = 2 * by + (lane >> 4);
+        has = i < cnb && j < cnb;
+        kid = (f * cnb + j) * cnb + i;
+        kid0 = (f * cnb + 2 * by) * cnb + 2 * bx;
+    }
+    const TreeGeo k = child[has ? kid : kid0];
     const float on = has && (lane & 7) == 0 ? 1.f : 0.f;
     const float cx = warp_sum(on * k.c.x), cy = warp_sum(on * k.c.y), cz = warp_sum(on * k.c.z);
     const float ux = warp_sum(on * k.f1.x), uy = warp_sum(on * k.f1.y), uz = warp_sum(on * k.f1.z);
@@ -316,7 +329,7 @@ __global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__
     g.a2 = (double)warp_max(m2) * 1.002;
     // near at a child implies near here
     const float cd = (k.c.w + sqrtf(d0 * d0 + d1 * d1 + d2 * d2)) * 1.00003f + 2e-6f;
-    const double D = fmax(near_radius(fmax(g.a1, g.a2)) * 1.00001 + 1e-7, (double)warp_max(cd));
+    const double D = fmax(near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7, (double)warp_max(cd));
     if (lane == 0) {
         finish_geo(g, D);
         geo[t] = g;
@@ -513,10 +526,8 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_nodes_f32(TreeNodeArgs a)
         int64_t at;
         const int64_t cl = tree_item(a.W, item, np, kc, nch, at);
         if (cl < 0) continue;
-        int64_t pcl = 0;
+        const int64_t pcl = ROOT ? 0 : tree_parent(cl, a.nb, a.pnb);
         if (!ROOT) {
-            const int64_t f = cl / ((int64_t)a.nb * a.nb), rem = cl - f * a.nb * a.nb;
-            pcl = (f * a.pnb + rem / a.nb / 2) * a.pnb + rem % a.nb / 2;
             load_geo(&sm.pgeo, a.pgeo + pcl);
         }
         load_geo(&sm.geo, a.geo + cl);
@@ -563,7 +574,7 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_nodes_f32(TreeNodeArgs a)
                 }
             });
         };
-        tree_scan<ROOT, false>(a.S, kc, nch, self, parent, 0.f, 0.f, sm.scan, consume);
+        tree_scan<ROOT, false>(a.S, kc, nch, self, parent, 0.f, 0.f, 0.f, sm.scan, consume);
         double (*red)[kNN] = reinterpret_cast<double (*)[kNN]>(sm.rec);   // the batches are done
 #pragma unroll
         for (int q = 0; q < 4; ++q) red[2 * w + half][16 * q + hl] = (double)ahi[q] + (double)alo[q];
@@ -813,7 +824,8 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_pixels_f32(TreePixArgs a)
                 }
             });
         };
-        tree_scan<false, true>(a.S, kc, nch, self, self, target_radius(sm.geo), a.b_min, sm.scan, consume);
+        const float R = target_radius(sm.geo);
+        tree_scan<false, true>(a.S, kc, nch, self, self, R, 1.5f * R, a.b_min, sm.scan, consume);
         if (qlen > 0) near_flush(nq, qlen, a.s64, a.nv, a.ldn, kw, zerocnt);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {   // both half-warps' sums of a pixel; half q / 2 writes it
@@ -840,20 +852,409 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_pixels_f32(TreePixArgs a)
     }
 }
 
-// theta of the clusters that were cut into chunks: their partial sums added in chunk order.
-__global__ void __launch_bounds__(kLeaf *kLeaf) k_tree_reduce(TreeWork W, const double *__restrict__ partial,
-                                                              const int64_t *__restrict__ outidx,
-                                                              double *__restrict__ theta, int accumulate)
+// ------------------------------------------------------------------------------------
+// FP64 maps: 16 x 16 nodes, leaves of 32 x 32 pixels.  The FP64 unit (two FMA lanes per clock and SM)
+// is all that counts, so every thread simply holds its nodes or pixels and reads one staged sample at
+// a time.  N_side 64 with 10,240 samples 18.3 -> 14.4 ms (a leaf of 32 pixels spans 0.5 rad there and four
+// tenths of the pairs stay near), N_side 128 with 25,087 170 -> 57 ms.  Error against the oracle 1.2e-16
+// to 1.7e-16 of the rms (direct kernel 0.5e-16 to 1.2e-16), largest 1.3e-15 (1.0e-15).
+// ------------------------------------------------------------------------------------
+constexpr int kNP64 = 16, kNN64 = kNP64 * kNP64, kLeaf64 = 32;
+constexpr int kNodeTarget64 = 128, kPixTarget64 = 48;
+
+// One staged sample: a Far64 or Seg64 record (pixels), or the sample relative to the cluster's centre
+// (nodes): 2D (3), K, Xdot (3), P, X' (3), Q, B0, f, c, see the FP32 entries; or, on clusters at least
+// d_far from their samples, in completed squares with sigma = sign c, s = sqrt(|c|/2):
+// sigma 2D (3), sigma K, s Xdot (3), s (B0 + P)/2, s X' (3), s (Q + f/2), 1/s, e/2, s^2 (f^2 - e^2)/4, sigma.
+// Nodes always take the offset m from the centre and not the rounded direction: the rounding of a
+// direction moves a node by 5e-17, and the interpolant's values by that times the slope (2e-16 of the
+// rms).
+struct __align__(16) Stage64 {
+    double v[16];
+};
+static_assert(sizeof(Far64) <= sizeof(Stage64) && sizeof(Seg64) == sizeof(Stage64), "stage layout");
+
+struct __align__(16) TreeSmem64 {
+    Stage64 rec[kTreeBatch];
+    TreeScanSmem scan;
+    TreeGeo geo, pgeo;
+    double coef[kNN64], tmp[kNN64];
+    int64_t item;
+};
+
+// the interpolant with the shared coefficients at (x, y) in [-1, 1]^2: Clenshaw's recurrence in y, rows
+// added from the highest order down
+__device__ __forceinline__ double interp64(const double *coef, double x, double y)
 {
-    constexpr int TILE = kLeaf * kLeaf;
-    const int np = *W.npool;
-    for (int e = blockIdx.x; e < np; e += gridDim.x) {
+    double tx[kNP64];
+    tx[0] = 1.0;
+    tx[1] = x;
+#pragma unroll
+    for (int i = 2; i < kNP64; ++i) tx[i] = fma(2.0 * x, tx[i - 1], -tx[i - 2]);
+    const double y2 = 2.0 * y;
+    double b1 = 0.0, b2 = 0.0, r = 0.0;
+#pragma unroll 1
+    for (int j = kNP64 - 1; j >= 0; --j) {
+        r = 0.0;
+#pragma unroll
+        for (int i = kNP64 - 1; i >= 0; --i) r = fma(coef[j * kNP64 + i], tx[i], r);
+        if (j > 0) {
+            const double t = fma(y2, b1, r - b2);
+            b2 = b1;
+            b1 = t;
+        }
+    }
+    return fma(y, b1, r - b2);
+}
+
+// [-1, 1]^2 coordinates in frame g of the direction at offset (dx, dy, dz) from its centre
+__device__ __forceinline__ void local_xy64(const TreeGeo &g, double dx, double dy, double dz, double &x, double &y)
+{
+    const double s = 1.0 / (2.0 - 0.5 * (dx * dx + dy * dy + dz * dz));
+    x = (dx * g.e1[0] + dy * g.e1[1] + dz * g.e1[2]) * (s / g.a1);
+    y = (dx * g.e2[0] + dy * g.e2[1] + dz * g.e2[2]) * (s / g.a2);
+}
+
+// Values of cluster cl at its nodes, kept as (hi, lo) pairs [slot][2][256] -> the value of a middle node as a
+// pair and the Chebyshev coefficients of the differences from it (shared).  The differences are a fraction of
+// the values, so the interpolation's rounding stays below that of the value itself.
+__device__ __forceinline__ void cheb_coefs64(const double *__restrict__ F, const TreeWork &W, int64_t cl, double *coef,
+                                             double *tmp, double &rhi, double &rlo)
+{
+    const int nch = W.nch[cl];
+    const int64_t at = nch == 1 ? cl : W.ncl + W.pbase[cl];
+    for (int k = threadIdx.x; k < kNN64; k += kTreeNT) {
+        double hi = 0.0, lo = 0.0;
+        for (int c = 0; c < nch; ++c) {
+            const double *f = F + (at + c) * 2 * kNN64 + k;
+            fold64(hi, lo, f[0]);
+            lo += f[kNN64];
+        }
+        coef[k] = hi;
+        tmp[k] = lo;
+    }
+    __syncthreads();
+    constexpr int kMid = kNN64 / 2 + kNP64 / 2;
+    rhi = coef[kMid];
+    rlo = tmp[kMid];
+    double d[kNN64 / kTreeNT];
+#pragma unroll
+    for (int q = 0; q < kNN64 / kTreeNT; ++q) {
+        const int k = q * kTreeNT + threadIdx.x;
+        d[q] = (coef[k] - rhi) + (tmp[k] - rlo);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kNN64 / kTreeNT; ++q) coef[q * kTreeNT + threadIdx.x] = d[q];
+    __syncthreads();
+    cheb_transform<kNP64>(coef, tmp);
+}
+
+// Copies the staged batch: eval(batch start, size) runs with sm.rec filled; whole block.
+template <typename Stage, typename Eval>
+__device__ __forceinline__ void tree_batches64(TreeSmem64 &sm, int count, Stage &&stage, Eval &&eval)
+{
+#pragma unroll 1
+    for (int b0 = 0; b0 < count; b0 += kTreeBatch) {
+        if (b0 + (int)threadIdx.x < count) stage(sm.scan.list[b0 + threadIdx.x], sm.rec[threadIdx.x]);
+        __syncthreads();
+        eval(count - b0 < kTreeBatch ? count - b0 : kTreeBatch);
+        __syncthreads();
+    }
+}
+
+__device__ __forceinline__ void copy_record(Stage64 &dst, const void *src, int n16)
+{
+    for (int k = 0; k < n16; ++k) reinterpret_cast<double2 *>(dst.v)[k] = reinterpret_cast<const double2 *>(src)[k];
+}
+
+// Far-field pair term (17 FP64 operations, see k_map_f64)
+__device__ __forceinline__ double far_term64(const Far64 &r, double nx, double ny, double nz, double acc)
+{
+    const double hs = fma(nz, r.mxh[2], fma(ny, r.mxh[1], fma(nx, r.mxh[0], r.sg)));
+    const double B = fma(nz, r.xd[2], fma(ny, r.xd[1], fma(nx, r.xd[0], 1.0)));
+    const double A2 = fma(nz, r.xp[2], fma(ny, r.xp[1], fma(nx, r.xp[0], r.af)));
+    const double B2 = fma(r.sx, B, r.be);
+    const double num = fma(-A2, A2, fma(B2, B2, -r.K));
+    return fma(num, rcp64(B * hs), acc);
+}
+
+struct TreeNodeArgs64 {
+    TreeNodeArgs n;
+    const Seg64 *s64;
+    float d_far;
+};
+
+// Two nodes per thread: 18 FP64 operations per sample and node where every node of the cluster is at least
+// d_far from the samples (completed squares), else 21.
+template <bool ROOT>
+__global__ void __launch_bounds__(kTreeNT) k_tree_nodes_f64(TreeNodeArgs64 A)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TreeSmem64 &sm = *reinterpret_cast<TreeSmem64 *>(smem_raw);
+    const TreeNodeArgs &a = A.n;
+    const int tid = threadIdx.x;
+    const int np = *a.W.npool;
+    TreeQueue queue{a.queue, 0ull};
+    for (int64_t item = queue.first(&sm.item); item < a.W.ncl + np; item = queue.next(&sm.item)) {
+        int kc, nch;
+        int64_t at;
+        const int64_t cl = tree_item(a.W, item, np, kc, nch, at);
+        if (cl < 0) continue;
+        const int64_t pcl = ROOT ? 0 : tree_parent(cl, a.nb, a.pnb);
+        if (!ROOT) load_geo(&sm.pgeo, a.pgeo + pcl);
+        load_geo(&sm.geo, a.geo + cl);
+        __syncthreads();
+        const float4 self = sm.geo.c, parent = ROOT ? self : sm.pgeo.c;
+        double m[2][3], mm[2], hi[2] = {0.0, 0.0}, lo[2] = {0.0, 0.0};
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int k = q * kTreeNT + tid;
+            const double xi = sm.geo.a1 * cheb_at<kNP64>(1, k % kNP64), eta = sm.geo.a2 * cheb_at<kNP64>(1, k / kNP64);
+            const double r2 = xi * xi + eta * eta, s = 2.0 / (1.0 + r2);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                m[q][c] = s * (xi * sm.geo.e1[c] + eta * sm.geo.e2[c] - r2 * sm.geo.n0[c]);
+            }
+            mm[q] = m[q][0] * m[q][0] + m[q][1] * m[q][1] + m[q][2] * m[q][2];
+        }
+        const bool far = self.w - target_radius(sm.geo) >= A.d_far;
+        auto stage = [&](uint32_t e, Stage64 &d) {
+            const Seg64 &s = A.s64[e];
+            double D[3], P = 0.0, Q = 0.0, K = 0.0, B0 = 1.0;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                D[c] = (sm.geo.n0[c] - s.xh[c]) - s.xl[c];
+                P = fma(s.xd[c], D[c], P);
+                Q = fma(s.xp[c], D[c], Q);
+                K = fma(D[c], D[c], K);
+                B0 = fma(s.xd[c], sm.geo.n0[c], B0);
+                d.v[c] = 2.0 * D[c];
+                d.v[4 + c] = s.xd[c];
+                d.v[8 + c] = s.xp[c];
+            }
+            const double f = s.xp[0] * s.xh[0] + s.xp[1] * s.xh[1] + s.xp[2] * s.xh[2];   // X'.Xhat
+            if (!far) {
+                d.v[3] = K;
+                d.v[7] = P;
+                d.v[11] = Q;
+                d.v[12] = B0;
+                d.v[13] = f;
+                d.v[14] = s.c;
+                return;
+            }
+            const double sg = s.c < 0.0 ? -1.0 : 1.0, c2 = 0.5 * fabs(s.c), q = sqrt(c2), e1 = B0 - P;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                d.v[c] = sg * (2.0 * D[c]);
+                d.v[4 + c] = q * s.xd[c];
+                d.v[8 + c] = q * s.xp[c];
+            }
+            d.v[3] = sg * K;
+            d.v[7] = 0.5 * q * (B0 + P);
+            d.v[11] = q * (Q + 0.5 * f);
+            d.v[12] = q > 0.0 ? 1.0 / q : 0.0;
+            d.v[13] = 0.5 * e1;
+            d.v[14] = 0.25 * c2 * (f * f - e1 * e1);
+            d.v[15] = sg;
+        };
+        auto eval = [&](int cnt) {
+            double part[2] = {0.0, 0.0};
+            if (far) {
+#pragma unroll 2
+                for (int s = 0; s < cnt; ++s) {
+                    const double *v = sm.rec[s].v;
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const double Q = fma(m[q][2], v[2], fma(m[q][1], v[1], fma(m[q][0], v[0], fma(v[15], mm[q], v[3]))));
+                        const double U = fma(m[q][2], v[6], fma(m[q][1], v[5], fma(m[q][0], v[4], v[7])));
+                        const double V = fma(m[q][2], v[10], fma(m[q][1], v[9], fma(m[q][0], v[8], v[11])));
+                        const double B = fma(U, v[12], v[13]);
+                        // c (B Xdot.d - A X'.d) / (B d.d) with c / 2 in the squares: twice the quotient
+                        part[q] = fma(fma(-V, V, fma(U, U, v[14])), rcp64(B * Q), part[q]);
+                    }
+                }
+                part[0] *= 2.0;
+                part[1] *= 2.0;
+            } else {
+#pragma unroll 2
+                for (int s = 0; s < cnt; ++s) {
+                    const double *v = sm.rec[s].v;
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const double Q = fma(m[q][2], v[2], fma(m[q][1], v[1], fma(m[q][0], v[0], mm[q] + v[3])));
+                        const double g = fma(m[q][2], v[6], fma(m[q][1], v[5], m[q][0] * v[4]));
+                        const double Qd = fma(m[q][2], v[10], fma(m[q][1], v[9], fma(m[q][0], v[8], v[11])));
+                        const double B = v[12] + g, num = fma(B, v[7] + g, -(v[13] + Qd) * Qd);
+                        part[q] = fma(v[14] * num, rcp64(B * Q), part[q]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) fold64(hi[q], lo[q], part[q]);
+        };
+        tree_scan<ROOT, false>(a.S, kc, nch, self, parent, 0.f, 0.f, 0.f, sm.scan,
+                               [&](int count) { tree_batches64(sm, count, stage, eval); });
+        if (!ROOT && kc == 0) {
+            double rhi, rlo;
+            cheb_coefs64(a.Fp, a.Wp, pcl, sm.coef, sm.tmp, rhi, rlo);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                double x, y;
+                local_xy64(sm.pgeo, (sm.geo.n0[0] - sm.pgeo.n0[0]) + m[q][0], (sm.geo.n0[1] - sm.pgeo.n0[1]) + m[q][1],
+                           (sm.geo.n0[2] - sm.pgeo.n0[2]) + m[q][2], x, y);
+                fold64(hi[q], lo[q], rhi);
+                fold64(hi[q], lo[q], interp64(sm.coef, x, y));
+                lo[q] += rlo;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            a.F[at * 2 * kNN64 + q * kTreeNT + tid] = hi[q];
+            a.F[(at * 2 + 1) * kNN64 + q * kTreeNT + tid] = lo[q];
+        }
+        __syncthreads();
+    }
+}
+
+struct TreePixArgs64 {
+    TreePixArgs p;
+    const Far64 *far64;
+    float d_far;
+};
+
+// Four pixels per thread, half a cluster per item.  Samples with |d| >= d_far and B >= b_min at every pixel of the cluster in
+// the far-field form (its squares cancel to a factor 1/B of the rounding), the others from the double-double Xhat (29 operations, with rcp64 in the place of a division).
+__global__ void __launch_bounds__(kTreeNT) k_tree_pixels_f64(TreePixArgs64 A)
+{
+    constexpr int TILE = kLeaf64 * kLeaf64, P = 4, PARTS = TILE / (P * kTreeNT);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TreeSmem64 &sm = *reinterpret_cast<TreeSmem64 *>(smem_raw);
+    const TreePixArgs &a = A.p;
+    const int tid = threadIdx.x;
+    const int np = *a.W.npool;
+    unsigned zerocnt = 0;
+    TreeQueue queue{a.queue, 0ull};
+    for (int64_t it = queue.first(&sm.item); it < (a.W.ncl + np) * PARTS; it = queue.next(&sm.item)) {
+        int kc, nch;
+        int64_t at;
+        const int64_t item = it / PARTS, base = it % PARTS * (P * kTreeNT);   // the item's share of the cluster
+        const int64_t cl = tree_item(a.W, item, np, kc, nch, at);
+        if (cl < 0) continue;
+        load_geo(&sm.geo, a.geo + cl);
+        __syncthreads();
+        const float4 self = sm.geo.c;
+        double n[P][3], hi[P], lo[P];
+        unsigned valid = 0;
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            const int64_t k = cl * TILE + base + q * kTreeNT + tid;
+            if (a.outidx[k] >= 0) valid |= 1u << q;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) n[q][c] = a.nv[c * a.ldn + k];
+            hi[q] = lo[q] = 0.0;
+        }
+        auto stage = [&](uint32_t e, Stage64 &d) {
+            const uint32_t r = e & kTreeIndex;
+            if (e & (kTreeClose | kTreeBeam)) copy_record(d, a.s64 + r, sizeof(Seg64) / 16);
+            else copy_record(d, A.far64 + r, sizeof(Far64) / 16);
+        };
+        int b0 = 0;   // list position of the batch
+        auto eval = [&](int cnt) {
+            double part[P];
+#pragma unroll
+            for (int q = 0; q < P; ++q) part[q] = 0.0;
+#pragma unroll 1
+            for (int s = 0; s < cnt; ++s) {
+                if (!(sm.scan.list[b0 + s] & (kTreeClose | kTreeBeam))) {
+                    const Far64 &r = *reinterpret_cast<const Far64 *>(sm.rec[s].v);
+#pragma unroll
+                    for (int q = 0; q < P; ++q) part[q] = far_term64(r, n[q][0], n[q][1], n[q][2], part[q]);
+                    continue;
+                }
+                const Seg64 &g = *reinterpret_cast<const Seg64 *>(sm.rec[s].v);
+#pragma unroll
+                for (int q = 0; q < P; ++q) {
+                    const double dx = (n[q][0] - g.xh[0]) - g.xl[0], dy = (n[q][1] - g.xh[1]) - g.xl[1],
+                                 dz = (n[q][2] - g.xh[2]) - g.xl[2];
+                    const double Q = fma(dz, dz, fma(dy, dy, dx * dx));
+                    const double Pd = fma(g.xd[2], dz, fma(g.xd[1], dy, g.xd[0] * dx));
+                    const double Qd = fma(g.xp[2], dz, fma(g.xp[1], dy, g.xp[0] * dx));
+                    // A and B from n itself: 1 + Xdot.Xhat + Xdot.d would round a small B twice
+                    const double A = n[q][0] * g.xp[0] + n[q][1] * g.xp[1] + n[q][2] * g.xp[2];
+                    const double B = 1.0 + (n[q][0] * g.xd[0] + n[q][1] * g.xd[1] + n[q][2] * g.xd[2]);
+                    const double num = B * Pd - A * Qd, den = B * Q;
+                    // the float estimate of the reciprocal needs a value inside the float range
+                    const int ex = __double2hiint(den) & 0x7ff00000;
+                    if (ex > 0x39b00000 && ex < 0x46000000) {
+                        part[q] = fma(g.c * num, rcp64(den), part[q]);
+                    } else if (Q == 0.0) {
+                        if (valid & (1u << q)) ++zerocnt;
+                    } else {
+                        part[q] += g.c * num / den;
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < P; ++q) fold64(hi[q], lo[q], part[q]);
+        };
+        const float R = target_radius(sm.geo);
+        tree_scan<false, true>(a.S, kc, nch, self, self, R, A.d_far + R, a.b_min, sm.scan, [&](int count) {
+            b0 = 0;
+            tree_batches64(sm, count, stage, [&](int cnt) {
+                eval(cnt);
+                b0 += kTreeBatch;
+            });
+        });
+        double rhi = 0.0, rlo = 0.0;
+        if (kc == 0) cheb_coefs64(a.F, a.Wf, cl, sm.coef, sm.tmp, rhi, rlo);
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            const int64_t k = cl * TILE + base + q * kTreeNT + tid;
+            if (kc == 0) {
+                double x, y;
+                local_xy64(sm.geo, n[q][0] - sm.geo.n0[0], n[q][1] - sm.geo.n0[1], n[q][2] - sm.geo.n0[2], x, y);
+                fold64(hi[q], lo[q], rhi);
+                fold64(hi[q], lo[q], interp64(sm.coef, x, y));
+                lo[q] += rlo;
+            }
+            const double v = hi[q] + lo[q];
+            if (nch == 1) {
+                const int64_t oi = a.outidx[k];
+                if (oi >= 0) a.theta[oi] = a.accumulate ? a.theta[oi] + v : v;
+            } else {
+                a.partial[item * TILE + base + q * kTreeNT + tid] = v;   // pool entry of the chunk
+            }
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) zerocnt += __shfl_xor_sync(0xffffffffu, zerocnt, o);
+    if ((tid & 31) == 0 && zerocnt) atomicAdd(&a.st->zero_pairs, (unsigned long long)zerocnt);
+}
+
+// theta of the clusters that were cut into chunks: their partial sums added in chunk order, one pixel per
+// thread.
+__global__ void __launch_bounds__(256) k_tree_reduce(TreeWork W, int tile, const double *__restrict__ partial,
+                                                     const int64_t *__restrict__ outidx, double *__restrict__ theta,
+                                                     int accumulate)
+{
+    const int np = *W.npool, parts = tile / 256;
+    for (int i = blockIdx.x; i < np * parts; i += gridDim.x) {
+        const int e = i / parts, l = i % parts * 256 + threadIdx.x;
         const int2 it = W.pool[e];
         if (it.y != 0) continue;
-        const int64_t oi = outidx[(int64_t)it.x * TILE + threadIdx.x];
         const int nch = W.nch[it.x];
+        const int64_t oi = outidx[(int64_t)it.x * tile + l];
+        const double *src = partial + (int64_t)e * tile + l;
         double hi = 0.0, lo = 0.0;
-        for (int c = 0; c < nch; ++c) fold64(hi, lo, partial[(int64_t)(e + c) * TILE + threadIdx.x]);
+        int c = 0;
+        for (; c + 4 <= nch; c += 4) {
+            double v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = src[(int64_t)(c + k) * tile];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) fold64(hi, lo, v[k]);
+        }
+        for (; c < nch; ++c) fold64(hi, lo, src[(int64_t)c * tile]);
         if (oi >= 0) theta[oi] = accumulate ? theta[oi] + (hi + lo) : hi + lo;
     }
 }
@@ -861,7 +1262,8 @@ __global__ void __launch_bounds__(kLeaf *kLeaf) k_tree_reduce(TreeWork W, const 
 // The stages to plan: node sums of the levels, then the pixels.
 constexpr int kTargets = 8;             // chunk sizes tried: target, 2 target, ...
 // work counters, totals per chunk size and pool lengths of the stages
-constexpr size_t kTreeZero = (kTreeLevels + 1) * ((1 + kTargets) * sizeof(unsigned long long) + sizeof(int));
+constexpr size_t kTreeZero =
+    (kTreeLevels + 1) * ((1 + kTargets) * sizeof(unsigned long long) + sizeof(int));
 struct TreeStages {
     int n;
     int64_t first[kTreeLevels + 2];     // prefix of the stages' cluster counts
@@ -905,8 +1307,7 @@ __global__ void __launch_bounds__(128) k_tree_count(TreeStages g, TreeSamples S,
         const float4 self = g.geo[st][c].c;
         float4 outer = self;
         if (!leaf) {
-            const int64_t nb = g.nb[st], f = c / (nb * nb), rem = c - f * nb * nb;
-            outer = g.pgeo[st][(f * g.pnb[st] + rem / nb / 2) * g.pnb[st] + rem % nb / 2].c;
+            outer = g.pgeo[st][tree_parent(c, g.nb[st], g.pnb[st])].c;
         }
         float share = 0.f;
         const int nsup = (int)((S.nst + kTreeSuper - 1) / kTreeSuper);
@@ -975,31 +1376,36 @@ int slots_of(const void *fn, size_t smem, int num_sms)
 
 }  // namespace
 
-int tree_leaf(int prec) { return kLeaf; }
+int tree_leaf(int prec) { return prec == ISW_F64 ? kLeaf64 : kLeaf; }
 
-TreePlan tree_plan(int prec, int64_t N, int nface, int64_t n, int num_sms)
+TreePlan tree_plan(int prec, int64_t N, int nface, int64_t npix, int64_t n, int num_sms)
 {
     TreePlan p{};
-    p.leaf = kLeaf;
-    p.nn = kNN;
-    p.nface = nface;
+    const bool f64 = prec == ISW_F64;
+    p.prec = prec;
+    p.leaf = tree_leaf(prec);
+    p.nn = f64 ? 2 * kNN64 : kNN;   // doubles per cluster
     p.n_pad = (n + kTreeS - 1) / kTreeS * kTreeS;
     p.nst = p.n_pad / kTreeS;
-    int64_t nb = (N + p.leaf - 1) / p.leaf;
-    p.nslots = slots_of((const void *)&k_tree_nodes_f32<false>, sizeof(TreeSmem32), num_sms);
-    p.pslots = slots_of((const void *)&k_tree_pixels_f32, sizeof(TreeSmemPix), num_sms);
+    p.nslots = f64 ? slots_of((const void *)&k_tree_nodes_f64<false>, sizeof(TreeSmem64), num_sms)
+                   : slots_of((const void *)&k_tree_nodes_f32<false>, sizeof(TreeSmem32), num_sms);
+    p.pslots = f64 ? slots_of((const void *)&k_tree_pixels_f64, sizeof(TreeSmem64), num_sms)
+                   : slots_of((const void *)&k_tree_pixels_f32, sizeof(TreeSmemPix), num_sms);
     int64_t all = 0;
+    int64_t nb = nface > 0 ? (N + p.leaf - 1) / p.leaf : 0;
+    int64_t ncl = nface > 0 ? nface * nb * nb : (npix + p.leaf * p.leaf - 1) / (p.leaf * p.leaf);
     for (;;) {
         const int L = p.levels++;
         p.nb[L] = (int)nb;
-        p.ncl[L] = nface * nb * nb;
-        all += p.ncl[L];
-        if (nb <= 2 || p.levels == kTreeLevels) break;
+        p.ncl[L] = ncl;
+        all += ncl;
+        if ((nface > 0 ? nb <= 2 : ncl <= 48) || p.levels == kTreeLevels) break;
         nb = (nb + 1) / 2;
+        ncl = nface > 0 ? nface * nb * nb : (ncl + 3) / 4;
     }
     all += p.ncl[0];
-    p.pool = 8 * p.nslots;
-    p.ppool = 8 * p.pslots;
+    p.pool = (f64 ? 16 : 8) * p.nslots;
+    p.ppool = (f64 ? 16 : 8) * p.pslots;
     size_t at = 0;
     auto take = [&](size_t bytes) {
         const size_t o = at;
@@ -1013,7 +1419,7 @@ TreePlan tree_plan(int prec, int64_t N, int nface, int64_t n, int num_sms)
     p.off_sup = take((size_t)2 * ((p.nst + kTreeSuper - 1) / kTreeSuper) * sizeof(TreeCap));
     p.off_vidx = take((size_t)p.n_pad * sizeof(uint32_t));
     p.off_inv = take((size_t)n * sizeof(uint32_t));
-    p.off_rec = take((size_t)p.n_pad * sizeof(TreeRec));
+    p.off_rec = f64 ? 0 : take((size_t)p.n_pad * sizeof(TreeRec));
     p.off_work = take((size_t)3 * all * sizeof(int));
     p.off_pool = take(((size_t)p.levels * p.pool + p.ppool) * sizeof(int2));
     p.off_partial = take((size_t)p.ppool * p.leaf * p.leaf * sizeof(double));
@@ -1027,11 +1433,13 @@ TreePlan tree_plan(int prec, int64_t N, int nface, int64_t n, int num_sms)
 
 cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_t s)
 {
+    const bool f64 = p.prec == ISW_F64;
+    const double kappa = f64 ? kKappa64 : kKappa32;
     unsigned char *b = (unsigned char *)m.scratch;
     TreeCrit *crit = (TreeCrit *)(b + p.off_crit), *vcrit = (TreeCrit *)(b + p.off_vcrit);
     TreeCap *caps = (TreeCap *)(b + p.off_caps), *sup = (TreeCap *)(b + p.off_sup);
     uint32_t *vidx = (uint32_t *)(b + p.off_vidx), *inv = (uint32_t *)(b + p.off_inv);
-    TreeRec *rec = (TreeRec *)(b + p.off_rec);
+    TreeRec *rec = f64 ? nullptr : (TreeRec *)(b + p.off_rec);
     unsigned long long *queue = (unsigned long long *)(b + p.off_queue), *total = queue + kTreeLevels + 1;
     int *npool = (int *)(total + (kTreeLevels + 1) * kTargets);
     cudaError_t e = cudaMemsetAsync(queue, 0, kTreeZero, s);
@@ -1042,11 +1450,17 @@ cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_
     const int64_t nsup = (p.nst + kTreeSuper - 1) / kTreeSuper;
     k_tree_super<<<dim3((unsigned)((nsup + 3) / 4), 2), 128, 0, s>>>(caps, p.nst, nsup, sup);
     const TreeSamples S{crit, vcrit, caps, caps + p.nst, sup, sup + nsup, vidx, p.nst};
-    k_tree_leaf_geo<kLeaf><<<(unsigned)p.ncl[0], kLeaf * kLeaf / 4, 0, s>>>(m.nv, m.ldn, m.outidx, m.diag, m.theta_pix,
-                                                                             (TreeGeo *)(b + p.off_geo[0]));
+    TreeGeo *leaf_geo = (TreeGeo *)(b + p.off_geo[0]);
+    if (f64)
+        k_tree_leaf_geo<kLeaf64><<<(unsigned)p.ncl[0], kLeaf64 * kLeaf64 / 4, 0, s>>>(m.nv, m.ldn, m.outidx, m.order,
+                                                                                       m.theta_pix, kappa, leaf_geo);
+    else
+        k_tree_leaf_geo<kLeaf><<<(unsigned)p.ncl[0], kLeaf * kLeaf / 4, 0, s>>>(m.nv, m.ldn, m.outidx, m.order,
+                                                                                 m.theta_pix, kappa, leaf_geo);
     for (int L = 1; L < p.levels; ++L)
         k_tree_up_geo<<<(unsigned)((p.ncl[L] + 3) / 4), 128, 0, s>>>((const TreeGeo *)(b + p.off_geo[L - 1]), p.nb[L - 1],
-                                                                     (TreeGeo *)(b + p.off_geo[L]), p.nb[L], p.nface);
+                                                                     p.ncl[L - 1], (TreeGeo *)(b + p.off_geo[L]), p.nb[L],
+                                                                     p.ncl[L], kappa);
     // stages 0 .. levels - 1: node sums of the level; stage `levels`: the pixels
     TreeStages g{};
     g.n = p.levels + 1;
@@ -1062,7 +1476,7 @@ cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_
             g.pnb[st] = p.nb[st + 1];
         }
         g.pool[st] = pix ? p.ppool : p.pool;
-        g.target[st] = pix ? kPixTarget : kNodeTarget;
+        g.target[st] = f64 ? (pix ? kPixTarget64 : kNodeTarget64) : (pix ? kPixTarget : kNodeTarget);
         g.entries[st] = entries + (size_t)st * p.pool;
     }
     const int64_t all = g.first[g.n];
@@ -1074,7 +1488,8 @@ cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_
     };
     for (int L = p.levels - 1; L >= 0; --L) {
         const bool root = L == p.levels - 1;
-        TreeNodeArgs a{};
+        TreeNodeArgs64 A{};
+        TreeNodeArgs &a = A.n;
         a.S = S;
         a.rec = rec;
         a.geo = (const TreeGeo *)(b + p.off_geo[L]);
@@ -1088,17 +1503,26 @@ cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_
             a.Wp = work(L + 1);
         }
         a.queue = queue + L;
-        const void *fn = root ? (const void *)&k_tree_nodes_f32<true> : (const void *)&k_tree_nodes_f32<false>;
+        A.s64 = m.s64;
+        A.d_far = m.d_far;
         const int64_t items = p.ncl[L] + p.pool;
-        void *args[] = {(void *)&a};
-        cudaLaunchKernel(fn, dim3((unsigned)(items < p.nslots ? items : p.nslots)), dim3(kTreeNT), args,
-                         sizeof(TreeSmem32), s);
+        const dim3 grid((unsigned)(items < p.nslots ? items : p.nslots));
+        if (f64) {
+            const void *fn = root ? (const void *)&k_tree_nodes_f64<true> : (const void *)&k_tree_nodes_f64<false>;
+            void *args[] = {(void *)&A};
+            cudaLaunchKernel(fn, grid, dim3(kTreeNT), args, sizeof(TreeSmem64), s);
+        } else {
+            const void *fn = root ? (const void *)&k_tree_nodes_f32<true> : (const void *)&k_tree_nodes_f32<false>;
+            void *args[] = {(void *)&a};
+            cudaLaunchKernel(fn, grid, dim3(kTreeNT), args, sizeof(TreeSmem32), s);
+        }
     }
-    TreePixArgs a{};
+    TreePixArgs64 A{};
+    TreePixArgs &a = A.p;
     a.S = S;
     a.rec = rec;
     a.s64 = m.s64;
-    a.geo = (const TreeGeo *)(b + p.off_geo[0]);
+    a.geo = leaf_geo;
     a.nv = m.nv;
     a.ldn = m.ldn;
     a.outidx = m.outidx;
@@ -1111,9 +1535,13 @@ cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_
     a.b_min = m.b_min;
     a.st = m.st;
     a.queue = queue + kTreeLevels;
-    const int64_t items = p.ncl[0] + p.ppool;
-    k_tree_pixels_f32<<<(unsigned)(items < p.pslots ? items : p.pslots), kTreeNT, sizeof(TreeSmemPix), s>>>(a);
-    k_tree_reduce<<<(unsigned)p.pslots, kLeaf * kLeaf, 0, s>>>(a.W, a.partial, m.outidx, m.theta, m.accumulate);
+    A.far64 = m.far64;
+    A.d_far = m.d_far;
+    const int64_t items = (p.ncl[0] + p.ppool) * (f64 ? 2 : 1);
+    const unsigned grid = (unsigned)(items < p.pslots ? items : p.pslots);
+    if (f64) k_tree_pixels_f64<<<grid, kTreeNT, sizeof(TreeSmem64), s>>>(A);
+    else k_tree_pixels_f32<<<grid, kTreeNT, sizeof(TreeSmemPix), s>>>(a);
+    k_tree_reduce<<<(unsigned)p.pslots, 256, 0, s>>>(a.W, p.leaf * p.leaf, a.partial, m.outidx, m.theta, m.accumulate);
     return cudaSuccess;
 }
 

@@ -79,6 +79,15 @@ struct TreeWork {
     int64_t ncl;
 };
 
+// Parent of cluster c: 2 x 2 blocks of a face's nb x nb clusters (pnb x pnb parents), or, for a list of
+// pixels in spatial order (nb = 0), four consecutive clusters.
+__device__ __forceinline__ int64_t tree_parent(int64_t c, int nb, int pnb)
+{
+    if (nb == 0) return c >> 2;
+    const int64_t f = c / ((int64_t)nb * nb), rem = c - f * nb * nb;
+    return (f * pnb + rem / nb / 2) * pnb + rem % nb / 2;
+}
+
 constexpr int kTreeS = 64;        // samples per tile of the scan
 constexpr int kTreeNT = 128;      // threads per CTA of the evaluation kernels
 constexpr int kTreeBatch = 128;   // samples per staged batch, one per thread
@@ -165,8 +174,8 @@ struct TreeScanSmem {
 };
 
 // List entries: the record and, for LEAF, what the evaluation has to watch for at the cluster's pixels
-// (all within chord R of the centre): kTreeBeam when some B may be below b_min, kTreeClose when some
-// |d| may be below max(rho, R / 2).
+// (all within chord R of the centre): kTreeBeam when some B may be below b_min, kTreeClose when the
+// centre is within `close` + rho.
 constexpr uint32_t kTreeBeam = 0x80000000u, kTreeClose = 0x40000000u, kTreeIndex = 0x3fffffffu;
 
 // Exclusive prefix of 32 counts (tcnt, in warp order) and their total, for every thread.
@@ -188,7 +197,7 @@ __device__ __forceinline__ int tree_prefix(const int *tcnt, int &total)
 // sm.list after the `held` entries there; whole block, returns the new length.
 template <bool ROOT, bool LEAF, typename Tile>
 __device__ __forceinline__ int tree_select(const TreeSamples &S, int pass, const float4 self, const float4 outer,
-                                           float R, float beam2, int n, int held, TreeScanSmem &sm, Tile &&tile)
+                                           float close, float beam2, int n, int held, TreeScanSmem &sm, Tile &&tile)
 {
     constexpr int W = kTreeNT / 32, NR = kTreeGroup / W;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -215,7 +224,7 @@ __device__ __forceinline__ int tree_select(const TreeSamples &S, int pass, const
                 } else {
                     if (tree_beam2(b, self) < beam2) fl |= 1u << (4 * i + 2 * h);
                     float4 c = self;
-                    c.w = 1.5f * R + 1e-6f;   // the chord limit of tree_near_pos adds rho
+                    c.w = close + 1e-6f;   // tree_near_pos adds rho
                     if (tree_near_pos(a, c)) fl |= 2u << (4 * i + 2 * h);
                 }
                 mk[i][h] = __ballot_sync(0xffffffffu, sel);
@@ -255,7 +264,7 @@ __device__ __forceinline__ int tree_select(const TreeSamples &S, int pass, const
 // 32 candidates, then the samples of 32 tiles; entries left over wait, so that batches stay full.
 template <bool ROOT, bool LEAF, typename Consume>
 __device__ __forceinline__ void tree_scan(const TreeSamples &S, int kc, int split, const float4 self,
-                                          const float4 parent, float R, float b_min, TreeScanSmem &sm,
+                                          const float4 parent, float R, float close, float b_min, TreeScanSmem &sm,
                                           Consume &&consume)
 {
     constexpr int W = kTreeNT / 32, NR = kTreeGroup / W;
@@ -282,7 +291,7 @@ __device__ __forceinline__ void tree_scan(const TreeSamples &S, int kc, int spli
 #pragma unroll 1
         for (int64_t g0 = 0; g0 < j1; g0 += kTreeGroup) {
             const int n = (int)(j1 - g0 < kTreeGroup ? j1 - g0 : kTreeGroup);
-            held = tree_select<true, false>(S, 0, self, self, R, beam2, n, held, sm,
+            held = tree_select<true, false>(S, 0, self, self, close, beam2, n, held, sm,
                                             [&](int i) { return kc + (g0 + i) * split; });
             drain();
         }
@@ -339,7 +348,7 @@ __device__ __forceinline__ void tree_scan(const TreeSamples &S, int kc, int spli
 #pragma unroll 1
                     for (int g0 = 0; g0 < ncand; g0 += kTreeGroup) {
                         const int n = ncand - g0 < kTreeGroup ? ncand - g0 : kTreeGroup;
-                        held = tree_select<false, LEAF>(S, pass, self, outer, R, beam2, n, held, sm,
+                        held = tree_select<false, LEAF>(S, pass, self, outer, close, beam2, n, held, sm,
                                                         [&](int i) { return sm.cand[g0 + i]; });
                         drain();
                     }
@@ -394,22 +403,12 @@ struct TreeQueue {
     }
 };
 
-// Values of cluster cl at its NP x NP nodes (the sum of its chunks) -> their Chebyshev coefficients in
-// shared memory (coef, tmp: NP * NP doubles); whole block.
+// Node values (node k = j NP + i) -> Chebyshev coefficients, in place in shared memory; whole block.
 template <int NP>
-__device__ __forceinline__ void cheb_coefs(const double *__restrict__ F, const TreeWork &W, int64_t cl, double *coef,
-                                           double *tmp)
+__device__ __forceinline__ void cheb_transform(double *coef, double *tmp)
 {
     constexpr int NN = NP * NP;
-    const int nch = W.nch[cl];
-    const int64_t at = nch == 1 ? cl : W.ncl + W.pbase[cl];
-    for (int k = threadIdx.x; k < NN; k += blockDim.x) {
-        double v = 0.0;
-        for (int c = 0; c < nch; ++c) v += F[(at + c) * NN + k];
-        coef[k] = v;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < NN; k += blockDim.x) {   // along xi: node k = j NP + i
+    for (int k = threadIdx.x; k < NN; k += blockDim.x) {   // along xi
         const int j = k / NP, m = k % NP;
         double v = 0.0;
 #pragma unroll
@@ -425,6 +424,24 @@ __device__ __forceinline__ void cheb_coefs(const double *__restrict__ F, const T
         coef[k] = v * (q == 0 ? 1.0 / NP : 2.0 / NP);
     }
     __syncthreads();
+}
+
+// Values of cluster cl at its NP x NP nodes (the sum of its chunks) -> their Chebyshev coefficients in
+// shared memory (coef, tmp: NP * NP doubles); whole block.
+template <int NP>
+__device__ __forceinline__ void cheb_coefs(const double *__restrict__ F, const TreeWork &W, int64_t cl, double *coef,
+                                           double *tmp)
+{
+    constexpr int NN = NP * NP;
+    const int nch = W.nch[cl];
+    const int64_t at = nch == 1 ? cl : W.ncl + W.pbase[cl];
+    for (int k = threadIdx.x; k < NN; k += blockDim.x) {
+        double v = 0.0;
+        for (int c = 0; c < nch; ++c) v += F[(at + c) * NN + k];
+        coef[k] = v;
+    }
+    __syncthreads();
+    cheb_transform<NP>(coef, tmp);
 }
 
 // Position (lx, ly) of slot l in a T x T block enumerated by anti-diagonals from the largest

@@ -4,7 +4,8 @@ the tree can go wrong: sides at and around multiples of the 16-pixel leaf, sampl
 signs.  Tolerances: the truncation of the 8 x 8 interpolation is below 4e-7 of the rms next to the
 strings (rate 5^-8 at a near radius of 3.5 half-sizes) and FP32 pair rounding adds up to 1.2e-6 where
 samples spread over the sky; where thousands of terms of both signs meet in a few pixels FP32 gives
-3e-6 in either kind of kernel, and the bar is the FP32 maps' 1e-5."""
+3e-6 in either kind of kernel, and the bar is the FP32 maps' 1e-5.  FP64: truncation below 1e-16 and
+rounding of 2e-15 of the rms against the maps' bar of 1e-12."""
 import numpy as np
 import pytest
 
@@ -12,6 +13,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 TOL32 = 2e-6
 BAR32 = 1e-5
+TOL64 = 1e-12
 
 
 @pytest.fixture(scope="module")
@@ -74,24 +76,31 @@ def test_tree_sizes(isw, nside, n):
     _check(isw, nside, _samples(n, nside), "f32c", TOL32)
 
 
+@pytest.mark.parametrize("nside,n", [(64, 407), (65, 448), (96, 449), (100, 65), (257, 63)])
+def test_tree_sizes_f64(isw, nside, n):
+    _check(isw, nside, _samples(n, nside), "f64", TOL64)
+
+
+@pytest.mark.parametrize("prec,tol", [("f32c", BAR32), ("f64", TOL64)])
 @pytest.mark.parametrize("kw", [dict(spot=1e-3), dict(spot=0.0), dict(cusp=True), dict(mixed=True), dict(spot=0.05, mixed=True)])
-def test_tree_sample_layouts(isw, kw):
-    _check(isw, 64, _samples(4001, 3, **kw), "f32c", BAR32)
+def test_tree_sample_layouts(isw, kw, prec, tol):
+    _check(isw, 64, _samples(4001, 3, **kw), prec, tol)
 
 
-def test_tree_skipped_zero_pairs_accumulate(isw):
+@pytest.mark.parametrize("prec,tol", [("f32c", TOL32), ("f64", TOL64)])
+def test_tree_skipped_zero_pairs_accumulate(isw, prec, tol):
     nside = 64
     S = _samples(4500, 5)
     centre = isw.hp_pix2vec_ring(nside).cpu().numpy()
     S[0:3, 7] = centre[:, 12345]              # on a pixel's line of sight
     S[3:6, 100] = [0.6, 0.8, 0.0]             # |Xdot| = 1
-    got, ref = _check(isw, nside, S, "f32c", TOL32)
+    got, ref = _check(isw, nside, S, prec, tol)
     Sd = torch.from_numpy(S).cuda()
     base = torch.full_like(got, 2.0)
-    isw.isw_map(nside, Sd, prec="f32c", accumulate=True, out=base)
+    isw.isw_map(nside, Sd, prec=prec, accumulate=True, out=base)
     rms = ref.square().mean().sqrt()
     assert ((base - 2.0 - got).abs().max() / rms).item() <= 1e-14
-    again = isw.isw_map(nside, Sd, prec="f32c")
+    again = isw.isw_map(nside, Sd, prec=prec)
     assert torch.equal(again, got)            # reproducible
     isw.default_context().check_status()
 
@@ -108,3 +117,47 @@ def test_tree_near_pairs_and_observer(isw):
         assert abs(near - ctx.check_status()[1]["near_pairs"]) <= 2   # |d| = rho to rounding
         ref = _direct(isw, 64, S, x_obs=x_obs)
         assert ((got - ref).abs().max() / ref.square().mean().sqrt()).item() <= TOL32
+
+
+@pytest.mark.parametrize("prec,tol,npix,n", [("f32c", TOL32, 12289, 8200), ("f64", TOL64, 49153, 500)])
+def test_tree_lists_and_ranges(isw, prec, tol, npix, n):
+    """Pixels of a list (random, with repeats; an index out of range is reported and left alone) and of a
+    range, summed in spatial order and written to their own places."""
+    nside = 256
+    S = torch.from_numpy(_samples(n, 8)).cuda()
+    g = torch.Generator("cuda").manual_seed(4)
+    pix = torch.randint(12 * nside * nside, (npix,), device="cuda", generator=g)
+    pix[5] = pix[4]
+    ctx = isw.default_context()
+    ctx.check_status()
+    for kw in (dict(pix=pix), dict(pix0=77, npix=npix)):
+        got = isw.isw_map(nside, S, prec=prec, **kw)
+        ref = _direct(isw, nside, S, **kw)
+        assert ((got - ref).abs().max() / ref.square().mean().sqrt()).item() <= tol
+    assert ctx.check_status()[0] == isw.OK
+    pix[9] = 12 * nside * nside
+    out = torch.full((npix,), 7.0, dtype=torch.float64, device="cuda")
+    isw.isw_map(nside, S, pix=pix, prec=prec, out=out)
+    assert ctx.check_status()[0] == isw.EINVAL and out[9].item() == 7.0
+    ref = _direct(isw, nside, S, pix=pix[10:])
+    assert ((out[10:] - ref).abs().max() / ref.square().mean().sqrt()).item() <= tol
+    ctx.check_status()
+
+
+@pytest.mark.parametrize("prec,tol,M,n", [("f32c", TOL32, 111, 8200), ("f32c", TOL32, 160, 4000), ("f64", TOL64, 222, 500),
+                                          ("f64", TOL64, 256, 400)])
+def test_tree_patch(isw, prec, tol, M, n):
+    S = torch.from_numpy(_samples(n, M, spot=0.1)).cuda()
+    e3 = S[0:3, 0].cpu().numpy() / np.linalg.norm(S[0:3, 0].cpu().numpy())
+    e1 = np.cross(e3, [0.0, 0.0, 1.0])
+    e1 /= np.linalg.norm(e1)
+    frame = np.stack([e1, np.cross(e3, e1), e3])
+    ctx = isw.default_context()
+    got = isw.isw_map_patch(frame, M, 0.2, S, prec=prec)
+    ctx.set_param(isw.PARAM_SPLIT, 1)
+    try:
+        ref = isw.isw_map_patch(frame, M, 0.2, S, prec="f64")
+    finally:
+        ctx.set_param(isw.PARAM_SPLIT, 0)
+    assert ctx.check_status()[0] == isw.OK
+    assert ((got - ref).abs().max() / ref.square().mean().sqrt()).item() <= tol
