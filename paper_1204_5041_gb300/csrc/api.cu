@@ -848,6 +848,22 @@ int isw_map_patch(isw_ctx *c, const double *frame, int64_t M, double width, cons
         return ISW_OK;
     }
     const bool f64 = prec == ISW_F64;
+    if (c->split_override == 0 && flat_tree_rule(M, n)) {
+        const FlatTreePlan tp = flat_tree_plan(f64, M, n, c->num_sms);
+        if ((r = ensure_ws(c, kWsFlat, (size_t)tp.n_pad * flat_record_bytes()))) return r;
+        if ((r = ensure_ws(c, kWsTree, tp.bytes))) return r;
+        unsigned char *rec = (unsigned char *)c->ws[kWsFlat];
+        void *r32 = rec, *r64 = rec + (size_t)tp.n_pad * (flat_record_bytes() / 2);
+        const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
+        launch_flat_pack(samples, n, ld, p, xo[0], xo[1], xo[2], GU, tp.n_pad, r32, r64, s);
+        const int ti = timing_begin(c, s);
+        cudaError_t e = launch_map_flat_tree(tp, r32, r64, n, M, width, theta_out, accumulate, c->ws[kWsTree], s);
+        if (e != cudaSuccess) return cuda_err(c, e, "isw_map_patch launch");
+        timing_end(c, ti, s);
+        c->n_launch += 1 + flat_tree_launches(tp);
+        c->n_pair += 1;
+        return check_launch(c, "isw_map_patch launch");
+    }
     const int S = flat_seg_tile(), tx = flat_tx(), ty = flat_ty();
     const int64_t ntiles = ((M + tx - 1) / tx) * ((M + ty - 1) / ty), tot = ntiles * tx * ty;
     const int64_t n_pad = (n + S - 1) / S * S, nst = n_pad / S;

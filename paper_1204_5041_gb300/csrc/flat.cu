@@ -10,19 +10,12 @@
 // behind the patch plane (Z <= 0) get zero weight; d = 0 contributes zero.
 #include <type_traits>
 
+#include "flat.cuh"
 #include "isw_internal.cuh"
 #include "kernels.cuh"
 #include "pipeline.cuh"
 
 namespace isw {
-
-struct __align__(16) Flat32 {
-    float4 a;   // xi_s hi, eta_s hi, xi_s lo, eta_s lo
-    float4 b;   // w1, w2, 0, 0
-};
-struct __align__(16) Flat64 {
-    double xs, ys, w1, w2;
-};
 
 constexpr int kFlatNT = 128, kFlatP = 4, kFlatS = 128;
 

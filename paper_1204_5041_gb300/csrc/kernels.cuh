@@ -89,6 +89,9 @@ size_t sort_scratch_bytes(int64_t n, int orders);
 const uint32_t *launch_spatial_order(const double *S, int64_t n, int64_t ld, double xo0, double xo1, double xo2,
                                      void *scratch, int orders, cudaStream_t s);
 int spatial_order_launches();
+// stable sort of 24-bit keys already in the scratch: keys [orders][n], indices [orders][n] after twice as
+// many words
+const uint32_t *launch_sort_keys(int64_t n, int orders, void *scratch, cudaStream_t s);
 // the same for the selected pixels (a range, or a list when pix_list is given): perm[npix] of positions
 const uint32_t *launch_pixel_order(int64_t N, int64_t pix0, int64_t npix, const int64_t *pix_list, void *scratch,
                                    cudaStream_t s);
@@ -191,6 +194,24 @@ int tree_leaf(int prec);
 TreePlan tree_plan(int prec, int64_t N, int nface, int64_t npix, int64_t n, int num_sms);
 cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_t s);
 inline int tree_launches(const TreePlan &p) { return 2 * p.levels + 7; }
+
+// flattree.cu: flat-sky patch maps over a tree of pixel clusters
+struct FlatTreePlan {
+    bool f64;
+    int leaf, levels, nb[kTreeLevels];    // leaf side in pixels, clusters per side from the leaves
+    int64_t n_pad, nst;
+    int nslots, pslots, pool, ppool;
+    size_t off_queue, off_crit, off_caps, off_sup, off_rec, off_sort, off_work, off_pool, off_partial, off_A[kTreeLevels], bytes;
+};
+// from 3e7 pairs: its 20 launches take 0.1 ms, the direct kernel 3.5e7 pairs' time of FP32
+inline bool flat_tree_rule(int64_t M, int64_t n)
+{
+    return M >= 32 && (double)M * (double)M * (double)n >= 3e7 && n < (int64_t(1) << 30);
+}
+FlatTreePlan flat_tree_plan(bool f64, int64_t M, int64_t n, int num_sms);
+cudaError_t launch_map_flat_tree(const FlatTreePlan &p, const void *r32, const void *r64, int64_t n, int64_t M, double width,
+                                 double *theta, int accumulate, void *scratch, cudaStream_t s);
+inline int flat_tree_launches(const FlatTreePlan &p) { return p.levels + 17; }
 
 // adjoint.cu
 struct AdjArgs {

@@ -243,6 +243,11 @@ const uint32_t *launch_pixel_order(int64_t N, int64_t pix0, int64_t npix, const 
     return sort_passes(npix, 1, p, s);
 }
 
+const uint32_t *launch_sort_keys(int64_t n, int orders, void *scratch, cudaStream_t s)
+{
+    return sort_passes(n, orders, reinterpret_cast<uint32_t *>(scratch), s);
+}
+
 int spatial_order_launches() { return 1 + 3 * 3; }
 
 }  // namespace isw

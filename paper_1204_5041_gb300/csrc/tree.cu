@@ -35,44 +35,6 @@ __device__ __forceinline__ double near_radius(double kappa, double a)
     return 2.0 * z / sqrt(1.0 + z * z);
 }
 
-__device__ __forceinline__ float warp_sum(float v)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ float warp_max(float v)
-{
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
-// ball around the mean of the lane's two points (w = enlargement, < 0: no point); radius < 0 when empty
-__device__ __forceinline__ TreeCap warp_ball(const float4 (&x)[2])
-{
-    float sx = 0.f, sy = 0.f, sz = 0.f, cnt = 0.f, r = -1.f;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-        if (x[h].w >= 0.f) {
-            sx += x[h].x;
-            sy += x[h].y;
-            sz += x[h].z;
-            cnt += 1.f;
-        }
-    cnt = fmaxf(warp_sum(cnt), 1.f);
-    sx = warp_sum(sx) / cnt;
-    sy = warp_sum(sy) / cnt;
-    sz = warp_sum(sz) / cnt;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-        if (x[h].w >= 0.f) {
-            const float dx = x[h].x - sx, dy = x[h].y - sy, dz = x[h].z - sz;
-            r = fmaxf(r, sqrtf(dx * dx + dy * dy + dz * dz) * 1.0001f + 1e-6f + x[h].w);
-        }
-    TreeCap c;
-    c.a = make_float4(sx, sy, sz, warp_max(r));
-    return c;
-}
-
 // One warp per tile of 64 records (position order): decision data, evaluation records, caps, and the
 // record of every input sample.
 __global__ void __launch_bounds__(256) k_tree_crit(const Seg32 *__restrict__ s32, const Seg64 *__restrict__ s64,
@@ -145,26 +107,6 @@ __global__ void __launch_bounds__(256) k_tree_vcrit(const TreeCrit *__restrict__
     }
     const TreeCap c = warp_ball(x);
     if (lane == 0) vcaps[t] = c;
-}
-
-// Balls over kTreeSuper tiles, one warp each: around the mean of the tiles' centres.  Position order in
-// blockIdx.y = 0, velocity order in 1 (caps and sup hold both, nst and nsup apart).
-__global__ void __launch_bounds__(128) k_tree_super(const TreeCap *__restrict__ caps, int64_t nst, int64_t nsup,
-                                                    TreeCap *__restrict__ sup)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t u = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (u >= nsup) return;
-    const int64_t t = u * kTreeSuper + lane;
-    float4 a = make_float4(0.f, 0.f, 0.f, -1.f);
-    if (t < nst) a = caps[blockIdx.y * nst + t].a;
-    const float on = a.w >= 0.f ? 1.f : 0.f, cnt = fmaxf(warp_sum(on), 1.f);
-    const float sx = warp_sum(on * a.x) / cnt, sy = warp_sum(on * a.y) / cnt, sz = warp_sum(on * a.z) / cnt;
-    const float dx = a.x - sx, dy = a.y - sy, dz = a.z - sz;
-    const float r = warp_max(on > 0.f ? sqrtf(dx * dx + dy * dy + dz * dz) * 1.0001f + 1e-6f + a.w : -1.f);
-    TreeCap c;
-    c.a = make_float4(sx, sy, sz, r);
-    if (lane == 0) sup[blockIdx.y * nsup + u] = c;
 }
 
 // frame from a centre direction and a rough tangent; extents are filled in by the caller
@@ -1229,139 +1171,6 @@ __global__ void __launch_bounds__(kTreeNT) k_tree_pixels_f64(TreePixArgs64 A)
     }
     for (int o = 16; o > 0; o >>= 1) zerocnt += __shfl_xor_sync(0xffffffffu, zerocnt, o);
     if ((tid & 31) == 0 && zerocnt) atomicAdd(&a.st->zero_pairs, (unsigned long long)zerocnt);
-}
-
-// theta of the clusters that were cut into chunks: their partial sums added in chunk order, one pixel per
-// thread.
-__global__ void __launch_bounds__(256) k_tree_reduce(TreeWork W, int tile, const double *__restrict__ partial,
-                                                     const int64_t *__restrict__ outidx, double *__restrict__ theta,
-                                                     int accumulate)
-{
-    const int np = *W.npool, parts = tile / 256;
-    for (int i = blockIdx.x; i < np * parts; i += gridDim.x) {
-        const int e = i / parts, l = i % parts * 256 + threadIdx.x;
-        const int2 it = W.pool[e];
-        if (it.y != 0) continue;
-        const int nch = W.nch[it.x];
-        const int64_t oi = outidx[(int64_t)it.x * tile + l];
-        const double *src = partial + (int64_t)e * tile + l;
-        double hi = 0.0, lo = 0.0;
-        int c = 0;
-        for (; c + 4 <= nch; c += 4) {
-            double v[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) v[k] = src[(int64_t)(c + k) * tile];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) fold64(hi, lo, v[k]);
-        }
-        for (; c < nch; ++c) fold64(hi, lo, src[(int64_t)c * tile]);
-        if (oi >= 0) theta[oi] = accumulate ? theta[oi] + (hi + lo) : hi + lo;
-    }
-}
-
-// The stages to plan: node sums of the levels, then the pixels.
-constexpr int kTargets = 8;             // chunk sizes tried: target, 2 target, ...
-// work counters, totals per chunk size and pool lengths of the stages
-constexpr size_t kTreeZero =
-    (kTreeLevels + 1) * ((1 + kTargets) * sizeof(unsigned long long) + sizeof(int));
-struct TreeStages {
-    int n;
-    int64_t first[kTreeLevels + 2];     // prefix of the stages' cluster counts
-    const TreeGeo *geo[kTreeLevels + 1], *pgeo[kTreeLevels + 1];   // the clusters, their parents (nodes only)
-    int nb[kTreeLevels + 1], pnb[kTreeLevels + 1];
-    int pool[kTreeLevels + 1];          // pool entries
-    int target[kTreeLevels + 1];        // smallest chunk
-    int2 *entries[kTreeLevels + 1];
-};
-
-// Share of a tile's samples that lies within the near chord of a cluster, from the tile's ball (a
-// linear ramp across the ball): position tiles by distance, beam tiles by B.
-__device__ __forceinline__ float tile_share(const TreeCap &t, const float4 &c, int pass)
-{
-    if (t.a.w < 0.f) return 0.f;
-    float x;
-    if (pass) {
-        const float b = 1.f + (c.x * t.a.x + c.y * t.a.y + c.z * t.a.z);
-        x = 0.5f * c.w * c.w - b;
-    } else {
-        const float dx = c.x - t.a.x, dy = c.y - t.a.y, dz = c.z - t.a.z;
-        x = c.w - sqrtf(dx * dx + dy * dy + dz * dz);
-    }
-    return fminf(fmaxf(0.5f + 0.5f * x / (t.a.w + 1e-6f), 0.f), 1.f);
-}
-
-// Estimate of every cluster's samples from the tile balls; all of them at the root.  And, for each chunk
-// size, the pool entries that it would take.  One warp per (stage, cluster).
-__global__ void __launch_bounds__(128) k_tree_count(TreeStages g, TreeSamples S, int64_t n, int *__restrict__ est,
-                                                    unsigned long long *__restrict__ total)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (k >= g.first[g.n]) return;
-    int st = 0;
-    while (k >= g.first[st + 1]) ++st;
-    const int64_t c = k - g.first[st];
-    const bool leaf = st == g.n - 1;
-    int64_t v = n;
-    if (leaf || g.pgeo[st]) {
-        const float4 self = g.geo[st][c].c;
-        float4 outer = self;
-        if (!leaf) {
-            outer = g.pgeo[st][tree_parent(c, g.nb[st], g.pnb[st])].c;
-        }
-        float share = 0.f;
-        const int nsup = (int)((S.nst + kTreeSuper - 1) / kTreeSuper);
-        for (int pass = 0; pass < 2; ++pass) {
-            const TreeCap *sup = pass ? S.vsup : S.sup, *caps = pass ? S.vcaps : S.caps;
-            for (int u0 = 0; u0 < nsup; u0 += 32) {
-                bool in = false;
-                if (u0 + lane < nsup) {
-                    const TreeCap cap = sup[u0 + lane];
-                    in = pass ? tree_tile_beam(cap, outer) : tree_tile_pos(cap, outer);
-                }
-                unsigned m = __ballot_sync(0xffffffffu, in);
-                for (; m; m &= m - 1u) {
-                    const int64_t t = (int64_t)(u0 + __ffs(m) - 1) * kTreeSuper + lane;
-                    if (t < S.nst) {
-                        const TreeCap cap = caps[t];
-                        const float f = tile_share(cap, outer, pass);
-                        share += leaf || pass ? f : fmaxf(f - tile_share(cap, self, pass), 0.f);
-                    }
-                }
-            }
-        }
-        v = (int64_t)(warp_sum(share) * (float)kTreeS);
-        if (v > n) v = n;
-    }
-    if (lane == 0) est[k] = (int)v;
-    if (lane < kTargets) {
-        const int64_t T = (int64_t)g.target[st] << lane;
-        if (v >= T) atomicAdd(total + st * kTargets + lane, (unsigned long long)(1 + v / T));
-    }
-}
-
-// Chunks per cluster: with the smallest chunk size whose entries fit the pool (none: no cluster is
-// cut).  Where a cluster's entries lie in the pool depends on the order of the atomics; what they hold
-// does not.
-__global__ void __launch_bounds__(128) k_tree_plan(TreeStages g, const int *__restrict__ est,
-                                                   const unsigned long long *__restrict__ total, int *__restrict__ nch,
-                                                   int *__restrict__ pbase, int *__restrict__ npool)
-{
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= g.first[g.n]) return;
-    int st = 0;
-    while (k >= g.first[st + 1]) ++st;
-    int j = 0;
-    while (j < kTargets && total[st * kTargets + j] > (unsigned long long)g.pool[st]) ++j;
-    const int64_t T = (int64_t)g.target[st] << j;
-    const int m = j == kTargets || est[k] < T ? 1 : (int)(1 + est[k] / T);
-    int b = 0;
-    if (m > 1) {
-        b = atomicAdd(npool + st, m);
-        for (int i = 0; i < m; ++i) g.entries[st][b + i] = make_int2((int)(k - g.first[st]), i);
-    }
-    nch[k] = m;
-    pbase[k] = b;
 }
 
 size_t up256(size_t x) { return (x + 255) & ~size_t(255); }

@@ -161,3 +161,37 @@ def test_tree_patch(isw, prec, tol, M, n):
         ctx.set_param(isw.PARAM_SPLIT, 0)
     assert ctx.check_status()[0] == isw.OK
     assert ((got - ref).abs().max() / ref.square().mean().sqrt()).item() <= tol
+
+
+@pytest.mark.parametrize("prec,tol", [("f32c", TOL32), ("f64", TOL64)])
+@pytest.mark.parametrize("M,width,n", [(33, 0.1, 30000), (64, 0.3, 8191), (100, 0.05, 3000), (512, 0.13, 129), (543, 0.2, 1000)])
+def test_flat_tree(isw, prec, tol, M, width, n):
+    """Flat-sky patches over the series tree against the direct kernel: both leaf sizes, ragged sides,
+    samples in the field, beyond it and behind its plane, one exactly on a pixel.  The flat sky has no FP64
+    near field: a pixel next to a sample is one term of any size, good to FP32's few ulp of itself, so the
+    FP32 bound is tol * rms + 1e-6 of the value."""
+    S = _samples(n, M, spot=0.1)
+    S[0:3, : n // 8] = _samples(n // 8, M + 1)[0:3]        # all over the sky: half of these behind
+    e3 = np.array([0.3, -0.5, 0.4]) / np.sqrt(0.5)
+    e1 = np.cross(e3, [0.0, 0.0, 1.0])
+    e1 /= np.linalg.norm(e1)
+    frame = np.stack([e1, np.cross(e3, e1), e3])
+    i, j = M // 2, M // 3
+    S[0:3, 1] = 0.5 * (e3 + (i + 0.5 - 0.5 * M) * width / M * e1 + (j + 0.5 - 0.5 * M) * width / M * np.cross(e3, e1))
+    Sd = torch.from_numpy(S).cuda()
+    ctx = isw.default_context()
+    got = isw.isw_map_patch(frame, M, width, Sd, prec=prec, approx=isw.FLATSKY)
+    base = torch.full_like(got, 3.0)
+    isw.isw_map_patch(frame, M, width, Sd, prec=prec, approx=isw.FLATSKY, accumulate=True, out=base)
+    ctx.set_param(isw.PARAM_SPLIT, 1)
+    try:
+        ref = isw.isw_map_patch(frame, M, width, Sd, prec="f64", approx=isw.FLATSKY)
+    finally:
+        ctx.set_param(isw.PARAM_SPLIT, 0)
+    assert ctx.check_status()[0] == isw.OK
+    keep = torch.ones_like(ref, dtype=torch.bool)
+    keep[j, i] = False       # 1 / |d| of a rounding error: any value
+    rms = ref[keep].square().mean().sqrt()
+    own = 1e-6 if prec == "f32c" else 1e-13
+    assert ((got - ref).abs() <= tol * rms + own * ref.abs())[keep].all()
+    assert ((base - 3.0 - got).abs() <= 1e-13 * (rms + ref.abs()))[keep].all()
