@@ -970,6 +970,52 @@ int isw_map_adjoint(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const
         return ISW_OK;
     }
     const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
+    if (prec == ISW_F32C && c->split_override == 0 && tree_rule(prec, npix, n) && npix < (int64_t(1) << 32)) {
+        const bool full = !pix_list && pix0 == 0 && npix == 12 * nside * nside;
+        const AdjTreePlan p = adj_tree_plan(nside, full ? 12 : 0, npix, n, c->num_sms);
+        const int64_t tot = p.map.ncl[0] * p.map.leaf * p.map.leaf;
+        const size_t sort_bytes = (sort_scratch_bytes(n, 2) + 255) / 256 * 256;
+        if ((r = ensure_ws(c, kWsNv, (size_t)tot * 3 * sizeof(double)))) return r;
+        if ((r = ensure_ws(c, kWsOut, (size_t)tot * sizeof(int64_t)))) return r;
+        if ((r = ensure_ws(c, kWsS32, (size_t)p.n_pad * sizeof(Seg32)))) return r;
+        if ((r = ensure_ws(c, kWsS64, (size_t)p.n_pad * sizeof(Seg64)))) return r;
+        if ((r = ensure_ws(c, kWsSort, sort_bytes + (full ? 0 : sort_scratch_bytes(npix, 1))))) return r;
+        if ((r = ensure_ws(c, kWsTree, p.bytes))) return r;
+        double *nv = (double *)c->ws[kWsNv];
+        int64_t *outidx = (int64_t *)c->ws[kWsOut];
+        Seg32 *s32 = (Seg32 *)c->ws[kWsS32];
+        Seg64 *s64 = (Seg64 *)c->ws[kWsS64];
+        unsigned char *sort = (unsigned char *)c->ws[kWsSort];
+        const uint32_t *pp = full ? nullptr : launch_pixel_order(nside, pix0, npix, pix_list, sort + sort_bytes, s);
+        launch_pixel_table(nside, full ? 0 : (pix_list ? 2 : 1), pix0, npix, pix_list, p.map.leaf, p.map.leaf, p.map.ncl[0],
+                           nv, tot, outidx, nullptr, c->d_status, s, pp);
+        AdjTreeCall m{};
+        m.theta_pix = std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
+        m.perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], sort, 2, s);
+        launch_pack(samples, n, ld, xo[0], xo[1], xo[2], GU, m.theta_pix, c->near_k, p.n_pad, m.perm, s32, s64, nullptr,
+                    nullptr, nullptr, c->d_status, s);
+        m.nv = nv;
+        m.ldn = tot;
+        m.outidx = outidx;
+        m.order = full ? kSlotsDiag : kSlotsList;
+        m.g = dL_dtheta;
+        m.s32 = s32;
+        m.s64 = s64;
+        m.n = n;
+        m.b_min = (float)c->b_min;
+        m.ngrad = ngrad;
+        m.grad = grad_out;
+        m.ld_g = ld_g;
+        m.st = c->d_status;
+        m.scratch = c->ws[kWsTree];
+        const int ti = timing_begin(c, s);
+        cudaError_t e = launch_adjoint_tree(p, m, s);
+        if (e != cudaSuccess) return cuda_err(c, e, "isw_map_adjoint launch");
+        timing_end(c, ti, s);
+        c->n_pair += 1;
+        c->n_launch += spatial_order_launches() * (full ? 1 : 2) + 2 + adj_tree_launches(p);
+        return check_launch(c, "isw_map_adjoint launch");
+    }
     const int NT = adj_seg_tile(prec), TP = adj_pix_tile(prec);
     const Variant pv{0, 0, 0, 32, TP / 32};
     const PixelPlan pp = plan_pixels(nside, pix0, npix, pix_list, pv);

@@ -371,8 +371,6 @@ __global__ void __launch_bounds__(256) k_flat_reduce(TreeWork W, const double *_
     }
 }
 
-size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
-
 const void *pixel_kernel(bool f64, int leaf)
 {
     if (leaf == 32) return f64 ? (const void *)&k_flat_pixels<true, 32> : (const void *)&k_flat_pixels<false, 32>;

@@ -213,6 +213,36 @@ cudaError_t launch_map_flat_tree(const FlatTreePlan &p, const void *r32, const v
                                  double *theta, int accumulate, void *scratch, cudaStream_t s);
 inline int flat_tree_launches(const FlatTreePlan &p) { return p.levels + 17; }
 
+// treeadj.cu: FP32 adjoint over the cluster tree
+struct AdjTreePlan {
+    TreePlan map;                         // levels and clusters
+    int64_t n_pad;
+    int slots;
+    size_t off_queue, off_crit, off_vcrit, off_caps, off_vidx, off_inv, off_rec, off_pix, off_low, off_partial, bytes;
+    size_t off_geo[kTreeLevels], off_node[kTreeLevels];
+};
+struct AdjTreeCall {
+    const double *nv;                     // pixel table as in TreeMapArgs
+    int64_t ldn;
+    const int64_t *outidx;
+    int order;
+    double theta_pix;
+    const double *g;                      // dL/dTheta by output index
+    const Seg32 *s32;                     // n_pad records
+    const Seg64 *s64;
+    const uint32_t *perm;
+    int64_t n;
+    float b_min;
+    int ngrad;
+    double *grad;
+    int64_t ld_g;
+    DevStatus *st;
+    void *scratch;
+};
+AdjTreePlan adj_tree_plan(int64_t N, int nface, int64_t npix, int64_t n, int num_sms);
+cudaError_t launch_adjoint_tree(const AdjTreePlan &p, const AdjTreeCall &m, cudaStream_t s);
+inline int adj_tree_launches(const AdjTreePlan &p) { return 2 * p.map.levels + 5; }
+
 // adjoint.cu
 struct AdjArgs {
     const Pix32 *p32;        // pixel records in tile order

@@ -681,6 +681,309 @@ __global__ void __launch_bounds__(256) k_tree_reduce(TreeWork W, int tile, const
     }
 }
 
+constexpr int kNP = 8, kNN = kNP * kNP;   // FP32: 8 x 8 nodes
+constexpr int kLeaf = 16;                 // and 16 x 16 pixel leaves
+// Near radius in stereographic half-sizes.  FP32 (8 x 8 nodes): 4 gives 2.2e-8 of the rms at N_side 100 and 10.1 ms at N_side 512
+// with 2e5 samples, 3.5 2.6e-8 and 9.2 ms, 3 5.1e-8 and 8.5 ms.
+// FP64 (16 x 16 nodes): in 80-bit arithmetic, with clusters set next to the strings, the truncation is
+// 9e-16 of the rms at 4 and 1e-17 at 5; 4.5 keeps it below the rounding of the sums.
+constexpr double kKappa32 = 3.5, kKappa64 = 4.5;
+
+__device__ __forceinline__ double near_radius(double kappa, double a)
+{
+    // chord of stereographic radius kappa a
+    const double z = kappa * a;
+    return 2.0 * z / sqrt(1.0 + z * z);
+}
+
+// One warp per tile of 64 records (position order): decision data, evaluation records, caps, and the
+// record of every input sample.
+__global__ void __launch_bounds__(256) k_tree_crit(const Seg32 *__restrict__ s32, const Seg64 *__restrict__ s64,
+                                                   const uint32_t *__restrict__ perm, int64_t n, int64_t ntile,
+                                                   TreeCrit *__restrict__ crit, TreeCap *__restrict__ caps,
+                                                   TreeRec *__restrict__ rec, uint32_t *__restrict__ inv)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (t >= ntile) return;
+    float4 x[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int64_t s = t * kTreeS + 32 * h + lane;
+        TreeCrit cr;
+        cr.a = make_float4(0.f, 0.f, 0.f, 0.f);
+        cr.b = make_float4(0.f, 0.f, 0.f, kCritSkip);
+        x[h] = make_float4(0.f, 0.f, 0.f, -1.f);
+        const Seg32 f = s32[s];
+        if (s < n) {
+            inv[perm[s]] = (uint32_t)s;
+            if (f.b.w >= 0.f) {
+                cr.a = make_float4(f.a.x, f.a.y, f.a.z, sqrtf(f.b.w) * 1.0001f);
+                cr.b = make_float4(-f.k.x, -f.k.y, -f.k.z, (float)s64[s].om);
+                x[h] = cr.a;
+            }
+        }
+        crit[s] = cr;
+        if (rec) {
+            float4 *dst = rec[s].v;
+            dst[0] = f.a;
+            dst[1] = make_float4(f.b.x, f.b.y, f.b.z, f.e.w);
+            dst[2] = make_float4(f.d.x, f.d.y, f.d.z, f.k.w);
+            dst[3] = make_float4(f.e.x, f.e.y, f.e.z, f.b.w);
+        }
+    }
+    const TreeCap c = warp_ball(x);
+    if (lane == 0) caps[t] = c;
+}
+
+// One warp per tile of 64 samples in velocity order.
+__global__ void __launch_bounds__(256) k_tree_vcrit(const TreeCrit *__restrict__ crit, const Seg32 *__restrict__ s32,
+                                                    const uint32_t *__restrict__ vperm,
+                                                    const uint32_t *__restrict__ inv, int64_t n, int64_t ntile,
+                                                    TreeCrit *__restrict__ vcrit, TreeCap *__restrict__ vcaps,
+                                                    uint32_t *__restrict__ vidx)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (t >= ntile) return;
+    float4 x[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int64_t k = t * kTreeS + 32 * h + lane;
+        TreeCrit cr;
+        cr.a = make_float4(0.f, 0.f, 0.f, 0.f);
+        cr.b = make_float4(0.f, 0.f, 0.f, kCritSkip);
+        x[h] = make_float4(0.f, 0.f, 0.f, -1.f);
+        uint32_t r = 0;
+        if (k < n) {
+            r = inv[vperm[k]];
+            cr = crit[r];
+            if (cr.b.w < kCritSkip) {
+                const float4 d = s32[r].d;
+                x[h] = make_float4(d.x, d.y, d.z, 0.f);
+            }
+        }
+        vcrit[k] = cr;
+        vidx[k] = r;
+    }
+    const TreeCap c = warp_ball(x);
+    if (lane == 0) vcaps[t] = c;
+}
+
+// frame from a centre direction and a rough tangent; extents are filled in by the caller
+__device__ __forceinline__ void make_frame(double cx, double cy, double cz, double tx, double ty, double tz,
+                                           TreeGeo &g)
+{
+    const double r = 1.0 / sqrt(cx * cx + cy * cy + cz * cz);
+    g.n0[0] = cx * r;
+    g.n0[1] = cy * r;
+    g.n0[2] = cz * r;
+    double t = tx * g.n0[0] + ty * g.n0[1] + tz * g.n0[2];
+    double ux = tx - t * g.n0[0], uy = ty - t * g.n0[1], uz = tz - t * g.n0[2];
+    double u2 = ux * ux + uy * uy + uz * uz;
+    if (!(u2 > 1e-12 * (tx * tx + ty * ty + tz * tz)) || !(u2 > 0.0)) {   // no tangent: any will do
+        ux = fabs(g.n0[2]) < 0.9 ? -g.n0[1] : 0.0;
+        uy = fabs(g.n0[2]) < 0.9 ? g.n0[0] : -g.n0[2];
+        uz = fabs(g.n0[2]) < 0.9 ? 0.0 : g.n0[1];
+        u2 = ux * ux + uy * uy + uz * uz;
+    }
+    const double ru = 1.0 / sqrt(u2);
+    g.e1[0] = ux * ru;
+    g.e1[1] = uy * ru;
+    g.e1[2] = uz * ru;
+    // once more against the rounding of the first projection
+    t = g.e1[0] * g.n0[0] + g.e1[1] * g.n0[1] + g.e1[2] * g.n0[2];
+    for (int c = 0; c < 3; ++c) g.e1[c] -= t * g.n0[c];
+    const double rv = 1.0 / sqrt(g.e1[0] * g.e1[0] + g.e1[1] * g.e1[1] + g.e1[2] * g.e1[2]);
+    for (int c = 0; c < 3; ++c) g.e1[c] *= rv;
+    g.e2[0] = g.n0[1] * g.e1[2] - g.n0[2] * g.e1[1];
+    g.e2[1] = g.n0[2] * g.e1[0] - g.n0[0] * g.e1[2];
+    g.e2[2] = g.n0[0] * g.e1[1] - g.n0[1] * g.e1[0];
+}
+
+// the float copies of a finished geometry, with the near radius D
+__device__ __forceinline__ void finish_geo(TreeGeo &g, double D)
+{
+    g.pad = 0.0;
+    g.c = make_float4((float)g.n0[0], (float)g.n0[1], (float)g.n0[2], (float)D);
+    g.l = make_float4((float)(g.n0[0] - (double)g.c.x), (float)(g.n0[1] - (double)g.c.y),
+                      (float)(g.n0[2] - (double)g.c.z), 0.f);
+    g.f1 = make_float4((float)g.e1[0], (float)g.e1[1], (float)g.e1[2], (float)(1.0 / g.a1));
+    g.f2 = make_float4((float)g.e2[0], (float)g.e2[1], (float)g.e2[2], (float)(1.0 / g.a2));
+}
+
+// One CTA of T*T/4 threads per finest cluster.  Sums in float are enough: they only choose the
+// centre and frame, and the extents are measured from the pixels afterwards.
+template <int T>
+__global__ void __launch_bounds__(T *T / 4) k_tree_leaf_geo(const double *__restrict__ nv, int64_t ldn,
+                                                            const int64_t *__restrict__ outidx, int order,
+                                                            double theta_pix, double kappa, TreeGeo *__restrict__ geo)
+{
+    constexpr int NT = T * T / 4, W = NT / 32;
+    __shared__ float red[6][W];
+    __shared__ TreeGeo g;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int64_t t = blockIdx.x;
+    float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int l = tid; l < T * T; l += NT) {
+        const int64_t k = t * T * T + l;
+        if (outidx[k] < 0) continue;
+        int lx = T / 2, ly;
+        if (order == kSlotsDiag) diag_slot_square(l, T, lx, ly);
+        else if (order == kSlotsRows) lx = l % T;
+        // a list has no axis of its own: the frame is then any
+        const float f = order == kSlotsList ? 0.f : (float)lx - 0.5f * (float)(T - 1);
+        for (int c = 0; c < 3; ++c) {
+            const float v = (float)nv[c * ldn + k];
+            s[c] += v;
+            s[3 + c] += f * v;
+        }
+    }
+    for (int c = 0; c < 6; ++c) {
+        for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
+        if (lane == 0) red[c][w] = s[c];
+    }
+    __syncthreads();
+    if (tid == 0) {
+        double a[6];
+        for (int c = 0; c < 6; ++c) {
+            a[c] = 0.0;
+            for (int i = 0; i < W; ++i) a[c] += red[c][i];
+        }
+        make_frame(a[0], a[1], a[2], a[3], a[4], a[5], g);
+    }
+    __syncthreads();
+    const float e1x = (float)g.e1[0], e1y = (float)g.e1[1], e1z = (float)g.e1[2];
+    const float e2x = (float)g.e2[0], e2y = (float)g.e2[1], e2z = (float)g.e2[2];
+    float m1 = 0.f, m2 = 0.f;
+    for (int l = tid; l < T * T; l += NT) {
+        const int64_t k = t * T * T + l;
+        if (outidx[k] < 0) continue;
+        const float dx = (float)(nv[k] - g.n0[0]), dy = (float)(nv[ldn + k] - g.n0[1]),
+                    dz = (float)(nv[2 * ldn + k] - g.n0[2]);
+        const float s = 1.f / (2.f - 0.5f * (dx * dx + dy * dy + dz * dz));
+        m1 = fmaxf(m1, fabsf(dx * e1x + dy * e1y + dz * e1z) * s);
+        m2 = fmaxf(m2, fabsf(dx * e2x + dy * e2y + dz * e2z) * s);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+        m2 = fmaxf(m2, __shfl_xor_sync(0xffffffffu, m2, o));
+    }
+    __syncthreads();
+    if (lane == 0) {
+        red[0][w] = m1;
+        red[1][w] = m2;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int i = 0; i < W; ++i) {
+            m1 = fmaxf(m1, red[0][i]);
+            m2 = fmaxf(m2, red[1][i]);
+        }
+        // margin for the float arithmetic; a single pixel still gets a square of a quarter pixel
+        g.a1 = fmax((double)m1 * 1.00001, 0.125 * theta_pix);
+        g.a2 = fmax((double)m2 * 1.00001, 0.125 * theta_pix);
+        finish_geo(g, near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7);
+        geo[t] = g;
+    }
+}
+
+// One warp per parent cluster (tree_parent of the child level): lane l
+// takes point l % 8 (corners and edge midpoints) of the rectangle of child l / 8.  Offsets from the
+// parent's centre are differences of FP64 centres plus a float offset, so they keep their relative
+// accuracy for small clusters.
+__global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__ child, int cnb, int64_t cncl,
+                                                     TreeGeo *__restrict__ geo, int nb, int64_t ncl, double kappa)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (t >= ncl) return;
+    int64_t kid, kid0;
+    bool has;
+    if (nb == 0) {
+        kid0 = 4 * t;
+        kid = kid0 + (lane >> 3);
+        has = kid < cncl;
+    } else {
+        const int64_t f = t / ((int64_t)nb * nb);
+        const int by = (int)(t - f * nb * nb) / nb, bx = (int)(t - f * nb * nb) % nb;
+        const int i = 2 * bx + (lane >> 3 & 1), j = 2 * by + (lane >> 4);
+        has = i < cnb && j < cnb;
+        kid = (f * cnb + j) * cnb + i;
+        kid0 = (f * cnb + 2 * by) * cnb + 2 * bx;
+    }
+    const TreeGeo k = child[has ? kid : kid0];
+    const float on = has && (lane & 7) == 0 ? 1.f : 0.f;
+    const float cx = warp_sum(on * k.c.x), cy = warp_sum(on * k.c.y), cz = warp_sum(on * k.c.z);
+    const float ux = warp_sum(on * k.f1.x), uy = warp_sum(on * k.f1.y), uz = warp_sum(on * k.f1.z);
+    TreeGeo g;
+    make_frame(cx, cy, cz, ux, uy, uz, g);
+    const float d0 = (float)(k.n0[0] - g.n0[0]), d1 = (float)(k.n0[1] - g.n0[1]), d2 = (float)(k.n0[2] - g.n0[2]);
+    const int q = lane & 7, pt = q < 4 ? q : q + 1;   // 3 x 3 points without the middle one
+    const float xi = (float)(pt % 3 - 1) * (float)k.a1, eta = (float)(pt / 3 - 1) * (float)k.a2;
+    const float r2 = xi * xi + eta * eta, s = 2.f / (1.f + r2);
+    const float x = d0 + s * (xi * k.f1.x + eta * k.f2.x - r2 * k.c.x);
+    const float y = d1 + s * (xi * k.f1.y + eta * k.f2.y - r2 * k.c.y);
+    const float z = d2 + s * (xi * k.f1.z + eta * k.f2.z - r2 * k.c.z);
+    const float ps = 1.f / (2.f - 0.5f * (x * x + y * y + z * z));
+    const float m1 = fabsf(x * (float)g.e1[0] + y * (float)g.e1[1] + z * (float)g.e1[2]) * ps;
+    const float m2 = fabsf(x * (float)g.e2[0] + y * (float)g.e2[1] + z * (float)g.e2[2]) * ps;
+    g.a1 = (double)warp_max(m1) * 1.002;
+    g.a2 = (double)warp_max(m2) * 1.002;
+    // near at a child implies near here
+    const float cd = (k.c.w + sqrtf(d0 * d0 + d1 * d1 + d2 * d2)) * 1.00003f + 2e-6f;
+    const double D = fmax(near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7, (double)warp_max(cd));
+    if (lane == 0) {
+        finish_geo(g, D);
+        geo[t] = g;
+    }
+}
+
+__device__ __forceinline__ void load_geo(TreeGeo *dst, const TreeGeo *src)
+{
+    constexpr int W = sizeof(TreeGeo) / 4;
+    static_assert(sizeof(TreeGeo) % 4 == 0 && W <= kTreeNT, "geometry copy");
+    if ((int)threadIdx.x < W) reinterpret_cast<uint32_t *>(dst)[threadIdx.x] = reinterpret_cast<const uint32_t *>(src)[threadIdx.x];
+}
+
+__device__ __forceinline__ float comp(const float4 &v, int c) { return c == 0 ? v.x : (c == 1 ? v.y : v.z); }
+
+// Coordinates in [-1, 1]^2 of direction n0 + d (float offset d from the centre)
+__device__ __forceinline__ void local_xy(const TreeGeo &g, float dx, float dy, float dz, float &x, float &y)
+{
+    const float s = __fdividef(1.f, 2.f - 0.5f * fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
+    x = fmaf(dz, g.f1.z, fmaf(dy, g.f1.y, dx * g.f1.x)) * (s * g.f1.w);
+    y = fmaf(dz, g.f2.z, fmaf(dy, g.f2.y, dx * g.f2.x)) * (s * g.f2.w);
+}
+
+// chord from the centre to the farthest point of the cluster's rectangle
+__device__ __forceinline__ float target_radius(const TreeGeo &g)
+{
+    const float r2 = (float)(g.a1 * g.a1 + g.a2 * g.a2);
+    return 2.f * sqrtf(r2 / (1.f + r2)) * 1.0001f + 1e-7f;
+}
+
+__device__ __forceinline__ uint64_t dup2(float v) { return f2_pack(v, v); }
+
+// offset from the centre of the node at (xi, eta)
+__device__ __forceinline__ void node_offset(const TreeGeo &g, int k, float (&m)[3])
+{
+    const float xi = (float)(g.a1 * cheb_at<kNP>(1, k % kNP)), eta = (float)(g.a2 * cheb_at<kNP>(1, k / kNP));
+    const float r2 = fmaf(xi, xi, eta * eta), s = 2.f / (1.f + r2);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) m[c] = s * fmaf(xi, comp(g.f1, c), fmaf(eta, comp(g.f2, c), -r2 * comp(g.c, c)));
+}
+
+size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
+
+int slots_of(const void *fn, size_t smem, int num_sms)
+{
+    int nb = 0;
+    if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kTreeNT, smem);
+    return (nb > 0 ? nb : 1) * num_sms;
+}
+
 }  // namespace
 
 }  // namespace isw

@@ -195,3 +195,49 @@ def test_flat_tree(isw, prec, tol, M, width, n):
     own = 1e-6 if prec == "f32c" else 1e-13
     assert ((got - ref).abs() <= tol * rms + own * ref.abs())[keep].all()
     assert ((base - 3.0 - got).abs() <= 1e-13 * (rms + ref.abs()))[keep].all()
+
+
+def _adjoint(isw, nside, S, g, prec, ngrad, split=0, **kw):
+    ctx = isw.default_context()
+    ctx.set_param(isw.PARAM_SPLIT, split)
+    try:
+        return isw.isw_map_adjoint(nside, S, g, prec=prec, ngrad=ngrad, **kw)
+    finally:
+        ctx.set_param(isw.PARAM_SPLIT, 0)
+
+
+@pytest.mark.parametrize("nside,n,ngrad,kw", [(32, 8139, 6, {}), (33, 8193, 10, {}), (47, 4000, 9, dict(spot=0.05, mixed=True)),
+                                              (64, 2561, 6, dict(spot=1e-3)), (100, 900, 10, {}), (257, 127, 6, {})])
+def test_adjoint_tree(isw, nside, n, ngrad, kw):
+    """FP32 gradients over the tree against the direct FP64 kernel, per block of rows, relative to the
+    block's largest entry (the adjoint's bar, 1e-6); skipped samples get zero rows; reproducible."""
+    S = _samples(n, nside, **kw)
+    S[3:6, n // 2] = [0.0, 0.6, 0.8]
+    Sd = torch.from_numpy(S).cuda()
+    g = torch.randn(12 * nside * nside, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    ctx = isw.default_context()
+    ctx.check_status()
+    got = _adjoint(isw, nside, Sd, g, "f32c", ngrad)
+    status, counts = ctx.check_status()
+    ref = _adjoint(isw, nside, Sd, g, "f64", ngrad, split=4)
+    assert status == isw.EDOMAIN and counts["skipped_samples"] == 1 and ctx.check_status()[1]["skipped_samples"] == 1
+    assert (got[:, n // 2] == 0).all()
+    used = torch.arange(n, device="cuda") != n // 2
+    for a in range(0, ngrad, 3):
+        b = (slice(a, min(a + 3, ngrad)), used)
+        assert ((got - ref)[b].abs().max() / ref[b].abs().max()).item() <= 1e-6
+    assert torch.equal(got, _adjoint(isw, nside, Sd, g, "f32c", ngrad))
+    ctx.check_status()
+
+
+def test_adjoint_tree_list(isw):
+    nside, npix, n = 256, 12301, 8200
+    S = torch.from_numpy(_samples(n, 12)).cuda()
+    pix = torch.randint(12 * nside * nside, (npix,), device="cuda", generator=torch.Generator("cuda").manual_seed(2))
+    g = torch.randn(npix, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    for kw in (dict(pix=pix), dict(pix0=1234, npix=npix)):
+        got = _adjoint(isw, nside, S, g, "f32c", 6, **kw)
+        ref = _adjoint(isw, nside, S, g, "f64", 6, split=4, **kw)
+        for b in (slice(0, 3), slice(3, 6)):
+            assert ((got - ref)[b].abs().max() / ref[b].abs().max()).item() <= 1e-6
+    assert isw.default_context().check_status()[0] == isw.OK
