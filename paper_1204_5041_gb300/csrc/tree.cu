@@ -18,6 +18,8 @@
 // quarter of its time) and by the tests that find them.
 #include "tree.cuh"
 
+#include <algorithm>
+
 namespace isw {
 
 namespace {
@@ -494,20 +496,14 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_pixels_f32(TreePixArgs a)
 // ------------------------------------------------------------------------------------
 // FP64 maps: 16 x 16 nodes, leaves of 32 x 32 pixels.  The FP64 unit (two FMA lanes per clock and SM)
 // is all that counts, so every thread simply holds its nodes or pixels and reads one staged sample at
-// a time.  N_side 64 with 10,240 samples 18.3 -> 14.4 ms (a leaf of 32 pixels spans 0.5 rad there and four
-// tenths of the pairs stay near), N_side 128 with 25,087 170 -> 57 ms.  Error against the oracle 1.2e-16
+// a time.  N_side 64 with 10,240 samples 18.3 -> 12.3 ms (a leaf of 32 pixels spans 0.5 rad there and four
+// tenths of the pairs stay near), N_side 128 with 25,087 170 -> 46 ms.  Error against the oracle 1.2e-16
 // to 1.7e-16 of the rms (direct kernel 0.5e-16 to 1.2e-16), largest 1.3e-15 (1.0e-15).
 // ------------------------------------------------------------------------------------
 constexpr int kNP64 = 16, kNN64 = kNP64 * kNP64, kLeaf64 = 32;
 constexpr int kNodeTarget64 = 128, kPixTarget64 = 48;
 
-// One staged sample: a Far64 or Seg64 record (pixels), or the sample relative to the cluster's centre
-// (nodes): 2D (3), K, Xdot (3), P, X' (3), Q, B0, f, c, see the FP32 entries; or, on clusters at least
-// d_far from their samples, in completed squares with sigma = sign c, s = sqrt(|c|/2):
-// sigma 2D (3), sigma K, s Xdot (3), s (B0 + P)/2, s X' (3), s (Q + f/2), 1/s, e/2, s^2 (f^2 - e^2)/4, sigma.
-// Nodes always take the offset m from the centre and not the rounded direction: the rounding of a
-// direction moves a node by 5e-17, and the interpolant's values by that times the slope (2e-16 of the
-// rms).
+// A staged Far64 or Seg64 record.
 struct __align__(16) Stage64 {
     double v[16];
 };
@@ -590,8 +586,8 @@ __device__ __forceinline__ void cheb_coefs64(const double *__restrict__ F, const
 }
 
 // Copies the staged batch: eval(batch start, size) runs with sm.rec filled; whole block.
-template <typename Stage, typename Eval>
-__device__ __forceinline__ void tree_batches64(TreeSmem64 &sm, int count, Stage &&stage, Eval &&eval)
+template <typename Smem, typename Stage, typename Eval>
+__device__ __forceinline__ void tree_batches64(Smem &sm, int count, Stage &&stage, Eval &&eval)
 {
 #pragma unroll 1
     for (int b0 = 0; b0 < count; b0 += kTreeBatch) {
@@ -621,18 +617,41 @@ __device__ __forceinline__ double far_term64(const Far64 &r, double nx, double n
 struct TreeNodeArgs64 {
     TreeNodeArgs n;
     const Seg64 *s64;
-    float d_far;
 };
 
-// Two nodes per thread: 18 FP64 operations per sample and node where every node of the cluster is at least
-// d_far from the samples (completed squares), else 21.
+// Node (xi, eta) of a cluster is n0 + (xi e1 + eta e2 - r^2 n0) / w with r^2 = xi^2 + eta^2 and w = (1 + r^2) / 2,
+// so w times anything linear in n is a polynomial in xi plus one in eta:
+//   w (a + v.m) = [a/2 + xi v.e1 + xi^2 (a/2 - v.n0)] + [eta v.e2 + eta^2 (a/2 - v.n0)],
+// and w |d|^2 likewise (|m|^2 w = 2 r^2).  The pair term is a quotient of degree 2 over degree 2 in such forms: w
+// cancels.  With the 2 x 16 values of the five forms |d|^2, B, c Xdot.d, A and c X'.d in tables per sample, a
+// node costs five additions and 12 FP64 operations in all (18 to 21 from the node's offset), the tables
+// one per node.  Offsets and not directions: the rounding of a direction moves a node by 5e-17, and the
+// interpolant's values by that times the slope (2e-16 of the rms).
+constexpr int kForms64 = 5, kTabBatch = 16;
+struct __align__(16) NodeCoef64 {
+    double v[kForms64][4], pad[2];   // constant, xi, eta, square; odd multiple of 16 bytes
+};
+struct __align__(16) NodeForms64 {
+    double v[kForms64 + 1];
+};
+struct __align__(16) TreeNodeSmem64 {
+    NodeCoef64 rec[kTreeBatch];
+    NodeForms64 tab[kTabBatch][2 * kNP64];
+    TreeScanSmem scan;
+    TreeGeo geo, pgeo;
+    double coef[kNN64], tmp[kNN64];
+    int64_t item;
+};
+
+// Two nodes per thread.  Bound by the FP64 unit (85% busy); N_side 128 with 25,087 samples, both levels: 20.6 ms
+// from the nodes' offsets, 15.9 ms from tables.
 template <bool ROOT>
 __global__ void __launch_bounds__(kTreeNT) k_tree_nodes_f64(TreeNodeArgs64 A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TreeSmem64 &sm = *reinterpret_cast<TreeSmem64 *>(smem_raw);
+    TreeNodeSmem64 &sm = *reinterpret_cast<TreeNodeSmem64 *>(smem_raw);
     const TreeNodeArgs &a = A.n;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int np = *a.W.npool;
     TreeQueue queue{a.queue, 0ull};
     for (int64_t item = queue.first(&sm.item); item < a.W.ncl + np; item = queue.next(&sm.item)) {
@@ -645,87 +664,65 @@ __global__ void __launch_bounds__(kTreeNT) k_tree_nodes_f64(TreeNodeArgs64 A)
         load_geo(&sm.geo, a.geo + cl);
         __syncthreads();
         const float4 self = sm.geo.c, parent = ROOT ? self : sm.pgeo.c;
-        double m[2][3], mm[2], hi[2] = {0.0, 0.0}, lo[2] = {0.0, 0.0};
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int k = q * kTreeNT + tid;
-            const double xi = sm.geo.a1 * cheb_at<kNP64>(1, k % kNP64), eta = sm.geo.a2 * cheb_at<kNP64>(1, k / kNP64);
-            const double r2 = xi * xi + eta * eta, s = 2.0 / (1.0 + r2);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                m[q][c] = s * (xi * sm.geo.e1[c] + eta * sm.geo.e2[c] - r2 * sm.geo.n0[c]);
-            }
-            mm[q] = m[q][0] * m[q][0] + m[q][1] * m[q][1] + m[q][2] * m[q][2];
-        }
-        const bool far = self.w - target_radius(sm.geo) >= A.d_far;
-        auto stage = [&](uint32_t e, Stage64 &d) {
+        double hi[2] = {0.0, 0.0}, lo[2] = {0.0, 0.0};
+        const double xt = ((lane & 8) == 0 ? sm.geo.a1 : sm.geo.a2) * cheb_at<kNP64>(1, lane & 7), x2 = xt * xt;
+        auto stage = [&](uint32_t e, NodeCoef64 &d) {
             const Seg64 &s = A.s64[e];
+            const double *n0 = sm.geo.n0, *e1 = sm.geo.e1, *e2 = sm.geo.e2;
             double D[3], P = 0.0, Q = 0.0, K = 0.0, B0 = 1.0;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                D[c] = (sm.geo.n0[c] - s.xh[c]) - s.xl[c];
+                D[c] = (n0[c] - s.xh[c]) - s.xl[c];
                 P = fma(s.xd[c], D[c], P);
                 Q = fma(s.xp[c], D[c], Q);
                 K = fma(D[c], D[c], K);
-                B0 = fma(s.xd[c], sm.geo.n0[c], B0);
-                d.v[c] = 2.0 * D[c];
-                d.v[4 + c] = s.xd[c];
-                d.v[8 + c] = s.xp[c];
+                B0 = fma(s.xd[c], n0[c], B0);
             }
             const double f = s.xp[0] * s.xh[0] + s.xp[1] * s.xh[1] + s.xp[2] * s.xh[2];   // X'.Xhat
-            if (!far) {
-                d.v[3] = K;
-                d.v[7] = P;
-                d.v[11] = Q;
-                d.v[12] = B0;
-                d.v[13] = f;
-                d.v[14] = s.c;
-                return;
-            }
-            const double sg = s.c < 0.0 ? -1.0 : 1.0, c2 = 0.5 * fabs(s.c), q = sqrt(c2), e1 = B0 - P;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                d.v[c] = sg * (2.0 * D[c]);
-                d.v[4 + c] = q * s.xd[c];
-                d.v[8 + c] = q * s.xp[c];
-            }
-            d.v[3] = sg * K;
-            d.v[7] = 0.5 * q * (B0 + P);
-            d.v[11] = q * (Q + 0.5 * f);
-            d.v[12] = q > 0.0 ? 1.0 / q : 0.0;
-            d.v[13] = 0.5 * e1;
-            d.v[14] = 0.25 * c2 * (f * f - e1 * e1);
-            d.v[15] = sg;
+            auto dot = [](const double *u, const double *v) { return fma(u[2], v[2], fma(u[1], v[1], u[0] * v[0])); };
+            auto put = [&](int k, double con, double x, double y, double sq) {
+                d.v[k][0] = con;
+                d.v[k][1] = x;
+                d.v[k][2] = y;
+                d.v[k][3] = sq;
+            };
+            put(0, 0.5 * K, 2.0 * dot(D, e1), 2.0 * dot(D, e2), 2.0 + fma(-2.0, dot(D, n0), 0.5 * K));
+            const double p0 = dot(s.xd, n0), p1 = dot(s.xd, e1), p2 = dot(s.xd, e2);
+            put(1, 0.5 * B0, p1, p2, fma(0.5, B0, -p0));
+            put(2, s.c * (0.5 * P), s.c * p1, s.c * p2, s.c * fma(0.5, P, -p0));
+            const double q0 = dot(s.xp, n0), q1 = dot(s.xp, e1), q2 = dot(s.xp, e2), A0 = f + Q;
+            put(3, 0.5 * A0, q1, q2, fma(0.5, A0, -q0));
+            put(4, s.c * (0.5 * Q), s.c * q1, s.c * q2, s.c * fma(0.5, Q, -q0));
         };
         auto eval = [&](int cnt) {
             double part[2] = {0.0, 0.0};
-            if (far) {
-#pragma unroll 2
-                for (int s = 0; s < cnt; ++s) {
-                    const double *v = sm.rec[s].v;
+#pragma unroll 1
+            for (int b0 = 0; b0 < cnt; b0 += kTabBatch) {
+                const int nb = cnt - b0 < kTabBatch ? cnt - b0 : kTabBatch;
+                if (b0 > 0) __syncthreads();
+#pragma unroll 1
+                for (int s = tid >> 4; s < nb; s += kTreeNT / 16) {   // entries for xt and -xt
+                    const NodeCoef64 &c = sm.rec[b0 + s];
+                    const bool xi = (lane & 8) == 0;
+                    NodeForms64 *t = sm.tab[s] + (xi ? 0 : kNP64);
 #pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const double Q = fma(m[q][2], v[2], fma(m[q][1], v[1], fma(m[q][0], v[0], fma(v[15], mm[q], v[3]))));
-                        const double U = fma(m[q][2], v[6], fma(m[q][1], v[5], fma(m[q][0], v[4], v[7])));
-                        const double V = fma(m[q][2], v[10], fma(m[q][1], v[9], fma(m[q][0], v[8], v[11])));
-                        const double B = fma(U, v[12], v[13]);
-                        // c (B Xdot.d - A X'.d) / (B d.d) with c / 2 in the squares: twice the quotient
-                        part[q] = fma(fma(-V, V, fma(U, U, v[14])), rcp64(B * Q), part[q]);
+                    for (int k = 0; k < kForms64; ++k) {
+                        const double2 u = *reinterpret_cast<const double2 *>(&c.v[k][0]), v = *reinterpret_cast<const double2 *>(&c.v[k][2]);
+                        const double even = fma(x2, v.y, xi ? u.x : 0.0), lin = xi ? u.y : v.x;
+                        t[lane & 7].v[k] = fma(xt, lin, even);
+                        t[kNP64 - 1 - (lane & 7)].v[k] = fma(-xt, lin, even);
                     }
                 }
-                part[0] *= 2.0;
-                part[1] *= 2.0;
-            } else {
+                __syncthreads();
 #pragma unroll 2
-                for (int s = 0; s < cnt; ++s) {
-                    const double *v = sm.rec[s].v;
+                for (int s = 0; s < nb; ++s) {
+                    const NodeForms64 F = sm.tab[s][tid % kNP64];
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
-                        const double Q = fma(m[q][2], v[2], fma(m[q][1], v[1], fma(m[q][0], v[0], mm[q] + v[3])));
-                        const double g = fma(m[q][2], v[6], fma(m[q][1], v[5], m[q][0] * v[4]));
-                        const double Qd = fma(m[q][2], v[10], fma(m[q][1], v[9], fma(m[q][0], v[8], v[11])));
-                        const double B = v[12] + g, num = fma(B, v[7] + g, -(v[13] + Qd) * Qd);
-                        part[q] = fma(v[14] * num, rcp64(B * Q), part[q]);
+                        const NodeForms64 G = sm.tab[s][kNP64 + q * (kTreeNT / kNP64) + tid / kNP64];
+                        const double Q = F.v[0] + G.v[0], B = F.v[1] + G.v[1], Pd = F.v[2] + G.v[2];
+                        const double An = F.v[3] + G.v[3], Qd = F.v[4] + G.v[4];
+                        part[q] = fma(fma(B, Pd, -(An * Qd)), rcp64(B * Q), part[q]);
                     }
                 }
             }
@@ -739,9 +736,14 @@ __global__ void __launch_bounds__(kTreeNT) k_tree_nodes_f64(TreeNodeArgs64 A)
             cheb_coefs64(a.Fp, a.Wp, pcl, sm.coef, sm.tmp, rhi, rlo);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                double x, y;
-                local_xy64(sm.pgeo, (sm.geo.n0[0] - sm.pgeo.n0[0]) + m[q][0], (sm.geo.n0[1] - sm.pgeo.n0[1]) + m[q][1],
-                           (sm.geo.n0[2] - sm.pgeo.n0[2]) + m[q][2], x, y);
+                const int k = q * kTreeNT + tid;
+                const double xi = sm.geo.a1 * cheb_at<kNP64>(1, k % kNP64), eta = sm.geo.a2 * cheb_at<kNP64>(1, k / kNP64);
+                const double r2 = xi * xi + eta * eta, s = 2.0 / (1.0 + r2);
+                double m[3], x, y;
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    m[c] = (sm.geo.n0[c] - sm.pgeo.n0[c]) + s * (xi * sm.geo.e1[c] + eta * sm.geo.e2[c] - r2 * sm.geo.n0[c]);
+                local_xy64(sm.pgeo, m[0], m[1], m[2], x, y);
                 fold64(hi[q], lo[q], rhi);
                 fold64(hi[q], lo[q], interp64(sm.coef, x, y));
                 lo[q] += rlo;
@@ -883,7 +885,8 @@ TreePlan tree_plan(int prec, int64_t N, int nface, int64_t npix, int64_t n, int 
     p.nn = f64 ? 2 * kNN64 : kNN;   // doubles per cluster
     p.n_pad = (n + kTreeS - 1) / kTreeS * kTreeS;
     p.nst = p.n_pad / kTreeS;
-    p.nslots = f64 ? slots_of((const void *)&k_tree_nodes_f64<false>, sizeof(TreeSmem64), num_sms)
+    p.nslots = f64 ? std::min(slots_of((const void *)&k_tree_nodes_f64<false>, sizeof(TreeNodeSmem64), num_sms),
+                              slots_of((const void *)&k_tree_nodes_f64<true>, sizeof(TreeNodeSmem64), num_sms))
                    : slots_of((const void *)&k_tree_nodes_f32<false>, sizeof(TreeSmem32), num_sms);
     p.pslots = f64 ? slots_of((const void *)&k_tree_pixels_f64, sizeof(TreeSmem64), num_sms)
                    : slots_of((const void *)&k_tree_pixels_f32, sizeof(TreeSmemPix), num_sms);
@@ -1000,13 +1003,12 @@ cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_
         }
         a.queue = queue + L;
         A.s64 = m.s64;
-        A.d_far = m.d_far;
         const int64_t items = p.ncl[L] + p.pool;
         const dim3 grid((unsigned)(items < p.nslots ? items : p.nslots));
         if (f64) {
             const void *fn = root ? (const void *)&k_tree_nodes_f64<true> : (const void *)&k_tree_nodes_f64<false>;
             void *args[] = {(void *)&A};
-            cudaLaunchKernel(fn, grid, dim3(kTreeNT), args, sizeof(TreeSmem64), s);
+            cudaLaunchKernel(fn, grid, dim3(kTreeNT), args, sizeof(TreeNodeSmem64), s);
         } else {
             const void *fn = root ? (const void *)&k_tree_nodes_f32<true> : (const void *)&k_tree_nodes_f32<false>;
             void *args[] = {(void *)&a};
