@@ -232,6 +232,7 @@ int map_tree_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const i
     } else if (full) {
         launch_pixel_table(nside, 0, 0, npix, nullptr, p.leaf, p.leaf, p.ncl[0], nv, tot, outidx, nullptr, c->d_status, s);
         m.order = kSlotsDiag;
+        m.nside = nside;
     } else {
         const uint32_t *pp = launch_pixel_order(nside, pix0, npix, pix_list, sort + sort_bytes, s);
         launch_pixel_table(nside, pix_list ? 2 : 1, pix0, npix, pix_list, p.leaf, p.leaf, p.ncl[0], nv, tot, outidx,

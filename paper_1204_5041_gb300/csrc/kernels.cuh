@@ -177,6 +177,7 @@ struct TreeMapArgs {
     int64_t ldn;
     const int64_t *outidx;
     int order;                // slots of a cluster
+    int64_t nside;            // N_side of a full-sky map, else 0
     double theta_pix;
     const Seg32 *s32;
     const Seg64 *s64;

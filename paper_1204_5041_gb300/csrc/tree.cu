@@ -496,26 +496,18 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_pixels_f32(TreePixArgs a)
 // ------------------------------------------------------------------------------------
 // FP64 maps: 16 x 16 nodes, leaves of 32 x 32 pixels.  The FP64 unit (two FMA lanes per clock and SM)
 // is all that counts, so every thread simply holds its nodes or pixels and reads one staged sample at
-// a time.  N_side 64 with 10,240 samples 18.3 -> 12.3 ms (a leaf of 32 pixels spans 0.5 rad there and four
-// tenths of the pairs stay near), N_side 128 with 25,087 170 -> 46 ms.  Error against the oracle 1.2e-16
-// to 1.7e-16 of the rms (direct kernel 0.5e-16 to 1.2e-16), largest 1.3e-15 (1.0e-15).
+// a time.  N_side 64 with 10,240 samples 18.3 -> 10.5 ms (a leaf of 32 pixels spans 0.5 rad there and four
+// tenths of the pairs stay near), N_side 128 with 25,087 170 -> 41 ms.  Error against the oracle 1.2e-16
+// to 1.9e-16 of the rms (direct kernel 0.5e-16 to 1.2e-16), largest 1.9e-15 (1.0e-15).
 // ------------------------------------------------------------------------------------
 constexpr int kNP64 = 16, kNN64 = kNP64 * kNP64, kLeaf64 = 32;
 constexpr int kNodeTarget64 = 128, kPixTarget64 = 48;
 
-// A staged Far64 or Seg64 record.
+// A staged Far64 record.
 struct __align__(16) Stage64 {
     double v[16];
 };
-static_assert(sizeof(Far64) <= sizeof(Stage64) && sizeof(Seg64) == sizeof(Stage64), "stage layout");
-
-struct __align__(16) TreeSmem64 {
-    Stage64 rec[kTreeBatch];
-    TreeScanSmem scan;
-    TreeGeo geo, pgeo;
-    double coef[kNN64], tmp[kNN64];
-    int64_t item;
-};
+static_assert(sizeof(Far64) <= sizeof(Stage64) && sizeof(Far64) % 16 == 0, "stage layout");
 
 // the interpolant with the shared coefficients at (x, y) in [-1, 1]^2: Clenshaw's recurrence in y, rows
 // added from the highest order down
@@ -596,11 +588,6 @@ __device__ __forceinline__ void tree_batches64(Smem &sm, int count, Stage &&stag
         eval(count - b0 < kTreeBatch ? count - b0 : kTreeBatch);
         __syncthreads();
     }
-}
-
-__device__ __forceinline__ void copy_record(Stage64 &dst, const void *src, int n16)
-{
-    for (int k = 0; k < n16; ++k) reinterpret_cast<double2 *>(dst.v)[k] = reinterpret_cast<const double2 *>(src)[k];
 }
 
 // Far-field pair term (17 FP64 operations, see k_map_f64)
@@ -762,77 +749,292 @@ struct TreePixArgs64 {
     TreePixArgs p;
     const Far64 *far64;
     float d_far;
+    int64_t nside;   // full-sky maps
+    int nb;
 };
 
-// Four pixels per thread, half a cluster per item.  Samples with |d| >= d_far and B >= b_min at every pixel of the cluster in
-// the far-field form (its squares cancel to a factor 1/B of the rounding), the others from the double-double Xhat (29 operations, with rcp64 in the place of a division).
-__global__ void __launch_bounds__(kTreeNT) k_tree_pixels_f64(TreePixArgs64 A)
+// Ring form of the far-field pair term.  A pixel of a ring (z, s = sin theta) at azimuth phi has n / s =
+// (cos phi, sin phi, z / s), so a linear form over s is a function of the ring plus one of the azimuth, and the
+// quotient of degree 2 over degree 2 does not change.  On an equatorial leaf pixel (x, y) has ring x + y and
+// azimuth x - y: tables of 63 + 63 values per sample leave 11 FP64 operations per pixel of 17.  A polar pixel
+// has its own azimuth and takes two operations per form in the place of three (14).  The tables cost 0.8 per
+// pixel.
+// |d|^2 / (2 s) = [(z - zX)^2 + (s - sX)^2] / (2 s) + sX |u - uX|^2 / 2 with azimuth directions u and uX: a sum
+// of squares, so that it keeps its relative accuracy next to the sample, where 1 - n.Xhat cancels (error of
+// a map 3.1e-16 of the rms with that, 1.9e-16 with the squares); a block of polar pixels away from the sample
+// takes - uX.u for the last square.
+constexpr int kRings = 2 * kLeaf64 - 1, kTabPix = 4;
+struct __align__(16) RingForms {
+    double v[6];   // sigma |d|^2 / 2, B, s A - s f/2 (see Far64), -s e/2, -K; the first for the other azimuth part
+};
+struct __align__(16) AzForms {
+    double v[4];   // the first three's azimuth parts
+};
+// A block of pixels: two slots of every lane of a warp
+constexpr int kPix64 = kLeaf64 * kLeaf64 / kTreeNT, kBlocks64 = kPix64 / 2;
+
+struct __align__(16) TreePixSmem64 {
+    Stage64 rec[kTreeBatch];
+    union {
+        double n[3][kLeaf64 * kLeaf64];   // lists and patches: directions
+        struct {
+            double2 u[kLeaf64 * kLeaf64];   // (cos phi, sin phi)
+            RingForms F[kTabPix][kRings + 1];
+            AzForms G[kTabPix][kRings + 1];
+        } sky;
+    };
+    double ring[5][kRings + 1], az[2][kRings + 1];   // z, s, 1/s, z/s, 1/s^2; cos, sin
+    float4 cap[kTreeNT / 32][kBlocks64];
+    TreeScanSmem scan;
+    TreeGeo geo;
+    double coef[kNN64], tmp[kNN64];
+    int64_t item;
+};
+
+// Slot of pixel (lx, ly) in the order of diag_slot_square
+__device__ __forceinline__ int diag_index_square(int lx, int ly, int T)
 {
-    constexpr int TILE = kLeaf64 * kLeaf64, P = 4, PARTS = TILE / (P * kTreeNT);
+    const int k = lx + ly < T - 1 ? lx + ly : 2 * T - 2 - lx - ly, h = k * (k + 1) / 2;
+    return lx + ly < T - 1 ? T * T - 1 - h - ly : h + T - 1 - ly;
+}
+
+// Ring of the table, 0 .. 2 T - 2, and place of the azimuth: even ones first, a warp's pixels then lie in
+// neighbouring entries
+__device__ __forceinline__ int az_place(int l) { return (l >> 1) + (l & 1) * kLeaf64; }
+
+// Eight pixels per thread, one cluster per item: four blocks of 8 x 8 pixels per warp (full sky) or of 64
+// consecutive slots.  Bound by the FP64 unit.  N_side 64 with 10,240 samples 10.2 ms with 17 operations for every
+// pixel -> 8.4 ms, N_side 128 with 30,001 33.5 -> 26.7 ms.  Samples that the cluster's test flags are tested again per block: with |d| >= d_far and
+// B >= b_min on the block they too take the far-field form (its squares cancel to a factor 1/B of the rounding),
+// else the pair term from the double-double Xhat (29 operations).
+template <bool SKY>
+__global__ void __launch_bounds__(kTreeNT, 3) k_tree_pixels_f64(TreePixArgs64 A)
+{
+    constexpr int TILE = kLeaf64 * kLeaf64, P = kPix64;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TreeSmem64 &sm = *reinterpret_cast<TreeSmem64 *>(smem_raw);
+    TreePixSmem64 &sm = *reinterpret_cast<TreePixSmem64 *>(smem_raw);
     const TreePixArgs &a = A.p;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int np = *a.W.npool;
     unsigned zerocnt = 0;
     TreeQueue queue{a.queue, 0ull};
-    for (int64_t it = queue.first(&sm.item); it < (a.W.ncl + np) * PARTS; it = queue.next(&sm.item)) {
+    for (int64_t item = queue.first(&sm.item); item < a.W.ncl + np; item = queue.next(&sm.item)) {
         int kc, nch;
         int64_t at;
-        const int64_t item = it / PARTS, base = it % PARTS * (P * kTreeNT);   // the item's share of the cluster
         const int64_t cl = tree_item(a.W, item, np, kc, nch, at);
         if (cl < 0) continue;
         load_geo(&sm.geo, a.geo + cl);
+        const int64_t k0 = cl * TILE;
+        int slot[P], place[P];   // slot in the cluster; SKY: ring and azimuth entries
+        unsigned valid = 0, eq = 0;
+        if (SKY) {
+            const int64_t N = A.nside, f = cl / ((int64_t)A.nb * A.nb), rem = cl - f * A.nb * A.nb;
+            const int64_t y0 = rem / A.nb * kLeaf64, x0 = rem % A.nb * kLeaf64;
+            const int64_t jr0 = (f < 4 ? 2 : f < 8 ? 3 : 4) * N - x0 - y0 - 1;   // HEALPix ring of entry r: jr0 - r
+            if (tid < kRings) {
+                const int64_t jr = jr0 - tid, i = jr < N ? jr : jr > 3 * N ? 4 * N - jr : N;
+                const double N3 = 3.0 * (double)N;
+                double z, st;
+                if (jr < N || jr > 3 * N) {
+                    const double q = (double)(i * i) / (N3 * (double)N);
+                    z = jr < N ? 1.0 - q : q - 1.0;
+                    st = sqrt((double)(6 * N * N - i * i)) * (double)i / (N3 * (double)N);
+                } else {
+                    z = (double)(4 * N - 2 * jr) / N3;
+                    st = sqrt((double)((2 * jr - N) * (7 * N - 2 * jr))) / N3;
+                }
+                if (!(i > 0)) z = 0.0, st = 1.0;   // past the pole: padding only
+                const double iw = 1.0 / st;
+                sm.ring[0][tid] = z;
+                sm.ring[1][tid] = st;
+                sm.ring[2][tid] = iw;
+                sm.ring[3][tid] = z * iw;
+                sm.ring[4][tid] = iw * iw;
+            } else if (tid >= 64 && tid - 64 < kRings) {
+                const int l = tid - 64;
+                const int64_t jp = f < 4 ? 2 * f + 1 : f < 8 ? 2 * (f - 4) : 2 * (f - 8) + 1;
+                double sp, cp;
+                sincospi_frac(jp * N + x0 - y0 + l - (kLeaf64 - 1), 4 * N, sp, cp);
+                sm.az[0][az_place(l)] = cp;
+                sm.az[1][az_place(l)] = sp;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const int blk = w * kBlocks64 + q / 2, lx = blk % 4 * 8 + (lane & 7), ly = blk / 4 * 8 + q % 2 * 4 + (lane >> 3);
+                slot[q] = diag_index_square(lx, ly, kLeaf64);
+                place[q] = (lx + ly) | az_place(lx - ly + kLeaf64 - 1) << 8;
+                const int64_t jr = jr0 - lx - ly;
+                if (__all_sync(0xffffffffu, jr >= N && jr <= 3 * N)) eq |= 1u << q;
+                if (a.outidx[k0 + slot[q]] >= 0) valid |= 1u << q;
+                const double iw = sm.ring[2][lx + ly];
+                sm.sky.u[q * kTreeNT + tid] = make_double2(a.nv[k0 + slot[q]] * iw, a.nv[a.ldn + k0 + slot[q]] * iw);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                slot[q] = (w * P + q) * 32 + lane;
+                place[q] = 0;
+                if (a.outidx[k0 + slot[q]] >= 0) valid |= 1u << q;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) sm.n[c][q * kTreeNT + tid] = a.nv[c * a.ldn + k0 + slot[q]];
+            }
+        }
+        // balls of the blocks (radius < 0: no pixel)
+#pragma unroll
+        for (int p = 0; p < kBlocks64; ++p) {
+            float4 x[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int64_t k = k0 + slot[2 * p + u];
+                x[u] = make_float4((float)a.nv[k], (float)a.nv[a.ldn + k], (float)a.nv[2 * a.ldn + k],
+                                   valid >> (2 * p + u) & 1 ? 0.f : -1.f);
+            }
+            const TreeCap c = warp_ball(x);
+            if (lane == 0) sm.cap[w][p] = c.a;
+        }
         __syncthreads();
         const float4 self = sm.geo.c;
-        double n[P][3], hi[P], lo[P];
-        unsigned valid = 0;
+        double hi[P], lo[P];
 #pragma unroll
-        for (int q = 0; q < P; ++q) {
-            const int64_t k = cl * TILE + base + q * kTreeNT + tid;
-            if (a.outidx[k] >= 0) valid |= 1u << q;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) n[q][c] = a.nv[c * a.ldn + k];
-            hi[q] = lo[q] = 0.0;
-        }
+        for (int q = 0; q < P; ++q) hi[q] = lo[q] = 0.0;
         auto stage = [&](uint32_t e, Stage64 &d) {
-            const uint32_t r = e & kTreeIndex;
-            if (e & (kTreeClose | kTreeBeam)) copy_record(d, a.s64 + r, sizeof(Seg64) / 16);
-            else copy_record(d, A.far64 + r, sizeof(Far64) / 16);
+            const double2 *src = reinterpret_cast<const double2 *>(A.far64 + (e & kTreeIndex));
+#pragma unroll
+            for (int k = 0; k < (int)sizeof(Far64) / 16; ++k) reinterpret_cast<double2 *>(d.v)[k] = src[k];
+            if (SKY) {   // sigma sX, sigma / (2 sX)
+                const double sX = sqrt(fma(d.v[1], d.v[1], d.v[0] * d.v[0]));
+                d.v[14] = copysign(sX, d.v[3]);
+                d.v[15] = sX > 0.0 ? 0.5 / d.v[14] : 0.0;
+            }
         };
-        int b0 = 0;   // list position of the batch
+        // the far-field form at one block
+        auto far_block = [&](const Stage64 &rec, int p, int ts, bool close, double &p0, double &p1) {
+            double *const part[2] = {&p0, &p1};
+            const Far64 &r = *reinterpret_cast<const Far64 *>(rec.v);
+            if (SKY) {
+                const bool e2 = (eq >> (2 * p) & 3) == 3;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int q = 2 * p + u;
+                    const RingForms &F = sm.sky.F[ts][place[q] & 0xff];
+                    double hs, B, A2;
+                    if (e2) {
+                        const AzForms &G = sm.sky.G[ts][place[q] >> 8];
+                        hs = F.v[0] + G.v[0];
+                        B = F.v[1] + G.v[1];
+                        A2 = F.v[2] + G.v[2];
+                    } else {
+                        const double2 n = sm.sky.u[q * kTreeNT + tid];
+                        if (close) {
+                            const double *v = rec.v;
+                            const double x = fma(v[14], n.x, v[0]), y = fma(v[14], n.y, v[1]);
+                            hs = fma(v[15], fma(y, y, x * x), F.v[0]);
+                        } else {
+                            hs = fma(n.y, r.mxh[1], fma(n.x, r.mxh[0], F.v[5]));
+                        }
+                        B = fma(n.y, r.xd[1], fma(n.x, r.xd[0], F.v[1]));
+                        A2 = fma(n.y, r.xp[1], fma(n.x, r.xp[0], F.v[2]));
+                    }
+                    const double B2 = fma(r.sx, B, F.v[3]);
+                    *part[u] = fma(fma(-A2, A2, fma(B2, B2, F.v[4])), rcp64(B * hs), *part[u]);
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int i = (2 * p + u) * kTreeNT + tid;
+                    *part[u] = far_term64(r, sm.n[0][i], sm.n[1][i], sm.n[2][i], *part[u]);
+                }
+            }
+        };
+        auto near_block = [&](const Seg64 &g, int p, double &p0, double &p1) {
+            double *const part[2] = {&p0, &p1};
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int q = 2 * p + u;
+                const int64_t k = k0 + slot[q];
+                const double nx = a.nv[k], ny = a.nv[a.ldn + k], nz = a.nv[2 * a.ldn + k];
+                const double dx = (nx - g.xh[0]) - g.xl[0], dy = (ny - g.xh[1]) - g.xl[1], dz = (nz - g.xh[2]) - g.xl[2];
+                const double Q = fma(dz, dz, fma(dy, dy, dx * dx));
+                const double Pd = fma(g.xd[2], dz, fma(g.xd[1], dy, g.xd[0] * dx));
+                const double Qd = fma(g.xp[2], dz, fma(g.xp[1], dy, g.xp[0] * dx));
+                // A and B from n itself: 1 + Xdot.Xhat + Xdot.d would round a small B twice
+                const double An = nx * g.xp[0] + ny * g.xp[1] + nz * g.xp[2];
+                const double B = 1.0 + (nx * g.xd[0] + ny * g.xd[1] + nz * g.xd[2]);
+                const double num = B * Pd - An * Qd, den = B * Q;
+                // the estimate of the reciprocal needs a normal value
+                const int ex = __double2hiint(den) & 0x7ff00000;
+                if (ex > 0x39b00000 && ex < 0x46000000) {
+                    *part[u] = fma(g.c * num, rcp64(den), *part[u]);
+                } else if (Q == 0.0) {
+                    if (valid >> q & 1) ++zerocnt;
+                } else {
+                    *part[u] += g.c * num / den;
+                }
+            }
+        };
+        // whether a flagged sample may take the far-field form on block p
+        auto far_on = [&](const float4 xh, const float4 bm, int p) {
+            const float4 c = sm.cap[w][p];
+            float x = c.x - xh.x, y = c.y - xh.y, z = c.z - xh.z;
+            const float d = sqrtf(x * x + y * y + z * z) - c.w;
+            x = c.x - bm.x, y = c.y - bm.y, z = c.z - bm.z;
+            const float h = fmaxf(sqrtf(x * x + y * y + z * z) - c.w, 0.f);
+            return c.w < 0.f || (d >= A.d_far && fmaf(0.5f * (1.f - bm.w) * h, h, bm.w) >= a.b_min);
+        };
+        int l0 = 0;   // list position of the batch
         auto eval = [&](int cnt) {
             double part[P];
 #pragma unroll
             for (int q = 0; q < P; ++q) part[q] = 0.0;
 #pragma unroll 1
-            for (int s = 0; s < cnt; ++s) {
-                if (!(sm.scan.list[b0 + s] & (kTreeClose | kTreeBeam))) {
-                    const Far64 &r = *reinterpret_cast<const Far64 *>(sm.rec[s].v);
-#pragma unroll
-                    for (int q = 0; q < P; ++q) part[q] = far_term64(r, n[q][0], n[q][1], n[q][2], part[q]);
-                    continue;
+            for (int b0 = 0; b0 < cnt; b0 += kTabPix) {
+                const int nb = cnt - b0 < kTabPix ? cnt - b0 : kTabPix;
+                if (SKY) {
+                    if (b0 > 0) __syncthreads();
+                    if (tid < kRings) {
+                        const double z = sm.ring[0][tid], st = sm.ring[1][tid], iw = sm.ring[2][tid], zw = sm.ring[3][tid],
+                                     iw2 = sm.ring[4][tid];
+                        for (int s = 0; s < nb; ++s) {
+                            const Far64 &r = *reinterpret_cast<const Far64 *>(sm.rec[b0 + s].v);
+                            RingForms &F = sm.sky.F[s][tid];
+                            const double S = sm.rec[b0 + s].v[14], x = fma(r.sg, z, r.mxh[2]), y = fma(r.sg, st, -S);
+                            const double h = fma(y, y, x * x) * (0.5 * r.sg * iw);
+                            F.v[0] = h;
+                            F.v[5] = h + S;
+                            F.v[1] = fma(r.xd[2], zw, iw);
+                            F.v[2] = fma(r.xp[2], zw, r.af * iw);
+                            F.v[3] = r.be * iw;
+                            F.v[4] = -r.K * iw2;
+                        }
+                    } else if (tid >= 64 && tid - 64 < kRings) {
+                        const double c = sm.az[0][tid - 64], d = sm.az[1][tid - 64];
+                        for (int s = 0; s < nb; ++s) {
+                            const Far64 &r = *reinterpret_cast<const Far64 *>(sm.rec[b0 + s].v);
+                            AzForms &G = sm.sky.G[s][tid - 64];
+                            const double *v = sm.rec[b0 + s].v;
+                            const double x = fma(v[14], c, v[0]), y = fma(v[14], d, v[1]);
+                            G.v[0] = v[15] * fma(y, y, x * x);
+                            G.v[1] = fma(r.xd[1], d, r.xd[0] * c);
+                            G.v[2] = fma(r.xp[1], d, r.xp[0] * c);
+                        }
+                    }
+                    __syncthreads();
                 }
-                const Seg64 &g = *reinterpret_cast<const Seg64 *>(sm.rec[s].v);
+#pragma unroll 1
+                for (int s = 0; s < nb; ++s) {
+                    const uint32_t e = sm.scan.list[l0 + b0 + s];
+                    const Stage64 &r = sm.rec[b0 + s];
+                    if (!(e & (kTreeClose | kTreeBeam))) {
 #pragma unroll
-                for (int q = 0; q < P; ++q) {
-                    const double dx = (n[q][0] - g.xh[0]) - g.xl[0], dy = (n[q][1] - g.xh[1]) - g.xl[1],
-                                 dz = (n[q][2] - g.xh[2]) - g.xl[2];
-                    const double Q = fma(dz, dz, fma(dy, dy, dx * dx));
-                    const double Pd = fma(g.xd[2], dz, fma(g.xd[1], dy, g.xd[0] * dx));
-                    const double Qd = fma(g.xp[2], dz, fma(g.xp[1], dy, g.xp[0] * dx));
-                    // A and B from n itself: 1 + Xdot.Xhat + Xdot.d would round a small B twice
-                    const double A = n[q][0] * g.xp[0] + n[q][1] * g.xp[1] + n[q][2] * g.xp[2];
-                    const double B = 1.0 + (n[q][0] * g.xd[0] + n[q][1] * g.xd[1] + n[q][2] * g.xd[2]);
-                    const double num = B * Pd - A * Qd, den = B * Q;
-                    // the float estimate of the reciprocal needs a value inside the float range
-                    const int ex = __double2hiint(den) & 0x7ff00000;
-                    if (ex > 0x39b00000 && ex < 0x46000000) {
-                        part[q] = fma(g.c * num, rcp64(den), part[q]);
-                    } else if (Q == 0.0) {
-                        if (valid & (1u << q)) ++zerocnt;
-                    } else {
-                        part[q] += g.c * num / den;
+                        for (int p = 0; p < kBlocks64; ++p) far_block(r, p, s, false, part[2 * p], part[2 * p + 1]);
+                        continue;
+                    }
+                    const float4 xh = a.S.crit[e & kTreeIndex].a, bm = a.S.crit[e & kTreeIndex].b;
+#pragma unroll
+                    for (int p = 0; p < kBlocks64; ++p) {
+                        if (far_on(xh, bm, p)) far_block(r, p, s, true, part[2 * p], part[2 * p + 1]);
+                        else near_block(a.s64[e & kTreeIndex], p, part[2 * p], part[2 * p + 1]);
                     }
                 }
             }
@@ -841,20 +1043,20 @@ __global__ void __launch_bounds__(kTreeNT) k_tree_pixels_f64(TreePixArgs64 A)
         };
         const float R = target_radius(sm.geo);
         tree_scan<false, true>(a.S, kc, nch, self, self, R, A.d_far + R, a.b_min, sm.scan, [&](int count) {
-            b0 = 0;
+            l0 = 0;
             tree_batches64(sm, count, stage, [&](int cnt) {
                 eval(cnt);
-                b0 += kTreeBatch;
+                l0 += kTreeBatch;
             });
         });
         double rhi = 0.0, rlo = 0.0;
         if (kc == 0) cheb_coefs64(a.F, a.Wf, cl, sm.coef, sm.tmp, rhi, rlo);
 #pragma unroll
         for (int q = 0; q < P; ++q) {
-            const int64_t k = cl * TILE + base + q * kTreeNT + tid;
+            const int64_t k = k0 + slot[q];
             if (kc == 0) {
                 double x, y;
-                local_xy64(sm.geo, n[q][0] - sm.geo.n0[0], n[q][1] - sm.geo.n0[1], n[q][2] - sm.geo.n0[2], x, y);
+                local_xy64(sm.geo, a.nv[k] - sm.geo.n0[0], a.nv[a.ldn + k] - sm.geo.n0[1], a.nv[2 * a.ldn + k] - sm.geo.n0[2], x, y);
                 fold64(hi[q], lo[q], rhi);
                 fold64(hi[q], lo[q], interp64(sm.coef, x, y));
                 lo[q] += rlo;
@@ -864,12 +1066,13 @@ __global__ void __launch_bounds__(kTreeNT) k_tree_pixels_f64(TreePixArgs64 A)
                 const int64_t oi = a.outidx[k];
                 if (oi >= 0) a.theta[oi] = a.accumulate ? a.theta[oi] + v : v;
             } else {
-                a.partial[item * TILE + base + q * kTreeNT + tid] = v;   // pool entry of the chunk
+                a.partial[item * TILE + slot[q]] = v;   // pool entry of the chunk
             }
         }
+        __syncthreads();
     }
     for (int o = 16; o > 0; o >>= 1) zerocnt += __shfl_xor_sync(0xffffffffu, zerocnt, o);
-    if ((tid & 31) == 0 && zerocnt) atomicAdd(&a.st->zero_pairs, (unsigned long long)zerocnt);
+    if (lane == 0 && zerocnt) atomicAdd(&a.st->zero_pairs, (unsigned long long)zerocnt);
 }
 
 }  // namespace
@@ -888,7 +1091,8 @@ TreePlan tree_plan(int prec, int64_t N, int nface, int64_t npix, int64_t n, int 
     p.nslots = f64 ? std::min(slots_of((const void *)&k_tree_nodes_f64<false>, sizeof(TreeNodeSmem64), num_sms),
                               slots_of((const void *)&k_tree_nodes_f64<true>, sizeof(TreeNodeSmem64), num_sms))
                    : slots_of((const void *)&k_tree_nodes_f32<false>, sizeof(TreeSmem32), num_sms);
-    p.pslots = f64 ? slots_of((const void *)&k_tree_pixels_f64, sizeof(TreeSmem64), num_sms)
+    p.pslots = f64 ? std::min(slots_of((const void *)&k_tree_pixels_f64<false>, sizeof(TreePixSmem64), num_sms),
+                              slots_of((const void *)&k_tree_pixels_f64<true>, sizeof(TreePixSmem64), num_sms))
                    : slots_of((const void *)&k_tree_pixels_f32, sizeof(TreeSmemPix), num_sms);
     int64_t all = 0;
     int64_t nb = nface > 0 ? (N + p.leaf - 1) / p.leaf : 0;
@@ -1035,9 +1239,12 @@ cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_
     a.queue = queue + kTreeLevels;
     A.far64 = m.far64;
     A.d_far = m.d_far;
-    const int64_t items = (p.ncl[0] + p.ppool) * (f64 ? 2 : 1);
+    A.nside = m.nside;
+    A.nb = p.nb[0];
+    const int64_t items = p.ncl[0] + p.ppool;
     const unsigned grid = (unsigned)(items < p.pslots ? items : p.pslots);
-    if (f64) k_tree_pixels_f64<<<grid, kTreeNT, sizeof(TreeSmem64), s>>>(A);
+    if (f64 && m.nside > 0) k_tree_pixels_f64<true><<<grid, kTreeNT, sizeof(TreePixSmem64), s>>>(A);
+    else if (f64) k_tree_pixels_f64<false><<<grid, kTreeNT, sizeof(TreePixSmem64), s>>>(A);
     else k_tree_pixels_f32<<<grid, kTreeNT, sizeof(TreeSmemPix), s>>>(a);
     k_tree_reduce<<<(unsigned)p.pslots, 256, 0, s>>>(a.W, p.leaf * p.leaf, a.partial, m.outidx, m.theta, m.accumulate);
     return cudaSuccess;

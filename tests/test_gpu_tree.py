@@ -81,6 +81,24 @@ def test_tree_sizes_f64(isw, nside, n):
     _check(isw, nside, _samples(n, nside), "f64", TOL64)
 
 
+@pytest.mark.parametrize("nside", [64, 65, 95, 130])
+def test_tree_rings_f64(isw, nside):
+    """Samples and beams at the poles, on the border of the polar caps and at azimuths where faces meet: the
+    pixels' ring and azimuth forms have their edges there."""
+    S = _samples(600, nside + 1)
+    k = 0
+    for z in (1.0, -1.0, 2 / 3, -2 / 3, 0.0, 1 - 1e-12, 0.6666):
+        for phi in np.arange(8) * np.pi / 4:
+            s = np.sqrt(1 - z * z)
+            v = np.array([s * np.cos(phi), s * np.sin(phi), z]) if abs(z) < 1 else np.array([0.0, 0.0, z])
+            S[0:3, k] = 0.4 * v
+            t = np.cross(v, [0.3, 0.5, 0.8])
+            t /= np.linalg.norm(t)
+            S[3:6, k + 1], S[6:9, k + 1] = -0.999 * v, np.sqrt(1 - 0.999**2) * t
+            k += 2
+    _check(isw, nside, S, "f64", TOL64)
+
+
 @pytest.mark.parametrize("prec,tol", [("f32c", BAR32), ("f64", TOL64)])
 @pytest.mark.parametrize("kw", [dict(spot=1e-3), dict(spot=0.0), dict(cusp=True), dict(mixed=True), dict(spot=0.05, mixed=True)])
 def test_tree_sample_layouts(isw, kw, prec, tol):
