@@ -971,11 +971,13 @@ int isw_map_adjoint(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const
         return ISW_OK;
     }
     const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
-    if (prec == ISW_F32C && c->split_override == 0 && tree_rule(prec, npix, n) && npix < (int64_t(1) << 32)) {
+    if (c->split_override == 0 && tree_rule(prec, npix, n) && npix < (int64_t(1) << 32)) {
+        const bool f64 = prec == ISW_F64;
+        const int orders = f64 ? 1 : 2;
         const bool full = !pix_list && pix0 == 0 && npix == 12 * nside * nside;
-        const AdjTreePlan p = adj_tree_plan(nside, full ? 12 : 0, npix, n, c->num_sms);
+        const AdjTreePlan p = (f64 ? adj_tree_plan64 : adj_tree_plan)(nside, full ? 12 : 0, npix, n, c->num_sms);
         const int64_t tot = p.map.ncl[0] * p.map.leaf * p.map.leaf;
-        const size_t sort_bytes = (sort_scratch_bytes(n, 2) + 255) / 256 * 256;
+        const size_t sort_bytes = (sort_scratch_bytes(n, orders) + 255) / 256 * 256;
         if ((r = ensure_ws(c, kWsNv, (size_t)tot * 3 * sizeof(double)))) return r;
         if ((r = ensure_ws(c, kWsOut, (size_t)tot * sizeof(int64_t)))) return r;
         if ((r = ensure_ws(c, kWsS32, (size_t)p.n_pad * sizeof(Seg32)))) return r;
@@ -992,7 +994,7 @@ int isw_map_adjoint(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const
                            nv, tot, outidx, nullptr, c->d_status, s, pp);
         AdjTreeCall m{};
         m.theta_pix = std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
-        m.perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], sort, 2, s);
+        m.perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], sort, orders, s);
         launch_pack(samples, n, ld, xo[0], xo[1], xo[2], GU, m.theta_pix, c->near_k, p.n_pad, m.perm, s32, s64, nullptr,
                     nullptr, nullptr, c->d_status, s);
         m.nv = nv;
@@ -1004,13 +1006,14 @@ int isw_map_adjoint(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const
         m.s64 = s64;
         m.n = n;
         m.b_min = (float)c->b_min;
+        m.d_far = (float)c->d_far;
         m.ngrad = ngrad;
         m.grad = grad_out;
         m.ld_g = ld_g;
         m.st = c->d_status;
         m.scratch = c->ws[kWsTree];
         const int ti = timing_begin(c, s);
-        cudaError_t e = launch_adjoint_tree(p, m, s);
+        cudaError_t e = f64 ? launch_adjoint_tree64(p, m, s) : launch_adjoint_tree(p, m, s);
         if (e != cudaSuccess) return cuda_err(c, e, "isw_map_adjoint launch");
         timing_end(c, ti, s);
         c->n_pair += 1;

@@ -791,13 +791,6 @@ struct __align__(16) TreePixSmem64 {
     int64_t item;
 };
 
-// Slot of pixel (lx, ly) in the order of diag_slot_square
-__device__ __forceinline__ int diag_index_square(int lx, int ly, int T)
-{
-    const int k = lx + ly < T - 1 ? lx + ly : 2 * T - 2 - lx - ly, h = k * (k + 1) / 2;
-    return lx + ly < T - 1 ? T * T - 1 - h - ly : h + T - 1 - ly;
-}
-
 // Ring of the table, 0 .. 2 T - 2, and place of the azimuth: even ones first, a warp's pixels then lie in
 // neighbouring entries
 __device__ __forceinline__ int az_place(int l) { return (l >> 1) + (l & 1) * kLeaf64; }

@@ -464,6 +464,13 @@ __device__ __forceinline__ void diag_slot_square(int l, int T, int &lx, int &ly)
     }
 }
 
+// Slot of pixel (lx, ly) in the order of diag_slot_square
+__device__ __forceinline__ int diag_index_square(int lx, int ly, int T)
+{
+    const int k = lx + ly < T - 1 ? lx + ly : 2 * T - 2 - lx - ly, h = k * (k + 1) / 2;
+    return lx + ly < T - 1 ? T * T - 1 - h - ly : h + T - 1 - ly;
+}
+
 namespace {
 
 __device__ __forceinline__ float warp_sum(float v)

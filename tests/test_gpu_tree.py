@@ -259,3 +259,46 @@ def test_adjoint_tree_list(isw):
         for b in (slice(0, 3), slice(3, 6)):
             assert ((got - ref)[b].abs().max() / ref[b].abs().max()).item() <= 1e-6
     assert isw.default_context().check_status()[0] == isw.OK
+
+
+@pytest.mark.parametrize("nside,n,ngrad,kw", [(64, 407, 6, {}), (65, 448, 10, {}), (67, 449, 9, dict(spot=0.05, mixed=True)),
+                                              (96, 4001, 6, dict(spot=1e-3)), (100, 1001, 10, dict(cusp=True)), (257, 63, 9, {})])
+def test_adjoint_tree_f64(isw, nside, n, ngrad, kw):
+    """FP64 gradients over the tree against the direct FP64 kernel, per block of rows relative to the block's
+    largest entry; samples on the line of sight of a pixel, at a pole, skipped.  Bound: the two sum ~1e5 terms of
+    either sign in different orders, 1e-15 of the largest terms, and a beam with 1 - |Xdot| = 1e-8 magnifies the
+    rounding of B by up to 1e-16 / 1e-8 against the largest entry's own size; hence 1e-12 (1e-7 with cusps)."""
+    S = _samples(n, nside, **kw)
+    S[3:6, n // 2] = [0.0, 0.6, 0.8]
+    S[0:3, 3] = [0.0, 0.0, 0.5]
+    S[0:3, 7] = isw.hp_pix2vec_ring(nside).cpu().numpy()[:, 12345]
+    Sd = torch.from_numpy(S).cuda()
+    g = torch.randn(12 * nside * nside, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    ctx = isw.default_context()
+    ctx.check_status()
+    got = _adjoint(isw, nside, Sd, g, "f64", ngrad)
+    status, counts = ctx.check_status()
+    ref = _adjoint(isw, nside, Sd, g, "f64", ngrad, split=4)
+    status_d, counts_d = ctx.check_status()
+    assert status == status_d and counts["skipped_samples"] == counts_d["skipped_samples"] == 1
+    assert counts["zero_pairs"] == counts_d["zero_pairs"]
+    assert (got[:, n // 2] == 0).all()
+    used = torch.arange(n, device="cuda") != n // 2
+    for a in range(0, ngrad, 3):
+        b = (slice(a, min(a + 3, ngrad)), used)
+        assert ((got - ref)[b].abs().max() / ref[b].abs().max()).item() <= (1e-7 if "cusp" in kw else 1e-12)
+    assert torch.equal(got, _adjoint(isw, nside, Sd, g, "f64", ngrad))
+    ctx.check_status()
+
+
+def test_adjoint_tree_list_f64(isw):
+    nside, npix, n = 256, 49153, 500
+    S = torch.from_numpy(_samples(n, 12)).cuda()
+    pix = torch.randint(12 * nside * nside, (npix,), device="cuda", generator=torch.Generator("cuda").manual_seed(2))
+    g = torch.randn(npix, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    for kw in (dict(pix=pix), dict(pix0=1234, npix=npix)):
+        got = _adjoint(isw, nside, S, g, "f64", 6, **kw)
+        ref = _adjoint(isw, nside, S, g, "f64", 6, split=4, **kw)
+        for b in (slice(0, 3), slice(3, 6)):
+            assert ((got - ref)[b].abs().max() / ref[b].abs().max()).item() <= 1e-12
+    assert isw.default_context().check_status()[0] == isw.OK
