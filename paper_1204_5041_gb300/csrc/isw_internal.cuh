@@ -23,9 +23,33 @@ __device__ __forceinline__ double dsqrt(double a) { return __dsqrt_rn(a); }
 // pi rounded to the nearest double
 constexpr double kPi = 3.14159265358979323846264338327950288;
 
+// a / C rounded to nearest, C an integer below 1024.  With r = RN(1/C), q = RN(a r) is off by less than two
+// ulps, so a - C q is exact, and q plus its correction is off by far less than an ulp / (2 C), the least
+// distance of a / C from a rounding boundary (no quotient lies on one: an odd 54-bit number times C has no
+// 53-bit product).  Three operations instead of the division's chain (the 20 divisions of a sine and cosine
+// bound the light-cone solve's latency, 218 -> 141 us for 10,240 segments, and the pixel tables); where the product underflows, q and the
+// quotient may differ in the last subnormal digit.
+template <int C>
+__device__ __forceinline__ double ddiv_const(double a)
+{
+    static_assert(C > 0 && C < 1024, "range of the proof");
+    constexpr double r = 1.0 / C;
+    const double q = dmul(a, r);
+    return __fma_rn(__fma_rn(-(double)C, q, a), r, q);
+}
+
+template <int K>
+__device__ __forceinline__ void sincos_terms(double x2, double (&st)[11], double (&ct)[11])
+{
+    st[K] = ddiv_const<2 * K * (2 * K + 1)>(dmul(st[K - 1], x2));
+    ct[K] = ddiv_const<(2 * K - 1) * 2 * K>(dmul(ct[K - 1], x2));
+    if constexpr (K < 10) sincos_terms<K + 1>(x2, st, ct);
+}
+
 // sin and cos of x = f * pi/4, f in [0, 1]: Taylor series, ten terms after the first, each
 // term obtained from the previous one by (term * x^2) / ((2k)(2k+1)) (sin) or
-// / ((2k-1)(2k)) (cos), summed from the smallest term up.
+// / ((2k-1)(2k)) (cos), summed from the smallest term up.  A term small enough to be subnormal is lost in the
+// sum (the first term of either series is larger by 1e200), so the result is that of the divisions.
 __device__ __forceinline__ void sincos_octant(double f, double &s, double &c)
 {
     const double quarter_pi = kPi * 0.25;
@@ -34,11 +58,7 @@ __device__ __forceinline__ void sincos_octant(double f, double &s, double &c)
     double st[11], ct[11];
     st[0] = x;
     ct[0] = 1.0;
-#pragma unroll
-    for (int k = 1; k <= 10; ++k) {
-        st[k] = ddiv(dmul(st[k - 1], x2), (double)((2 * k) * (2 * k + 1)));
-        ct[k] = ddiv(dmul(ct[k - 1], x2), (double)((2 * k - 1) * (2 * k)));
-    }
+    sincos_terms<1>(x2, st, ct);
     double S = 0.0, C = 0.0;
 #pragma unroll
     for (int k = 10; k >= 0; --k) {
