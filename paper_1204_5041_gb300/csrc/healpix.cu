@@ -91,6 +91,85 @@ __global__ void k_pixel_table(int64_t N, int mode, int64_t pix0, int64_t npix, c
     }
 }
 
+// The same table for a full sky in T x T blocks (T <= 32), with the same bits.  Pixel (ix, iy) of faces 0-3
+// and pixel (N - 1 - ix, N - 1 - iy) of faces 8-11 have rings mirrored about the equator and, folded into an
+// octant, the same azimuth fraction 1 - |ix - iy| / nr (nr pixels per quarter ring); the four equatorial
+// faces share |ix - iy| / N.  So a CTA takes one block of all eight (four) faces: rings (z, sin theta) and the
+// equatorial azimuths are computed once per block, a polar azimuth once per eight pixels.  One sine and
+// cosine per eight pixels instead of one each: at N_side 1024 0.27 ms instead of 3.5 (the stores take 0.06).
+__global__ void __launch_bounds__(256) k_sky_table(int64_t N, int T, int64_t nb, double *__restrict__ nv, int64_t ldn,
+                                                   int64_t *__restrict__ outidx)
+{
+    __shared__ double rz[64], rs[64], as[64], ac[64];
+    const int tid = threadIdx.x;
+    const bool belt = (int64_t)blockIdx.x >= nb * nb;   // faces 4-7
+    const int64_t t = blockIdx.x - (belt ? nb * nb : 0), x0 = t % nb * T, y0 = t / nb * T;
+    const int64_t jr0 = (belt ? 3 : 2) * N - x0 - y0 - 1;   // ring of ix + iy = x0 + y0
+    if (tid < 2 * T - 1) {
+        const int64_t i = jr0 - tid;
+        if (i >= 1 && i < N) {
+            rz[tid] = ddiv((double)(3 * N * N - i * i), (double)(3 * N * N));
+            rs[tid] = ddiv(dmul((double)i, dsqrt((double)(6 * N * N - i * i))), (double)(3 * N * N));
+        } else if (i >= N) {
+            rz[tid] = ddiv((double)(4 * N - 2 * i), (double)(3 * N));
+            rs[tid] = ddiv(dsqrt((double)((2 * i - N) * (7 * N - 2 * i))), (double)(3 * N));
+        }
+    } else if (tid >= 64 && tid - 64 < 2 * T - 1) {
+        const int64_t d = x0 - y0 + (tid - 64) - (T - 1), m = d < 0 ? -d : d;
+        if (m <= N) sincos_octant(ddiv((double)(belt ? m : N - m), (double)N), as[tid - 64], ac[tid - 64]);
+    }
+    __syncthreads();
+    const int64_t ncap = 2 * N * (N - 1), npix = 12 * N * N, blocks = nb * nb;
+    for (int l = tid; l < T * T; l += 256) {
+        int lx, ly;
+        diag_slot_square(l, T, lx, ly);
+        const int64_t ix = x0 + lx, iy = y0 + ly;
+        const int64_t k0 = t * T * T + l;   // slot on face 0
+        if (ix >= N || iy >= N) {
+            for (int f = 0; f < (belt ? 4 : 8); ++f) {
+                const int64_t k = k0 + (belt ? 4 + f : f < 4 ? f : 4 + f) * blocks * T * T;
+                nv[k] = nv[ldn + k] = 0.0;
+                nv[2 * ldn + k] = 1.0;
+                outidx[k] = -1;
+            }
+            continue;
+        }
+        const int64_t jr = jr0 - lx - ly, d = ix - iy, nr = jr < N ? jr : N;
+        const double z = rz[lx + ly], st = rs[lx + ly];
+        double sf, cf;
+        if (jr < N) {
+            sincos_octant(ddiv((double)(nr - (d < 0 ? -d : d)), (double)nr), sf, cf);
+        } else {
+            sf = as[lx - ly + T - 1];
+            cf = ac[lx - ly + T - 1];
+        }
+        const int64_t kshift = jr < N ? 0 : (jr - N) & 1;
+        auto put = [&](int64_t k, int jp_face, int64_t dd, double zz, int64_t before) {
+            double s, c;
+            octant_unfold(jp_face + (dd < 0 ? 7 : 8), sf, cf, s, c);
+            int64_t jp = ((int64_t)jp_face * nr + dd + 1 + kshift + 8 * nr) / 2 - 4 * nr;
+            if (jp > 4 * nr) jp -= 4 * nr;
+            if (jp < 1) jp += 4 * nr;
+            nv[k] = dmul(st, c);
+            nv[ldn + k] = dmul(st, s);
+            nv[2 * ldn + k] = zz;
+            outidx[k] = before + jp - 1;
+        };
+        if (belt) {
+            for (int f = 0; f < 4; ++f) put(k0 + (4 + f) * blocks * T * T, 2 * f, d, z, ncap + (jr - N) * 4 * N);
+        } else {
+            const int mx = (int)(N - 1 - ix), my = (int)(N - 1 - iy);
+            const int64_t km = (my / T * nb + mx / T) * T * T + diag_index_square(mx % T, my % T, T);
+            const int64_t north = jr < N ? 2 * nr * (nr - 1) : ncap + (jr - N) * 4 * N;
+            const int64_t south = jr < N ? npix - 2 * nr * (nr + 1) : ncap + (3 * N - jr) * 4 * N;
+            for (int f = 0; f < 4; ++f) {
+                put(k0 + f * blocks * T * T, 2 * f + 1, d, z, north);
+                put(km + (8 + f) * blocks * T * T, 2 * f + 1, -d, -z, south);
+            }
+        }
+    }
+}
+
 // Bounding cap of each pixel tile: centre = normalised mean direction, radius = largest
 // chord from the centre (valid pixels only).  One block of 256 threads per tile.
 __global__ void k_pixel_caps(const double *__restrict__ nv, int64_t ldn, const int64_t *__restrict__ outidx,
@@ -202,7 +281,11 @@ void launch_pixel_table(int64_t N, int mode, int64_t pix0, int64_t npix, const i
     const int threads = 256;
     int64_t blocks = (total + threads - 1) / threads;
     if (blocks > 152 * 64) blocks = 152 * 64;
-    k_pixel_table<<<(unsigned)blocks, threads, 0, s>>>(N, mode, pix0, npix, pix_list, tx, ty, ntiles, nv, ldn, outidx,
+    const int64_t nb = (N + tx - 1) / tx;
+    if (mode == 0 && tx == ty && tx <= 32 && nb < 30000)
+        k_sky_table<<<(unsigned)(2 * nb * nb), 256, 0, s>>>(N, tx, nb, nv, ldn, outidx);
+    else
+        k_pixel_table<<<(unsigned)blocks, threads, 0, s>>>(N, mode, pix0, npix, pix_list, tx, ty, ntiles, nv, ldn, outidx,
                                                        perm, st);
     if (caps) k_pixel_caps<<<(unsigned)ntiles, 256, 0, s>>>(nv, ldn, outidx, tx * ty, caps);
 }

@@ -238,6 +238,33 @@ __device__ __forceinline__ int64_t vec2pix_ring(int64_t N, double vx, double vy,
     return 12 * N * N - 2 * ir * (ir + 1) + ip;
 }
 
+// Position (lx, ly) of slot l in a T x T block enumerated by anti-diagonals from the largest
+// lx + ly down (the slot order of the full-sky pixel tables).
+__device__ __forceinline__ void diag_slot_square(int l, int T, int &lx, int &ly)
+{
+    const int half = T * (T + 1) / 2;
+    const bool upper = l < half;
+    const int m = upper ? l : T * T - 1 - l;
+    int k = (int)((sqrtf(8.f * (float)m + 1.f) - 1.f) * 0.5f);
+    while (k * (k + 1) / 2 > m) --k;
+    while ((k + 1) * (k + 2) / 2 <= m) ++k;
+    const int o = m - k * (k + 1) / 2;
+    if (upper) {
+        lx = T - 1 - k + o;
+        ly = T - 1 - o;
+    } else {
+        lx = k - o;
+        ly = o;
+    }
+}
+
+// Slot of pixel (lx, ly) in the order of diag_slot_square
+__device__ __forceinline__ int diag_index_square(int lx, int ly, int T)
+{
+    const int k = lx + ly < T - 1 ? lx + ly : 2 * T - 2 - lx - ly, h = k * (k + 1) / 2;
+    return lx + ly < T - 1 ? T * T - 1 - h - ly : h + T - 1 - ly;
+}
+
 // RING index of the pixel at (ix, iy) of base face f (0..11).  The twelve base pixels of
 // Gorski et al. (2005, Sec. 4) are rhombi in three rings of four: face f is centred on ring
 // jr(f) * N, jr = 2 (north faces 0-3), 3 (equatorial faces 4-7), 4 (south faces 8-11), with its

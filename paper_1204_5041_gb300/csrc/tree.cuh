@@ -444,33 +444,6 @@ __device__ __forceinline__ void cheb_coefs(const double *__restrict__ F, const T
     cheb_transform<NP>(coef, tmp);
 }
 
-// Position (lx, ly) of slot l in a T x T block enumerated by anti-diagonals from the largest
-// lx + ly down (the slot order of the full-sky pixel tables).
-__device__ __forceinline__ void diag_slot_square(int l, int T, int &lx, int &ly)
-{
-    const int half = T * (T + 1) / 2;
-    const bool upper = l < half;
-    const int m = upper ? l : T * T - 1 - l;
-    int k = (int)((sqrtf(8.f * (float)m + 1.f) - 1.f) * 0.5f);
-    while (k * (k + 1) / 2 > m) --k;
-    while ((k + 1) * (k + 2) / 2 <= m) ++k;
-    const int o = m - k * (k + 1) / 2;
-    if (upper) {
-        lx = T - 1 - k + o;
-        ly = T - 1 - o;
-    } else {
-        lx = k - o;
-        ly = o;
-    }
-}
-
-// Slot of pixel (lx, ly) in the order of diag_slot_square
-__device__ __forceinline__ int diag_index_square(int lx, int ly, int T)
-{
-    const int k = lx + ly < T - 1 ? lx + ly : 2 * T - 2 - lx - ly, h = k * (k + 1) / 2;
-    return lx + ly < T - 1 ? T * T - 1 - h - ly : h + T - 1 - ly;
-}
-
 namespace {
 
 __device__ __forceinline__ float warp_sum(float v)

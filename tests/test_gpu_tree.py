@@ -302,3 +302,23 @@ def test_adjoint_tree_list_f64(isw):
         for b in (slice(0, 3), slice(3, 6)):
             assert ((got - ref)[b].abs().max() / ref[b].abs().max()).item() <= 1e-12
     assert isw.default_context().check_status()[0] == isw.OK
+
+
+@pytest.mark.parametrize("nside", [32, 33, 63, 64, 130])
+def test_sky_table_bits(isw, nside):
+    """The pixel directions of a full-sky map are those of a list of all pixels, bit for bit: one sample of
+    weight, every pair in FP64, so a map value is one term of the pixel's direction."""
+    npix = 12 * nside * nside
+    S = _samples(100_000_000 // npix + 1, 9)
+    S[9, 1:] = 0.0
+    S = torch.from_numpy(S).cuda()
+    pix = torch.arange(npix, device="cuda")
+    ctx = isw.default_context()
+    near_k = ctx.get_param(isw.PARAM_NEAR_K)
+    ctx.set_param(isw.PARAM_NEAR_K, 1e5)
+    try:
+        sky, lst = isw.isw_map(nside, S), isw.isw_map(nside, S, pix=pix)
+    finally:
+        ctx.set_param(isw.PARAM_NEAR_K, near_k)
+    assert (sky != 0).all() and torch.equal(sky, lst)
+    ctx.check_status()
