@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(256) k_sky_table(int64_t N, int T, int64_t nb,
     }
     __syncthreads();
     const int64_t ncap = 2 * N * (N - 1), npix = 12 * N * N, blocks = nb * nb;
-    for (int l = tid; l < T * T; l += 256) {
+    for (int l = blockIdx.y * 256 + tid; l < T * T; l += 256 * gridDim.y) {
         int lx, ly;
         diag_slot_square(l, T, lx, ly);
         const int64_t ix = x0 + lx, iy = y0 + ly;
@@ -283,7 +283,7 @@ void launch_pixel_table(int64_t N, int mode, int64_t pix0, int64_t npix, const i
     if (blocks > 152 * 64) blocks = 152 * 64;
     const int64_t nb = (N + tx - 1) / tx;
     if (mode == 0 && tx == ty && tx <= 32 && nb < 30000)
-        k_sky_table<<<(unsigned)(2 * nb * nb), 256, 0, s>>>(N, tx, nb, nv, ldn, outidx);
+        k_sky_table<<<dim3((unsigned)(2 * nb * nb), tx == 32 ? 4 : 1), 256, 0, s>>>(N, tx, nb, nv, ldn, outidx);
     else
         k_pixel_table<<<(unsigned)blocks, threads, 0, s>>>(N, mode, pix0, npix, pix_list, tx, ty, ntiles, nv, ldn, outidx,
                                                        perm, st);

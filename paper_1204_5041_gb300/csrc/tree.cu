@@ -1148,15 +1148,11 @@ cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_
     const TreeSamples S{crit, vcrit, caps, caps + p.nst, sup, sup + nsup, vidx, p.nst};
     TreeGeo *leaf_geo = (TreeGeo *)(b + p.off_geo[0]);
     if (f64)
-        k_tree_leaf_geo<kLeaf64><<<(unsigned)p.ncl[0], kLeaf64 * kLeaf64 / 4, 0, s>>>(m.nv, m.ldn, m.outidx, m.order,
-                                                                                       m.theta_pix, kappa, leaf_geo);
+        launch_leaf_geo<kLeaf64>(m.nv, m.ldn, m.outidx, m.order, m.theta_pix, kappa, p.ncl[0], leaf_geo, s);
     else
-        k_tree_leaf_geo<kLeaf><<<(unsigned)p.ncl[0], kLeaf * kLeaf / 4, 0, s>>>(m.nv, m.ldn, m.outidx, m.order,
-                                                                                 m.theta_pix, kappa, leaf_geo);
+        launch_leaf_geo<kLeaf>(m.nv, m.ldn, m.outidx, m.order, m.theta_pix, kappa, p.ncl[0], leaf_geo, s);
     for (int L = 1; L < p.levels; ++L)
-        k_tree_up_geo<<<(unsigned)((p.ncl[L] + 3) / 4), 128, 0, s>>>((const TreeGeo *)(b + p.off_geo[L - 1]), p.nb[L - 1],
-                                                                     p.ncl[L - 1], (TreeGeo *)(b + p.off_geo[L]), p.nb[L],
-                                                                     p.ncl[L], kappa);
+        launch_up_geo((const TreeGeo *)(b + p.off_geo[L - 1]), p.nb[L - 1], p.ncl[L - 1], (TreeGeo *)(b + p.off_geo[L]), p.nb[L], p.ncl[L], kappa, s);
     // stages 0 .. levels - 1: node sums of the level; stage `levels`: the pixels
     TreeStages g{};
     g.n = p.levels + 1;

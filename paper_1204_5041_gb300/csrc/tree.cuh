@@ -634,30 +634,36 @@ __global__ void __launch_bounds__(128) k_tree_plan(TreeStages g, const int *__re
 }
 
 // theta of the clusters that were cut into chunks: their partial sums added in chunk order, one pixel per
-// thread.
+// thread.  With few clusters a warp takes 32 pixels of one, since the FP64 additions of clusters with many
+// chunks are the bound (N_side 64 in FP64, 48 clusters of 150 chunks: 375 us by 256 pixels, 103 us by 32); with
+// more clusters than warps it takes a cluster, most of which have one chunk (N_side 1024: 44 us by 32 pixels, 34 us
+// so).
 __global__ void __launch_bounds__(256) k_tree_reduce(TreeWork W, int tile, const double *__restrict__ partial,
                                                      const int64_t *__restrict__ outidx, double *__restrict__ theta,
                                                      int accumulate)
 {
-    const int np = *W.npool, parts = tile / 256;
-    for (int i = blockIdx.x; i < np * parts; i += gridDim.x) {
-        const int e = i / parts, l = i % parts * 256 + threadIdx.x;
-        const int2 it = W.pool[e];
-        if (it.y != 0) continue;
-        const int nch = W.nch[it.x];
-        const int64_t oi = outidx[(int64_t)it.x * tile + l];
-        const double *src = partial + (int64_t)e * tile + l;
-        double hi = 0.0, lo = 0.0;
-        int c = 0;
-        for (; c + 4 <= nch; c += 4) {
-            double v[4];
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
+    const int parts = W.ncl < warps ? tile / 32 : 1, share = tile / parts;
+    for (int64_t i = threadIdx.x / 32 * (int64_t)gridDim.x + blockIdx.x; i < W.ncl * parts; i += warps) {
+        const int64_t cl = i / parts;
+        const int nch = W.nch[cl];
+        if (nch == 1) continue;
+        const int l0 = (int)(i - cl * parts) * share;
+        for (int l = l0 + (threadIdx.x & 31); l < l0 + share; l += 32) {
+            const int64_t oi = outidx[cl * tile + l];
+            const double *src = partial + (int64_t)W.pbase[cl] * tile + l;
+            double hi = 0.0, lo = 0.0;
+            int c = 0;
+            for (; c + 8 <= nch; c += 8) {
+                double v[8];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) v[k] = src[(int64_t)(c + k) * tile];
+                for (int k = 0; k < 8; ++k) v[k] = src[(int64_t)(c + k) * tile];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) fold64(hi, lo, v[k]);
+                for (int k = 0; k < 8; ++k) fold64(hi, lo, v[k]);
+            }
+            for (; c < nch; ++c) fold64(hi, lo, src[(int64_t)c * tile]);
+            if (oi >= 0) theta[oi] = accumulate ? theta[oi] + (hi + lo) : hi + lo;
         }
-        for (; c < nch; ++c) fold64(hi, lo, src[(int64_t)c * tile]);
-        if (oi >= 0) theta[oi] = accumulate ? theta[oi] + (hi + lo) : hi + lo;
     }
 }
 
@@ -792,131 +798,176 @@ __device__ __forceinline__ void finish_geo(TreeGeo &g, double D)
     g.f2 = make_float4((float)g.e2[0], (float)g.e2[1], (float)g.e2[2], (float)(1.0 / g.a2));
 }
 
-// One CTA of T*T/4 threads per finest cluster.  Sums in float are enough: they only choose the
-// centre and frame, and the extents are measured from the pixels afterwards.
-template <int T>
-__global__ void __launch_bounds__(T *T / 4) k_tree_leaf_geo(const double *__restrict__ nv, int64_t ldn,
-                                                            const int64_t *__restrict__ outidx, int order,
-                                                            double theta_pix, double kappa, TreeGeo *__restrict__ geo)
+// (float)x truncated, in integer instructions: a conversion takes a slot of the FP64 unit (two per clock and SM)
+__device__ __forceinline__ float trunc_float(double x)
 {
-    constexpr int NT = T * T / 4, W = NT / 32;
-    __shared__ float red[6][W];
-    __shared__ TreeGeo g;
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int64_t t = blockIdx.x;
-    float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int l = tid; l < T * T; l += NT) {
-        const int64_t k = t * T * T + l;
-        if (outidx[k] < 0) continue;
-        int lx = T / 2, ly;
-        if (order == kSlotsDiag) diag_slot_square(l, T, lx, ly);
-        else if (order == kSlotsRows) lx = l % T;
-        // a list has no axis of its own: the frame is then any
-        const float f = order == kSlotsList ? 0.f : (float)lx - 0.5f * (float)(T - 1);
-        for (int c = 0; c < 3; ++c) {
-            const float v = (float)nv[c * ldn + k];
-            s[c] += v;
-            s[3 + c] += f * v;
+    const int hi = __double2hiint(x), e = (hi >> 20 & 0x7ff) - 896;
+    const unsigned m = (unsigned)(hi & 0xfffff) << 3 | (unsigned)__double2loint(x) >> 29;
+    return e <= 0 ? 0.f : __int_as_float((int)((unsigned)hi & 0x80000000u | (unsigned)e << 23 | m));
+}
+
+// Finest clusters, W warps each and G clusters per CTA; the frames of a CTA's clusters are made by as many lanes
+// of one warp.  Sums in float are enough: they only choose the centre and frame, and the extents are measured
+// from the pixels afterwards.
+template <int T, int W, int G>
+__global__ void __launch_bounds__(32 * W * G) k_tree_leaf_geo(const double *__restrict__ nv, int64_t ldn,
+                                                              const int64_t *__restrict__ outidx, int order, double theta_pix,
+                                                              double kappa, int64_t ncl, TreeGeo *__restrict__ geo)
+{
+    __shared__ float red[G][W][6];
+    __shared__ TreeGeo gs[G];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid / 32 % W, own = tid / (32 * W);
+    const int64_t t = blockIdx.x * (int64_t)G + own;
+    if (t < ncl) {
+        float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int l = 32 * w + lane; l < T * T; l += 32 * W) {
+            const int64_t k = t * T * T + l;
+            if (outidx[k] < 0) continue;
+            int lx = T / 2, ly;
+            if (order == kSlotsDiag) diag_slot_square(l, T, lx, ly);
+            else if (order == kSlotsRows) lx = l % T;
+            // a list has no axis of its own: the frame is then any
+            const float f = order == kSlotsList ? 0.f : (float)lx - 0.5f * (float)(T - 1);
+            for (int c = 0; c < 3; ++c) {
+                const float v = trunc_float(nv[c * ldn + k]);
+                s[c] += v;
+                s[3 + c] += f * v;
+            }
+        }
+        for (int c = 0; c < 6; ++c) {
+            s[c] = warp_sum(s[c]);
+            if (lane == 0) red[own][w][c] = s[c];
         }
     }
-    for (int c = 0; c < 6; ++c) {
-        for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
-        if (lane == 0) red[c][w] = s[c];
-    }
     __syncthreads();
-    if (tid == 0) {
+    const int64_t t1 = blockIdx.x * (int64_t)G + tid;   // the cluster whose frame this thread makes
+    const bool maker = tid < G && t1 < ncl;
+    if (maker) {
         double a[6];
         for (int c = 0; c < 6; ++c) {
             a[c] = 0.0;
-            for (int i = 0; i < W; ++i) a[c] += red[c][i];
+            for (int i = 0; i < W; ++i) a[c] += red[tid][i][c];
         }
-        make_frame(a[0], a[1], a[2], a[3], a[4], a[5], g);
+        make_frame(a[0], a[1], a[2], a[3], a[4], a[5], gs[tid]);
     }
     __syncthreads();
-    const float e1x = (float)g.e1[0], e1y = (float)g.e1[1], e1z = (float)g.e1[2];
-    const float e2x = (float)g.e2[0], e2y = (float)g.e2[1], e2z = (float)g.e2[2];
-    float m1 = 0.f, m2 = 0.f;
-    for (int l = tid; l < T * T; l += NT) {
-        const int64_t k = t * T * T + l;
-        if (outidx[k] < 0) continue;
-        const float dx = (float)(nv[k] - g.n0[0]), dy = (float)(nv[ldn + k] - g.n0[1]),
-                    dz = (float)(nv[2 * ldn + k] - g.n0[2]);
-        const float s = 1.f / (2.f - 0.5f * (dx * dx + dy * dy + dz * dz));
-        m1 = fmaxf(m1, fabsf(dx * e1x + dy * e1y + dz * e1z) * s);
-        m2 = fmaxf(m2, fabsf(dx * e2x + dy * e2y + dz * e2z) * s);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-        m2 = fmaxf(m2, __shfl_xor_sync(0xffffffffu, m2, o));
+    if (t < ncl) {
+        const TreeGeo &g = gs[own];
+        const float e1x = trunc_float(g.e1[0]), e1y = trunc_float(g.e1[1]), e1z = trunc_float(g.e1[2]);
+        const float e2x = trunc_float(g.e2[0]), e2y = trunc_float(g.e2[1]), e2z = trunc_float(g.e2[2]);
+        float m1 = 0.f, m2 = 0.f;
+        for (int l = 32 * w + lane; l < T * T; l += 32 * W) {
+            const int64_t k = t * T * T + l;
+            if (outidx[k] < 0) continue;
+            const float dx = trunc_float(nv[k] - g.n0[0]), dy = trunc_float(nv[ldn + k] - g.n0[1]),
+                        dz = trunc_float(nv[2 * ldn + k] - g.n0[2]);
+            const float s = 1.f / (2.f - 0.5f * (dx * dx + dy * dy + dz * dz));
+            m1 = fmaxf(m1, fabsf(dx * e1x + dy * e1y + dz * e1z) * s);
+            m2 = fmaxf(m2, fabsf(dx * e2x + dy * e2y + dz * e2z) * s);
+        }
+        m1 = warp_max(m1);
+        m2 = warp_max(m2);
+        if (lane == 0) {
+            red[own][w][0] = m1;
+            red[own][w][1] = m2;
+        }
     }
     __syncthreads();
-    if (lane == 0) {
-        red[0][w] = m1;
-        red[1][w] = m2;
-    }
-    __syncthreads();
-    if (tid == 0) {
+    if (maker) {
+        TreeGeo &g = gs[tid];
+        float m1 = 0.f, m2 = 0.f;
         for (int i = 0; i < W; ++i) {
-            m1 = fmaxf(m1, red[0][i]);
-            m2 = fmaxf(m2, red[1][i]);
+            m1 = fmaxf(m1, red[tid][i][0]);
+            m2 = fmaxf(m2, red[tid][i][1]);
         }
         // margin for the float arithmetic; a single pixel still gets a square of a quarter pixel
         g.a1 = fmax((double)m1 * 1.00001, 0.125 * theta_pix);
         g.a2 = fmax((double)m2 * 1.00001, 0.125 * theta_pix);
         finish_geo(g, near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7);
-        geo[t] = g;
+        geo[t1] = g;
     }
 }
+// With 16 clusters for every SM the FP64 unit bounds a CTA per cluster, whose frame is the work of one thread:
+// a warp per cluster and 16 per CTA take 270 us at N_side 1024 (49,152 clusters) instead of 719.  With fewer the
+// latency of a CTA counts: at N_side 64 (192 clusters) 12 us with a CTA each, 17 with 16 per CTA.
+template <int T>
+void launch_leaf_geo(const double *nv, int64_t ldn, const int64_t *outidx, int order, double theta_pix, double kappa, int64_t ncl,
+                     TreeGeo *geo, cudaStream_t s)
+{
+    constexpr int W = T * T / 128;
+    if (ncl < 16 * 152)
+        k_tree_leaf_geo<T, W, 1><<<(unsigned)ncl, 32 * W, 0, s>>>(nv, ldn, outidx, order, theta_pix, kappa, ncl, geo);
+    else
+        k_tree_leaf_geo<T, 1, 16><<<(unsigned)((ncl + 15) / 16), 512, 0, s>>>(nv, ldn, outidx, order, theta_pix, kappa, ncl, geo);
+}
 
-// One warp per parent cluster (tree_parent of the child level): lane l
-// takes point l % 8 (corners and edge midpoints) of the rectangle of child l / 8.  Offsets from the
-// parent's centre are differences of FP64 centres plus a float offset, so they keep their relative
-// accuracy for small clusters.
+// Four lanes per parent cluster (tree_parent of the child level), a lane per child: points of the child's
+// rectangle (corners and edge midpoints).  Offsets from the parent's centre are differences of FP64 centres plus a
+// float offset, so they keep their relative accuracy for small clusters.  With a warp per parent every lane
+// repeated the frame's FP64 work (N_side 1024, five levels: 178 us, so 50 us).
 __global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__ child, int cnb, int64_t cncl,
                                                      TreeGeo *__restrict__ geo, int nb, int64_t ncl, double kappa)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (t >= ncl) return;
+    const int c = threadIdx.x & 3;
+    const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 2, t = p < ncl ? p : ncl - 1;
     int64_t kid, kid0;
     bool has;
     if (nb == 0) {
         kid0 = 4 * t;
-        kid = kid0 + (lane >> 3);
+        kid = kid0 + c;
         has = kid < cncl;
     } else {
         const int64_t f = t / ((int64_t)nb * nb);
         const int by = (int)(t - f * nb * nb) / nb, bx = (int)(t - f * nb * nb) % nb;
-        const int i = 2 * bx + (lane >> 3 & 1), j = 2 * by + (lane >> 4);
+        const int i = 2 * bx + (c & 1), j = 2 * by + (c >> 1);
         has = i < cnb && j < cnb;
         kid = (f * cnb + j) * cnb + i;
         kid0 = (f * cnb + 2 * by) * cnb + 2 * bx;
     }
     const TreeGeo k = child[has ? kid : kid0];
-    const float on = has && (lane & 7) == 0 ? 1.f : 0.f;
-    const float cx = warp_sum(on * k.c.x), cy = warp_sum(on * k.c.y), cz = warp_sum(on * k.c.z);
-    const float ux = warp_sum(on * k.f1.x), uy = warp_sum(on * k.f1.y), uz = warp_sum(on * k.f1.z);
+    const float on = has ? 1.f : 0.f;
+    auto sum4 = [](float v) {
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        return v + __shfl_xor_sync(0xffffffffu, v, 2);
+    };
+    auto max4 = [](float v) {
+        v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
+        return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2));
+    };
+    const float cx = sum4(on * k.c.x), cy = sum4(on * k.c.y), cz = sum4(on * k.c.z);
+    const float ux = sum4(on * k.f1.x), uy = sum4(on * k.f1.y), uz = sum4(on * k.f1.z);
     TreeGeo g;
     make_frame(cx, cy, cz, ux, uy, uz, g);
     const float d0 = (float)(k.n0[0] - g.n0[0]), d1 = (float)(k.n0[1] - g.n0[1]), d2 = (float)(k.n0[2] - g.n0[2]);
-    const int q = lane & 7, pt = q < 4 ? q : q + 1;   // 3 x 3 points without the middle one
-    const float xi = (float)(pt % 3 - 1) * (float)k.a1, eta = (float)(pt / 3 - 1) * (float)k.a2;
-    const float r2 = xi * xi + eta * eta, s = 2.f / (1.f + r2);
-    const float x = d0 + s * (xi * k.f1.x + eta * k.f2.x - r2 * k.c.x);
-    const float y = d1 + s * (xi * k.f1.y + eta * k.f2.y - r2 * k.c.y);
-    const float z = d2 + s * (xi * k.f1.z + eta * k.f2.z - r2 * k.c.z);
-    const float ps = 1.f / (2.f - 0.5f * (x * x + y * y + z * z));
-    const float m1 = fabsf(x * (float)g.e1[0] + y * (float)g.e1[1] + z * (float)g.e1[2]) * ps;
-    const float m2 = fabsf(x * (float)g.e2[0] + y * (float)g.e2[1] + z * (float)g.e2[2]) * ps;
-    g.a1 = (double)warp_max(m1) * 1.002;
-    g.a2 = (double)warp_max(m2) * 1.002;
+    const float a1 = (float)k.a1, a2 = (float)k.a2;
+    const float g1x = (float)g.e1[0], g1y = (float)g.e1[1], g1z = (float)g.e1[2];
+    const float g2x = (float)g.e2[0], g2y = (float)g.e2[1], g2z = (float)g.e2[2];
+    float m1 = 0.f, m2 = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int pt = q < 4 ? q : q + 1;   // 3 x 3 points without the middle one
+        const float xi = (float)(pt % 3 - 1) * a1, eta = (float)(pt / 3 - 1) * a2;
+        const float r2 = xi * xi + eta * eta, s = 2.f / (1.f + r2);
+        const float x = d0 + s * (xi * k.f1.x + eta * k.f2.x - r2 * k.c.x);
+        const float y = d1 + s * (xi * k.f1.y + eta * k.f2.y - r2 * k.c.y);
+        const float z = d2 + s * (xi * k.f1.z + eta * k.f2.z - r2 * k.c.z);
+        const float ps = 1.f / (2.f - 0.5f * (x * x + y * y + z * z));
+        m1 = fmaxf(m1, fabsf(x * g1x + y * g1y + z * g1z) * ps);
+        m2 = fmaxf(m2, fabsf(x * g2x + y * g2y + z * g2z) * ps);
+    }
+    g.a1 = (double)max4(m1) * 1.002;
+    g.a2 = (double)max4(m2) * 1.002;
     // near at a child implies near here
     const float cd = (k.c.w + sqrtf(d0 * d0 + d1 * d1 + d2 * d2)) * 1.00003f + 2e-6f;
-    const double D = fmax(near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7, (double)warp_max(cd));
-    if (lane == 0) {
+    const double D = fmax(near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7, (double)max4(cd));
+    if (c == 0 && p < ncl) {
         finish_geo(g, D);
-        geo[t] = g;
+        geo[p] = g;
     }
+}
+void launch_up_geo(const TreeGeo *child, int cnb, int64_t cncl, TreeGeo *geo, int nb, int64_t ncl, double kappa, cudaStream_t s)
+{
+    k_tree_up_geo<<<(unsigned)((ncl + 31) / 32), 128, 0, s>>>(child, cnb, cncl, geo, nb, ncl, kappa);
 }
 
 __device__ __forceinline__ void load_geo(TreeGeo *dst, const TreeGeo *src)

@@ -680,8 +680,7 @@ cudaError_t launch_adjoint_tree(const AdjTreePlan &p, const AdjTreeCall &m, cuda
         u.nb = t.nb[L];
         u.node = node;
         if (L == 0) {
-            k_tree_leaf_geo<kLeaf><<<(unsigned)t.ncl[0], kLeaf * kLeaf / 4, 0, s>>>(m.nv, m.ldn, m.outidx, m.order, m.theta_pix,
-                                                                                     kKappaAdj, geo);
+            launch_leaf_geo<kLeaf>(m.nv, m.ldn, m.outidx, m.order, m.theta_pix, kKappaAdj, t.ncl[0], geo, s);
             u.nv = m.nv;
             u.ldn = m.ldn;
             u.outidx = m.outidx;
@@ -690,8 +689,7 @@ cudaError_t launch_adjoint_tree(const AdjTreePlan &p, const AdjTreeCall &m, cuda
             u.low = (AdjLow *)(b + p.off_low);
             k_adj_up<true><<<(unsigned)t.ncl[0], 128, 0, s>>>(u);
         } else {
-            k_tree_up_geo<<<(unsigned)((t.ncl[L] + 3) / 4), 128, 0, s>>>(a.geo[L - 1], t.nb[L - 1], t.ncl[L - 1], geo, t.nb[L],
-                                                                         t.ncl[L], kKappaAdj);
+            launch_up_geo(a.geo[L - 1], t.nb[L - 1], t.ncl[L - 1], geo, t.nb[L], t.ncl[L], kKappaAdj, s);
             u.cgeo = a.geo[L - 1];
             u.cnb = t.nb[L - 1];
             u.cncl = t.ncl[L - 1];

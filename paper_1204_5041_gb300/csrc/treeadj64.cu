@@ -480,8 +480,7 @@ cudaError_t launch_adjoint_tree64(const AdjTreePlan &p, const AdjTreeCall &m, cu
         u.nb = t.nb[L];
         u.node = node;
         if (L == 0) {
-            k_tree_leaf_geo<kLeaf64><<<(unsigned)t.ncl[0], kLeaf64 * kLeaf64 / 4, 0, s>>>(m.nv, m.ldn, m.outidx, m.order,
-                                                                                           m.theta_pix, kKappa64, geo);
+            launch_leaf_geo<kLeaf64>(m.nv, m.ldn, m.outidx, m.order, m.theta_pix, kKappa64, t.ncl[0], geo, s);
             u.nv = m.nv;
             u.ldn = m.ldn;
             u.outidx = m.outidx;
@@ -490,8 +489,7 @@ cudaError_t launch_adjoint_tree64(const AdjTreePlan &p, const AdjTreeCall &m, cu
             u.pix = (AdjPix64 *)(b + p.off_pix);
             k_adj_up64<true><<<(unsigned)t.ncl[0], kNN64, 0, s>>>(u);
         } else {
-            k_tree_up_geo<<<(unsigned)((t.ncl[L] + 3) / 4), 128, 0, s>>>(a.geo[L - 1], t.nb[L - 1], t.ncl[L - 1], geo, t.nb[L],
-                                                                         t.ncl[L], kKappa64);
+            launch_up_geo(a.geo[L - 1], t.nb[L - 1], t.ncl[L - 1], geo, t.nb[L], t.ncl[L], kKappa64, s);
             u.cgeo = a.geo[L - 1];
             u.cnb = t.nb[L - 1];
             u.cncl = t.ncl[L - 1];
