@@ -52,7 +52,8 @@ __device__ __forceinline__ double pair64_fast(double nx, double ny, double nz, c
     const double Pd = g.xd[0] * dx + g.xd[1] * dy + g.xd[2] * dz;
     const double Qd = g.xp[0] * dx + g.xp[1] * dy + g.xp[2] * dz;
     const double den = B * Q, num = g.c * (B * Pd - A * Qd);
-    if (fabs(den) > 1e-30 && fabs(den) < 1e30) return num * rcp64(den);
+    const int ex = __double2hiint(den) & 0x7ff00000;   // 2^-100 <= |den| < 2^101
+    if (ex >= 0x39b00000 && ex < 0x46400000) return num * rcp64(den);
     if (Q == 0.0) {
         ++zero;
         return 0.0;

@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_nodes_f32(TreeNodeArgs a)
         tree_scan<ROOT, false>(a.S, kc, nch, self, parent, 0.f, 0.f, 0.f, sm.scan, consume);
         double (*red)[kNN] = reinterpret_cast<double (*)[kNN]>(sm.rec);   // the batches are done
 #pragma unroll
-        for (int q = 0; q < 4; ++q) red[2 * w + half][16 * q + hl] = (double)ahi[q] + (double)alo[q];
+        for (int q = 0; q < 4; ++q) red[2 * w + half][16 * q + hl] = widen(ahi[q]) + widen(alo[q]);
         __syncthreads();
         double v = 0.0;
         if (tid < kNN) {
@@ -332,26 +332,32 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_pixels_f32(TreePixArgs a)
         int qlen = 0;
         uint64_t m[2][3], ml[2][3], mm[2];   // offsets from the centre as float pairs, |m|^2
         const int64_t kw = cl * TILE + w * 64;   // pixel 16 q + hl of the warp is the lane's q-th
-#pragma unroll
-        for (int pp = 0; pp < 2; ++pp) {
-            float h[2][3], l[2][3];
+        {
+            // two pixels per lane, the other two from the lane of the other half-warp that has the same ones
+            float h[2][3], l[2][3], oh[2][3], ol[2][3];
+            unsigned own = 0;
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                const int64_t k = kw + 16 * (2 * pp + u) + hl;
-                if (a.outidx[k] >= 0) valid |= 1u << (2 * pp + u);
+                const int64_t k = kw + 16 * (2 * half + u) + hl;
+                if (a.outidx[k] >= 0) own |= 1u << (2 * half + u);
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    const double v = a.nv[c * a.ldn + k] - sm.geo.n0[c];
-                    h[u][c] = __double2float_rn(v);
-                    l[u][c] = __double2float_rn(v - (double)h[u][c]);
+                    split_float(a.nv[c * a.ldn + k] - sm.geo.n0[c], h[u][c], l[u][c]);
+                    oh[u][c] = __shfl_xor_sync(0xffffffffu, h[u][c], 16);
+                    ol[u][c] = __shfl_xor_sync(0xffffffffu, l[u][c], 16);
                 }
             }
+            valid = own | __shfl_xor_sync(0xffffffffu, own, 16);
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                m[pp][c] = f2_pack(h[0][c], h[1][c]);
-                ml[pp][c] = f2_pack(l[0][c], l[1][c]);
+                m[0][c] = half ? f2_pack(oh[0][c], oh[1][c]) : f2_pack(h[0][c], h[1][c]);
+                m[1][c] = half ? f2_pack(h[0][c], h[1][c]) : f2_pack(oh[0][c], oh[1][c]);
+                ml[0][c] = half ? f2_pack(ol[0][c], ol[1][c]) : f2_pack(l[0][c], l[1][c]);
+                ml[1][c] = half ? f2_pack(l[0][c], l[1][c]) : f2_pack(ol[0][c], ol[1][c]);
             }
-            mm[pp] = f2_fma(m[pp][2], m[pp][2], f2_fma(m[pp][1], m[pp][1], f2_mul(m[pp][0], m[pp][0])));
+#pragma unroll
+            for (int pp = 0; pp < 2; ++pp)
+                mm[pp] = f2_fma(m[pp][2], m[pp][2], f2_fma(m[pp][1], m[pp][1], f2_mul(m[pp][0], m[pp][0])));
         }
         double far[2] = {0.0, 0.0};   // of the lane's pixels 2 half and 2 half + 1
         if (kc == 0) {
@@ -468,12 +474,21 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_pixels_f32(TreePixArgs a)
         const float R = target_radius(sm.geo);
         tree_scan<false, true>(a.S, kc, nch, self, self, R, 1.5f * R, a.b_min, sm.scan, consume);
         if (qlen > 0) near_flush(nq, qlen, a.s64, a.nv, a.ldn, kw, zerocnt);
+        float sh[2] = {0.f, 0.f}, sl[2] = {0.f, 0.f};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {   // both half-warps' sums of a pixel; half q / 2 writes it
-            double v = (double)ahi[q] + (double)alo[q];
-            v += __shfl_xor_sync(0xffffffffu, v, 16);
-            if (half != q / 2) continue;
-            v = (v + nq.acc[16 * q + hl]) + far[q & 1];
+            const float bh = __shfl_xor_sync(0xffffffffu, ahi[q], 16), bl = __shfl_xor_sync(0xffffffffu, alo[q], 16);
+            float h = ahi[q], l = alo[q] + bl;
+            fold(h, l, bh);
+            if (half == q / 2) {
+                sh[q & 1] = h;
+                sl[q & 1] = l;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int q = 2 * half + u;
+            const double v = ((widen(sh[u]) + widen(sl[u])) + nq.acc[16 * q + hl]) + far[u];
             const int64_t k = kw + 16 * q + hl;
             if (nch == 1) {
                 const int64_t oi = a.outidx[k];

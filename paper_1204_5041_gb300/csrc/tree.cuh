@@ -446,6 +446,30 @@ __device__ __forceinline__ void cheb_coefs(const double *__restrict__ F, const T
 
 namespace {
 
+// Conversions in integer instructions: a conversion takes a slot of the FP64 unit (two per clock and SM), and the
+// FP32 kernels' few FP64 operations per pixel bound them where clusters have few samples.
+// (float)x truncated; below the normal range 0; finite values
+__device__ __forceinline__ float trunc_float(double x)
+{
+    const int hi = __double2hiint(x), e = (hi >> 20 & 0x7ff) - 896;
+    const unsigned m = (unsigned)(hi & 0xfffff) << 3 | (unsigned)__double2loint(x) >> 29;
+    return e <= 0 ? 0.f : __int_as_float((int)((unsigned)hi & 0x80000000u | (unsigned)e << 23 | m));
+}
+// x as a float pair, h truncated to 24 bits
+__device__ __forceinline__ void split_float(double x, float &h, float &l)
+{
+    const double t = __hiloint2double(__double2hiint(x), __double2loint(x) & (int)0xe0000000);
+    h = trunc_float(t);
+    l = trunc_float(x - t);
+}
+// (double)x; below the normal range 0
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = (unsigned)__float_as_int(x), e = b >> 23 & 0xff;
+    const unsigned hi = (b & 0x80000000u) | (e == 0xff ? 0x7ffu : e + 896) << 20 | (b & 0x7fffff) >> 3;
+    return e == 0 ? 0.0 : __hiloint2double((int)hi, (int)(b << 29));
+}
+
 __device__ __forceinline__ float warp_sum(float v)
 {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -796,14 +820,6 @@ __device__ __forceinline__ void finish_geo(TreeGeo &g, double D)
                       (float)(g.n0[2] - (double)g.c.z), 0.f);
     g.f1 = make_float4((float)g.e1[0], (float)g.e1[1], (float)g.e1[2], (float)(1.0 / g.a1));
     g.f2 = make_float4((float)g.e2[0], (float)g.e2[1], (float)g.e2[2], (float)(1.0 / g.a2));
-}
-
-// (float)x truncated, in integer instructions: a conversion takes a slot of the FP64 unit (two per clock and SM)
-__device__ __forceinline__ float trunc_float(double x)
-{
-    const int hi = __double2hiint(x), e = (hi >> 20 & 0x7ff) - 896;
-    const unsigned m = (unsigned)(hi & 0xfffff) << 3 | (unsigned)__double2loint(x) >> 29;
-    return e <= 0 ? 0.f : __int_as_float((int)((unsigned)hi & 0x80000000u | (unsigned)e << 23 | m));
 }
 
 // Finest clusters, W warps each and G clusters per CTA; the frames of a CTA's clusters are made by as many lanes
