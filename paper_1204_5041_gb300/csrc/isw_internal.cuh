@@ -23,19 +23,19 @@ __device__ __forceinline__ double dsqrt(double a) { return __dsqrt_rn(a); }
 // pi rounded to the nearest double
 constexpr double kPi = 3.14159265358979323846264338327950288;
 
-// a / C rounded to nearest, C an integer below 1024.  With r = RN(1/C), q = RN(a r) is off by less than two
-// ulps, so a - C q is exact, and q plus its correction is off by far less than an ulp / (2 C), the least
-// distance of a / C from a rounding boundary (no quotient lies on one: an odd 54-bit number times C has no
-// 53-bit product).  Three operations instead of the division's chain (the 20 divisions of a sine and cosine
-// bound the light-cone solve's latency, 218 -> 141 us for 10,240 segments, and the pixel tables); where the product underflows, q and the
-// quotient may differ in the last subnormal digit.
+// a / C rounded to nearest, C an integer below 1024: a (h + l) with h = RN(1/C) and h + l = 1/C to 106 bits, one
+// rounded product and one fused operation.  Before its last rounding the sum is off by less than 2^-50 ulp, and
+// a / C is at least an ulp / (2 C) away from a rounding boundary (none lies on one: an odd 54-bit number times C
+// has no 53-bit product).  Two operations instead of the division's chain (the 20 divisions of a sine and cosine
+// bound the light-cone solve, 218 us for 10,240 segments, and the pixel tables); where the product underflows,
+// the last subnormal digit may differ.
 template <int C>
 __device__ __forceinline__ double ddiv_const(double a)
 {
     static_assert(C > 0 && C < 1024, "range of the proof");
-    constexpr double r = 1.0 / C;
-    const double q = dmul(a, r);
-    return __fma_rn(__fma_rn(-(double)C, q, a), r, q);
+    constexpr double h = 1.0 / C, t = h * 134217729.0, hh = t - (t - h), hl = h - hh;   // h in halves: C hh, C hl exact
+    constexpr double l = ((1.0 - C * hh) - C * hl) / C;
+    return __fma_rn(a, h, dmul(a, l));
 }
 
 template <int K>

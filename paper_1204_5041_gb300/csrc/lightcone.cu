@@ -11,38 +11,68 @@ namespace isw {
 //   a(u) = L/(2 pi m) (sin 2 pi m u/L, -cos 2 pi m u/L, 0),
 //   b(v) = L/(2 pi n) (sin 2 pi n v/L, -cos psi cos 2 pi n v/L, -sin psi cos 2 pi n v/L);
 // Xdot = R (b' - a')/2, X' = R (a' + b')/2.  P is double[17][ldp]: c(3) R(9) L m n psi t0.
-__device__ __forceinline__ void burden_worldsheet(const double *__restrict__ P, int64_t ldp, int64_t id, double sigma,
-                                                  double t, double X[3], double Xd[3], double Xp[3])
-{
-    const double two_pi = 2.0 * kPi;
-    const double L = P[12 * ldp + id], m = P[13 * ldp + id], n = P[14 * ldp + id];
-    const double psi = P[15 * ldp + id], t0 = P[16 * ldp + id];
-    const double dt = dsub(t, t0);
-    const double u = dsub(sigma, dt), v = dadd(sigma, dt);
-    double sa, ca, sb, cb, sp, cp;
-    sincos_turns(ddiv(dmul(m, u), L), sa, ca);
-    sincos_turns(ddiv(dmul(n, v), L), sb, cb);
-    sincos_turns(ddiv(psi, two_pi), sp, cp);
-    const double ra = ddiv(L, dmul(two_pi, m)), rb = ddiv(L, dmul(two_pi, n));
-    const double a[3] = {dmul(ra, sa), -dmul(ra, ca), 0.0};
-    const double b[3] = {dmul(rb, sb), -dmul(rb, dmul(cp, cb)), -dmul(rb, dmul(sp, cb))};
-    const double ap[3] = {ca, sa, 0.0};
-    const double bp[3] = {cb, dmul(cp, sb), dmul(sp, sb)};
-    double h[3], hd[3], hp[3];
+//
+// What does not depend on t is read and computed once per node: the sine and cosine of psi and the radii would
+// be a third of a Newton step.
+struct BurdenLoop {
+    double c[3], R[9], L, m, n, t0, sp, cp, ra, rb;
+    double h[4];   // sa, ca, sb, cb at the last t
+
+    __device__ __forceinline__ void load(const double *__restrict__ P, int64_t ldp, int64_t id)
+    {
+        const double two_pi = 2.0 * kPi;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        h[k] = dmul(0.5, dadd(a[k], b[k]));
-        hd[k] = dmul(0.5, dsub(bp[k], ap[k]));
-        hp[k] = dmul(0.5, dadd(ap[k], bp[k]));
-    }
+        for (int k = 0; k < 3; ++k) c[k] = P[k * ldp + id];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const double r0 = P[(3 + 3 * k) * ldp + id], r1 = P[(4 + 3 * k) * ldp + id], r2 = P[(5 + 3 * k) * ldp + id];
-        X[k] = dadd(P[k * ldp + id], dadd(dadd(dmul(r0, h[0]), dmul(r1, h[1])), dmul(r2, h[2])));
-        Xd[k] = dadd(dadd(dmul(r0, hd[0]), dmul(r1, hd[1])), dmul(r2, hd[2]));
-        Xp[k] = dadd(dadd(dmul(r0, hp[0]), dmul(r1, hp[1])), dmul(r2, hp[2]));
+        for (int k = 0; k < 9; ++k) R[k] = P[(3 + k) * ldp + id];
+        L = P[12 * ldp + id];
+        m = P[13 * ldp + id];
+        n = P[14 * ldp + id];
+        t0 = P[16 * ldp + id];
+        sincos_turns(ddiv(P[15 * ldp + id], two_pi), sp, cp);
+        ra = ddiv(L, dmul(two_pi, m));
+        rb = ddiv(L, dmul(two_pi, n));
     }
-}
+    __device__ __forceinline__ double rot(int k, const double (&x)[3]) const
+    {
+        return dadd(dadd(dmul(R[3 * k], x[0]), dmul(R[3 * k + 1], x[1])), dmul(R[3 * k + 2], x[2]));
+    }
+    // X and Xdot at (sigma, t)
+    __device__ __forceinline__ void at(double sigma, double t, double X[3], double Xd[3])
+    {
+        const double dt = dsub(t, t0);
+        const double u = dsub(sigma, dt), v = dadd(sigma, dt);
+        double &sa = h[0], &ca = h[1], &sb = h[2], &cb = h[3];
+        sincos_turns(ddiv(dmul(m, u), L), sa, ca);
+        sincos_turns(ddiv(dmul(n, v), L), sb, cb);
+        const double a[3] = {dmul(ra, sa), -dmul(ra, ca), 0.0};
+        const double b[3] = {dmul(rb, sb), -dmul(rb, dmul(cp, cb)), -dmul(rb, dmul(sp, cb))};
+        const double ap[3] = {ca, sa, 0.0};
+        const double bp[3] = {cb, dmul(cp, sb), dmul(sp, sb)};
+        double x[3], xd[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            x[k] = dmul(0.5, dadd(a[k], b[k]));
+            xd[k] = dmul(0.5, dsub(bp[k], ap[k]));
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            X[k] = dadd(c[k], rot(k, x));
+            Xd[k] = rot(k, xd);
+        }
+    }
+    // X' at the last point of at()
+    __device__ __forceinline__ void tangent(double Xp[3]) const
+    {
+        const double ap[3] = {h[1], h[0], 0.0};
+        const double bp[3] = {h[3], dmul(cp, h[2]), dmul(sp, h[2])};
+        double x[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) x[k] = dmul(0.5, dadd(ap[k], bp[k]));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) Xp[k] = rot(k, x);
+    }
+};
 
 __device__ __forceinline__ int solve_node(int mode, const double *__restrict__ nodes, int64_t ld, int64_t s,
                                           const double *__restrict__ P, int64_t nloops, int64_t ldp, double t_box,
@@ -98,8 +128,10 @@ __device__ __forceinline__ int solve_node(int mode, const double *__restrict__ n
             // f(t) = |X(s, t) - x_obs| - (t_obs - t) is increasing (f' = 1 + rhat.Xdot > 0):
             // Newton steps, replaced by bisection when they leave the bracket or fail to halve
             // the step taken two iterations earlier
+            BurdenLoop loop;
+            loop.load(P, ldp, id);
             for (int it = 0; it < max_iter; ++it) {
-                burden_worldsheet(P, ldp, id, sigma, t, X, Xd, Xp);
+                loop.at(sigma, t, X, Xd);
                 const double r[3] = {dsub(X[0], xo0), dsub(X[1], xo1), dsub(X[2], xo2)};
                 const double rn = dsqrt(dadd(dadd(dmul(r[0], r[0]), dmul(r[1], r[1])), dmul(r[2], r[2])));
                 const double f = dsub(rn, dsub(t_obs, t));
@@ -121,6 +153,7 @@ __device__ __forceinline__ int solve_node(int mode, const double *__restrict__ n
                 step1 = fabs(dsub(tn, t));
                 if (it + 1 < max_iter) t = tn;
             }
+            if (max_iter > 0) loop.tangent(Xp);
         }
     }
     return st;
@@ -182,6 +215,11 @@ __global__ void k_lightcone_shells(const double *__restrict__ nodes, int64_t n, 
     }
 }
 
+// One warp per CTA: each of its FP64 instructions takes 64 cycles of a quarter SM's unit, so the time of a small
+// call is one warp's instructions (some 300 per Newton step) as long as no unit has two of them (10,240 nodes:
+// 133 us in CTAs of 128 threads, 122 us in warps).
+constexpr int kSolveNT = 32;
+
 static unsigned grid_for(int64_t n, int threads)
 {
     int64_t b = (n + threads - 1) / threads;
@@ -196,7 +234,7 @@ void launch_lightcone(int mode, const double *nodes, int64_t n, int64_t ld, cons
                       cudaStream_t s)
 {
     if (n <= 0) return;
-    k_lightcone<<<grid_for(n, 128), 128, 0, s>>>(mode, nodes, n, ld, P, nloops, ldp, t_box, xo0, xo1, xo2, t_obs, tol,
+    k_lightcone<<<grid_for(n, kSolveNT), kSolveNT, 0, s>>>(mode, nodes, n, ld, P, nloops, ldp, t_box, xo0, xo1, xo2, t_obs, tol,
                                                   max_iter, out, ld_out, tau, status, st);
 }
 
@@ -206,7 +244,7 @@ void launch_lightcone_shells(const double *nodes, int64_t n, int64_t ld, const i
                              int64_t ld_out, DevStatus *st, cudaStream_t s)
 {
     if (n <= 0) return;
-    k_lightcone_shells<<<grid_for(n, 128), 128, 0, s>>>(nodes, n, ld, shell_off, nshell, t_box, mode, P, nloops, ldp,
+    k_lightcone_shells<<<grid_for(n, kSolveNT), kSolveNT, 0, s>>>(nodes, n, ld, shell_off, nshell, t_box, mode, P, nloops, ldp,
                                                          xo0, xo1, xo2, t_obs, tol, out, ld_out, st);
 }
 
