@@ -192,11 +192,13 @@ void timing_end(isw_ctx *c, int k, cudaStream_t s)
     c->n_timed = k + 1;
 }
 
-// Whether a map runs over the cluster tree (a variant or a chunk count set by the caller asks for the
-// direct kernels).
-bool use_tree(const isw_ctx *c, int64_t npix, int64_t n, int prec)
+// A chunk count or a wait limit set by the caller asks for the direct kernels: the tree's have neither.
+bool default_kernels(const isw_ctx *c) { return c->split_override == 0 && c->wait_polls == kWaitPolls; }
+
+// Whether a map runs over the cluster tree (an FP32 variant set by the caller asks for the direct kernels, too).
+bool use_tree(const isw_ctx *c, TreeUse use, int64_t npix, int64_t n, int prec)
 {
-    return c->split_override == 0 && (prec == ISW_F64 || c->tile_override < 0) && tree_rule(prec, npix, n) &&
+    return default_kernels(c) && (prec == ISW_F64 || c->tile_override < 0) && tree_rule(prec, use, npix, n) &&
            npix < (int64_t(1) << 32);
 }
 
@@ -281,7 +283,8 @@ int map_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_
         }
         return ISW_OK;
     }
-    if (tune_waves == 0 && use_tree(c, npix, n, prec))
+    const TreeUse use = patch ? kTreePatch : !pix_list && pix0 == 0 && npix == 12 * nside * nside ? kTreeSky : kTreePixelList;
+    if (tune_waves == 0 && use_tree(c, use, npix, n, prec))
         return map_tree_impl(c, nside, pix0, npix, pix_list, patch, samples, n, ld, xo, GU, prec, accumulate, theta, s);
     int vidx = 0;
     if (prec == ISW_F32C) {
@@ -849,7 +852,7 @@ int isw_map_patch(isw_ctx *c, const double *frame, int64_t M, double width, cons
         return ISW_OK;
     }
     const bool f64 = prec == ISW_F64;
-    if (c->split_override == 0 && flat_tree_rule(M, n)) {
+    if (default_kernels(c) && flat_tree_rule(M, n)) {
         const FlatTreePlan tp = flat_tree_plan(f64, M, n, c->num_sms);
         if ((r = ensure_ws(c, kWsFlat, (size_t)tp.n_pad * flat_record_bytes()))) return r;
         if ((r = ensure_ws(c, kWsTree, tp.bytes))) return r;
@@ -971,7 +974,7 @@ int isw_map_adjoint(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const
         return ISW_OK;
     }
     const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
-    if (c->split_override == 0 && tree_rule(prec, npix, n) && npix < (int64_t(1) << 32)) {
+    if (default_kernels(c) && tree_rule(prec, kTreeAdjoint, npix, n) && npix < (int64_t(1) << 32)) {
         const bool f64 = prec == ISW_F64;
         const int orders = f64 ? 1 : 2;
         const bool full = !pix_list && pix0 == 0 && npix == 12 * nside * nside;
@@ -1164,7 +1167,7 @@ int isw_map_batched(isw_ctx *c, int64_t nside, const double *nodes, int64_t ld, 
 
     // autotuner: time every FP32 variant on a prefix of the samples, keep the fastest
     if ((flags & ISW_AUTOTUNE) && prec == ISW_F32C && n > 0 && c->tile_override < 0 &&
-        !use_tree(c, npix, n, prec) &&
+        !use_tree(c, kTreeSky, npix, n, prec) &&
         !(c->tuned_nside == nside && c->tuned_n == n)) {
         if (!skip_lc) {
             launch_lightcone_shells(nodes, n, ld, d_off, nshell, d_tbox, d_mode, loop_params, nloops, ldp, xo[0],

@@ -149,15 +149,25 @@ void launch_reduce_partials(const MapArgs &a, int tile_sz, cudaStream_t s);
 
 // tree.cu: the map over a cluster tree of the pixels
 constexpr int kTreeLevels = 20;
-// Whether a map of default settings runs over the tree: from 1e8 pairs in FP32, where its dozen extra
-// launches (0.15 ms) are made up for (N_side 64 with 10,240 samples, 5e8 pairs: 0.6 against 2.5 ms), and
-// from 2e7 in FP64; with enough pixels for the leaves' nodes to be fewer than the pixels.  The list
-// entries hold 30-bit record numbers.
-inline bool tree_rule(int prec, int64_t npix, int64_t n)
+// Whether a call of default settings runs over the tree, by pairs (both sides timed from N_side 4 to 90, samples of
+// strings and scattered ones; direct / tree in ms):
+//   FP32 full sky  1e6: N_side 16 with 500 0.69 / 0.29 and 0.29 / 0.21, N_side 64 with 500 0.78 / 0.38 and
+//                  0.21 / 0.22.  The direct kernel sums a string's near pairs lane by lane in FP64.
+//   FP32 patch     5e7: 128 x 128 with 5,000 0.91 / 0.36 with a string in it, 0.21 / 0.25 with none near
+//   FP32 list      3e8: 20,000 pixels and samples 0.79 / 0.71, a quarter of the pairs 0.37 / 0.43.
+//   FP32 adjoint   3e8, N_side 32: 12,288 pixels and 20,000 samples 0.64 / 0.64, N_side 53 with 10,000 0.92 / 0.81,
+//                  with 5,000 0.54 / 0.68.
+//   FP64 map       6e7: N_side 64 with 2,500 4.4 / 3.4 and 8.5 / 3.4, with 1,000 1.9 / 2.2 and 3.7 / 2.2; the
+//                  leaves have 32 x 32 pixels, so at least four faces of half that.
+//   FP64 adjoint   6e6, N_side 32: N_side 32 with 500 1.18 / 0.80, with 250 0.64 / 0.56; N_side 22 with 5,000 4.2 / 5.0.
+// The list entries hold 30-bit record numbers.
+enum TreeUse : int { kTreeSky = 0, kTreePatch = 1, kTreePixelList = 2, kTreeAdjoint = 3 };
+inline bool tree_rule(int prec, TreeUse use, int64_t npix, int64_t n)
 {
-    const bool f64 = prec == ISW_F64;
-    return npix >= (f64 ? 48 * 1024 : 12 * 1024) && (double)npix * (double)n >= (f64 ? 2e7 : 1e8) &&
-           n < (int64_t(1) << 30);
+    const bool f64 = prec == ISW_F64, adj = use == kTreeAdjoint;
+    const int64_t pix = adj ? 12 * 1024 : f64 ? 4096 : 192;
+    const double pairs = adj ? (f64 ? 6e6 : 3e8) : f64 ? 6e7 : use == kTreeSky ? 1e6 : use == kTreePatch ? 5e7 : 3e8;
+    return npix >= pix && (double)npix * (double)n >= pairs && n < (int64_t(1) << 30);
 }
 // slot order of the pixel tables: anti-diagonals (full sky), rows (patch), spatially sorted list
 enum : int { kSlotsDiag = 0, kSlotsRows = 1, kSlotsList = 2 };

@@ -170,7 +170,7 @@ extern "C" int isw_map_f32c_noalloc(int64_t nside, int64_t pix0, int64_t npix, c
     int sms = 0;
     int r = scratch_address(dev, &base, &sms);
     if (r) return r;
-    if (tree_rule(ISW_F32C, npix, n)) {   // the cluster tree, as isw_map, when it fits
+    if (tree_rule(ISW_F32C, pix0 == 0 && npix == 12 * nside * nside ? kTreeSky : kTreePixelList, npix, n)) {   // the cluster tree, as isw_map, when it fits
         r = map_tree_noalloc(nside, pix0, npix, samples, n, ld, x_obs, GU, theta_out, (unsigned char *)base, sms, s);
         if (r != ISW_EINVAL) return r == ISW_OK ? finish(base, status_out, s) : r;
     }

@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_pixels_f32(TreePixArgs a)
 // to 1.9e-16 of the rms (direct kernel 0.5e-16 to 1.2e-16), largest 1.9e-15 (1.0e-15).
 // ------------------------------------------------------------------------------------
 constexpr int kNP64 = 16, kNN64 = kNP64 * kNP64, kLeaf64 = 32;
-constexpr int kNodeTarget64 = 128, kPixTarget64 = 48;
+constexpr int kNodeTarget64 = 32, kPixTarget64 = 12;
 
 // A staged Far64 record.
 struct __align__(16) Stage64 {
@@ -766,6 +766,7 @@ struct TreePixArgs64 {
     float d_far;
     int64_t nside;   // full-sky maps
     int nb;
+    int parts;       // items of a cluster (and chunk): 1, or 4 with a block per warp each
 };
 
 // Ring form of the far-field pair term.  A pixel of a ring (z, s = sin theta) at azimuth phi has n / s =
@@ -810,7 +811,9 @@ struct __align__(16) TreePixSmem64 {
 // neighbouring entries
 __device__ __forceinline__ int az_place(int l) { return (l >> 1) + (l & 1) * kLeaf64; }
 
-// Eight pixels per thread, one cluster per item: four blocks of 8 x 8 pixels per warp (full sky) or of 64
+// Eight pixels per thread, one cluster per item, or a quarter of one with fewer than two (cluster, sample
+// tile) pairs for every CTA slot (N_side 64 with 1,000 samples 2.6 -> 2.2 ms, N_side 16 with 250 1.2 -> 0.6;
+// with 2,500 samples at N_side 64 the quarters' tables cost more, 3.4 -> 4.4): four blocks of 8 x 8 pixels per warp (full sky) or of 64
 // consecutive slots.  Bound by the FP64 unit.  N_side 64 with 10,240 samples 10.2 ms with 17 operations for every
 // pixel -> 8.4 ms, N_side 128 with 30,001 33.5 -> 26.7 ms.  Samples that the cluster's test flags are tested again per block: with |d| >= d_far and
 // B >= b_min on the block they too take the far-field form (its squares cancel to a factor 1/B of the rounding),
@@ -826,15 +829,18 @@ __global__ void __launch_bounds__(kTreeNT, 3) k_tree_pixels_f64(TreePixArgs64 A)
     const int np = *a.W.npool;
     unsigned zerocnt = 0;
     TreeQueue queue{a.queue, 0ull};
-    for (int64_t item = queue.first(&sm.item); item < a.W.ncl + np; item = queue.next(&sm.item)) {
+    const int per = kBlocks64 / A.parts;   // blocks per warp of an item
+    for (int64_t it = queue.first(&sm.item); it < (a.W.ncl + np) * A.parts; it = queue.next(&sm.item)) {
         int kc, nch;
         int64_t at;
+        const int64_t item = it / A.parts;
+        const int pb = (int)(it - item * A.parts) * per;   // first block
         const int64_t cl = tree_item(a.W, item, np, kc, nch, at);
         if (cl < 0) continue;
         load_geo(&sm.geo, a.geo + cl);
         const int64_t k0 = cl * TILE;
         int slot[P], place[P];   // slot in the cluster; SKY: ring and azimuth entries
-        unsigned valid = 0, eq = 0;
+        unsigned valid = 0, eq = 0, live = 0;   // live: blocks of this item that have pixels
         if (SKY) {
             const int64_t N = A.nside, f = cl / ((int64_t)A.nb * A.nb), rem = cl - f * A.nb * A.nb;
             const int64_t y0 = rem / A.nb * kLeaf64, x0 = rem % A.nb * kLeaf64;
@@ -900,6 +906,7 @@ __global__ void __launch_bounds__(kTreeNT, 3) k_tree_pixels_f64(TreePixArgs64 A)
             }
             const TreeCap c = warp_ball(x);
             if (lane == 0) sm.cap[w][p] = c.a;
+            if (c.a.w >= 0.f && p >= pb && p < pb + per) live |= 1u << p;
         }
         __syncthreads();
         const float4 self = sm.geo.c;
@@ -988,7 +995,7 @@ __global__ void __launch_bounds__(kTreeNT, 3) k_tree_pixels_f64(TreePixArgs64 A)
             const float d = sqrtf(x * x + y * y + z * z) - c.w;
             x = c.x - bm.x, y = c.y - bm.y, z = c.z - bm.z;
             const float h = fmaxf(sqrtf(x * x + y * y + z * z) - c.w, 0.f);
-            return c.w < 0.f || (d >= A.d_far && fmaf(0.5f * (1.f - bm.w) * h, h, bm.w) >= a.b_min);
+            return (d >= A.d_far && fmaf(0.5f * (1.f - bm.w) * h, h, bm.w) >= a.b_min);
         };
         int l0 = 0;   // list position of the batch
         auto eval = [&](int cnt) {
@@ -1035,12 +1042,14 @@ __global__ void __launch_bounds__(kTreeNT, 3) k_tree_pixels_f64(TreePixArgs64 A)
                     const Stage64 &r = sm.rec[b0 + s];
                     if (!(e & (kTreeClose | kTreeBeam))) {
 #pragma unroll
-                        for (int p = 0; p < kBlocks64; ++p) far_block(r, p, s, false, part[2 * p], part[2 * p + 1]);
+                        for (int p = 0; p < kBlocks64; ++p)
+                            if (live >> p & 1u) far_block(r, p, s, false, part[2 * p], part[2 * p + 1]);
                         continue;
                     }
                     const float4 xh = a.S.crit[e & kTreeIndex].a, bm = a.S.crit[e & kTreeIndex].b;
 #pragma unroll
                     for (int p = 0; p < kBlocks64; ++p) {
+                        if (!(live >> p & 1u)) continue;
                         if (far_on(xh, bm, p)) far_block(r, p, s, true, part[2 * p], part[2 * p + 1]);
                         else near_block(a.s64[e & kTreeIndex], p, part[2 * p], part[2 * p + 1]);
                     }
@@ -1061,8 +1070,9 @@ __global__ void __launch_bounds__(kTreeNT, 3) k_tree_pixels_f64(TreePixArgs64 A)
         if (kc == 0) cheb_coefs64(a.F, a.Wf, cl, sm.coef, sm.tmp, rhi, rlo);
 #pragma unroll
         for (int q = 0; q < P; ++q) {
+            if (q / 2 < pb || q / 2 >= pb + per) continue;
             const int64_t k = k0 + slot[q];
-            if (kc == 0) {
+            if (kc == 0 && live >> q / 2 & 1u) {
                 double x, y;
                 local_xy64(sm.geo, a.nv[k] - sm.geo.n0[0], a.nv[a.ldn + k] - sm.geo.n0[1], a.nv[2 * a.ldn + k] - sm.geo.n0[2], x, y);
                 fold64(hi[q], lo[q], rhi);
@@ -1245,7 +1255,8 @@ cudaError_t launch_map_tree(const TreePlan &p, const TreeMapArgs &m, cudaStream_
     A.d_far = m.d_far;
     A.nside = m.nside;
     A.nb = p.nb[0];
-    const int64_t items = p.ncl[0] + p.ppool;
+    A.parts = p.ncl[0] * p.nst < 2 * (int64_t)p.pslots ? kBlocks64 : 1;
+    const int64_t items = (p.ncl[0] + p.ppool) * (f64 ? A.parts : 1);
     const unsigned grid = (unsigned)(items < p.pslots ? items : p.pslots);
     if (f64 && m.nside > 0) k_tree_pixels_f64<true><<<grid, kTreeNT, sizeof(TreePixSmem64), s>>>(A);
     else if (f64) k_tree_pixels_f64<false><<<grid, kTreeNT, sizeof(TreePixSmem64), s>>>(A);
