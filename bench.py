@@ -40,6 +40,9 @@ FLOPS_PER_PAIR = 36          # algorithmic flops of one Eq. (1)-(2) pair term, F
 # algorithmic flops of one pair of the adjoint (dL/dX, dL/dXdot: the derivative sums of
 # isw_map_adjoint in textbook form, FMA = 2, the two reciprocals not counted)
 ADJ_FLOPS_PER_PAIR = 66
+# pairs are counted as the all-pairs sum has them; the cluster tree sums far pairs at nodes
+EQUIVALENT = "equivalent, not executed: {} textbook flops for each pixel-sample pair of the sum (above 1 where the " \
+             "cluster tree sums most pairs at its nodes) of the "
 FP32_LANES = 128             # FP32 FMA lanes per SM (Blackwell)
 
 
@@ -304,8 +307,8 @@ def run_gpu(args):
         ach64 = FLOPS_PER_PAIR * pairs_step / (k64 / 1e3) / 1e12
         fp64 = {"value": pairs_step / (ms64 / 1e3), "unit": UNIT, "ms_per_step": ms64,
                 "roofline": {"bound": "alu", "achieved": ach64, "peak": fma64, "unit": "TFLOP/s",
-                             "frac": ach64 / fma64, "frac_kind": "algorithmic (36 flop/pair) of measured",
-                             "traffic": None, "kernel": "isw::k_map_f64 (+ chunk reduce)",
+                             "frac": ach64 / fma64, "frac_kind": EQUIVALENT.format(36) + "measured FP64 peak",
+                             "traffic": None, "kernel": "isw::k_tree_nodes_f64, k_tree_pixels_f64 (cluster tree)",
                              "kernel_ms": k64, "flops_per_pair": FLOPS_PER_PAIR,
                              "peak_note": "measured: FP64 FMA-chain calibration kernel on every SM "
                                           "(isw_fma_rate), this run"}}
@@ -349,13 +352,13 @@ def run_gpu(args):
                             "fp64_value": p3 / (ms3_64 / 1e3), "fp64_ms": ms3_64,
                             "roofline": {"bound": "alu", "achieved": a32, "peak": peak32, "unit": "TFLOP/s",
                                          "frac": a32 / peak32, "flops_per_pair": ADJ_FLOPS_PER_PAIR,
-                                         "frac_kind": "algorithmic (66 flop/pair) of the derived FP32 peak",
-                                         "kernel": "isw::k_adj_f32c (+ chunk reduce)",
+                                         "frac_kind": EQUIVALENT.format(66) + "derived FP32 peak",
+                                         "kernel": "isw::k_adj_tree (cluster tree)",
                                          "kernel_ms": ka32, "traffic": None},
                             "fp64_roofline": {"bound": "alu", "achieved": a64, "peak": fma64, "unit": "TFLOP/s",
                                               "frac": a64 / fma64, "flops_per_pair": ADJ_FLOPS_PER_PAIR,
-                                              "frac_kind": "algorithmic (66 flop/pair) of the measured FP64 peak",
-                                              "kernel": "isw::k_adj_f64 (+ chunk reduce)",
+                                              "frac_kind": EQUIVALENT.format(66) + "measured FP64 peak",
+                                              "kernel": "isw::k_adj_tree64 (cluster tree)",
                                               "kernel_ms": ka64, "traffic": None}}
         # gradient through the light-cone solve: map adjoint with the dsigma row, then the
         # loop-parameter chain (98 Burden loops)
@@ -438,11 +441,12 @@ def run_gpu(args):
     map_avg_ms = map_ms / max(map_launches, 1)
     achieved = FLOPS_PER_PAIR * pairs_step / (map_avg_ms / 1e3) / 1e12
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "frac_kind": "algorithmic: 36 textbook flops per pair (the far-field form executes ~15 FP32 "
-                         "lane operations per pair) of the derived FP32 peak",
+            "frac_kind": EQUIVALENT.format(36) + "derived FP32 peak (the default workload's 6.3e11 pairs are "
+                         "summed by 3e9 pair terms at cluster nodes and 6e8 at pixels)",
             "fma_pipe_busy_far_pass": (profiled_fma_busy(variant_used) if args.nside is None else None),
             "traffic": (profiled_traffic(variant_used) if args.nside is None else None),
-            "kernel": f"pair kernels: isw::k_map_f32c (far field) + k_map_f32c_near + chunk reduce, variant {variant_used}",
+            "kernel": "isw::k_tree_nodes_f32 + k_tree_pixels_f32 (cluster tree) and their set-up; below 1e6 pairs or "
+                      f"with a variant set, k_map_f32c + k_map_f32c_near + chunk reduce, variant {variant_used}",
             "flops_per_pair": FLOPS_PER_PAIR, "kernel_ms": map_avg_ms, "kernel_launches": map_launches,
             "peak_note": f"derived: {sm_count} SMs (device) x {FP32_LANES} FP32 lanes x 2 flop x {mhz:.0f} MHz "
                          f"(max SM clock); measured FP32 FMA calibration kernel: {fma32:.1f} TFLOP/s"}

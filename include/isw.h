@@ -93,7 +93,14 @@ const char *isw_last_error(const isw_ctx *ctx);
  * non-finite weight), pairs that the FP32 path evaluated in FP64 (near field). */
 int isw_check_status(isw_ctx *ctx, void *stream, int64_t *counts);
 
-/* Tunables: ISW_PARAM_NEAR_K (default 2): a pair is "near" when the chord |n - Xhat| is
+/* Maps and adjoints with many pairs run over a cluster tree of the pixels: the samples far from a
+ * cluster (by position and by beam) are summed at Chebyshev nodes and interpolated, the others pixel
+ * by pixel, to the working precision of the call.  It is taken by default settings of
+ * ISW_PARAM_SPLIT and ISW_PARAM_WAIT_POLLS (and, for FP32 maps, ISW_PARAM_VARIANT) from a number of
+ * pairs that depends on the call; any other value of these keeps the direct kernels, which sum every
+ * pair and which these three tunables describe.
+ *
+ * Tunables: ISW_PARAM_NEAR_K (default 2): a pair is "near" when the chord |n - Xhat| is
  * below near_k * max(pixel size, angular length of the sample's segment); ISW_PARAM_B_MIN
  * (default 0.01): a pair with 1 + n.Xdot below b_min is evaluated in FP64 by the FP32 path;
  * ISW_PARAM_SPLIT: number of segment chunks of the forward maps (0 = automatic: enough
@@ -104,9 +111,9 @@ int isw_check_status(isw_ctx *ctx, void *stream, int64_t *counts);
  * segment tiles whose every pair is at least this chord apart from the pixel tile use the
  * FP32 far-field form (d.d = 2 (1 - n.Xhat), Xdot.d and X'.d from per-sample constants);
  * 4 disables it; ISW_PARAM_TIMING (default 0):
- * when 1, every launch of the pair kernel (the all-pairs sum of isw_map and
- * isw_map_batched: the FP32 far- and near-field passes and the chunk reduction between them, or
- * the FP64 kernel and its reduction) is bracketed by CUDA events on its stream, read by
+ * when 1, every launch of the pair work (the all-pairs sum of isw_map and
+ * isw_map_batched: the kernels of the tree; or the FP32 far- and near-field passes and the chunk
+ * reduction between them, or the FP64 kernel and its reduction) is bracketed by CUDA events on its stream, read by
  * isw_get_timing.  ISW_PARAM_WAIT_POLLS (default 2^22; a negative value restores it): the
  * limit, in mbarrier try_wait polls, of every wait of the pair kernels (isw_map, isw_map_batched,
  * isw_map_adjoint, isw_map_patch) for a stage of records to land in shared memory.  A wait that
