@@ -314,7 +314,8 @@ int lightcone_adjoint(isw_ctx *ctx, int mode, const double *nodes_in, int64_t n,
  * nshell; loop_params as in lightcone_intersect.  The light-cone solve of every shell and
  * one map over all samples are enqueued (flags: ISW_SKIP_LIGHTCONE when nodes are already
  * samples on the cone; ISW_GRAPH to capture the sequence in a CUDA graph that later calls
- * with the same arguments replay; ISW_AUTOTUNE to pick the FP32 kernel variant by timing).
+ * with the same arguments replay; ISW_AUTOTUNE to pick the FP32 kernel variant of the
+ * direct kernels by timing, where these are taken).
  * theta_out: device double[12 N^2] (RING), written or accumulated as in isw_map. */
 int isw_map_batched(isw_ctx *ctx, int64_t nside, const double *nodes, int64_t ld, const int64_t *shell_off,
                     int64_t nshell, const double *t_box, const int32_t *mode, const double *loop_params,
@@ -339,8 +340,9 @@ int isw_map_batched(isw_ctx *ctx, int64_t nside, const double *nodes, int64_t ld
  *     without ordering) race on the array and produce wrong maps.
  *   - Arguments as in isw_map (device samples double[10][ld] and theta_out double[npix] on the
  *     current device, host x_obs or NULL); kernel variant, segment chunks, near-field and b_min
- *     settings are those of isw_map with default settings (the chunk count capped by the
- *     scratch), so the map equals isw_map's.
+ *     settings are those of isw_map with default settings, so the map equals isw_map's (the chunk
+ *     count is capped by the scratch, and where isw_map would take the cluster tree but its scratch
+ *     does not fit, the direct kernels run: the two then agree to the FP32 path's precision).
  *   - status_out (host, may be NULL): when given, the call waits for `stream` and stores the
  *     status the kernels recorded: ISW_OK, ISW_EDOMAIN (a sample with |Xdot| >= 1 or a
  *     non-finite weight was skipped) or ISW_ETIMEOUT (a bounded device wait ran out: the map is
