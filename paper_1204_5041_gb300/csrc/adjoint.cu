@@ -22,7 +22,7 @@
 // operations and two reciprocals per pair); other tiles go through the checked loop (float-pair
 // d, cancellation-free B, FP64 for near pairs).  FP64 kernel: the same sums in FP64 from Pix64
 // records, far tiles in the far-field form with Newton-refined reciprocals (rcp64), the others
-// pair by pair in the d form with IEEE divisions.  Per-chunk gradients are reduced over chunks in
+// pair by pair in the d form.  Per-chunk gradients are reduced over chunks in
 // a fixed order (deterministic).
 #include "adjoint.cuh"
 #include "isw_internal.cuh"

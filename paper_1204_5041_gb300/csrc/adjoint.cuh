@@ -2,6 +2,7 @@
 #pragma once
 
 #include "isw_internal.cuh"
+#include "pipeline.cuh"
 
 namespace isw {
 
@@ -31,7 +32,7 @@ __device__ __forceinline__ void adj_pair64(double nx, double ny, double nz, doub
     const double B = 1.0 + (nx * s.xd[0] + ny * s.xd[1] + nz * s.xd[2]);
     const double Pd = s.xd[0] * dx + s.xd[1] * dy + s.xd[2] * dz;
     const double Qd = s.xp[0] * dx + s.xp[1] * dy + s.xp[2] * dz;
-    const double iQ = 1.0 / Q, iB = 1.0 / B;
+    const double iQ = rcp64(Q), iB = rcp64(B);
     const double AB = A * iB;
     const double uX = (s.xd[0] * s.xh[0] + s.xd[1] * s.xh[1] + s.xd[2] * s.xh[2]) -
                       AB * (s.xp[0] * s.xh[0] + s.xp[1] * s.xh[1] + s.xp[2] * s.xh[2]);

@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(NT, (P <= 4 ? 512 : 256) / NT) k_map_f32c_near
 // t = (c/2) [B (B - e) - A (A - f)] / [B (1 - n.Xhat)], written with completed squares scaled by
 // sqrt(|c|/2) (Far64 records: 17 FP64 operations per pair; the cancellation in 1 - n.Xhat costs
 // at most a factor 2/d_far^2 = 32 of the 1e-16 rounding); the others pair by pair from
-// d = n - Xhat formed from the double-double Xhat, with the IEEE division.
+// d = n - Xhat formed from the double-double Xhat.
 template <int NT, int P, int S>
 __global__ void __launch_bounds__(NT) k_map_f64(MapArgs a)
 {

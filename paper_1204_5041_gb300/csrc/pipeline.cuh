@@ -8,24 +8,6 @@ namespace isw {
 
 constexpr int kStages = 4;
 
-// FP64 pair term (d = (n - Xhat_hi) - Xhat_lo keeps full relative accuracy near the string)
-__device__ __forceinline__ double pair64(double nx, double ny, double nz, const Seg64 &g, unsigned &zero)
-{
-    const double dx = (nx - g.xh[0]) - g.xl[0];
-    const double dy = (ny - g.xh[1]) - g.xl[1];
-    const double dz = (nz - g.xh[2]) - g.xl[2];
-    const double Q = dx * dx + dy * dy + dz * dz;
-    if (Q == 0.0) {
-        ++zero;
-        return 0.0;
-    }
-    const double A = nx * g.xp[0] + ny * g.xp[1] + nz * g.xp[2];
-    const double B = 1.0 + (nx * g.xd[0] + ny * g.xd[1] + nz * g.xd[2]);
-    const double Pd = g.xd[0] * dx + g.xd[1] * dy + g.xd[2] * dz;
-    const double Qd = g.xp[0] * dx + g.xp[1] * dy + g.xp[2] * dz;
-    return g.c * (B * Pd - A * Qd) / (B * Q);
-}
-
 // 1/x for a nonzero normal double of either sign whose reciprocal is normal: the estimate r from the high
 // word of x (relative error e = 1 - x r at most 2^-19.9) refined by one third-order step of the iteration
 // for 1/x, r (1 + e + e^2) (error e^3 < 2^-59, a hundredth of an ulp):
@@ -39,9 +21,11 @@ __device__ __forceinline__ double rcp64(double x)
     return fma(r, fma(e, e, e), r);
 }
 
-// pair64 with the third-order reciprocal in the place of the IEEE division (an ulp or two; B and Q
-// are far above the float range's lower end: Q >= 1e-30 for distinct directions, B > 1e-12)
-__device__ __forceinline__ double pair64_fast(double nx, double ny, double nz, const Seg64 &g, unsigned &zero)
+// Pair term of Eq. (1)-(2) in FP64 from the double-double Xhat, c [B Xdot.d - A X'.d] / (B d.d); a pixel on the
+// sample's line of sight adds nothing and is counted.  The third-order reciprocal in the place of an IEEE
+// division costs an ulp or two and saves some ten FP64 operations (a direct FP64 map of N_side 22 with 5,000
+// samples 2.54 -> 2.26 ms, its error 0.9e-16 of the rms with either).
+__device__ __forceinline__ double pair64(double nx, double ny, double nz, const Seg64 &g, unsigned &zero)
 {
     const double dx = (nx - g.xh[0]) - g.xl[0];
     const double dy = (ny - g.xh[1]) - g.xl[1];

@@ -289,7 +289,7 @@ __device__ __noinline__ void near_flush(TreeNearQueue &q, int cnt, const Seg64 *
     if (on) {
         const Seg64 g = s64[q.src[lane]];
         const int64_t k = kw + px;
-        v = pair64_fast(nv[k], nv[ldn + k], nv[2 * ldn + k], g, zerocnt);
+        v = pair64(nv[k], nv[ldn + k], nv[2 * ldn + k], g, zerocnt);
     }
     q.val[lane] = v;
     __syncwarp();
