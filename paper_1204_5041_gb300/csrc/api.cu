@@ -645,10 +645,13 @@ int lightcone_adjoint(isw_ctx *c, int mode, const double *nodes_in, int64_t n, i
     cudaStream_t s = (cudaStream_t)stream;
     int *runs = nullptr;
     int64_t *first = nullptr, *last = nullptr;
+    double *contrib = nullptr;
     if (mode == ISW_BURDEN) {
         const size_t nl = (size_t)nloops;
-        if ((r = ensure_ws(c, kWsLoops, nl * (2 * sizeof(int64_t) + sizeof(int)) + 16))) return r;
-        first = (int64_t *)c->ws[kWsLoops];
+        const size_t terms = (size_t)n * 15 * sizeof(double);
+        if ((r = ensure_ws(c, kWsLoops, terms + nl * (2 * sizeof(int64_t) + sizeof(int)) + 16))) return r;
+        contrib = (double *)c->ws[kWsLoops];
+        first = (int64_t *)(contrib + (size_t)n * 15);
         last = first + nl;
         runs = (int *)(last + nl);
         cudaError_t e = cudaMemsetAsync(runs, 0, nl * sizeof(int), s);
@@ -657,7 +660,7 @@ int lightcone_adjoint(isw_ctx *c, int mode, const double *nodes_in, int64_t n, i
     const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
     launch_lightcone_adjoint(mode, nodes_in, n, ld, loop_params, nloops, ldp, t_box, xo[0], xo[1], xo[2], tau,
                              grad_samples, ld_gs, ngrad, grad_nodes, ld_gn, grad_loops, ld_gl, runs, first, last,
-                             c->d_status, s);
+                             contrib, c->d_status, s);
     c->n_launch += (n > 0 ? 1 : 0) + (mode == ISW_BURDEN ? 1 : 0);
     return check_launch(c, "lightcone_adjoint launch");
 }

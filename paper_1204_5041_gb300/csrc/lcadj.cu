@@ -7,8 +7,8 @@
 //   lambda = (g_X . dX/dt + g_Xd . dXdot/dt + g_Xp . dX'/dt) / (1 + rhat . Xdot),
 //   gamma = g_X - lambda rhat,
 // dL/dq = gamma . dX/dq|_t + g_Xd . dXdot/dq|_t + g_Xp . dX'/dq|_t for every parameter q.
-// One thread per node writes the node gradients; for Burden loops one warp per loop sums the
-// loop-parameter gradients over the loop's samples in a fixed order (deterministic).
+// One thread per node writes the node gradients and, for Burden loops, its terms of the loop-parameter
+// gradients, which one warp per loop sums over the loop's samples in a fixed order (deterministic).
 #include "isw_internal.cuh"
 #include "kernels.cuh"
 
@@ -85,7 +85,7 @@ __device__ __forceinline__ void load_gs(const double *__restrict__ gs, int64_t l
 }
 
 // One Burden sample: gamma-weighted derivatives.  Returns false when rhat is undefined or
-// 1 + rhat.Xdot <= 0.  contrib (optional): centre (3), rotation (9), L, psi, t0.
+// 1 + rhat.Xdot <= 0.  contrib: centre (3), rotation (9), L, psi, t0.
 __device__ __forceinline__ bool burden_sample(const double *__restrict__ P, int64_t ldp, int64_t id, double sigma,
                                               double t, const double xo[3], const double gX[3], const double gXd[3],
                                               const double gXp[3], double &g_sigma, double *contrib)
@@ -113,23 +113,21 @@ __device__ __forceinline__ bool burden_sample(const double *__restrict__ P, int6
 #pragma unroll
     for (int k = 0; k < 3; ++k) gam[k] = gX[k] - lam * (r[k] / rn);
     g_sigma = dot3(gam, Xp) + dot3(gXd, Xdp) + dot3(gXp, Xdd);
-    if (contrib) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            contrib[k] = gam[k];
+    for (int k = 0; k < 3; ++k) {
+        contrib[k] = gam[k];
 #pragma unroll
-            for (int j = 0; j < 3; ++j) contrib[3 + 3 * k + j] = gam[k] * J.h[j] + gXd[k] * J.hd[j] + gXp[k] * J.hp[j];
-        }
-        double v1[3], v2[3], v3[3];
-        rot(R, J.hL, v1);
-        rot(R, J.hdL, v2);
-        rot(R, J.hpL, v3);
-        contrib[12] = dot3(gam, v1) + dot3(gXd, v2) + dot3(gXp, v3);
-        rot(R, J.hs, v1);
-        rot(R, J.hds, v2);
-        contrib[13] = dot3(gam, v1) + dot3(gXd, v2) + dot3(gXp, v2);
-        contrib[14] = -(dot3(gam, Xd) + dot3(gXd, Xdd) + dot3(gXp, Xdp));
+        for (int j = 0; j < 3; ++j) contrib[3 + 3 * k + j] = gam[k] * J.h[j] + gXd[k] * J.hd[j] + gXp[k] * J.hp[j];
     }
+    double v1[3], v2[3], v3[3];
+    rot(R, J.hL, v1);
+    rot(R, J.hdL, v2);
+    rot(R, J.hpL, v3);
+    contrib[12] = dot3(gam, v1) + dot3(gXd, v2) + dot3(gXp, v3);
+    rot(R, J.hs, v1);
+    rot(R, J.hds, v2);
+    contrib[13] = dot3(gam, v1) + dot3(gXd, v2) + dot3(gXp, v2);
+    contrib[14] = -(dot3(gam, Xd) + dot3(gXd, Xdd) + dot3(gXp, Xdp));
     return true;
 }
 
@@ -140,13 +138,17 @@ __device__ __forceinline__ int64_t loop_id(const double *__restrict__ nodes, int
     return (id >= 0 && id < nloops) ? id : -1;
 }
 
-// Node gradients; Burden mode also marks the first and one-past-last sample of every run of
-// equal loop ids (runs[l] counts the runs of loop l: 1 when its samples are contiguous).
+// Node gradients, and in Burden mode the node's terms of the loop-parameter gradients (contrib[15][n]).  Here as many
+// threads as there are nodes compute them, 27 us for 5,120 nodes; the loops' warps, computing them themselves, took
+// 16 nodes' dependent FP64 work per lane: 320 us for 10 loops of 512 nodes, now 26 us.  Burden mode also marks the
+// first and one-past-last sample of every run of equal loop ids (runs[l] counts the runs of loop l: 1 when its
+// samples are contiguous).
 __global__ void k_lcadj_nodes(int mode, const double *__restrict__ nodes, int64_t n, int64_t ld,
                               const double *__restrict__ P, int64_t nloops, int64_t ldp, double t_box, double xo0,
                               double xo1, double xo2, const double *__restrict__ tau, const double *__restrict__ gs,
                               int64_t ldgs, int ngs, double *__restrict__ gn, int64_t ldgn, int *__restrict__ runs,
-                              int64_t *__restrict__ first, int64_t *__restrict__ last, DevStatus *ds)
+                              int64_t *__restrict__ first, int64_t *__restrict__ last, double *__restrict__ contrib,
+                              DevStatus *ds)
 {
     const double xo[3] = {xo0, xo1, xo2};
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
@@ -184,9 +186,12 @@ __global__ void k_lcadj_nodes(int mode, const double *__restrict__ nodes, int64_
             if (id < 0) {
                 atomicOr(&ds->bits, kStatBadIndex);
             } else {
-                double gsigma = 0.0;
-                if (burden_sample(P, ldp, id, nodes[ld + s], t, xo, gX, gXd, gXp, gsigma, nullptr)) out[1] = gsigma;
+                double gsigma = 0.0, term[15];
+                const bool ok = burden_sample(P, ldp, id, nodes[ld + s], t, xo, gX, gXd, gXp, gsigma, term);
+                if (ok) out[1] = gsigma;
                 else atomicOr(&ds->bits, kStatDomain);
+#pragma unroll
+                for (int q = 0; q < 15; ++q) contrib[q * n + s] = ok ? term[q] : 0.0;
                 if (s == 0 || loop_id(nodes, s - 1, nloops) != id) {
                     atomicAdd(&runs[id], 1);
                     first[id] = s;
@@ -201,13 +206,10 @@ __global__ void k_lcadj_nodes(int mode, const double *__restrict__ nodes, int64_
 
 // Loop-parameter gradients: one warp per loop, lanes stride over the loop's samples, fixed
 // butterfly reduction.  Rows: centre (3), rotation (9), L, m (0), n (0), psi, t0.
-__global__ void k_lcadj_loops(const double *__restrict__ nodes, int64_t ld, const double *__restrict__ P,
-                              int64_t nloops, int64_t ldp, double xo0, double xo1, double xo2,
-                              const double *__restrict__ tau, const double *__restrict__ gs, int64_t ldgs, int ngs,
-                              const int *__restrict__ runs, const int64_t *__restrict__ first,
-                              const int64_t *__restrict__ last, double *__restrict__ gl, int64_t ldgl, DevStatus *ds)
+__global__ void k_lcadj_loops(const double *__restrict__ contrib, int64_t n, int64_t nloops, const int *__restrict__ runs,
+                              const int64_t *__restrict__ first, const int64_t *__restrict__ last,
+                              double *__restrict__ gl, int64_t ldgl, DevStatus *ds)
 {
-    const double xo[3] = {xo0, xo1, xo2};
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t l = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); l < nloops; l += warps) {
@@ -217,12 +219,8 @@ __global__ void k_lcadj_loops(const double *__restrict__ nodes, int64_t ld, cons
         for (int q = 0; q < 15; ++q) acc[q] = 0.0;
         if (nr == 1) {
             for (int64_t s = first[l] + lane; s < last[l]; s += 32) {
-                double gX[3], gXd[3], gXp[3], gsig, gsigma, contrib[15];
-                load_gs(gs, ldgs, ngs, s, gX, gXd, gXp, gsig);
-                if (burden_sample(P, ldp, l, nodes[ld + s], tau[s], xo, gX, gXd, gXp, gsigma, contrib)) {
 #pragma unroll
-                    for (int q = 0; q < 15; ++q) acc[q] += contrib[q];
-                }
+                for (int q = 0; q < 15; ++q) acc[q] += contrib[q * n + s];
             }
         }
 #pragma unroll
@@ -250,19 +248,19 @@ __global__ void k_lcadj_loops(const double *__restrict__ nodes, int64_t ld, cons
 void launch_lightcone_adjoint(int mode, const double *nodes, int64_t n, int64_t ld, const double *P, int64_t nloops,
                               int64_t ldp, double t_box, double xo0, double xo1, double xo2, const double *tau,
                               const double *gs, int64_t ldgs, int ngs, double *gn, int64_t ldgn, double *gl,
-                              int64_t ldgl, int *runs, int64_t *first, int64_t *last, DevStatus *st, cudaStream_t s)
+                              int64_t ldgl, int *runs, int64_t *first, int64_t *last, double *contrib, DevStatus *st,
+                              cudaStream_t s)
 {
     if (n > 0) {
         int64_t b = (n + 127) / 128;
         if (b > 152 * 32) b = 152 * 32;
         k_lcadj_nodes<<<(unsigned)b, 128, 0, s>>>(mode, nodes, n, ld, P, nloops, ldp, t_box, xo0, xo1, xo2, tau, gs,
-                                                  ldgs, ngs, gn, ldgn, runs, first, last, st);
+                                                  ldgs, ngs, gn, ldgn, runs, first, last, contrib, st);
     }
     if (mode == ISW_BURDEN && nloops > 0) {
         int64_t b = (nloops + 3) / 4;   // 4 warps per block
         if (b > 152 * 16) b = 152 * 16;
-        k_lcadj_loops<<<(unsigned)b, 128, 0, s>>>(nodes, ld, P, nloops, ldp, xo0, xo1, xo2, tau, gs, ldgs, ngs, runs,
-                                                  first, last, gl, ldgl, st);
+        k_lcadj_loops<<<(unsigned)b, 128, 0, s>>>(contrib, n, nloops, runs, first, last, gl, ldgl, st);
     }
 }
 
