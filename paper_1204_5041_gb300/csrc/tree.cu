@@ -12,10 +12,11 @@
 // maps are reproducible.
 //
 // FP32 maps, 8 x 8 nodes, near radius 3.5 half-sizes, leaves of 16 x 16 pixels: N_side 512 with 2e5 samples
-// 309 -> 8.3 ms (6.3e11 pairs; 3e9 pair terms at nodes, 6e8 at pixels), N_side 64 with 10,240 samples
-// 2.5 -> 0.6 ms; error against FP64 2.6e-8 of the rms (direct kernels 6.9e-8), largest 3e-7 (9e-7).  The
-// node kernels are bound by FP32 issue (FMA pipe 40-50%), the pixel kernel by its FP64 near pairs (a
-// quarter of its time) and by the tests that find them.
+// 309 -> 7.1 ms (6.3e11 pairs; 3e9 pair terms at nodes, 6e8 at pixels), N_side 64 with 10,240 samples
+// 3.1 -> 0.47 ms; error against FP64 2.6e-8 of the rms (direct kernels 6.9e-8), largest 3e-7 (9e-7).  The
+// node kernels are bound by FP32 issue (45-55% of the cycles, FMA pipe 35-57%) at the 16 warps per SM that their
+// registers allow, the pixel kernel by its FP64 near pairs and by the tests that find them (issue 41%, FP64
+// unit 21%).
 #include "tree.cuh"
 
 #include <algorithm>
