@@ -176,6 +176,7 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_nodes_f32(TreeNodeArgs a)
         load_geo(&sm.geo, a.geo + cl);
         __syncthreads();
         const float4 self = sm.geo.c, parent = ROOT ? self : sm.pgeo.c;
+        if (tree_empty(self)) continue;
         uint64_t m[2][3], mm[2];   // node offsets from the centre, |m|^2
 #pragma unroll
         for (int pp = 0; pp < 2; ++pp) {
@@ -329,6 +330,7 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_pixels_f32(TreePixArgs a)
         nq.acc[32 + lane] = 0.0;
         __syncthreads();
         const float4 self = sm.geo.c;
+        if (tree_empty(self)) continue;
         float ahi[4] = {0.f, 0.f, 0.f, 0.f}, alo[4] = {0.f, 0.f, 0.f, 0.f};
         unsigned valid = 0;
         int qlen = 0;
@@ -668,6 +670,7 @@ __global__ void __launch_bounds__(kTreeNT) k_tree_nodes_f64(TreeNodeArgs64 A)
         load_geo(&sm.geo, a.geo + cl);
         __syncthreads();
         const float4 self = sm.geo.c, parent = ROOT ? self : sm.pgeo.c;
+        if (tree_empty(self)) continue;
         double hi[2] = {0.0, 0.0}, lo[2] = {0.0, 0.0};
         const double xt = ((lane & 8) == 0 ? sm.geo.a1 : sm.geo.a2) * cheb_at<kNP64>(1, lane & 7), x2 = xt * xt;
         auto stage = [&](uint32_t e, NodeCoef64 &d) {
@@ -839,6 +842,7 @@ __global__ void __launch_bounds__(kTreeNT, 3) k_tree_pixels_f64(TreePixArgs64 A)
         const int pb = (int)(it - item * A.parts) * per;   // first block
         const int64_t cl = tree_item(a.W, item, np, kc, nch, at);
         if (cl < 0) continue;
+        if (!SKY && tree_empty(a.geo[cl].c)) continue;
         load_geo(&sm.geo, a.geo + cl);
         const int64_t k0 = cl * TILE;
         int slot[P], place[P];   // slot in the cluster; SKY: ring and azimuth entries

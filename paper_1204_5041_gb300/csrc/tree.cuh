@@ -69,6 +69,12 @@ struct __align__(16) TreeGeo {
     float4 f2;   // e2, 1 / a2
 };
 
+// Near radius of a cluster without pixels (the end of a list whose last entries are no pixel indices): a mark,
+// above every real radius.  Such a cluster has a finite frame that stands for nothing, takes no samples, and its
+// parents leave it out.
+constexpr float kEmptyRadius = 8.f;
+__device__ __forceinline__ bool tree_empty(const float4 &c) { return c.w >= kEmptyRadius; }
+
 // Work of one stage (a level's node sums, or the pixels): clusters with many samples are cut into
 // chunks, listed in the pool; the others are one item each.
 struct TreeWork {
@@ -593,7 +599,9 @@ __global__ void __launch_bounds__(128) k_tree_count(TreeStages g, TreeSamples S,
     const int64_t c = k - g.first[st];
     const bool leaf = st == g.n - 1;
     int64_t v = n;
-    if (leaf || g.pnb[st] != 0 || g.pgeo[st]) {
+    if (g.plane.pitch == 0.f && tree_empty(g.geo[st][c].c)) {
+        v = 0;
+    } else if (leaf || g.pnb[st] != 0 || g.pgeo[st]) {
         float4 self, outer;
         if (g.plane.pitch > 0.f) {
             self = plane_ball(g.plane, g.plane_level[st], c, g.nb[st]);
@@ -830,12 +838,12 @@ __global__ void __launch_bounds__(32 * W * G) k_tree_leaf_geo(const double *__re
                                                               const int64_t *__restrict__ outidx, int order, double theta_pix,
                                                               double kappa, int64_t ncl, TreeGeo *__restrict__ geo)
 {
-    __shared__ float red[G][W][6];
+    __shared__ float red[G][W][7];
     __shared__ TreeGeo gs[G];
     const int tid = threadIdx.x, lane = tid & 31, w = tid / 32 % W, own = tid / (32 * W);
     const int64_t t = blockIdx.x * (int64_t)G + own;
     if (t < ncl) {
-        float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        float s[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         for (int l = 32 * w + lane; l < T * T; l += 32 * W) {
             const int64_t k = t * T * T + l;
             if (outidx[k] < 0) continue;
@@ -849,8 +857,9 @@ __global__ void __launch_bounds__(32 * W * G) k_tree_leaf_geo(const double *__re
                 s[c] += v;
                 s[3 + c] += f * v;
             }
+            s[6] = 1.f;   // has pixels
         }
-        for (int c = 0; c < 6; ++c) {
+        for (int c = 0; c < 7; ++c) {
             s[c] = warp_sum(s[c]);
             if (lane == 0) red[own][w][c] = s[c];
         }
@@ -858,13 +867,15 @@ __global__ void __launch_bounds__(32 * W * G) k_tree_leaf_geo(const double *__re
     __syncthreads();
     const int64_t t1 = blockIdx.x * (int64_t)G + tid;   // the cluster whose frame this thread makes
     const bool maker = tid < G && t1 < ncl;
+    bool empty = false;
     if (maker) {
-        double a[6];
-        for (int c = 0; c < 6; ++c) {
+        double a[7];
+        for (int c = 0; c < 7; ++c) {
             a[c] = 0.0;
             for (int i = 0; i < W; ++i) a[c] += red[tid][i][c];
         }
-        make_frame(a[0], a[1], a[2], a[3], a[4], a[5], gs[tid]);
+        empty = a[6] == 0.0;
+        make_frame(a[0], a[1], empty ? 1.0 : a[2], a[3], a[4], a[5], gs[tid]);
     }
     __syncthreads();
     if (t < ncl) {
@@ -899,7 +910,7 @@ __global__ void __launch_bounds__(32 * W * G) k_tree_leaf_geo(const double *__re
         // margin for the float arithmetic; a single pixel still gets a square of a quarter pixel
         g.a1 = fmax((double)m1 * 1.00001, 0.125 * theta_pix);
         g.a2 = fmax((double)m2 * 1.00001, 0.125 * theta_pix);
-        finish_geo(g, near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7);
+        finish_geo(g, empty ? (double)kEmptyRadius : near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7);
         geo[t1] = g;
     }
 }
@@ -919,7 +930,9 @@ void launch_leaf_geo(const double *nv, int64_t ldn, const int64_t *outidx, int o
 
 // Four lanes per parent cluster (tree_parent of the child level), a lane per child: points of the child's
 // rectangle (corners and edge midpoints).  Offsets from the parent's centre are differences of FP64 centres plus a
-// float offset, so they keep their relative accuracy for small clusters.  With a warp per parent every lane
+// float offset, so they keep their relative accuracy for small clusters.  Children without pixels are left out
+// (a list's invalid entries sort last, so they are the last ones), and a parent of none but those is one itself.
+// With a warp per parent every lane
 // repeated the frame's FP64 work (N_side 1024, five levels: 178 us, so 50 us).
 __global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__ child, int cnb, int64_t cncl,
                                                      TreeGeo *__restrict__ geo, int nb, int64_t ncl, double kappa)
@@ -941,6 +954,7 @@ __global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__
         kid0 = (f * cnb + 2 * by) * cnb + 2 * bx;
     }
     const TreeGeo k = child[has ? kid : kid0];
+    has = has && !tree_empty(k.c);
     const float on = has ? 1.f : 0.f;
     auto sum4 = [](float v) {
         v += __shfl_xor_sync(0xffffffffu, v, 1);
@@ -952,8 +966,9 @@ __global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__
     };
     const float cx = sum4(on * k.c.x), cy = sum4(on * k.c.y), cz = sum4(on * k.c.z);
     const float ux = sum4(on * k.f1.x), uy = sum4(on * k.f1.y), uz = sum4(on * k.f1.z);
+    const bool empty = sum4(on) == 0.f;
     TreeGeo g;
-    make_frame(cx, cy, cz, ux, uy, uz, g);
+    make_frame(cx, cy, empty ? 1.f : cz, ux, uy, uz, g);
     const float d0 = (float)(k.n0[0] - g.n0[0]), d1 = (float)(k.n0[1] - g.n0[1]), d2 = (float)(k.n0[2] - g.n0[2]);
     const float a1 = (float)k.a1, a2 = (float)k.a2;
     const float g1x = (float)g.e1[0], g1y = (float)g.e1[1], g1z = (float)g.e1[2];
@@ -971,11 +986,13 @@ __global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__
         m1 = fmaxf(m1, fabsf(x * g1x + y * g1y + z * g1z) * ps);
         m2 = fmaxf(m2, fabsf(x * g2x + y * g2y + z * g2z) * ps);
     }
-    g.a1 = (double)max4(m1) * 1.002;
-    g.a2 = (double)max4(m2) * 1.002;
+    m1 = max4(has ? m1 : 0.f);
+    m2 = max4(has ? m2 : 0.f);
+    g.a1 = empty ? 1.0 : (double)m1 * 1.002;
+    g.a2 = empty ? 1.0 : (double)m2 * 1.002;
     // near at a child implies near here
-    const float cd = (k.c.w + sqrtf(d0 * d0 + d1 * d1 + d2 * d2)) * 1.00003f + 2e-6f;
-    const double D = fmax(near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7, (double)max4(cd));
+    const float cd = max4(has ? (k.c.w + sqrtf(d0 * d0 + d1 * d1 + d2 * d2)) * 1.00003f + 2e-6f : 0.f);
+    const double D = empty ? (double)kEmptyRadius : fmax(near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7, (double)cd);
     if (c == 0 && p < ncl) {
         finish_geo(g, D);
         geo[p] = g;

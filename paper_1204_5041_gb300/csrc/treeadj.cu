@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(128) k_adj_up(AdjUpArgs a)
                 has = i < a.cnb && j < a.cnb;
                 kid = (f * a.cnb + j) * a.cnb + i;
             }
-            if (has) {
+            if (has && !tree_empty(a.cgeo[kid].c)) {
                 const float *p = reinterpret_cast<const float *>(a.child + kid * kPairs + k / 2) + (k & 1);
                 const TreeGeo &cg = a.cgeo[kid];
                 for (int q3 = 0; q3 < 3; ++q3) d[q3] = p[2 * q3] + (float)(cg.n0[q3] - geo.n0[q3]);
@@ -380,6 +380,7 @@ __global__ void __launch_bounds__(kTreeNT) k_adj_tree(AdjTreeArgs a)
                 const int64_t cl = sm.stack_cl[sp];
                 load_geo(&sm.geo, a.geo[L] + cl);
                 const float4 self = a.geo[L][cl].c;
+                if (tree_empty(self)) continue;
                 bool act = real;
                 if (L < top) {
                     const float4 par = a.geo[L + 1][tree_parent(cl, a.nb[L], a.nb[L + 1])].c;

@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kNN64) k_adj_up64(AdjUp64Args a)
                     has = i < a.cnb && j < a.cnb;
                     kid = (f * a.cnb + j) * a.cnb + i;
                 }
-                if (has) {
+                if (has && !tree_empty(a.cgeo[kid].c)) {
                     const TreeGeo &cg = a.cgeo[kid];
                     node_offset64(cg, k, d);
                     for (int q = 0; q < 3; ++q) d[q] += cg.n0[q] - geo.n0[q];
@@ -353,6 +353,7 @@ __global__ void __launch_bounds__(kTreeNT, 3) k_adj_tree64(AdjTree64Args a)
                     const int L = sm.stack_lv[sp];
                     const int64_t cl = sm.stack_cl[sp];
                     const float4 self = a.geo[L][cl].c;
+                    if (tree_empty(self)) continue;
                     if (!tree_near_pos(ca, self) && !tree_near_beam(cb, self)) {
                         if (lane == 0) {
                             sm.flv[nfar] = L;
