@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_nodes_f32(TreeNodeArgs a)
 #pragma unroll
             for (int i = 0; i < kTreeNT / 16; ++i) v += red[i][tid];
         }
-        if (!ROOT && kc == 0) {   // the parent's interpolant at this cluster's nodes
+        if (!ROOT && kc == 0 && !tree_wide(parent)) {   // the parent's interpolant at this cluster's nodes
             cheb_coefs<kNP>(a.Fp, a.Wp, pcl, sm.coef, sm.tmp);
             float *cf = reinterpret_cast<float *>(sm.rec + kTreeNT / 16 * kNN / 2);
             coefs_to_float(sm.coef, cf);
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kTreeNT, 4) k_tree_pixels_f32(TreePixArgs a)
                 mm[pp] = f2_fma(m[pp][2], m[pp][2], f2_fma(m[pp][1], m[pp][1], f2_mul(m[pp][0], m[pp][0])));
         }
         double far[2] = {0.0, 0.0};   // of the lane's pixels 2 half and 2 half + 1
-        if (kc == 0) {
+        if (kc == 0 && !tree_wide(self)) {
             cheb_coefs<kNP>(a.F, a.Wf, cl, sm.coef, sm.tmp);
             float *cf = reinterpret_cast<float *>(sm.rec);
             coefs_to_float(sm.coef, cf);
@@ -738,7 +738,7 @@ __global__ void __launch_bounds__(kTreeNT) k_tree_nodes_f64(TreeNodeArgs64 A)
         };
         tree_scan<ROOT, false>(a.S, kc, nch, self, parent, 0.f, 0.f, 0.f, sm.scan,
                                [&](int count) { tree_batches64(sm, count, stage, eval); });
-        if (!ROOT && kc == 0) {
+        if (!ROOT && kc == 0 && !tree_wide(parent)) {
             double rhi, rlo;
             cheb_coefs64(a.Fp, a.Wp, pcl, sm.coef, sm.tmp, rhi, rlo);
 #pragma unroll
@@ -1073,12 +1073,13 @@ __global__ void __launch_bounds__(kTreeNT, 3) k_tree_pixels_f64(TreePixArgs64 A)
             });
         });
         double rhi = 0.0, rlo = 0.0;
-        if (kc == 0) cheb_coefs64(a.F, a.Wf, cl, sm.coef, sm.tmp, rhi, rlo);
+        const bool inner = kc == 0 && !tree_wide(self);
+        if (inner) cheb_coefs64(a.F, a.Wf, cl, sm.coef, sm.tmp, rhi, rlo);
 #pragma unroll
         for (int q = 0; q < P; ++q) {
             if (q / 2 < pb || q / 2 >= pb + per) continue;
             const int64_t k = k0 + slot[q];
-            if (kc == 0 && live >> q / 2 & 1u) {
+            if (inner && live >> q / 2 & 1u) {
                 double x, y;
                 local_xy64(sm.geo, a.nv[k] - sm.geo.n0[0], a.nv[a.ldn + k] - sm.geo.n0[1], a.nv[2 * a.ldn + k] - sm.geo.n0[2], x, y);
                 fold64(hi[q], lo[q], rhi);

@@ -69,6 +69,12 @@ struct __align__(16) TreeGeo {
     float4 f2;   // e2, 1 / a2
 };
 
+// Near radius of a cluster wider than a hemisphere (stereographic half-size above 1; scattered pixels of a short
+// list): above every chord, so all samples are near to it, and its interpolant is not used.  Its frame and
+// extents stand for nothing: its mean direction may be zero, a pixel may be the centre's antipode, where the
+// coordinates are infinite.
+constexpr float kWideRadius = 4.f;
+__device__ __forceinline__ bool tree_wide(const float4 &c) { return c.w >= kWideRadius; }
 // Near radius of a cluster without pixels (the end of a list whose last entries are no pixel indices): a mark,
 // above every real radius.  Such a cluster has a finite frame that stands for nothing, takes no samples, and its
 // parents leave it out.
@@ -792,7 +798,9 @@ __global__ void __launch_bounds__(256) k_tree_vcrit(const TreeCrit *__restrict__
 __device__ __forceinline__ void make_frame(double cx, double cy, double cz, double tx, double ty, double tz,
                                            TreeGeo &g)
 {
-    const double r = 1.0 / sqrt(cx * cx + cy * cy + cz * cz);
+    const double c2 = cx * cx + cy * cy + cz * cz;
+    if (!(c2 > 0.0)) cx = cy = 0.0, cz = 1.0;   // no mean direction: any will do
+    const double r = c2 > 0.0 ? 1.0 / sqrt(c2) : 1.0;
     g.n0[0] = cx * r;
     g.n0[1] = cy * r;
     g.n0[2] = cz * r;
@@ -819,9 +827,19 @@ __device__ __forceinline__ void make_frame(double cx, double cy, double cz, doub
     g.e2[2] = g.n0[0] * g.e1[1] - g.n0[1] * g.e1[0];
 }
 
-// the float copies of a finished geometry, with the near radius D
-__device__ __forceinline__ void finish_geo(TreeGeo &g, double D)
+// A direction at angle theta from the centre has 2 - d^2 / 2 = 1 + cos(theta); the corners of a rectangle of
+// half-sizes 1 have 2/3.
+constexpr float kWideDen = 0.6f, kWideExtent = 1e3f;
+
+// the float copies of a finished geometry, with the near radius D or the marks
+__device__ __forceinline__ void finish_geo(TreeGeo &g, double D, bool empty)
 {
+    if (empty) {
+        D = kEmptyRadius;
+    } else if (!(fmax(g.a1, g.a2) <= 1.0) || !(D < kWideRadius)) {
+        D = kWideRadius;
+        g.a1 = g.a2 = kWideExtent;
+    }
     g.pad = 0.0;
     g.c = make_float4((float)g.n0[0], (float)g.n0[1], (float)g.n0[2], (float)D);
     g.l = make_float4((float)(g.n0[0] - (double)g.c.x), (float)(g.n0[1] - (double)g.c.y),
@@ -875,7 +893,7 @@ __global__ void __launch_bounds__(32 * W * G) k_tree_leaf_geo(const double *__re
             for (int i = 0; i < W; ++i) a[c] += red[tid][i][c];
         }
         empty = a[6] == 0.0;
-        make_frame(a[0], a[1], empty ? 1.0 : a[2], a[3], a[4], a[5], gs[tid]);
+        make_frame(a[0], a[1], a[2], a[3], a[4], a[5], gs[tid]);
     }
     __syncthreads();
     if (t < ncl) {
@@ -888,9 +906,10 @@ __global__ void __launch_bounds__(32 * W * G) k_tree_leaf_geo(const double *__re
             if (outidx[k] < 0) continue;
             const float dx = trunc_float(nv[k] - g.n0[0]), dy = trunc_float(nv[ldn + k] - g.n0[1]),
                         dz = trunc_float(nv[2 * ldn + k] - g.n0[2]);
-            const float s = 1.f / (2.f - 0.5f * (dx * dx + dy * dy + dz * dz));
+            const float den = 2.f - 0.5f * (dx * dx + dy * dy + dz * dz), s = 1.f / den;
             m1 = fmaxf(m1, fabsf(dx * e1x + dy * e1y + dz * e1z) * s);
             m2 = fmaxf(m2, fabsf(dx * e2x + dy * e2y + dz * e2z) * s);
+            if (!(den > kWideDen)) m1 = kWideExtent;
         }
         m1 = warp_max(m1);
         m2 = warp_max(m2);
@@ -910,7 +929,7 @@ __global__ void __launch_bounds__(32 * W * G) k_tree_leaf_geo(const double *__re
         // margin for the float arithmetic; a single pixel still gets a square of a quarter pixel
         g.a1 = fmax((double)m1 * 1.00001, 0.125 * theta_pix);
         g.a2 = fmax((double)m2 * 1.00001, 0.125 * theta_pix);
-        finish_geo(g, empty ? (double)kEmptyRadius : near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7);
+        finish_geo(g, near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7, empty);
         geo[t1] = g;
     }
 }
@@ -968,7 +987,7 @@ __global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__
     const float ux = sum4(on * k.f1.x), uy = sum4(on * k.f1.y), uz = sum4(on * k.f1.z);
     const bool empty = sum4(on) == 0.f;
     TreeGeo g;
-    make_frame(cx, cy, empty ? 1.f : cz, ux, uy, uz, g);
+    make_frame(cx, cy, cz, ux, uy, uz, g);
     const float d0 = (float)(k.n0[0] - g.n0[0]), d1 = (float)(k.n0[1] - g.n0[1]), d2 = (float)(k.n0[2] - g.n0[2]);
     const float a1 = (float)k.a1, a2 = (float)k.a2;
     const float g1x = (float)g.e1[0], g1y = (float)g.e1[1], g1z = (float)g.e1[2];
@@ -982,9 +1001,10 @@ __global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__
         const float x = d0 + s * (xi * k.f1.x + eta * k.f2.x - r2 * k.c.x);
         const float y = d1 + s * (xi * k.f1.y + eta * k.f2.y - r2 * k.c.y);
         const float z = d2 + s * (xi * k.f1.z + eta * k.f2.z - r2 * k.c.z);
-        const float ps = 1.f / (2.f - 0.5f * (x * x + y * y + z * z));
+        const float den = 2.f - 0.5f * (x * x + y * y + z * z), ps = 1.f / den;
         m1 = fmaxf(m1, fabsf(x * g1x + y * g1y + z * g1z) * ps);
         m2 = fmaxf(m2, fabsf(x * g2x + y * g2y + z * g2z) * ps);
+        if (!(den > kWideDen)) m1 = kWideExtent;
     }
     m1 = max4(has ? m1 : 0.f);
     m2 = max4(has ? m2 : 0.f);
@@ -992,9 +1012,9 @@ __global__ void __launch_bounds__(128) k_tree_up_geo(const TreeGeo *__restrict__
     g.a2 = empty ? 1.0 : (double)m2 * 1.002;
     // near at a child implies near here
     const float cd = max4(has ? (k.c.w + sqrtf(d0 * d0 + d1 * d1 + d2 * d2)) * 1.00003f + 2e-6f : 0.f);
-    const double D = empty ? (double)kEmptyRadius : fmax(near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7, (double)cd);
+    const double D = fmax(near_radius(kappa, fmax(g.a1, g.a2)) * 1.00001 + 1e-7, (double)cd);
     if (c == 0 && p < ncl) {
-        finish_geo(g, D);
+        finish_geo(g, D, empty);
         geo[p] = g;
     }
 }

@@ -1,5 +1,5 @@
 """Lists and ranges of pixels over the cluster tree where a cluster is out of the ordinary: leaves without
-one valid pixel (indices out of range sort last).  The tolerances are those of test_gpu_tree.py, whose direct
+one valid pixel (indices out of range sort last), and leaves wider than a hemisphere.  The tolerances are those of test_gpu_tree.py, whose direct
 kernels are the reference."""
 import numpy as np
 import pytest
@@ -55,3 +55,43 @@ def test_adjoint_list_with_empty_leaves(isw, prec, tol, good, bad):  # noqa: F81
     for a in (0, 3, 6):
         assert ((got - ref)[a : a + 3].abs().max() / ref[a : a + 3].abs().max()).item() <= tol
     ctx.check_status()
+
+
+@pytest.mark.parametrize("nside", [49, 51, 52, 58, 59, 61, 62, 63])
+def test_map_equator_ring(isw, nside):  # noqa: F811
+    """One leaf around the whole equator: its mean direction is zero (49 to 58) or the rounding of its sum, with
+    a pixel at the antipode of the centre for odd N_side."""
+    S = torch.from_numpy(_samples(int(3.001e8 / (4 * nside)) + 1, nside)).cuda()
+    ring = dict(pix0=2 * nside * (nside - 1) + 4 * nside * nside, npix=4 * nside)
+    got, ref = isw.isw_map(nside, S, **ring), _direct(isw, nside, S, **ring)
+    assert ((got - ref).abs().max() / ref.square().mean().sqrt()).item() <= TOL32
+    assert isw.default_context().check_status()[0] == isw.OK
+
+
+def _antipodes(isw, nside, count, seed):  # noqa: F811
+    p = torch.randint(12 * nside * nside, (count // 2,), device="cuda", generator=torch.Generator("cuda").manual_seed(seed))
+    return torch.cat([p, isw.hp_vec2pix_ring(nside, -isw.hp_pix2vec_ring(nside, pix=p))])
+
+
+@pytest.mark.parametrize("prec,tol,count", [("f32c", TOL32, 192), ("f32c", TOL32, 260), ("f32c", TOL32, 1000), ("f64", TOL64, 4096),
+                                            ("f64", TOL64, 4100)])
+def test_map_antipodal_pairs(isw, prec, tol, count):  # noqa: F811
+    """Scattered pixels with their antipodes in few leaves; and the N_side 2 sky repeated."""
+    S = torch.from_numpy(_samples(int((3.001e8 if prec == "f32c" else 6.001e7) / count) + 1, 21)).cuda()
+    sky2 = torch.arange(48, device="cuda").repeat(count // 48 + 1)[:count]
+    for nside, pix in ((64, _antipodes(isw, 64, count, count)), (2, sky2)):
+        got, ref = isw.isw_map(nside, S, pix=pix, prec=prec), _direct(isw, nside, S, pix=pix)
+        assert ((got - ref).abs().max() / ref.square().mean().sqrt()).item() <= tol
+    assert isw.default_context().check_status()[0] == isw.OK
+
+
+@pytest.mark.parametrize("prec,tol,count", [("f32c", 1e-6, 12288), ("f64", 1e-12, 12288)])
+def test_adjoint_antipodal_pairs(isw, prec, tol, count):  # noqa: F811
+    S = torch.from_numpy(_samples(int((3.01e8 if prec == "f32c" else 6.1e6) / count) + 1, 22)).cuda()
+    g = torch.randn(count, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    for nside, pix in ((64, _antipodes(isw, 64, count, 2)), (2, torch.arange(48, device="cuda").repeat(count // 48))):
+        got = _adjoint(isw, nside, S, g, prec, 9, pix=pix)
+        ref = _adjoint(isw, nside, S, g, "f64", 9, split=1, pix=pix)
+        for a in (0, 3, 6):
+            assert ((got - ref)[a : a + 3].abs().max() / ref[a : a + 3].abs().max()).item() <= tol
+    assert isw.default_context().check_status()[0] == isw.OK
