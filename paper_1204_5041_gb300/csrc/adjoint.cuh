@@ -7,6 +7,8 @@
 namespace isw {
 
 constexpr int kAcc = 13;
+// sums in use: those after the tenth are for dL/dX'
+__host__ __device__ constexpr int adj_rows(bool ng9) { return ng9 ? kAcc : 10; }
 
 // Per-pair derivative sums.  With d = n - Xhat, Q = d.d, u = Xdot - (A/B) X', T = u.d / Q and
 // eta = 2T/Q, the n-dependent parts of the three gradients are accumulated as vectors along d

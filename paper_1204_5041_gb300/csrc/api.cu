@@ -77,10 +77,19 @@ int ensure_ws(isw_ctx *c, int slot, size_t bytes)
     cudaError_t e = cudaMalloc(&c->ws[slot], grown);
     if (e != cudaSuccess) {
         c->ws[slot] = nullptr;
+        cudaGetLastError();   // no launch of a later call is to report it
         return cuda_err(c, e, "cudaMalloc(workspace)");
     }
     c->ws_size[slot] = grown;
     return ISW_OK;
+}
+
+void release_ws(isw_ctx *c, int slot)
+{
+    drop_graph(c);
+    if (c->ws[slot]) cudaFree(c->ws[slot]);
+    c->ws[slot] = nullptr;
+    c->ws_size[slot] = 0;
 }
 
 int set_device(isw_ctx *c)
@@ -202,24 +211,40 @@ bool use_tree(const isw_ctx *c, TreeUse use, int64_t npix, int64_t n, int prec)
            npix < (int64_t(1) << 32);
 }
 
+// A tree call asks for its workspace before it launches anything.  Where the device has no room for it the direct
+// kernels run, whose workspace differs and grows less with the samples (the FP32 adjoint's partial sums), so that
+// nothing they can hold is refused; a capture takes the path of the call before it, which has sized the buffers.
+// r: the failed request's error.
+bool no_room(isw_ctx *c, int r)
+{
+    if (c->capturing) return true;
+    if (r != ISW_ENOMEM) return false;
+    release_ws(c, kWsTree);
+    release_ws(c, kWsSort);
+    return true;
+}
+
 // isw_map over the cluster tree: a full sky, a patch (M x M, one face), or a list or range of pixels in
-// spatial order.
+// spatial order.  direct: nothing was launched (no_room).
 int map_tree_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_t *pix_list,
                   const PatchSpec *patch, const double *samples, int64_t n, int64_t ld, const double xo[3], double GU,
-                  int prec, int accumulate, double *theta, cudaStream_t s)
+                  int prec, int accumulate, double *theta, cudaStream_t s, bool &direct)
 {
     const bool full = !patch && !pix_list && pix0 == 0 && npix == 12 * nside * nside, list = !patch && !full;
     const TreePlan p = tree_plan(prec, patch ? patch->M : nside, patch ? 1 : (full ? 12 : 0), npix, n, c->num_sms);
     const int64_t tot = p.ncl[0] * p.leaf * p.leaf;
     const size_t sort_bytes = (sort_scratch_bytes(n, 2) + 255) / 256 * 256;
-    int r;
-    if ((r = ensure_ws(c, kWsNv, (size_t)tot * 3 * sizeof(double)))) return r;
-    if ((r = ensure_ws(c, kWsOut, (size_t)tot * sizeof(int64_t)))) return r;
-    if ((r = ensure_ws(c, kWsS32, (size_t)p.n_pad * sizeof(Seg32)))) return r;
-    if ((r = ensure_ws(c, kWsS64, (size_t)p.n_pad * sizeof(Seg64)))) return r;
-    if (prec == ISW_F64 && (r = ensure_ws(c, kWsFar64, (size_t)p.n_pad * sizeof(Far64)))) return r;
-    if ((r = ensure_ws(c, kWsSort, sort_bytes + (list ? sort_scratch_bytes(npix, 1) : 0)))) return r;
-    if ((r = ensure_ws(c, kWsTree, p.bytes))) return r;
+    int r = ensure_ws(c, kWsNv, (size_t)tot * 3 * sizeof(double));
+    if (!r) r = ensure_ws(c, kWsOut, (size_t)tot * sizeof(int64_t));
+    if (!r) r = ensure_ws(c, kWsS32, (size_t)p.n_pad * sizeof(Seg32));
+    if (!r) r = ensure_ws(c, kWsS64, (size_t)p.n_pad * sizeof(Seg64));
+    if (!r && prec == ISW_F64) r = ensure_ws(c, kWsFar64, (size_t)p.n_pad * sizeof(Far64));
+    if (!r) r = ensure_ws(c, kWsSort, sort_bytes + (list ? sort_scratch_bytes(npix, 1) : 0));
+    if (!r) r = ensure_ws(c, kWsTree, p.bytes);
+    if (r) {
+        direct = no_room(c, r);
+        return r;
+    }
     TreeMapArgs m{};
     m.theta_pix = patch ? patch->width / (double)patch->M : std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
     double *nv = (double *)c->ws[kWsNv];
@@ -269,6 +294,64 @@ int map_tree_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const i
     return check_launch(c, "isw_map launch");
 }
 
+// isw_map_adjoint over the cluster tree.  direct: nothing was launched (no_room).
+int adjoint_tree_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_t *pix_list, const double *samples,
+                      int64_t n, int64_t ld, const double xo[3], double GU, int prec, const double *dL_dtheta,
+                      double *grad_out, int64_t ld_g, int ngrad, cudaStream_t s, bool &direct)
+{
+    const bool f64 = prec == ISW_F64;
+    const int orders = f64 ? 1 : 2;
+    const bool full = !pix_list && pix0 == 0 && npix == 12 * nside * nside;
+    const AdjTreePlan p = (f64 ? adj_tree_plan64 : adj_tree_plan)(nside, full ? 12 : 0, npix, n, ngrad, c->num_sms);
+    const int64_t tot = p.map.ncl[0] * p.map.leaf * p.map.leaf;
+    const size_t sort_bytes = (sort_scratch_bytes(n, orders) + 255) / 256 * 256;
+    int r = ensure_ws(c, kWsNv, (size_t)tot * 3 * sizeof(double));
+    if (!r) r = ensure_ws(c, kWsOut, (size_t)tot * sizeof(int64_t));
+    if (!r) r = ensure_ws(c, kWsS32, (size_t)p.n_pad * sizeof(Seg32));
+    if (!r) r = ensure_ws(c, kWsS64, (size_t)p.n_pad * sizeof(Seg64));
+    if (!r) r = ensure_ws(c, kWsSort, sort_bytes + (full ? 0 : sort_scratch_bytes(npix, 1)));
+    if (!r) r = ensure_ws(c, kWsTree, p.bytes);
+    if (r) {
+        direct = no_room(c, r);
+        return r;
+    }
+    double *nv = (double *)c->ws[kWsNv];
+    int64_t *outidx = (int64_t *)c->ws[kWsOut];
+    Seg32 *s32 = (Seg32 *)c->ws[kWsS32];
+    Seg64 *s64 = (Seg64 *)c->ws[kWsS64];
+    unsigned char *sort = (unsigned char *)c->ws[kWsSort];
+    const uint32_t *pp = full ? nullptr : launch_pixel_order(nside, pix0, npix, pix_list, sort + sort_bytes, s);
+    launch_pixel_table(nside, full ? 0 : (pix_list ? 2 : 1), pix0, npix, pix_list, p.map.leaf, p.map.leaf, p.map.ncl[0],
+                       nv, tot, outidx, nullptr, c->d_status, s, pp);
+    AdjTreeCall m{};
+    m.theta_pix = std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
+    m.perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], sort, orders, s);
+    launch_pack(samples, n, ld, xo[0], xo[1], xo[2], GU, m.theta_pix, c->near_k, p.n_pad, m.perm, s32, s64, nullptr,
+                nullptr, nullptr, c->d_status, s);
+    m.nv = nv;
+    m.ldn = tot;
+    m.outidx = outidx;
+    m.order = full ? kSlotsDiag : kSlotsList;
+    m.g = dL_dtheta;
+    m.s32 = s32;
+    m.s64 = s64;
+    m.n = n;
+    m.b_min = (float)c->b_min;
+    m.d_far = (float)c->d_far;
+    m.ngrad = ngrad;
+    m.grad = grad_out;
+    m.ld_g = ld_g;
+    m.st = c->d_status;
+    m.scratch = c->ws[kWsTree];
+    const int ti = timing_begin(c, s);
+    cudaError_t e = f64 ? launch_adjoint_tree64(p, m, s) : launch_adjoint_tree(p, m, s);
+    if (e != cudaSuccess) return cuda_err(c, e, "isw_map_adjoint launch");
+    timing_end(c, ti, s);
+    c->n_pair += 1;
+    c->n_launch += spatial_order_launches() * (full ? 1 : 2) + 2 + adj_tree_launches(p);
+    return check_launch(c, "isw_map_adjoint launch");
+}
+
 // Shared body of isw_map: pixel table, sample records, caps, map kernel, partial reduce.
 int map_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_t *pix_list, const double *samples,
              int64_t n, int64_t ld, const double *x_obs, double GU, int prec, int accumulate, double *theta,
@@ -284,8 +367,11 @@ int map_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_
         return ISW_OK;
     }
     const TreeUse use = patch ? kTreePatch : !pix_list && pix0 == 0 && npix == 12 * nside * nside ? kTreeSky : kTreePixelList;
-    if (tune_waves == 0 && use_tree(c, use, npix, n, prec))
-        return map_tree_impl(c, nside, pix0, npix, pix_list, patch, samples, n, ld, xo, GU, prec, accumulate, theta, s);
+    if (tune_waves == 0 && use_tree(c, use, npix, n, prec)) {
+        bool direct = false;
+        const int r = map_tree_impl(c, nside, pix0, npix, pix_list, patch, samples, n, ld, xo, GU, prec, accumulate, theta, s, direct);
+        if (!direct) return r;
+    }
     int vidx = 0;
     if (prec == ISW_F32C) {
         if (c->tile_override >= 0 && c->tile_override < num_f32_variants()) vidx = c->tile_override;
@@ -857,19 +943,22 @@ int isw_map_patch(isw_ctx *c, const double *frame, int64_t M, double width, cons
     const bool f64 = prec == ISW_F64;
     if (default_kernels(c) && flat_tree_rule(M, n)) {
         const FlatTreePlan tp = flat_tree_plan(f64, M, n, c->num_sms);
-        if ((r = ensure_ws(c, kWsFlat, (size_t)tp.n_pad * flat_record_bytes()))) return r;
-        if ((r = ensure_ws(c, kWsTree, tp.bytes))) return r;
-        unsigned char *rec = (unsigned char *)c->ws[kWsFlat];
-        void *r32 = rec, *r64 = rec + (size_t)tp.n_pad * (flat_record_bytes() / 2);
-        const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
-        launch_flat_pack(samples, n, ld, p, xo[0], xo[1], xo[2], GU, tp.n_pad, r32, r64, s);
-        const int ti = timing_begin(c, s);
-        cudaError_t e = launch_map_flat_tree(tp, r32, r64, n, M, width, theta_out, accumulate, c->ws[kWsTree], s);
-        if (e != cudaSuccess) return cuda_err(c, e, "isw_map_patch launch");
-        timing_end(c, ti, s);
-        c->n_launch += 1 + flat_tree_launches(tp);
-        c->n_pair += 1;
-        return check_launch(c, "isw_map_patch launch");
+        r = ensure_ws(c, kWsFlat, (size_t)tp.n_pad * flat_record_bytes());
+        if (!r) r = ensure_ws(c, kWsTree, tp.bytes);
+        if (r && !no_room(c, r)) return r;
+        if (!r) {
+            unsigned char *rec = (unsigned char *)c->ws[kWsFlat];
+            void *r32 = rec, *r64 = rec + (size_t)tp.n_pad * (flat_record_bytes() / 2);
+            const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
+            launch_flat_pack(samples, n, ld, p, xo[0], xo[1], xo[2], GU, tp.n_pad, r32, r64, s);
+            const int ti = timing_begin(c, s);
+            cudaError_t e = launch_map_flat_tree(tp, r32, r64, n, M, width, theta_out, accumulate, c->ws[kWsTree], s);
+            if (e != cudaSuccess) return cuda_err(c, e, "isw_map_patch launch");
+            timing_end(c, ti, s);
+            c->n_launch += 1 + flat_tree_launches(tp);
+            c->n_pair += 1;
+            return check_launch(c, "isw_map_patch launch");
+        }
     }
     const int S = flat_seg_tile(), tx = flat_tx(), ty = flat_ty();
     const int64_t ntiles = ((M + tx - 1) / tx) * ((M + ty - 1) / ty), tot = ntiles * tx * ty;
@@ -978,53 +1067,9 @@ int isw_map_adjoint(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const
     }
     const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
     if (default_kernels(c) && tree_rule(prec, kTreeAdjoint, npix, n) && npix < (int64_t(1) << 32)) {
-        const bool f64 = prec == ISW_F64;
-        const int orders = f64 ? 1 : 2;
-        const bool full = !pix_list && pix0 == 0 && npix == 12 * nside * nside;
-        const AdjTreePlan p = (f64 ? adj_tree_plan64 : adj_tree_plan)(nside, full ? 12 : 0, npix, n, c->num_sms);
-        const int64_t tot = p.map.ncl[0] * p.map.leaf * p.map.leaf;
-        const size_t sort_bytes = (sort_scratch_bytes(n, orders) + 255) / 256 * 256;
-        if ((r = ensure_ws(c, kWsNv, (size_t)tot * 3 * sizeof(double)))) return r;
-        if ((r = ensure_ws(c, kWsOut, (size_t)tot * sizeof(int64_t)))) return r;
-        if ((r = ensure_ws(c, kWsS32, (size_t)p.n_pad * sizeof(Seg32)))) return r;
-        if ((r = ensure_ws(c, kWsS64, (size_t)p.n_pad * sizeof(Seg64)))) return r;
-        if ((r = ensure_ws(c, kWsSort, sort_bytes + (full ? 0 : sort_scratch_bytes(npix, 1))))) return r;
-        if ((r = ensure_ws(c, kWsTree, p.bytes))) return r;
-        double *nv = (double *)c->ws[kWsNv];
-        int64_t *outidx = (int64_t *)c->ws[kWsOut];
-        Seg32 *s32 = (Seg32 *)c->ws[kWsS32];
-        Seg64 *s64 = (Seg64 *)c->ws[kWsS64];
-        unsigned char *sort = (unsigned char *)c->ws[kWsSort];
-        const uint32_t *pp = full ? nullptr : launch_pixel_order(nside, pix0, npix, pix_list, sort + sort_bytes, s);
-        launch_pixel_table(nside, full ? 0 : (pix_list ? 2 : 1), pix0, npix, pix_list, p.map.leaf, p.map.leaf, p.map.ncl[0],
-                           nv, tot, outidx, nullptr, c->d_status, s, pp);
-        AdjTreeCall m{};
-        m.theta_pix = std::sqrt(4.0 * M_PI / (12.0 * (double)nside * (double)nside));
-        m.perm = launch_spatial_order(samples, n, ld, xo[0], xo[1], xo[2], sort, orders, s);
-        launch_pack(samples, n, ld, xo[0], xo[1], xo[2], GU, m.theta_pix, c->near_k, p.n_pad, m.perm, s32, s64, nullptr,
-                    nullptr, nullptr, c->d_status, s);
-        m.nv = nv;
-        m.ldn = tot;
-        m.outidx = outidx;
-        m.order = full ? kSlotsDiag : kSlotsList;
-        m.g = dL_dtheta;
-        m.s32 = s32;
-        m.s64 = s64;
-        m.n = n;
-        m.b_min = (float)c->b_min;
-        m.d_far = (float)c->d_far;
-        m.ngrad = ngrad;
-        m.grad = grad_out;
-        m.ld_g = ld_g;
-        m.st = c->d_status;
-        m.scratch = c->ws[kWsTree];
-        const int ti = timing_begin(c, s);
-        cudaError_t e = f64 ? launch_adjoint_tree64(p, m, s) : launch_adjoint_tree(p, m, s);
-        if (e != cudaSuccess) return cuda_err(c, e, "isw_map_adjoint launch");
-        timing_end(c, ti, s);
-        c->n_pair += 1;
-        c->n_launch += spatial_order_launches() * (full ? 1 : 2) + 2 + adj_tree_launches(p);
-        return check_launch(c, "isw_map_adjoint launch");
+        bool direct = false;
+        r = adjoint_tree_impl(c, nside, pix0, npix, pix_list, samples, n, ld, xo, GU, prec, dL_dtheta, grad_out, ld_g, ngrad, s, direct);
+        if (!direct) return r;
     }
     const int NT = adj_seg_tile(prec), TP = adj_pix_tile(prec);
     const Variant pv{0, 0, 0, 32, TP / 32};

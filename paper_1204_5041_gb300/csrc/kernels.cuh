@@ -229,7 +229,7 @@ inline int flat_tree_launches(const FlatTreePlan &p) { return p.levels + 17; }
 struct AdjTreePlan {
     TreePlan map;                         // levels and clusters
     int64_t n_pad;
-    int slots, parts;                     // resident CTAs; shares of the root clusters (FP64)
+    int slots, parts;                     // resident CTAs; shares of the root clusters
     size_t off_queue, off_crit, off_vcrit, off_caps, off_vidx, off_inv, off_rec, off_pix, off_low, off_partial, bytes;
     size_t off_geo[kTreeLevels], off_node[kTreeLevels];
 };
@@ -251,9 +251,9 @@ struct AdjTreeCall {
     DevStatus *st;
     void *scratch;
 };
-AdjTreePlan adj_tree_plan64(int64_t N, int nface, int64_t npix, int64_t n, int num_sms);
+AdjTreePlan adj_tree_plan64(int64_t N, int nface, int64_t npix, int64_t n, int ngrad, int num_sms);
 cudaError_t launch_adjoint_tree64(const AdjTreePlan &p, const AdjTreeCall &m, cudaStream_t s);
-AdjTreePlan adj_tree_plan(int64_t N, int nface, int64_t npix, int64_t n, int num_sms);
+AdjTreePlan adj_tree_plan(int64_t N, int nface, int64_t npix, int64_t n, int ngrad, int num_sms);
 cudaError_t launch_adjoint_tree(const AdjTreePlan &p, const AdjTreeCall &m, cudaStream_t s);
 inline int adj_tree_launches(const AdjTreePlan &p) { return 2 * p.map.levels + (p.map.prec == ISW_F64 ? 3 : 5); }
 

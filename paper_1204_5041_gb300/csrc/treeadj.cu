@@ -10,18 +10,20 @@
 // A CTA holds 128 samples that are neighbours, so that its threads agree on near and far: in position order
 // for clusters near by position (and the roots), in velocity order for those near by beam only (a string's
 // samples beam in many directions: in position order a third of the clusters would be visited for one or
-// two lanes each).  The subtrees of the roots are dealt to kAdjParts items per CTA of samples, with
+// two lanes each).  The subtrees of the roots are dealt to up to kAdjParts items per CTA of samples, with
 // separate partial sums.
 // Bound by the FP32 sums of these pairs (40 operations each).  N_side 256, 50,176 samples: per sample ~1e4
 // nodes and pixels instead of 786,432 pixels, 4.1 ms against 43.7 ms pair by pair.
 #include "adjoint.cuh"
 #include "tree.cuh"
 
+#include <algorithm>
+
 namespace isw {
 
 namespace {
 
-constexpr int kAdjParts = 8, kSums = 13;
+constexpr int kAdjParts = 8, kSums = kAcc;   // most shares of the root clusters
 // Near radius in half-sizes: a sample's own gradient sees the truncation that the map averages over
 // samples.  Median error of dL/dXdot per sample against FP64: 1.7e-7 at 3.5, 1.4e-7 at 4 (direct kernel
 // 1.4e-7); 3.9 ms at 3.5, 4.3 ms at 4.
@@ -172,7 +174,8 @@ struct AdjTreeArgs {
     int64_t ldn;
     const int64_t *outidx;
     int64_t n_pad;                 // samples, padded to the tiles of 128
-    double *partial;               // [2][kAdjParts][13][n_pad]
+    int parts;
+    double *partial;               // [2][parts][adj_rows][n_pad]
     float b_min;
     DevStatus *st;
     unsigned long long *queue;
@@ -297,16 +300,16 @@ __global__ void __launch_bounds__(kTreeNT) k_adj_tree(AdjTreeArgs a)
     AdjSmem &sm = *reinterpret_cast<AdjSmem *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     AdjQueue &nq = sm.q[w];
-    const int64_t ntile = a.n_pad / kTreeNT, n_items = 2 * ntile * kAdjParts;
+    const int64_t ntile = a.n_pad / kTreeNT, n_items = 2 * ntile * a.parts;
     const int top = a.levels - 1;
     const uint64_t half2 = f2_pack(0.5f, 0.5f);
     const float b_tiny = a.b_min * 1e-3f;
     unsigned nearcnt = 0, zerocnt = 0;
     TreeQueue queue{a.queue, 0ull};
     for (int64_t item = queue.first(&sm.item); item < n_items; item = queue.next(&sm.item)) {
-        const int pass = (int)(item / (ntile * kAdjParts));
-        const int64_t tile = item / kAdjParts % ntile;
-        const int part = (int)(item % kAdjParts);
+        const int pass = (int)(item / (ntile * a.parts));
+        const int64_t tile = item / a.parts % ntile;
+        const int part = (int)(item % a.parts);
         const int64_t idx = tile * kTreeNT + tid;
         const uint32_t src = pass ? a.vidx[idx] : (uint32_t)idx;
         const float4 ca = (pass ? a.vcrit : a.crit)[idx].a, cb = (pass ? a.vcrit : a.crit)[idx].b;
@@ -365,7 +368,7 @@ __global__ void __launch_bounds__(kTreeNT) k_adj_tree(AdjTreeArgs a)
             r.B0 = dup2(B0);
             r.f = dup2(q[1].w);
         };
-        for (int64_t root = part; root < a.ncl[top]; root += kAdjParts) {
+        for (int64_t root = part; root < a.ncl[top]; root += a.parts) {
             int sp = 0;
             __syncthreads();
             if (tid == 0) {
@@ -570,8 +573,8 @@ __global__ void __launch_bounds__(kTreeNT) k_adj_tree(AdjTreeArgs a)
         }
         __syncwarp();
 #pragma unroll
-        for (int k = 0; k < kSums; ++k)
-            a.partial[((int64_t)(pass * kAdjParts + part) * kSums + k) * a.n_pad + idx] =
+        for (int k = 0; k < adj_rows(NG9); ++k)
+            a.partial[((int64_t)(pass * a.parts + part) * adj_rows(NG9) + k) * a.n_pad + idx] =
                 ((double)ahi[k] + (double)alo[k]) + sm.acc64[k][tid];
         __syncthreads();
     }
@@ -594,7 +597,7 @@ __global__ void k_adj_vpos(const uint32_t *__restrict__ vidx, int64_t n, uint32_
 
 // One thread per record: its sums over passes and parts in order, then the gradient rows at the sample's
 // place in the input.
-__global__ void __launch_bounds__(128) k_adj_finish(const double *__restrict__ partial, int64_t n, int64_t n_pad,
+__global__ void __launch_bounds__(128) k_adj_finish(const double *__restrict__ partial, int parts, int64_t n, int64_t n_pad,
                                                     const uint32_t *__restrict__ vpos, const uint32_t *__restrict__ perm,
                                                     const Seg64 *__restrict__ s64, int ngrad, double *__restrict__ grad,
                                                     int64_t ld)
@@ -603,13 +606,13 @@ __global__ void __launch_bounds__(128) k_adj_finish(const double *__restrict__ p
     if (s >= n) return;
     double acc[kSums];
     const int64_t vp = vpos[s];
-    const int nk = ngrad >= 9 ? kSums : 10;
+    const int nk = adj_rows(ngrad >= 9);
 #pragma unroll
     for (int k = 0; k < kSums; ++k) {
         double hi = 0.0, lo = 0.0;
         if (k < nk)
-            for (int c = 0; c < 2 * kAdjParts; ++c)
-                fold64(hi, lo, partial[((int64_t)c * kSums + k) * n_pad + (c < kAdjParts ? s : vp)]);
+            for (int c = 0; c < 2 * parts; ++c)
+                fold64(hi, lo, partial[((int64_t)c * nk + k) * n_pad + (c < parts ? s : vp)]);
         acc[k] = hi + lo;
     }
     double out[10];
@@ -620,7 +623,7 @@ __global__ void __launch_bounds__(128) k_adj_finish(const double *__restrict__ p
 
 }  // namespace
 
-AdjTreePlan adj_tree_plan(int64_t N, int nface, int64_t npix, int64_t n, int num_sms)
+AdjTreePlan adj_tree_plan(int64_t N, int nface, int64_t npix, int64_t n, int ngrad, int num_sms)
 {
     AdjTreePlan p{};
     p.map = tree_plan(ISW_F32C, N, nface, npix, n, num_sms);
@@ -645,13 +648,17 @@ AdjTreePlan adj_tree_plan(int64_t N, int nface, int64_t npix, int64_t n, int num
     }
     p.off_pix = take((size_t)p.map.ncl[0] * kPixPairs * sizeof(AdjPair));
     p.off_low = take((size_t)p.map.ncl[0] * kPixPairs * sizeof(AdjLow));
-    p.off_partial = take((size_t)2 * kAdjParts * kSums * p.n_pad * sizeof(double));
-    p.bytes = at;
     int nb = 0;
     cudaFuncSetAttribute((const void *)&k_adj_tree<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(AdjSmem));
     cudaFuncSetAttribute((const void *)&k_adj_tree<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(AdjSmem));
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void *)&k_adj_tree<true>, kTreeNT, sizeof(AdjSmem));
     p.slots = (nb > 0 ? nb : 1) * num_sms;
+    // as many shares as give every resident CTA 16 items: partial sums are 80 or 104 bytes per sample, pass and
+    // share, so with eight at any size 2e6 samples took 3.3 GB
+    const int64_t tiles = 2 * (p.n_pad / kTreeNT), want = 16 * (int64_t)p.slots;
+    p.parts = (int)std::min<int64_t>(kAdjParts, (want + tiles - 1) / tiles);
+    p.off_partial = take((size_t)2 * p.parts * adj_rows(ngrad >= 9) * p.n_pad * sizeof(double));
+    p.bytes = at;
     return p;
 }
 
@@ -715,15 +722,16 @@ cudaError_t launch_adjoint_tree(const AdjTreePlan &p, const AdjTreeCall &m, cuda
     a.ldn = m.ldn;
     a.outidx = m.outidx;
     a.n_pad = p.n_pad;
+    a.parts = p.parts;
     a.partial = (double *)(b + p.off_partial);
     a.b_min = m.b_min;
     a.st = m.st;
     a.queue = queue;
-    const int64_t items = 2 * (p.n_pad / kTreeNT) * kAdjParts;
+    const int64_t items = 2 * (p.n_pad / kTreeNT) * p.parts;
     const void *fn = m.ngrad >= 9 ? (const void *)&k_adj_tree<true> : (const void *)&k_adj_tree<false>;
     void *args[] = {(void *)&a};
     cudaLaunchKernel(fn, dim3((unsigned)(items < p.slots ? items : p.slots)), dim3(kTreeNT), args, sizeof(AdjSmem), s);
-    k_adj_finish<<<(unsigned)((m.n + 127) / 128), 128, 0, s>>>(a.partial, m.n, p.n_pad, inv, m.perm, m.s64, m.ngrad, m.grad,
+    k_adj_finish<<<(unsigned)((m.n + 127) / 128), 128, 0, s>>>(a.partial, p.parts, m.n, p.n_pad, inv, m.perm, m.s64, m.ngrad, m.grad,
                                                                m.ld_g);
     return cudaSuccess;
 }

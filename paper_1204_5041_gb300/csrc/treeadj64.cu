@@ -148,7 +148,7 @@ struct AdjTree64Args {
     int64_t ncl[kTreeLevels];
     const AdjPix64 *pix;
     int64_t n;
-    double *partial;   // [parts][13][n]
+    double *partial;   // [parts][adj_rows][n]
     float b_min, d_far;
     DevStatus *st;
     unsigned long long *queue;
@@ -393,12 +393,12 @@ __global__ void __launch_bounds__(kTreeNT, 3) k_adj_tree64(AdjTree64Args a)
         }
         double out = 0.0;
 #pragma unroll
-        for (int k = 0; k < (NG9 ? kSums : 10); ++k) {
+        for (int k = 0; k < adj_rows(NG9); ++k) {
             double v = acc[k];
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (lane == k) out = v;
         }
-        if (lane < (NG9 ? kSums : 10)) a.partial[((int64_t)part * kSums + lane) * a.n + s] = out;
+        if (lane < adj_rows(NG9)) a.partial[((int64_t)part * adj_rows(NG9) + lane) * a.n + s] = out;
     }
     for (int o = 16; o > 0; o >>= 1) zerocnt += __shfl_xor_sync(0xffffffffu, zerocnt, o);
     if (lane == 0 && zerocnt) atomicAdd(&a.st->zero_pairs, (unsigned long long)zerocnt);
@@ -412,12 +412,12 @@ __global__ void __launch_bounds__(128) k_adj_finish64(const double *__restrict__
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= n) return;
     double acc[kSums];
-    const int nk = ngrad >= 9 ? kSums : 10;
+    const int nk = adj_rows(ngrad >= 9);
 #pragma unroll
     for (int k = 0; k < kSums; ++k) {
         double hi = 0.0, lo = 0.0;
         if (k < nk)
-            for (int c = 0; c < parts; ++c) fold64(hi, lo, partial[((int64_t)c * kSums + k) * n + s]);
+            for (int c = 0; c < parts; ++c) fold64(hi, lo, partial[((int64_t)c * nk + k) * n + s]);
         acc[k] = hi + lo;
     }
     double out[10];
@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(128) k_adj_finish64(const double *__restrict__
 
 }  // namespace
 
-AdjTreePlan adj_tree_plan64(int64_t N, int nface, int64_t npix, int64_t n, int num_sms)
+AdjTreePlan adj_tree_plan64(int64_t N, int nface, int64_t npix, int64_t n, int ngrad, int num_sms)
 {
     AdjTreePlan p{};
     p.map = tree_plan(ISW_F64, N, nface, npix, n, num_sms);
@@ -455,7 +455,7 @@ AdjTreePlan adj_tree_plan64(int64_t N, int nface, int64_t npix, int64_t n, int n
         p.off_node[L] = take((size_t)p.map.ncl[L] * kNN64 * sizeof(double));
     }
     p.off_pix = take((size_t)p.map.ncl[0] * kPts * sizeof(AdjPix64));
-    p.off_partial = take((size_t)p.parts * kSums * n * sizeof(double));
+    p.off_partial = take((size_t)p.parts * adj_rows(ngrad >= 9) * n * sizeof(double));
     p.bytes = at;
     return p;
 }
