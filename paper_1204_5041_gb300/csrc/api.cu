@@ -734,10 +734,14 @@ int lightcone_adjoint(isw_ctx *c, int mode, const double *nodes_in, int64_t n, i
     double *contrib = nullptr;
     if (mode == ISW_BURDEN) {
         const size_t nl = (size_t)nloops;
-        const size_t terms = (size_t)n * 15 * sizeof(double);
-        if ((r = ensure_ws(c, kWsLoops, terms + nl * (2 * sizeof(int64_t) + sizeof(int)) + 16))) return r;
-        contrib = (double *)c->ws[kWsLoops];
-        first = (int64_t *)(contrib + (size_t)n * 15);
+        const size_t terms = (size_t)n * 15 * sizeof(double), bounds = nl * (2 * sizeof(int64_t) + sizeof(int)) + 16;
+        // without room for the samples' terms the loops' sums compute them again
+        r = ensure_ws(c, kWsLoops, terms + bounds);
+        const bool stored = r == ISW_OK;
+        if (r == ISW_ENOMEM) r = ensure_ws(c, kWsLoops, bounds);
+        if (r) return r;
+        contrib = stored ? (double *)c->ws[kWsLoops] : nullptr;
+        first = (int64_t *)c->ws[kWsLoops] + (stored ? (size_t)n * 15 : 0);
         last = first + nl;
         runs = (int *)(last + nl);
         cudaError_t e = cudaMemsetAsync(runs, 0, nl * sizeof(int), s);

@@ -69,7 +69,7 @@ void launch_lightcone_adjoint(int mode, const double *nodes, int64_t n, int64_t 
                               int64_t ldp, double t_box, double xo0, double xo1, double xo2, const double *tau,
                               const double *gs, int64_t ldgs, int ngs, double *gn, int64_t ldgn, double *gl,
                               int64_t ldgl, int *runs, int64_t *first, int64_t *last, double *contrib, DevStatus *st,
-                              cudaStream_t s);   // contrib: 15 n doubles (Burden mode)
+                              cudaStream_t s);   // contrib: 15 n doubles (Burden mode) or NULL
 
 // cone.cu: stacking with HEALPix cones
 void launch_vec2pix(int64_t N, const double *v, int64_t n, int64_t ld, int64_t *pix, DevStatus *st, cudaStream_t s);

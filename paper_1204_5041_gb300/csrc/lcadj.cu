@@ -191,7 +191,8 @@ __global__ void k_lcadj_nodes(int mode, const double *__restrict__ nodes, int64_
                 if (ok) out[1] = gsigma;
                 else atomicOr(&ds->bits, kStatDomain);
 #pragma unroll
-                for (int q = 0; q < 15; ++q) contrib[q * n + s] = ok ? term[q] : 0.0;
+                for (int q = 0; q < 15; ++q)
+                    if (contrib) contrib[q * n + s] = ok ? term[q] : 0.0;
                 if (s == 0 || loop_id(nodes, s - 1, nloops) != id) {
                     atomicAdd(&runs[id], 1);
                     first[id] = s;
@@ -206,9 +207,18 @@ __global__ void k_lcadj_nodes(int mode, const double *__restrict__ nodes, int64_
 
 // Loop-parameter gradients: one warp per loop, lanes stride over the loop's samples, fixed
 // butterfly reduction.  Rows: centre (3), rotation (9), L, m (0), n (0), psi, t0.
-__global__ void k_lcadj_loops(const double *__restrict__ contrib, int64_t n, int64_t nloops, const int *__restrict__ runs,
-                              const int64_t *__restrict__ first, const int64_t *__restrict__ last,
-                              double *__restrict__ gl, int64_t ldgl, DevStatus *ds)
+// The samples' inputs, for a call whose terms there was no room to store (15 doubles per sample): the warps
+// compute them again, the same sums in the same order.
+struct LcadjInputs {
+    const double *nodes, *P, *tau, *gs;
+    int64_t ld, ldp, ldgs;
+    int ngs;
+    double xo[3];
+};
+template <bool STORED>
+__global__ void k_lcadj_loops(const double *__restrict__ contrib, int64_t n, LcadjInputs in, int64_t nloops,
+                              const int *__restrict__ runs, const int64_t *__restrict__ first,
+                              const int64_t *__restrict__ last, double *__restrict__ gl, int64_t ldgl, DevStatus *ds)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -219,8 +229,17 @@ __global__ void k_lcadj_loops(const double *__restrict__ contrib, int64_t n, int
         for (int q = 0; q < 15; ++q) acc[q] = 0.0;
         if (nr == 1) {
             for (int64_t s = first[l] + lane; s < last[l]; s += 32) {
+                if (STORED) {
 #pragma unroll
-                for (int q = 0; q < 15; ++q) acc[q] += contrib[q * n + s];
+                    for (int q = 0; q < 15; ++q) acc[q] += contrib[q * n + s];
+                } else {
+                    double gX[3], gXd[3], gXp[3], gsig, gsigma, term[15];
+                    load_gs(in.gs, in.ldgs, in.ngs, s, gX, gXd, gXp, gsig);
+                    if (burden_sample(in.P, in.ldp, l, in.nodes[in.ld + s], in.tau[s], in.xo, gX, gXd, gXp, gsigma, term)) {
+#pragma unroll
+                        for (int q = 0; q < 15; ++q) acc[q] += term[q];
+                    }
+                }
             }
         }
 #pragma unroll
@@ -260,7 +279,9 @@ void launch_lightcone_adjoint(int mode, const double *nodes, int64_t n, int64_t 
     if (mode == ISW_BURDEN && nloops > 0) {
         int64_t b = (nloops + 3) / 4;   // 4 warps per block
         if (b > 152 * 16) b = 152 * 16;
-        k_lcadj_loops<<<(unsigned)b, 128, 0, s>>>(contrib, n, nloops, runs, first, last, gl, ldgl, st);
+        const LcadjInputs in{nodes, P, tau, gs, ld, ldp, ldgs, ngs, {xo0, xo1, xo2}};
+        if (contrib) k_lcadj_loops<true><<<(unsigned)b, 128, 0, s>>>(contrib, n, in, nloops, runs, first, last, gl, ldgl, st);
+        else k_lcadj_loops<false><<<(unsigned)b, 128, 0, s>>>(contrib, n, in, nloops, runs, first, last, gl, ldgl, st);
     }
 }
 

@@ -1,5 +1,5 @@
 """Calls whose cluster-tree workspace the device has no room for run the direct kernels, as they do by
-ISW_PARAM_WAIT_POLLS: the same bits.  The rest of the device's memory is held by one tensor meanwhile."""
+ISW_PARAM_WAIT_POLLS: the same bits.  The loop sums of lightcone_adjoint do without stored terms.  The rest of the device's memory is held by one tensor meanwhile."""
 import contextlib
 
 import numpy as np
@@ -57,5 +57,34 @@ def test_no_room_for_the_tree(isw, name):  # noqa: F811
         assert torch.equal(got, want)
         call()                             # with room
         assert ctx.timing()[2] != direct
+    finally:
+        ctx.close()
+
+
+def test_no_room_for_the_loop_terms(isw):  # noqa: F811
+    nloops, nodes = 900, 512
+    n = nloops * nodes
+    rng = np.random.default_rng(2)
+    P = rng.uniform(0.01, 0.1, (17, nloops))
+    P[0:3], P[3:12] = rng.normal(size=(3, nloops)), np.eye(3).ravel()[:, None]
+    P[13:15] = rng.integers(1, 6, (2, nloops))
+    X = np.zeros((10, n))
+    X[0], X[1] = np.repeat(np.arange(nloops), nodes), rng.uniform(0.0, 0.1, n)
+    P, X = torch.from_numpy(P).cuda(), torch.from_numpy(X).cuda()
+    gen = torch.Generator("cuda").manual_seed(1)
+    tau, gs = (torch.randn(s, dtype=torch.float64, device="cuda", generator=gen) for s in ((n,), (9, n)))
+    gn, gl = torch.empty(10, n, dtype=torch.float64, device="cuda"), torch.empty(17, nloops, dtype=torch.float64, device="cuda")
+    ctx = isw.Context()
+    try:
+        call = lambda: isw.lightcone_adjoint(isw.BURDEN, X, tau, gs, loop_params=P, out=gn, out_loops=gl, ctx=ctx)  # noqa: E731
+        call()
+        want = gn.clone(), gl.clone()
+        gl.zero_()
+        ctx.close()
+        ctx = isw.Context()
+        with _little_memory():
+            call()
+        assert torch.equal(gn, want[0]) and torch.equal(gl, want[1]) and gl.abs().sum() > 0
+        ctx.check_status()
     finally:
         ctx.close()
