@@ -215,10 +215,12 @@ struct FlatTreePlan {
     int nslots, pslots, pool, ppool;
     size_t off_queue, off_crit, off_caps, off_sup, off_rec, off_sort, off_work, off_pool, off_partial, off_A[kTreeLevels], bytes;
 };
-// from 3e7 pairs: its 20 launches take 0.1 ms, the direct kernel 3.5e7 pairs' time of FP32
-inline bool flat_tree_rule(int64_t M, int64_t n)
+// from 3e7 pairs: its 20 launches take 0.1 ms, the direct kernel 3.5e7 pairs' time of FP32; patches whose squared
+// distances leave the range of float go to the direct kernels (d >= pitch of a far sample, d < 1e18)
+inline bool flat_tree_rule(int64_t M, int64_t n, double width)
 {
-    return M >= 32 && (double)M * (double)M * (double)n >= 3e7 && n < (int64_t(1) << 30);
+    return M >= 32 && (double)M * (double)M * (double)n >= 3e7 && n < (int64_t(1) << 30) && width >= 1e-15 * (double)M &&
+           width <= 1e15;
 }
 FlatTreePlan flat_tree_plan(bool f64, int64_t M, int64_t n, int num_sms);
 cudaError_t launch_map_flat_tree(const FlatTreePlan &p, const void *r32, const void *r64, int64_t n, int64_t M, double width,
