@@ -23,6 +23,9 @@ namespace isw {
 namespace {
 
 constexpr float kFlatKappa = 3.5f;
+// Samples beyond this coordinate are placed at it for the decisions near or far (widths are at most 1e15): balls and
+// distances in float would be infinite from 1.8e19 on, and a tile with an infinite ball lost its other samples.
+constexpr double kFlatEdge = 1e18;
 constexpr int kSeriesTarget = 2048, kFlatPixTarget = 512;   // samples per chunk, at least
 template <bool F64>
 struct FlatNum {
@@ -84,8 +87,9 @@ __global__ void __launch_bounds__(256) k_flat_crit(const Flat32 *__restrict__ r3
             if (f64) s64[s] = g;
             else s32[s] = r32[src];
             if (g.w1 != 0.0 || g.w2 != 0.0) {
-                cr.a.x = (float)g.xs;
-                cr.a.y = (float)g.ys;
+                // a sample close to the patch plane is anywhere; its square is to stay finite
+                cr.a.x = (float)fmin(fmax(g.xs, -kFlatEdge), kFlatEdge);
+                cr.a.y = (float)fmin(fmax(g.ys, -kFlatEdge), kFlatEdge);
                 cr.b = make_float4(1e6f, 0.f, 0.f, 0.f);   // never near by beam
                 x[h] = cr.a;
             }
@@ -172,7 +176,12 @@ __global__ void __launch_bounds__(kTreeNT) k_flat_series(FlatTreeArgs a)
                     w2 = g.b.y;
                 }
                 const T inv = (T)1 / (dx * dx + dy * dy);
-                const T ux = dx * inv, uy = -dy * inv;                        // 1 / (z_s - z0)
+                T ux = dx * inv, uy = -dy * inv;                              // 1 / (z_s - z0)
+                if (inv < (T)(F64 ? 1e-300 : 1e-37)) {   // the square overflows; the weight grows like the distance
+                    const T sx = dx * (T)0x1p-66, sy = dy * (T)0x1p-66, si = (T)1 / (sx * sx + sy * sy);
+                    ux = sx * si * (T)0x1p-66;
+                    uy = -sy * si * (T)0x1p-66;
+                }
                 T tx = -(w1 * ux - w2 * uy), ty = -(w1 * uy + w2 * ux);       // -W u
                 const T vx = (T)R * ux, vy = (T)R * uy;
 #pragma unroll
