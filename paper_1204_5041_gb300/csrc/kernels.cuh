@@ -225,7 +225,7 @@ inline bool flat_tree_rule(int64_t M, int64_t n, double width)
 FlatTreePlan flat_tree_plan(bool f64, int64_t M, int64_t n, int num_sms);
 cudaError_t launch_map_flat_tree(const FlatTreePlan &p, const void *r32, const void *r64, int64_t n, int64_t M, double width,
                                  double *theta, int accumulate, void *scratch, cudaStream_t s);
-inline int flat_tree_launches(const FlatTreePlan &p) { return p.levels + 17; }
+inline int flat_tree_launches(const FlatTreePlan &p) { return p.levels + 16; }
 
 // treeadj.cu: FP32 adjoint over the cluster tree
 struct AdjTreePlan {
