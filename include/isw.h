@@ -96,9 +96,9 @@ int isw_check_status(isw_ctx *ctx, void *stream, int64_t *counts);
 /* Maps and adjoints with many pairs run over a cluster tree of the pixels: the samples far from a
  * cluster (by position and by beam) are summed at Chebyshev nodes and interpolated, the others pixel
  * by pixel, to the working precision of the call.  It is taken by default settings of
- * ISW_PARAM_SPLIT and ISW_PARAM_WAIT_POLLS (and, for FP32 maps, ISW_PARAM_VARIANT) from a number of
- * pairs that depends on the call; any other value of these keeps the direct kernels, which sum every
- * pair and which these three tunables describe.
+ * ISW_PARAM_SPLIT and ISW_PARAM_WAIT_POLLS (and, in FP32, of ISW_PARAM_D_FAR and, for maps,
+ * ISW_PARAM_VARIANT) from a number of pairs that depends on the call; any other value of these keeps
+ * the direct kernels, which sum every pair and which these tunables describe.
  *
  * Tunables: ISW_PARAM_NEAR_K (default 2): a pair is "near" when the chord |n - Xhat| is
  * below near_k * max(pixel size, angular length of the sample's segment); ISW_PARAM_B_MIN

@@ -204,11 +204,12 @@ void timing_end(isw_ctx *c, int k, cudaStream_t s)
 // A chunk count or a wait limit set by the caller asks for the direct kernels: the tree's have neither.
 bool default_kernels(const isw_ctx *c) { return c->split_override == 0 && c->wait_polls == kWaitPolls; }
 
-// Whether a map runs over the cluster tree (an FP32 variant set by the caller asks for the direct kernels, too).
+// Whether a map or adjoint runs over the cluster tree.  In FP32 a far-field distance set by the caller asks for the
+// direct kernels, too (the tree has no far-field form there), and for maps a variant.
 bool use_tree(const isw_ctx *c, TreeUse use, int64_t npix, int64_t n, int prec)
 {
-    return default_kernels(c) && (prec == ISW_F64 || c->tile_override < 0) && tree_rule(prec, use, npix, n) &&
-           npix < (int64_t(1) << 32);
+    return default_kernels(c) && (prec == ISW_F64 || (c->d_far == kDFar && (use == kTreeAdjoint || c->tile_override < 0))) &&
+           tree_rule(prec, use, npix, n) && npix < (int64_t(1) << 32);
 }
 
 // A tree call asks for its workspace before it launches anything.  Where the device has no room for it the direct
@@ -1070,7 +1071,7 @@ int isw_map_adjoint(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const
         return ISW_OK;
     }
     const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
-    if (default_kernels(c) && tree_rule(prec, kTreeAdjoint, npix, n) && npix < (int64_t(1) << 32)) {
+    if (use_tree(c, kTreeAdjoint, npix, n, prec)) {
         bool direct = false;
         r = adjoint_tree_impl(c, nside, pix0, npix, pix_list, samples, n, ld, xo, GU, prec, dL_dtheta, grad_out, ld_g, ngrad, s, direct);
         if (!direct) return r;

@@ -1,0 +1,28 @@
+"""Tunables and the cluster tree: those that the tree does not have ask for the direct kernels."""
+import pytest
+
+from test_gpu_tree import _samples, isw  # noqa: F401
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("kind", ["map", "adjoint"])
+@pytest.mark.parametrize("value", [0.1, 4.0])
+def test_far_field_distance(isw, kind, value):  # noqa: F811
+    """ISW_PARAM_D_FAR takes effect on FP32 calls of every size: the bits are those of the direct kernels."""
+    S = torch.from_numpy(_samples(9000, 3)).cuda()
+    g = torch.randn(12 * 64 * 64, dtype=torch.float64, device="cuda")
+    call = {"map": lambda: isw.isw_map(64, S, prec="f32c"), "adjoint": lambda: isw.isw_map_adjoint(64, S, g, prec="f32c")}[kind]
+    ctx = isw.default_context()
+    default, out = ctx.get_param(isw.PARAM_D_FAR), []
+    try:
+        for polls in (-1, 2**22 - 1):
+            ctx.set_param(isw.PARAM_D_FAR, value)
+            ctx.set_param(isw.PARAM_WAIT_POLLS, polls)
+            out.append(call())
+    finally:
+        ctx.set_param(isw.PARAM_D_FAR, default)
+        ctx.set_param(isw.PARAM_WAIT_POLLS, -1)
+    assert torch.equal(out[0], out[1])
+    assert not torch.equal(out[0], call())     # default settings: the tree
