@@ -371,6 +371,7 @@ int map_impl(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const int64_
     if (tune_waves == 0 && use_tree(c, use, npix, n, prec)) {
         bool direct = false;
         const int r = map_tree_impl(c, nside, pix0, npix, pix_list, patch, samples, n, ld, xo, GU, prec, accumulate, theta, s, direct);
+        if (!r && prec == ISW_F32C && !c->capturing) c->last_variant = -1;
         if (!direct) return r;
     }
     int vidx = 0;

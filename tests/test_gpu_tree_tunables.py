@@ -26,3 +26,20 @@ def test_far_field_distance(isw, kind, value):  # noqa: F811
         ctx.set_param(isw.PARAM_WAIT_POLLS, -1)
     assert torch.equal(out[0], out[1])
     assert not torch.equal(out[0], call())     # default settings: the tree
+
+
+def test_variant_of_the_last_map(isw):  # noqa: F811
+    S = torch.from_numpy(_samples(2000, 3)).cuda()
+    ctx = isw.Context()
+    try:
+        assert ctx.get_param(isw.PARAM_VARIANT) == -1
+        isw.isw_map(4, S, prec="f32c", ctx=ctx)            # 384,000 pairs: the direct kernels
+        assert ctx.get_param(isw.PARAM_VARIANT) == 0
+        isw.isw_map(64, S, prec="f32c", ctx=ctx)
+        assert ctx.get_param(isw.PARAM_VARIANT) == -1
+        isw.isw_map(64, S, prec="f64", ctx=ctx)
+        ctx.set_param(isw.PARAM_VARIANT, 1)
+        isw.isw_map(64, S, prec="f32c", ctx=ctx)
+        assert ctx.get_param(isw.PARAM_VARIANT) == 1
+    finally:
+        ctx.close()
