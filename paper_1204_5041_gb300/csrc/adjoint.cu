@@ -75,7 +75,10 @@ __global__ void k_pack_pixels(const double *__restrict__ nv, int64_t ldn, const 
             for (int c = 0; c < 3; ++c) d.n[c] = nv[c * ldn + k];
             d.g = g[oi];
         } else {
-            d.n[0] = d.n[1] = d.n[2] = 0.0;
+            // padding: zero weight half way from the centre, so that neither d (of a sample's unit vector or of a
+            // skipped sample's zero vector) nor B = 1 + n.Xdot is zero
+            d.n[0] = 0.5;
+            d.n[1] = d.n[2] = 0.0;
             d.g = 0.0;
         }
         float hi[3], lo[3];
