@@ -208,7 +208,8 @@ bool default_kernels(const isw_ctx *c) { return c->split_override == 0 && c->wai
 // direct kernels, too (the tree has no far-field form there), and for maps a variant.
 bool use_tree(const isw_ctx *c, TreeUse use, int64_t npix, int64_t n, int prec)
 {
-    return default_kernels(c) && (prec == ISW_F64 || (c->d_far == kDFar && (use == kTreeAdjoint || c->tile_override < 0))) &&
+    const bool adj = use == kTreeAdjointSky || use == kTreeAdjointList;
+    return default_kernels(c) && (prec == ISW_F64 || (c->d_far == kDFar && (adj || c->tile_override < 0))) &&
            tree_rule(prec, use, npix, n) && npix < (int64_t(1) << 32);
 }
 
@@ -1072,7 +1073,8 @@ int isw_map_adjoint(isw_ctx *c, int64_t nside, int64_t pix0, int64_t npix, const
         return ISW_OK;
     }
     const double xo[3] = {x_obs ? x_obs[0] : 0.0, x_obs ? x_obs[1] : 0.0, x_obs ? x_obs[2] : 0.0};
-    if (use_tree(c, kTreeAdjoint, npix, n, prec)) {
+    const bool sky = !pix_list && pix0 == 0 && npix == 12 * nside * nside;
+    if (use_tree(c, sky ? kTreeAdjointSky : kTreeAdjointList, npix, n, prec)) {
         bool direct = false;
         r = adjoint_tree_impl(c, nside, pix0, npix, pix_list, samples, n, ld, xo, GU, prec, dL_dtheta, grad_out, ld_g, ngrad, s, direct);
         if (!direct) return r;

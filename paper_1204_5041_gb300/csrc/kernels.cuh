@@ -155,20 +155,29 @@ constexpr int kTreeLevels = 20;
 //   FP32 full sky  1e6: N_side 16 with 500 0.69 / 0.29 and 0.29 / 0.21, N_side 64 with 500 0.78 / 0.38 and
 //                  0.21 / 0.22.  The direct kernel sums a string's near pairs lane by lane in FP64.
 //   FP32 patch     5e7: 128 x 128 with 5,000 0.91 / 0.36 with a string in it, 0.21 / 0.25 with none near
-//   FP32 list      3e8: 20,000 pixels and samples 0.79 / 0.71, a quarter of the pairs 0.37 / 0.43.
-//   FP32 adjoint   3e8, N_side 32: 12,288 pixels and 20,000 samples 0.64 / 0.64, N_side 53 with 10,000 0.92 / 0.81,
-//                  with 5,000 0.54 / 0.68.
-//   FP64 map       6e7: N_side 64 with 2,500 4.4 / 3.4 and 8.5 / 3.4, with 1,000 1.9 / 2.2 and 3.7 / 2.2; the
-//                  leaves have 32 x 32 pixels, so at least four faces of half that.
-//   FP64 adjoint   6e6, N_side 32: N_side 32 with 500 1.18 / 0.80, with 250 0.64 / 0.56; N_side 22 with 5,000 4.2 / 5.0.
+//   FP32 list      3e8: where the pixels lie is not known here.  A compact list of 5,000 with 60,000 samples 1.55 / 0.68,
+//                  pixels scattered over the sky 0.67 / 0.81; 20,000 with 15,000 1.23 / 0.53 and 0.57 / 0.63; from 50,000
+//                  scattered pixels on 1.1 to 2.2 times as fast.
+//   FP32 adjoint   8e8 (the latency of the deepest subtrees bounds small calls; 120 sky calls of loops at 6e8 to 8e8 were
+//                  0.8 to 1.5 times as fast, at 8e8 to 1e9 0.98 to 1.7, at 3e8 from 0.57 on); lists 2e9: 12,288
+//                  scattered pixels 4.97 / 4.64 and 4.96 / 5.16, 50,000 4.91 / 3.67, compact ones 4.48 / 2.54.
+//   FP64 map       9e7: sky calls of loops at 6e7 to 8e7 0.80 to 1.7 times as fast, from 9e7 on 1.01 and more; lists 0.76 to 1.9 at 6e7,
+//                  from 1.2e8 on 1.2 and more.  The leaves have 32 x 32 pixels, so at least four faces of half that.
+//   FP64 patch     6e7: 64 x 64 with 14,649 3.57 / 1.52 to 3.56 / 3.60 by width (0.05 to 0.5) and sample layout.
+//   FP64 adjoint   6e6, N_side 32: N_side 32 with 500 1.3 / 0.83; lists of 12,288 with 489 1.14 / 0.91.  Between N_side 32 and 45
+//                  a face's four leaves are less than half full: N_side 33 and 36 with 15,360 33 / 42, 40 37 / 42, 44 40 / 41, 45 44 / 41.
 // The list entries hold 30-bit record numbers.
-enum TreeUse : int { kTreeSky = 0, kTreePatch = 1, kTreePixelList = 2, kTreeAdjoint = 3 };
+enum TreeUse : int { kTreeSky = 0, kTreePatch = 1, kTreePixelList = 2, kTreeAdjointSky = 3, kTreeAdjointList = 4 };
 inline bool tree_rule(int prec, TreeUse use, int64_t npix, int64_t n)
 {
-    const bool f64 = prec == ISW_F64, adj = use == kTreeAdjoint;
+    const bool f64 = prec == ISW_F64, adj = use == kTreeAdjointSky || use == kTreeAdjointList;
     const int64_t pix = adj ? 12 * 1024 : f64 ? 4096 : 192;
-    const double pairs = adj ? (f64 ? 6e6 : 3e8) : f64 ? 6e7 : use == kTreeSky ? 1e6 : use == kTreePatch ? 5e7 : 3e8;
-    return npix >= pix && (double)npix * (double)n >= pairs && n < (int64_t(1) << 30);
+    double pairs;
+    if (adj) pairs = f64 ? 6e6 : use == kTreeAdjointSky ? 8e8 : 2e9;
+    else if (f64) pairs = use == kTreePatch ? 6e7 : 9e7;
+    else pairs = use == kTreeSky ? 1e6 : use == kTreePatch ? 5e7 : 3e8;
+    const bool sparse = f64 && use == kTreeAdjointSky && npix > 12 * 32 * 32 && npix < 12 * 45 * 45;   // leaves
+    return npix >= pix && (double)npix * (double)n >= pairs && n < (int64_t(1) << 30) && !sparse;
 }
 // slot order of the pixel tables: anti-diagonals (full sky), rows (patch), spatially sorted list
 enum : int { kSlotsDiag = 0, kSlotsRows = 1, kSlotsList = 2 };

@@ -26,7 +26,7 @@ LISTS64 = [(12288, 1), (49152, 1), (50176, 2), (50176, 2500), (1024, 49000)]
 def test_map_list_with_empty_leaves(isw, prec, tol, good, bad):  # noqa: F811
     """Indices out of range fill whole leaves, alone under their parent or next to leaves of valid pixels: the
     valid pixels keep their values, the others are reported and left alone."""
-    nside, pairs = 256, 3.01e8 if prec == "f32c" else 6.01e7
+    nside, pairs = 256, 3.01e8 if prec == "f32c" else 9.01e7
     S = torch.from_numpy(_samples(int(pairs / (good + bad)) + 1, 8)).cuda()
     pix, ok = _bad_list(nside, good, bad)
     ctx = isw.default_context()
@@ -42,7 +42,7 @@ def test_map_list_with_empty_leaves(isw, prec, tol, good, bad):  # noqa: F811
 
 @pytest.mark.parametrize("prec,tol,good,bad", [("f32c", 1e-6, *k) for k in LISTS32] + [("f64", 1e-12, *k) for k in LISTS64])
 def test_adjoint_list_with_empty_leaves(isw, prec, tol, good, bad):  # noqa: F811
-    nside, pairs = 256, 3.01e8 if prec == "f32c" else 6.1e6
+    nside, pairs = 256, 2.01e9 if prec == "f32c" else 6.1e6
     n = int(pairs / (good + bad)) + 1
     S = torch.from_numpy(_samples(n, 12)).cuda()
     pix, ok = _bad_list(nside, good, bad)
@@ -77,7 +77,7 @@ def _antipodes(isw, nside, count, seed):  # noqa: F811
                                             ("f64", TOL64, 4100)])
 def test_map_antipodal_pairs(isw, prec, tol, count):  # noqa: F811
     """Scattered pixels with their antipodes in few leaves; and the N_side 2 sky repeated."""
-    S = torch.from_numpy(_samples(int((3.001e8 if prec == "f32c" else 6.001e7) / count) + 1, 21)).cuda()
+    S = torch.from_numpy(_samples(int((3.001e8 if prec == "f32c" else 9.001e7) / count) + 1, 21)).cuda()
     sky2 = torch.arange(48, device="cuda").repeat(count // 48 + 1)[:count]
     for nside, pix in ((64, _antipodes(isw, 64, count, count)), (2, sky2)):
         got, ref = isw.isw_map(nside, S, pix=pix, prec=prec), _direct(isw, nside, S, pix=pix)
@@ -87,7 +87,7 @@ def test_map_antipodal_pairs(isw, prec, tol, count):  # noqa: F811
 
 @pytest.mark.parametrize("prec,tol,count", [("f32c", 1e-6, 12288), ("f64", 1e-12, 12288)])
 def test_adjoint_antipodal_pairs(isw, prec, tol, count):  # noqa: F811
-    S = torch.from_numpy(_samples(int((3.01e8 if prec == "f32c" else 6.1e6) / count) + 1, 22)).cuda()
+    S = torch.from_numpy(_samples(int((2.01e9 if prec == "f32c" else 6.1e6) / count) + 1, 22)).cuda()
     g = torch.randn(count, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
     for nside, pix in ((64, _antipodes(isw, 64, count, 2)), (2, torch.arange(48, device="cuda").repeat(count // 48))):
         got = _adjoint(isw, nside, S, g, prec, 9, pix=pix)

@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("value", [0.1, 4.0])
 def test_far_field_distance(isw, kind, value):  # noqa: F811
     """ISW_PARAM_D_FAR takes effect on FP32 calls of every size: the bits are those of the direct kernels."""
-    S = torch.from_numpy(_samples(9000, 3)).cuda()
+    S = torch.from_numpy(_samples(17000, 3)).cuda()
     g = torch.randn(12 * 64 * 64, dtype=torch.float64, device="cuda")
     call = {"map": lambda: isw.isw_map(64, S, prec="f32c"), "adjoint": lambda: isw.isw_map_adjoint(64, S, g, prec="f32c")}[kind]
     ctx = isw.default_context()
