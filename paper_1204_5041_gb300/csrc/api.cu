@@ -948,7 +948,7 @@ int isw_map_patch(isw_ctx *c, const double *frame, int64_t M, double width, cons
         return ISW_OK;
     }
     const bool f64 = prec == ISW_F64;
-    if (default_kernels(c) && flat_tree_rule(M, n, width)) {
+    if (default_kernels(c) && flat_tree_rule(f64, M, n, width)) {
         const FlatTreePlan tp = flat_tree_plan(f64, M, n, c->num_sms);
         r = ensure_ws(c, kWsFlat, (size_t)tp.n_pad * flat_record_bytes());
         if (!r) r = ensure_ws(c, kWsTree, tp.bytes);

@@ -224,11 +224,17 @@ struct FlatTreePlan {
     int nslots, pslots, pool, ppool;
     size_t off_queue, off_crit, off_caps, off_sup, off_rec, off_sort, off_work, off_pool, off_partial, off_A[kTreeLevels], bytes;
 };
-// from 3e7 pairs: its 20 launches take 0.1 ms, the direct kernel 3.5e7 pairs' time of FP32; patches whose squared
-// distances leave the range of float go to the direct kernels (d >= pitch of a far sample, d < 1e18)
-inline bool flat_tree_rule(int64_t M, int64_t n, double width)
+// Whether a flat-sky patch runs over the tree (2,600 drawn patches of 32 to 1,176 pixels a side, 100 to 182,000 samples):
+//   FP32  9e8 pairs, where the direct kernel's 3e11 to 4e11 pairs a second meet the 0.35 to 2 ms that the tree's 20
+//         launches and its near samples take: at 9e8 to 1e9 0.9 to 1.5 times as fast, at 2e9 1.6 to 2.9 times;
+//         at 1e8 0.3 to 0.8 times
+//   FP64  3e7 from 192 pixels a side (1.4 to 4 times as fast), 5e7 below (median 1.6 to 4.5, down to 0.4 where the
+//         whole patch lies on a string)
+// Patches whose squared distances leave the range of float go to the direct kernels (d >= pitch of a far sample, d < 1e18).
+inline bool flat_tree_rule(bool f64, int64_t M, int64_t n, double width)
 {
-    return M >= 32 && (double)M * (double)M * (double)n >= 3e7 && n < (int64_t(1) << 30) && width >= 1e-15 * (double)M &&
+    const double pairs = (double)M * (double)M * (double)n;
+    return M >= 32 && pairs >= (!f64 ? 9e8 : M >= 192 ? 3e7 : 5e7) && n < (int64_t(1) << 30) && width >= 1e-15 * (double)M &&
            width <= 1e15;
 }
 FlatTreePlan flat_tree_plan(bool f64, int64_t M, int64_t n, int num_sms);

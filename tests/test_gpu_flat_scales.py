@@ -29,8 +29,8 @@ def _field(n):
 @pytest.mark.parametrize("prec,tol,own", [("f32c", TOL32, 1e-6), ("f64", TOL64, 1e-13)])
 @pytest.mark.parametrize("z", [1e-17, 1e-21, 1e-25, 1e-32])
 def test_samples_next_to_the_plane(isw, z, prec, tol, own):  # noqa: F811
-    S = _field(8200)
-    S[2, ::410] = z
+    S = _field(221400)
+    S[2, ::11070] = z
     Sd = torch.from_numpy(S).cuda()
     args = (np.eye(3), 64, 0.3, Sd)
     got = isw.isw_map_patch(*args, prec=prec, approx=isw.FLATSKY)
@@ -42,7 +42,7 @@ def test_samples_next_to_the_plane(isw, z, prec, tol, own):  # noqa: F811
 @pytest.mark.parametrize("prec", ["f32c", "f64"])
 @pytest.mark.parametrize("width", [1e-50, 1e-40, 1e-25, 1e18, 1e30])
 def test_extreme_widths(isw, width, prec):  # noqa: F811
-    Sd = torch.from_numpy(_field(8200)).cuda()
+    Sd = torch.from_numpy(_field(221400)).cuda()
     ctx = isw.default_context()
     ctx.timing()
     got = isw.isw_map_patch(np.eye(3), 64, width, Sd, prec=prec, approx=isw.FLATSKY)

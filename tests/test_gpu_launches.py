@@ -39,7 +39,7 @@ CALLS = ["sky32", "sky64", "list32", "list64", "range32", "patch32", "patch64", 
 @pytest.mark.parametrize("name", CALLS)
 def test_launch_counts(isw, name, direct):  # noqa: F811
     kind, prec = name.split("_")[0].rstrip("0123456789"), "f64" if "64" in name else "f32c"
-    nside, n = 64, 160000
+    nside, n = 64, 230000
     S = torch.from_numpy(_samples(n, 3)).cuda()
     pix = torch.randint(12 * nside * nside, (12800,), device="cuda")
     M = 512 if "512" in name else 64

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import test_gpu_tree as tree
-from test_gpu_tree import TOL64, _adjoint, _check, _samples, isw  # noqa: F401
+from test_gpu_tree import TOL32, TOL64, _adjoint, _check, _samples, isw  # noqa: F401
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -13,7 +13,8 @@ SKY32 = [(4, 5209), (9, 1100), (16, 331), (32, 8139), (49, 4097), (100, 1000), (
 SKY64 = [(20, 18755), (33, 6913), (64, 1857), (65, 1823), (96, 833), (100, 769), (257, 127)]
 RINGS64 = [80, 95, 96, 97, 128, 130]
 PATCH = [("f32c", 111, 8200), ("f32c", 160, 4000), ("f64", 222, 1300), ("f64", 256, 1000)]
-FLAT = [(33, 30000), (64, 8191), (100, 3001), (512, 129), (543, 1000)]
+FLAT = [("f32c", TOL32, 33, 0.1, 826500), ("f32c", TOL32, 64, 0.3, 219800), ("f32c", TOL32, 100, 0.05, 90001), ("f32c", TOL32, 512, 0.13, 3457),
+        ("f32c", TOL32, 543, 0.2, 3073), ("f64", TOL64, 33, 0.1, 45953), ("f64", TOL64, 64, 0.3, 12225), ("f64", TOL64, 100, 0.05, 5001)]
 ADJOINT32 = [(32, 65201, 6, {}), (33, 61313, 10, {}), (47, 30209, 9, dict(spot=0.05, mixed=True)), (64, 16321, 6, dict(spot=1e-3)),
              (100, 6703, 10, {}), (257, 1023, 6, {})]
 ADJOINT64 = [(32, 501, 6, {}), (45, 263, 9, {}), (64, 407, 6, {}), (65, 448, 10, {}), (257, 63, 9, {})]
@@ -32,6 +33,11 @@ def test_rings_f64(isw, nside):  # noqa: F811
 @pytest.mark.parametrize("npix,n", [(49153, 1900), (4097, 22001)])
 def test_lists_and_ranges_f64(isw, npix, n):  # noqa: F811
     tree.test_tree_lists_and_ranges(isw, "f64", TOL64, npix, n)
+
+
+@pytest.mark.parametrize("prec,tol,M,width,n", FLAT)
+def test_flat(isw, prec, tol, M, width, n):  # noqa: F811
+    tree.test_flat_tree(isw, M=M, width=width, n=n, prec=prec, tol=tol)
 
 
 @pytest.mark.parametrize("nside,n,ngrad,kw", ADJOINT32)
@@ -59,11 +65,11 @@ def test_adjoint_lists(isw, prec, tol, nside, npix, n):  # noqa: F811
 
 TAKEN = ([("sky", "f32c", *k, None) for k in SKY32] + [("sky", "f64", *k, None) for k in SKY64 + [(k, 1300) for k in RINGS64] + [(64, 4001), (64, 4500)]]
          + [("list", "f32c", 256, 24600, 12289), ("list", "f64", 256, 1900, 49153), ("list", "f64", 256, 22001, 4097)]
-         + [("patch", *k, None) for k in PATCH] + [("flat", p, *k, 0.1) for p in ("f32c", "f64") for k in FLAT]
+         + [("patch", *k, None) for k in PATCH] + [("flat", p, M, n, w) for p, _, M, w, n in FLAT] + [("flat", "f64", 512, 129, 0.1), ("flat", "f64", 543, 1000, 0.1)]
          + [("adjoint", "f32c", *k[:2], None) for k in ADJOINT32] + [("adjoint", "f64", *k[:2], None) for k in ADJOINT64]
          + [("adjoint", "f32c", 256, 163000, 12301), ("adjoint", "f64", 256, 501, 12301)])
 DIRECT = [("sky", "f32c", 4, 5208, None), ("sky", "f64", 64, 1831, None), ("sky", "f64", 18, 40000, None), ("list", "f32c", 256, 24000, 12289),
-          ("list", "f64", 256, 1800, 49153), ("patch", "f64", 222, 1200, None), ("adjoint", "f32c", 64, 16200, None),
+          ("list", "f64", 256, 1800, 49153), ("flat", "f32c", 64, 219000, 0.1), ("flat", "f64", 100, 4990, 0.1), ("patch", "f64", 222, 1200, None), ("adjoint", "f32c", 64, 16200, None),
           ("adjoint", "f64", 44, 9000, None), ("adjoint", "f64", 33, 9000, None), ("adjoint", "f32c", 256, 160000, 12301)]
 
 
