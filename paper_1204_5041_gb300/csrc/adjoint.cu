@@ -75,9 +75,10 @@ __global__ void k_pack_pixels(const double *__restrict__ nv, int64_t ldn, const 
             for (int c = 0; c < 3; ++c) d.n[c] = nv[c * ldn + k];
             d.g = g[oi];
         } else {
-            // padding: zero weight half way from the centre, so that neither d (of a sample's unit vector or of a
-            // skipped sample's zero vector) nor B = 1 + n.Xdot is zero
-            d.n[0] = 0.5;
+            // padding: zero weight, next to the centre, so that it is a unit vector's length away from a sample's direction
+            // (a near pair of padding would go through FP64), and not at the zero vector of a skipped sample, where d
+            // and with it the term's denominator vanish
+            d.n[0] = 0x1p-10;
             d.n[1] = d.n[2] = 0.0;
             d.g = 0.0;
         }
