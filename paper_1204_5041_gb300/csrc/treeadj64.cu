@@ -180,7 +180,8 @@ __global__ void __launch_bounds__(kTreeNT, 3) k_adj_tree64(AdjTree64Args a)
     const int lane = threadIdx.x & 31;
     const int top = a.levels - 1;
     const int64_t n_items = a.n * a.parts;
-    const double d_far2 = (double)a.d_far * (double)a.d_far, b_min = (double)a.b_min;
+    // a pixel's far form takes d from the rounded direction, and a pixel on the line of sight has none: not below 1/16
+    const double d_far = fmax((double)a.d_far, 0.0625), d_far2 = d_far * d_far, b_min = (double)a.b_min;
     unsigned zerocnt = 0;
     for (;;) {
         unsigned long long item = 0;

@@ -43,3 +43,31 @@ def test_variant_of_the_last_map(isw):  # noqa: F811
         assert ctx.get_param(isw.PARAM_VARIANT) == 1
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("value", [0.0, 1e-3, 1.0])
+def test_far_field_distance_of_the_f64_adjoint(isw, value):  # noqa: F811
+    """Samples on and next to the pixels' lines of sight keep their gradients at any ISW_PARAM_D_FAR."""
+    nside = 64
+    S = _samples(3000, 3)
+    centre = isw.hp_pix2vec_ring(nside).cpu().numpy()
+    S[0:3, :300] = 0.5 * centre[:, 1000:1300]
+    S[0:3, 300:600] = 0.5 * centre[:, 2000:2300] + 1e-9
+    S = torch.from_numpy(S).cuda()
+    g = torch.randn(12 * nside * nside, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    ctx = isw.default_context()
+    default, out = ctx.get_param(isw.PARAM_D_FAR), {}
+    try:
+        for polls in (-1, 2**22 - 1):
+            ctx.set_param(isw.PARAM_D_FAR, value)
+            ctx.set_param(isw.PARAM_WAIT_POLLS, polls)
+            out[polls] = isw.isw_map_adjoint(nside, S, g, prec="f64", ngrad=9)
+    finally:
+        ctx.set_param(isw.PARAM_D_FAR, default)
+        ctx.set_param(isw.PARAM_WAIT_POLLS, -1)
+    got, ref = out.values()
+    for a in (0, 3, 6):
+        # relative to each sample's own gradient: those on a line of sight are 1e12 times the others
+        scale = ref[a : a + 3].norm(dim=0) + ref[a : a + 3].norm(dim=0).median()
+        assert (((got - ref)[a : a + 3].norm(dim=0)) / scale).max().item() <= 1e-11
+    ctx.check_status()
