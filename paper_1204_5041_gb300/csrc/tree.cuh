@@ -169,14 +169,6 @@ __device__ __forceinline__ bool tree_tile_beam(const TreeCap &t, const float4 &c
     return t.a.w >= 0.f && 2.f * b < c.w * c.w + 1e-5f;
 }
 
-__device__ __forceinline__ void cp_async16(void *dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 struct TreeScanSmem {
     uint32_t list[kTreeList];
     uint32_t cand[kTreeGroup * kTreeSuper];   // candidate tiles

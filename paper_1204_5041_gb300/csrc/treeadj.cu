@@ -469,10 +469,10 @@ __global__ void __launch_bounds__(kTreeNT) k_adj_tree(AdjTreeArgs a)
                 int qlen = 0;
 #pragma unroll 1
                 for (int p0 = 0; p0 < kPixPairs; p0 += 32) {
-                    // gq, ga, gT, -, v n0-weight, ge d (3), gq d + v m (3), gbQd n0-weight, gbA d + gbQd m (3)
-                    uint64_t p[15];
+                    // gq, ga, gT, v n0-weight, ge d (3), gq d + v m (3), gbQd n0-weight, gbA d + gbQd m (3)
+                    uint64_t p[14];
 #pragma unroll
-                    for (int k = 0; k < 15; ++k) p[k] = 0ull;
+                    for (int k = 0; k < 14; ++k) p[k] = 0ull;
 #pragma unroll 1
                     for (int i = p0; i < p0 + 32; ++i) {
                         const ulonglong2 ta = *reinterpret_cast<const ulonglong2 *>(&sm.tgt[i].a),
@@ -504,19 +504,19 @@ __global__ void __launch_bounds__(kTreeNT) k_adj_tree(AdjTreeArgs a)
                         p[0] = f2_add(p[0], gq);
                         p[1] = f2_add(p[1], ga);
                         p[2] = f2_add(p[2], gT);
-                        p[4] = f2_add(p[4], vn);
-                        p[5] = f2_fma(ge, dx, p[5]);
-                        p[6] = f2_fma(ge, dy, p[6]);
-                        p[7] = f2_fma(ge, dz, p[7]);
-                        p[8] = f2_fma(gq, dx, f2_fma(f2_neg(vn), mx, p[8]));
-                        p[9] = f2_fma(gq, dy, f2_fma(f2_neg(vn), my, p[9]));
-                        p[10] = f2_fma(gq, dz, f2_fma(f2_neg(vn), mz, p[10]));
+                        p[3] = f2_add(p[3], vn);
+                        p[4] = f2_fma(ge, dx, p[4]);
+                        p[5] = f2_fma(ge, dy, p[5]);
+                        p[6] = f2_fma(ge, dz, p[6]);
+                        p[7] = f2_fma(gq, dx, f2_fma(f2_neg(vn), mx, p[7]));
+                        p[8] = f2_fma(gq, dy, f2_fma(f2_neg(vn), my, p[8]));
+                        p[9] = f2_fma(gq, dz, f2_fma(f2_neg(vn), mz, p[9]));
                         if (NG9) {
                             const uint64_t bqn = f2_mul(gq, t1n);   // -g Qd/(BQ)
-                            p[11] = f2_add(p[11], bqn);
-                            p[12] = f2_fma(ga, dx, f2_fma(f2_neg(bqn), mx, p[12]));
-                            p[13] = f2_fma(ga, dy, f2_fma(f2_neg(bqn), my, p[13]));
-                            p[14] = f2_fma(ga, dz, f2_fma(f2_neg(bqn), mz, p[14]));
+                            p[10] = f2_add(p[10], bqn);
+                            p[11] = f2_fma(ga, dx, f2_fma(f2_neg(bqn), mx, p[11]));
+                            p[12] = f2_fma(ga, dy, f2_fma(f2_neg(bqn), my, p[12]));
+                            p[13] = f2_fma(ga, dz, f2_fma(f2_neg(bqn), mz, p[13]));
                         }
                         if (__any_sync(0xffffffffu, leaf && (n0 || n1))) {
                             const unsigned below = (1u << lane) - 1u;
@@ -549,9 +549,9 @@ __global__ void __launch_bounds__(kTreeNT) k_adj_tree(AdjTreeArgs a)
                         }
                     }
                     if (leaf) {
-                        float v[15];
+                        float v[14];
 #pragma unroll
-                        for (int k = 0; k < 15; ++k) {
+                        for (int k = 0; k < 14; ++k) {
                             float lo, hi;
                             f2_unpack(p[k], lo, hi);
                             v[k] = lo + hi;
@@ -562,9 +562,9 @@ __global__ void __launch_bounds__(kTreeNT) k_adj_tree(AdjTreeArgs a)
                         fold(ahi[3], alo[3], v[2]);
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
-                            fold(ahi[4 + c], alo[4 + c], 2.f * v[5 + c]);
-                            fold(ahi[7 + c], alo[7 + c], fmaf(-v[4], comp(sm.geo.c, c), v[8 + c]));
-                            if (NG9) fold(ahi[10 + c], alo[10 + c], fmaf(-v[11], comp(sm.geo.c, c), v[12 + c]));
+                            fold(ahi[4 + c], alo[4 + c], 2.f * v[4 + c]);
+                            fold(ahi[7 + c], alo[7 + c], fmaf(-v[3], comp(sm.geo.c, c), v[7 + c]));
+                            if (NG9) fold(ahi[10 + c], alo[10 + c], fmaf(-v[10], comp(sm.geo.c, c), v[11 + c]));
                         }
                     }
                 }
