@@ -98,11 +98,13 @@ int isw_check_status(isw_ctx *ctx, void *stream, int64_t *counts);
  * by pixel, to the working precision of the call.  It is taken by default settings of
  * ISW_PARAM_SPLIT and ISW_PARAM_WAIT_POLLS (and, in FP32, of ISW_PARAM_D_FAR and, for maps,
  * ISW_PARAM_VARIANT) from a number of pairs that depends on the call; any other value of these keeps
- * the direct kernels, which sum every pair and which these tunables describe.
+ * the direct kernels, which sum every pair and which these tunables describe.  A call whose tree does
+ * not fit the device's free memory runs the direct kernels, too.
  *
  * Tunables: ISW_PARAM_NEAR_K (default 2): a pair is "near" when the chord |n - Xhat| is
- * below near_k * max(pixel size, angular length of the sample's segment); ISW_PARAM_B_MIN
- * (default 0.01): a pair with 1 + n.Xdot below b_min is evaluated in FP64 by the FP32 path;
+ * below near_k * max(pixel size, angular length of the sample's segment), and at its pixel in FP64
+ * in the FP32 path; ISW_PARAM_B_MIN (default 0.01): at its pixel a pair with 1 + n.Xdot below b_min
+ * is evaluated with a form of 1 + n.Xdot that does not cancel, below b_min / 1000 in FP64;
  * ISW_PARAM_SPLIT: number of segment chunks of the forward maps (0 = automatic: enough
  * (pixel tile, chunk) work items to fill every resident CTA in near-equal waves and at least 64
  * per resident CTA, while each chunk keeps 256 segment tiles; chunk partials cost 8 bytes per
@@ -266,8 +268,8 @@ int isw_map_patch(isw_ctx *ctx, const double *frame, int64_t M, double width, co
  *   alm   : device double[2][lmax+1][lmax+1] (real plane, then imaginary; entry [m][l], zero for
  *           l < m) or NULL (kept in the context's workspace)
  *   cl    : device double[lmax+1]
- * Per-ring Fourier sums cost N_pix (lmax + 1) complex products (no FFT); the sums over rings
- * have a fixed order (deterministic). */
+ * The rings' Fourier sums are FFTs in shared memory (any ring length), the sums over rings cost four
+ * FP64 operations per ring pair, l and m and have a fixed order (deterministic). */
 int isw_map_cl(isw_ctx *ctx, int64_t nside, const double *theta, int64_t lmax, double *alm, double *cl,
                void *stream);
 
@@ -276,7 +278,9 @@ int isw_map_cl(isw_ctx *ctx, int64_t nside, const double *theta, int64_t lmax, d
  * selection), writes grad_out = device double[ngrad][ld_g] with rows dL/dX (3), dL/dXdot (3),
  * then dL/dX' (3) when ngrad >= 9 and dL/ddsigma when ngrad = 10 (ngrad is 6, 9 or 10), for
  * every sample.  Pair terms are recomputed, not stored; the reduction over pixels has a fixed
- * order (deterministic).  A skipped sample (|Xdot| >= 1) gets zero rows. */
+ * order (deterministic).  A skipped sample (|Xdot| >= 1) gets zero rows.  The workspace of partial sums
+ * takes 160 to 1664 bytes per sample in FP32 over the cluster tree (1664 up to 66,000 samples), 80 to 832
+ * in FP64. */
 int isw_map_adjoint(isw_ctx *ctx, int64_t nside, int64_t pix0, int64_t npix, const int64_t *pix_list,
                     const double *samples, int64_t n, int64_t ld, const double *x_obs, double GU, int prec,
                     const double *dL_dtheta, double *grad_out, int64_t ld_g, int ngrad, void *stream);

@@ -2,10 +2,10 @@
 // w.d / |d|^2 = Re[ W / (z - z_s) ], W = w1 + i w2: analytic away from the sample, so the samples far from
 // a cluster (centre z0, half-diagonal R, |z_s - z0| >= kappa R) act on it as one Taylor series
 //   sum_s W_s / (z - z_s) = sum_k a_k ((z - z0) / R)^k,   a_k = -sum_s (W_s u_s) (R u_s)^k,  u_s = 1 / (z_s - z0),
-// with an error kappa^-K of their terms after K of them: kappa = 3 with K = 16 in FP32 (2e-8, for
-// samples at the near radius and the cluster's corners) and K = 36 in FP64 (7e-18).  A sample goes to
+// with an error kappa^-K of their terms after K of them: kappa = 3.5 with K = 16 in FP32 (2e-9, for
+// samples at the near radius and the cluster's corners) and K = 32 in FP64 (4e-18).  A sample goes to
 // the first level, from the whole patch down, at which it is far, and to the pixels of the leaves
-// (16 x 16) to which it is near at every level.  A sample costs 6 K operations per cluster; the
+// (32 x 32, 16 x 16 below 512 pixels a side) to which it is near at every level.  A sample costs 6 K operations per cluster; the
 // selection of samples and the planning of chunks are those of tree.cuh, with positions in the plane and
 // no beams.
 //   k_flat_keys    spatial order of the samples
