@@ -95,3 +95,22 @@ def test_adjoint_antipodal_pairs(isw, prec, tol, count):  # noqa: F811
         for a in (0, 3, 6):
             assert ((got - ref)[a : a + 3].abs().max() / ref[a : a + 3].abs().max()).item() <= tol
     assert isw.default_context().check_status()[0] == isw.OK
+
+
+@pytest.mark.parametrize("prec,tol,tola", [("f32c", TOL32, 1e-6), ("f64", TOL64, 1e-12)])
+@pytest.mark.parametrize("one", [6200, 12200])
+def test_two_opposite_points(isw, prec, tol, tola, one):  # noqa: F811
+    """A list of two opposite pixels, over and over: compact leaves but for the one that holds both."""
+    nside, count = 64, 12400
+    a = torch.tensor([20011], device="cuda")
+    b = isw.hp_vec2pix_ring(nside, -isw.hp_pix2vec_ring(nside, pix=a))
+    pix = torch.cat([a.expand(one), b.expand(count - one)])[torch.randperm(count, device="cuda", generator=torch.Generator("cuda").manual_seed(1))]
+    S = torch.from_numpy(_samples(int((2.01e9 if prec == "f32c" else 9.1e7) / count) + 1, 23)).cuda()
+    got, ref = isw.isw_map(nside, S, pix=pix, prec=prec), _direct(isw, nside, S, pix=pix)
+    assert ((got - ref).abs().max() / ref.square().mean().sqrt()).item() <= tol
+    g = torch.randn(count, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    got = _adjoint(isw, nside, S, g, prec, 9, pix=pix)
+    ref = _adjoint(isw, nside, S, g, "f64", 9, split=1, pix=pix)
+    for k in (0, 3, 6):
+        assert ((got - ref)[k : k + 3].abs().max() / ref[k : k + 3].abs().max()).item() <= tola
+    assert isw.default_context().check_status()[0] == isw.OK
